@@ -9,7 +9,6 @@
 
 #include "moe_internal.h"
 
-#include <atomic>
 #include <chrono>
 
 namespace moe {
@@ -115,6 +114,11 @@ int32_t moe_create(int32_t device, moe_handle **out)
         delete h;
         return MOE_ERR_CUDA;
     }
+    e = routing_prepare(&h->routing_max_cluster);
+    if (e != cudaSuccess) {
+        delete h;
+        return MOE_ERR_CUDA;
+    }
     cudaEvent_t ev = nullptr;
     e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -124,12 +128,13 @@ int32_t moe_create(int32_t device, moe_handle **out)
     h->counts_event = ev;
     // the count mailbox: a few KB of pinned host memory that the GPU addresses directly.  Without it (the
     // allocation or the mapping refused) the whole-step calls copy the counts and synchronise instead.
+    constexpr size_t kMailBytes = (size_t)kMailWords * sizeof(unsigned long long);
     void *mail = nullptr, *mail_dev = nullptr;
-    if (cudaHostAlloc(&mail, (size_t)kMailInts * sizeof(int32_t), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
-        memset(mail, 0, (size_t)kMailInts * sizeof(int32_t));
+    if (cudaHostAlloc(&mail, kMailBytes, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
+        memset(mail, 0, kMailBytes);
         if (cudaHostGetDevicePointer(&mail_dev, mail, 0) == cudaSuccess && mail_dev) {
-            h->mail_host = static_cast<int32_t *>(mail);
-            h->mail_dev = static_cast<int32_t *>(mail_dev);
+            h->mail_host = static_cast<unsigned long long *>(mail);
+            h->mail_dev = static_cast<unsigned long long *>(mail_dev);
         } else {
             cudaFreeHost(mail);
         }
@@ -339,7 +344,7 @@ int32_t moe_build_routing(moe_handle *h, const int32_t *topk_idx, const moe_shap
     if (r->max_mtiles < max_mtiles_of(s, tile_m)) return MOE_ERR_SHAPE;
     if (const int32_t rc = require_handle_device(h, "moe_build_routing")) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, status_dev, nullptr, 0u, st);
+    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev, nullptr, 0u, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "routing launch");
     if (tile_counts_host) {
         e = cudaMemcpyAsync(tile_counts_host, r->tiles, (size_t)(s->E_tot + 1) * 4, cudaMemcpyDeviceToHost, st);
@@ -368,7 +373,7 @@ int32_t build_routing_mailed(moe_handle *h, const int32_t *topk_idx, const moe_s
     if (r->max_mtiles < max_mtiles_of(s, tile_m)) return MOE_ERR_SHAPE;
     if (const int32_t rc = require_handle_device(h, "moe_build_routing")) return rc;
     if (++h->mail_seq == 0u) h->mail_seq = 1u;
-    const cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, status_dev, h->mail_dev, h->mail_seq, st);
+    const cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev, h->mail_dev, h->mail_seq, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "routing launch");
     *seq = h->mail_seq;
     return MOE_OK;
@@ -382,31 +387,34 @@ int32_t wait_counts(moe_handle *h, uint32_t seq, int32_t E_tot, int32_t *tile_co
         const cudaError_t e = fallback_event ? cudaEventSynchronize(fallback_event) : cudaStreamSynchronize(st);
         return e == cudaSuccess ? MOE_OK : cuda_fail(h, e, "tile counts wait");
     }
-    volatile uint32_t *word = reinterpret_cast<volatile uint32_t *>(h->mail_host);
+    const volatile unsigned long long *words = h->mail_host;
     const auto t0 = std::chrono::steady_clock::now();
     uint32_t spins = 0;
-    while (*word != seq) {
-        if ((++spins & 2047u) == 0u) {
-            // the kernels finished or failed without the word arriving?
-            const cudaError_t q = cudaStreamQuery(st);
-            if (q != cudaErrorNotReady) {
-                if (*word == seq) break;
-                if (q != cudaSuccess) return cuda_fail(h, q, "routing build");
-                snprintf(h->err, sizeof h->err, "the routing build finished without delivering the tile counts");
-                return MOE_ERR_CUDA;
+    bool finished = false;
+    for (int32_t x = 0; x <= E_tot; ++x) {
+        unsigned long long v;
+        while ((uint32_t)((v = words[x]) >> 32) != seq) {
+            if ((++spins & 2047u) == 0u) {
+                // the kernels finished or failed without the word arriving?
+                if (finished) {
+                    snprintf(h->err, sizeof h->err, "the routing build finished without delivering the tile counts");
+                    return MOE_ERR_CUDA;
+                }
+                const cudaError_t q = cudaStreamQuery(st);
+                if (q == cudaSuccess) finished = true;      // one more look at the words
+                else if (q != cudaErrorNotReady) return cuda_fail(h, q, "routing build");
+                const double waited = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+                if (waited > 2.0 + 2e-9 * (double)h->wait_ns) {
+                    snprintf(h->err, sizeof h->err, "no tile counts from the routing build after %.1f s", waited);
+                    return MOE_ERR_CUDA;
+                }
             }
-            const double waited = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-            if (waited > 2.0 + 2e-9 * (double)h->wait_ns) {
-                snprintf(h->err, sizeof h->err, "no tile counts from the routing build after %.1f s", waited);
-                return MOE_ERR_CUDA;
-            }
-        }
 #if defined(__x86_64__) || defined(__i386__)
-        __builtin_ia32_pause();
+            __builtin_ia32_pause();
 #endif
+        }
+        tile_counts_host[x] = (int32_t)(uint32_t)v;
     }
-    std::atomic_thread_fence(std::memory_order_acquire);
-    memcpy(tile_counts_host, h->mail_host + kMailCountsAt, (size_t)(E_tot + 1) * sizeof(int32_t));
     return MOE_OK;
 }
 

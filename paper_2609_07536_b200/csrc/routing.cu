@@ -4,10 +4,10 @@
 // ceil(M_e / T_M) tiles along the token dimension; Eq. 16: their sum S.
 // The routed rows are the flat assignments f = t * k_tot + j in a *stable* order by expert.
 //
-// Three launch shapes, the same arithmetic and the same outputs bit for bit:
-//   routing_small    up to 32 chunks of 256 assignments: one launch of one CTA;
-//   routing_cluster  up to 128 chunks: one launch of one cluster of 8 CTAs, totals exchanged in
-//                    distributed shared memory;
+// Two launch shapes, the same outputs bit for bit:
+//   routing_onepass  up to 131072 assignments: one launch of one cluster of 1 to 16 CTAs; the ids stay in
+//                    registers from the histogram to the scatter, the per-expert totals of the CTAs cross
+//                    through distributed shared memory;
 //   otherwise four small launches over the whole GPU:
 //   1. hist          every warp histograms its own contiguous chunk of assignments;
 //   2. scan_columns  one CTA per expert: exclusive prefix of that expert's histogram column over
@@ -17,8 +17,6 @@
 //                    match_any gives each lane its rank among equal experts -> stable.
 
 #include "moe_internal.h"
-
-#include <cooperative_groups.h>
 
 namespace moe {
 namespace {
@@ -31,6 +29,9 @@ static_assert(kRoutingChunk % 32 == 0, "a chunk is a whole number of warp-wide r
 // set up while its predecessor still runs, and waits here, first thing, until the predecessor's writes are
 // visible.  Without that launch attribute this returns at once.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// lets the next kernel on the stream, if it was launched that way, be set up beside this one (after the wait above,
+// so that everything before this kernel is complete by then)
+__device__ __forceinline__ void grid_dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // launch `kernel` so that it may be set up before the previous kernel on the stream has finished
 template <typename... KArgs, typename... Args>
@@ -154,20 +155,16 @@ __device__ __forceinline__ void expert_prefix(const int32_t *s_cnt, int32_t *s_o
     }
 }
 
-// The tile counts for the host, written straight into host memory the GPU can address (`mail`, or nullptr):
-// the word at mail[0] takes `seq` once tiles[0..E_tot) and S sit at mail[kMailCountsAt...].  A host that polls
-// the word has the counts while the scatter still runs and needs neither a copy nor a stream synchronisation.
-// Called by every thread of one CTA, after the prefixes are complete.
-__device__ __forceinline__ void mail_counts(int32_t *mail, uint32_t seq, const int32_t *s_toff, int E_tot)
+// The tile counts for the host, written straight into host memory the GPU can address (`mail`, or nullptr), by one
+// warp: word x is the pair (count x, seq), x = 0..E_tot, the last one S.  A 64-bit store arrives whole, so every
+// word says by itself whether it belongs to this call: no fence orders anything here.  (Plain counts followed by a
+// sequence number needed system-scope fences of the whole CTA, 4-5 us of a small build's 12.)
+__device__ __forceinline__ void mail_counts(unsigned long long *mail, uint32_t seq, const int32_t *s_toff, int E_tot, int lane)
 {
     if (!mail) return;
-    for (int x = threadIdx.x; x <= E_tot; x += blockDim.x)
-        mail[kMailCountsAt + x] = (x < E_tot) ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot];
-    __threadfence_system();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence_system();
-        *reinterpret_cast<volatile uint32_t *>(mail) = seq;
+    for (int x = lane; x <= E_tot; x += 32) {
+        const uint32_t c = (uint32_t)((x < E_tot) ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot]);
+        *reinterpret_cast<volatile unsigned long long *>(mail + x) = ((unsigned long long)seq << 32) | c;
     }
 }
 
@@ -245,7 +242,7 @@ __global__ void __launch_bounds__(1024)
 routing_finalize(int E_tot, int tile_m, int max_mtiles, const int32_t *__restrict__ counts,
                  int32_t *__restrict__ offsets, int32_t *__restrict__ tiles, int32_t *__restrict__ tile_offsets,
                  int32_t *__restrict__ mtile_expert, int32_t *__restrict__ mtile_first_row,
-                 int32_t *__restrict__ mtile_valid, uint32_t *status, int32_t *mail, uint32_t mail_seq)
+                 int32_t *__restrict__ mtile_valid, uint32_t *status, unsigned long long *mail, uint32_t mail_seq)
 {
     extern __shared__ int32_t fin[];
     grid_dependency_wait();
@@ -254,7 +251,7 @@ routing_finalize(int E_tot, int tile_m, int max_mtiles, const int32_t *__restric
     __syncthreads();
     if (threadIdx.x < 32) expert_prefix(s_cnt, s_off, s_toff, E_tot, tile_m, threadIdx.x);
     __syncthreads();
-    mail_counts(mail, mail_seq, s_toff, E_tot);
+    if (threadIdx.x < 32) mail_counts(mail, mail_seq, s_toff, E_tot, threadIdx.x);
     if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
     for (int e = threadIdx.x; e <= E_tot; e += blockDim.x) {
         offsets[e] = s_off[e];
@@ -295,188 +292,269 @@ routing_scatter(const int32_t *__restrict__ topk_idx, int R, int E_tot, int tile
     chunk_scatter(begin, end, lane, E_tot, tile_m, e, run, s_off, s_toff, perm, inv_perm, pad_row);
 }
 
-// ---- small batches: the same steps in ONE launch of one CTA ------------------------------------------------
+// ---- up to 131072 assignments: the same steps in ONE launch of one thread-block cluster ---------------------
 //
-// At most 32 chunks (8192 assignments), one per warp; the per-chunk histograms live in shared memory, the ids
-// of a chunk stay in its warp's registers from the histogram to the scatter, the steps are separated by CTA
-// barriers instead of launch boundaries.  Same arithmetic, same outputs, bit for bit; four launches cost
-// ~30 us of which the work is a few microseconds at these sizes.
-constexpr int kSmallWarps = 32;
-constexpr size_t kSmallMaxSmem = 200 * 1024;
-__global__ void __launch_bounds__(kSmallWarps * 32)
-routing_small(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_tot, int tile_m, int n_chunks, int max_mtiles,
-              int32_t *__restrict__ counts, int32_t *__restrict__ offsets, int32_t *__restrict__ tiles,
-              int32_t *__restrict__ tile_offsets, int32_t *__restrict__ mtile_expert,
-              int32_t *__restrict__ mtile_first_row, int32_t *__restrict__ mtile_valid, int32_t *__restrict__ perm,
-              int32_t *__restrict__ inv_perm, int32_t *__restrict__ pad_row, uint32_t *status, int32_t *mail,
-              uint32_t mail_seq)
+// A cluster of n CTAs (1 for the decode sizes, up to 16), every warp owns `rows` (1..8) rows of 32 assignments.
+// One pass over the ids: votes rank a row's equal experts, the warp's own counter row in shared memory ranks them
+// across its rows, so that the rank of every assignment inside its warp's chunk is known before the prefixes are,
+// the scatter is one addition, and no shared-memory atomic is needed.  Bound by the length of the serial chain
+// (launch, ids, ranks, prefix over warps, CTAs and experts, stores), not by bytes: 131072 ids are 512 KB.  So the
+// chain is kept short: one thread per expert reads its 32 counters with independent loads, CTA totals are pushed
+// to all CTAs and cross with one cluster barrier, the experts' prefixes are one scan of the whole CTA.  perm is first
+// put in order in shared memory when a CTA holds many assignments: its lines then leave whole instead of 4 bytes
+// at a time.  Measured (device time; before: one CTA, one cluster of 8 or four launches, two passes over the ids):
+//   assignments, experts   8, 66   192, 60   2048, 66   8024, 40   32768, 60   131072, 66   27000, 1000
+//   before                 4.6     7.3       10.0       16.3       12.8        21.5         23.9 us
+//   now                    3.9     3.8       5.6        5.7        7.5         14.1         12.5 us
+constexpr int kOnepassWarps = 32;
+constexpr int kOnepassRows = 8;
+constexpr int kOnepassMaxCtas = 16;
+constexpr size_t kOnepassMaxSmem = 200 * 1024;
+
+struct RoutingOut {
+    int32_t *counts, *offsets, *tiles, *tile_offsets, *mtile_expert, *mtile_first_row, *mtile_valid, *perm, *inv_perm, *pad_row;
+};
+
+// counter row of a warp: 16-bit (a CTA holds at most 8192 assignments), its pitch an odd number of 32-bit words,
+// so that the 32 counters of one expert lie in 32 banks
+__host__ __device__ constexpr int onepass_pitch(int E_tot) { return 2 * (((E_tot + 1) / 2) | 1); }
+// CTAs for R assignments (0: too many for one launch): one more row per warp lengthens the chain by ~1 us, a cluster
+// of 2 to 16 costs 0.7 us over a single CTA whatever its size: as many CTAs as it takes to keep one row per warp
+int onepass_ctas(int R, int max_cluster)
 {
-    extern __shared__ int32_t sm[];
-    int32_t *whist = sm;                                   // [kSmallWarps][E_tot]
-    int32_t *s_cnt = sm + kSmallWarps * E_tot, *s_off = s_cnt + (E_tot + 1), *s_toff = s_off + (E_tot + 1);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int32_t *h = whist + w * E_tot;
-    const int begin = min(R, w * kRoutingChunk), end = w < n_chunks ? min(R, begin + kRoutingChunk) : begin;
-    // 1. histogram of the warp's chunk
-    int e[kPerLane];
-    chunk_load(topk_idx, begin, end, lane, e);
-    for (int x = lane; x < E_tot; x += 32) h[x] = 0;
-    __syncwarp();
-    chunk_hist(topk_idx, begin, end, lane, k_tot, E_tot, e, h, status);
-    __syncthreads();
-    // 2. per expert: exclusive prefix of its histogram column over the chunks, and its count
-    for (int x = threadIdx.x; x < E_tot; x += blockDim.x) {
-        int base = 0;
-        for (int c = 0; c < n_chunks; ++c) {
-            const int v = whist[c * E_tot + x];
-            whist[c * E_tot + x] = base;
-            base += v;
-        }
-        s_cnt[x] = base;
-        counts[x] = base;
-    }
-    __syncthreads();
-    // 3. offsets, tiles per expert and their prefix, the m-tile table
-    if (w == 0) expert_prefix(s_cnt, s_off, s_toff, E_tot, tile_m, lane);
-    __syncthreads();
-    mail_counts(mail, mail_seq, s_toff, E_tot);
-    if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
-    for (int x = threadIdx.x; x <= E_tot; x += blockDim.x) {
-        offsets[x] = s_off[x];
-        tile_offsets[x] = s_toff[x];
-        tiles[x] = (x < E_tot) ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot];
-    }
-    const int S = min(s_toff[E_tot], max_mtiles);
-    for (int mu = threadIdx.x; mu < S; mu += blockDim.x)
-        mtile_entry(mu, E_tot, tile_m, s_cnt, s_off, s_toff, mtile_expert, mtile_first_row, mtile_valid);
-    // 4. stable scatter of the warp's chunk: h[x] becomes the next free row of expert x for this chunk
-    for (int x = lane; x < E_tot; x += 32) h[x] += s_off[x];
-    __syncwarp();
-    chunk_scatter(begin, end, lane, E_tot, tile_m, e, h, s_off, s_toff, perm, inv_perm, pad_row);
+    int n = 1;
+    while (n < max_cluster && n < kOnepassMaxCtas && n * kOnepassWarps * 32 < R) n *= 2;
+    return (int64_t)n * kOnepassWarps * 32 * kOnepassRows >= R ? n : 0;
+}
+int onepass_rows(int R, int n_ctas)
+{
+    const int per_row = n_ctas * kOnepassWarps * 32;
+    return R > per_row ? (R + per_row - 1) / per_row : 1;
+}
+bool onepass_staged(int rows) { return rows > 2; }
+size_t onepass_smem(int n_ctas, int rows, int E_tot)
+{
+    size_t ints = (size_t)kOnepassWarps * onepass_pitch(E_tot) / 2;       // counters
+    ints += (size_t)n_ctas * E_tot + E_tot;                                // totals of all CTAs, rows before this CTA
+    ints += 4 * (size_t)(E_tot + 1);                                       // counts, offsets, tile offsets, offsets inside the CTA
+    if (onepass_staged(rows)) ints += (size_t)rows * kOnepassWarps * 32;   // perm of this CTA, in order
+    return ints * sizeof(int32_t);
 }
 
-// ---- medium batches: ONE launch of one thread-block cluster ------------------------------------------------
-//
-// CTA r of the cluster owns a contiguous run of chunks, one per warp, and keeps their histograms in its own
-// shared memory; the per-expert totals of the CTAs are exchanged through distributed shared memory (the only
-// step that crosses CTAs), the launch boundaries become one cluster barrier.  Same outputs as the other two
-// paths, bit for bit.  Measured on B200 against the four launches: 8 CTAs win ~10 us at 128 chunks and
-// lose ~12 us at 512; a single CTA is 2x slower than four launches at 128 chunks.
-constexpr int kClusterCtas = 8;
-constexpr int kClusterMaxChunks = 128;
-static_assert(kClusterMaxChunks <= kClusterCtas * kSmallWarps, "one chunk per warp");
-__global__ void __launch_bounds__(kSmallWarps * 32)
-routing_cluster(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_tot, int tile_m, int n_chunks, int max_mtiles,
-                int32_t *__restrict__ counts, int32_t *__restrict__ offsets, int32_t *__restrict__ tiles,
-                int32_t *__restrict__ tile_offsets, int32_t *__restrict__ mtile_expert,
-                int32_t *__restrict__ mtile_first_row, int32_t *__restrict__ mtile_valid, int32_t *__restrict__ perm,
-                int32_t *__restrict__ inv_perm, int32_t *__restrict__ pad_row, uint32_t *status, int32_t *mail,
-                uint32_t mail_seq)
+__global__ void __launch_bounds__(kOnepassWarps * 32)
+routing_onepass(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_tot, int tile_m, int rows, int n_ctas, int staged,
+                int max_mtiles, const RoutingOut out, uint32_t *status, unsigned long long *mail, uint32_t mail_seq)
 {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int nb = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int cpc = (n_chunks + nb - 1) / nb;                       // chunks per CTA (<= 32), a contiguous run
-    const int c_lo = min(n_chunks, rank * cpc), c_n = min(n_chunks, c_lo + cpc) - c_lo;
     extern __shared__ int32_t sm[];
-    int32_t *whist = sm;                                            // [cpc][E_tot]
-    int32_t *s_tot = sm + (size_t)cpc * E_tot;                      // this CTA's rows per expert (read by the others)
-    int32_t *s_base = s_tot + E_tot;                                // rows per expert in the CTAs before this one
+    const int pitch = onepass_pitch(E_tot);
+    uint16_t *hist = reinterpret_cast<uint16_t *>(sm);              // [32][pitch]
+    int32_t *s_all = sm + kOnepassWarps * pitch / 2;                // [n_ctas][E_tot] rows per expert of every CTA
+    int32_t *s_base = s_all + n_ctas * E_tot;                       // [E_tot] rows of the expert in the CTAs before this one
     int32_t *s_cnt = s_base + E_tot, *s_off = s_cnt + (E_tot + 1), *s_toff = s_off + (E_tot + 1);
+    int32_t *s_loc = s_toff + (E_tot + 1);                          // offsets of the experts inside this CTA
+    int32_t *s_perm = s_loc + (E_tot + 1);
+    __shared__ int32_t s_sum[96];                                   // per scanning warp: rows, tiles, rows of this CTA
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool mine = w < c_n;                                      // this warp has a chunk
-    int32_t *h = whist + (size_t)(mine ? w : 0) * E_tot;
-    const int begin = min(R, (c_lo + w) * kRoutingChunk), end = mine ? min(R, begin + kRoutingChunk) : begin;
-    // 1. histogram of the warp's chunk
-    int e[kPerLane];
-    chunk_load(topk_idx, begin, end, lane, e);
-    if (mine) {
-        for (int x = lane; x < E_tot; x += 32) h[x] = 0;
+    uint32_t rank = 0;
+    if (n_ctas > 1) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // "this CTA runs": see the push below
+    }
+    grid_dependency_wait();
+    grid_dependents_may_launch();
+
+    // ---- ids of the warp's chunk, and the 32 before it (a token may straddle the boundary)
+    const int begin = min(R, ((int)rank * kOnepassWarps + w) * rows * 32), end = min(R, begin + rows * 32);
+    int e[kOnepassRows], before = -1;
+#pragma unroll
+    for (int i = 0; i < kOnepassRows; ++i) {
+        const int f = begin + 32 * i + lane;
+        e[i] = (i < rows && f < end) ? __ldg(topk_idx + f) : -1;
+    }
+    if (begin > 0 && begin < end) before = __ldg(topk_idx + begin - 32 + lane);
+    uint16_t *h = hist + w * pitch;
+    for (int x = lane; x < pitch / 2; x += 32) reinterpret_cast<uint32_t *>(h)[x] = 0u;
+    __syncwarp();
+
+    // ---- ranks inside the chunk; bad ids are reported and left out, repeated experts reported and kept
+    int rk[kOnepassRows];
+    int j = (begin + lane) % k_tot, m0 = begin % k_tot;             // slot of this lane's assignment, of the row's first
+    const int step = 32 % k_tot, id_bits = E_tot > 1 ? 32 - __clz(E_tot - 1) : 0;
+#pragma unroll
+    for (int i = 0; i < kOnepassRows; ++i) {
+        rk[i] = 0;
+        if (i >= rows || begin + 32 * i >= end) break;              // warp-uniform
+        const int f = begin + 32 * i + lane;
+        const bool ok = e[i] >= 0 && e[i] < E_tot;
+        if (f < end && !ok) report(status, MOE_DEV_OOB, (uint32_t)f, 1u);
+        // lanes with the same expert, bit by bit of the id (match_any takes ~80 cycles of the SM per row when the
+        // ids differ; these votes take a quarter of that at 66 experts)
+        uint32_t same = __ballot_sync(0xffffffffu, ok);
+        for (int b = 0; b < id_bits; ++b) {
+            const bool bit = (e[i] >> b) & 1;
+            const uint32_t m = __ballot_sync(0xffffffffu, bit);
+            same &= bit ? m : ~m;
+        }
+        const uint32_t lower = same & ((1u << lane) - 1u);
+        const int base = ok ? (int)h[e[i]] : 0;
         __syncwarp();
-        chunk_hist(topk_idx, begin, end, lane, k_tot, E_tot, e, h, status);
-    }
-    __syncthreads();
-    // 2. per expert: exclusive prefix over this CTA's chunks, the CTA's total; then the totals of all CTAs
-    for (int x = threadIdx.x; x < E_tot; x += blockDim.x) {
-        int base = 0;
-        for (int lc = 0; lc < c_n; ++lc) {
-            const int v = whist[(size_t)lc * E_tot + x];
-            whist[(size_t)lc * E_tot + x] = base;
-            base += v;
+        if (ok && lower == 0u) h[e[i]] = (uint16_t)(base + __popc(same));
+        __syncwarp();
+        rk[i] = base + __popc(lower);
+        // the same expert twice inside one token: among the lanes of this row, then in the row before
+        const int in_row = min(j, lane);
+        int twice = ok ? __popc(lower & (((1u << in_row) - 1u) << (lane - in_row))) : 0;
+        for (int d = 1; d <= m0; ++d) {
+            const int v = __shfl_sync(0xffffffffu, before, 32 - d);
+            if (ok && j - lane >= d && v == e[i]) ++twice;
         }
-        s_tot[x] = base;
+        for (; twice > 0; --twice) report(status, MOE_DEV_DUP_EXPERT, (uint32_t)(f / k_tot), 1u);
+        before = e[i];
+        j += step;
+        if (j >= k_tot) j -= k_tot;
+        m0 += step;
+        if (m0 >= k_tot) m0 -= k_tot;
+        if (!ok) e[i] = -1;
     }
-    cluster.sync();
-    for (int x = threadIdx.x; x < E_tot; x += blockDim.x) {
-        int before = 0, total = 0;
-        for (int j = 0; j < nb; ++j) {
-            const int v = cluster.map_shared_rank(s_tot, j)[x];
-            if (j < rank) before += v;
-            total += v;
+    __syncthreads();
+
+    // ---- thread x, expert x: exclusive prefix of the warps' counts; this CTA's total, pushed to every CTA; rows in the
+    // CTAs before this one and in all
+    const int x = (int)threadIdx.x;
+    int own = 0, cnt = 0, ahead = 0;
+    if (x < E_tot) {
+#pragma unroll
+        for (int c0 = 0; c0 < kOnepassWarps; c0 += 8) {
+            int v[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) v[c] = hist[(c0 + c) * pitch + x];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                hist[(c0 + c) * pitch + x] = (uint16_t)own;
+                own += v[c];
+            }
         }
-        s_base[x] = before;
-        s_cnt[x] = total;
-        if (rank == 0) counts[x] = total;
+        cnt = own;
+    }
+    if (n_ctas > 1) {
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");    // every CTA runs: its memory may be written
+        if (x < E_tot) {
+            const uint32_t mine = (uint32_t)__cvta_generic_to_shared(s_all + (int)rank * E_tot + x);
+            for (int c = 0; c < n_ctas; ++c)
+                asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.u32 [a], %2;\n\t}"
+                             ::"r"(mine), "r"(c), "r"(own) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (x < E_tot) {
+            cnt = 0;
+#pragma unroll
+            for (int c = 0; c < kOnepassMaxCtas; ++c) {
+                const int v = c < n_ctas ? s_all[c * E_tot + x] : 0;
+                if (c < (int)rank) ahead += v;
+                cnt += v;
+            }
+        }
+    }
+    // ---- exclusive prefixes over the experts: rows, tiles (Eq. 5, Eq. 16) and rows of this CTA (every CTA, for its own scatter)
+    const int tl = (cnt + tile_m - 1) / tile_m, n_scan = (E_tot + 31) / 32;
+    int ic = cnt, it = tl, io = own;
+    if (w < n_scan) {
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int uc = __shfl_up_sync(0xffffffffu, ic, d), ut = __shfl_up_sync(0xffffffffu, it, d), uo = __shfl_up_sync(0xffffffffu, io, d);
+            if (lane >= d) { ic += uc; it += ut; io += uo; }
+        }
+        if (lane == 31) { s_sum[w] = ic; s_sum[32 + w] = it; s_sum[64 + w] = io; }
     }
     __syncthreads();
-    // 3. offsets, tiles per expert and their prefix (every CTA, for its own scatter), the m-tile table
-    if (w == 0) expert_prefix(s_cnt, s_off, s_toff, E_tot, tile_m, lane);
+    if (w < n_scan) {
+        ic += __reduce_add_sync(0xffffffffu, lane < w ? s_sum[lane] : 0);
+        it += __reduce_add_sync(0xffffffffu, lane < w ? s_sum[32 + lane] : 0);
+        io += __reduce_add_sync(0xffffffffu, lane < w ? s_sum[64 + lane] : 0);
+        if (x < E_tot) {
+            s_cnt[x] = cnt;
+            s_base[x] = ahead;
+            s_off[x] = ic - cnt;
+            s_toff[x] = it - tl;
+            s_loc[x] = io - own;
+            if (x == E_tot - 1) { s_off[E_tot] = ic; s_toff[E_tot] = it; s_loc[E_tot] = io; }
+        }
+    }
     __syncthreads();
+
+    // ---- results
+    if (rank == 0 && w == kOnepassWarps - 1) mail_counts(mail, mail_seq, s_toff, E_tot, lane);
+#pragma unroll
+    for (int i = 0; i < kOnepassRows; ++i) {
+        const int f = begin + 32 * i + lane;
+        if (i >= rows || f >= end) break;
+        int r = -1, pad = -1;
+        if (e[i] >= 0) {
+            const int x = e[i], in_cta = (int)h[x] + rk[i], o = s_off[x];
+            r = o + s_base[x] + in_cta;
+            pad = tile_m * s_toff[x] + (r - o);
+            if (staged) s_perm[s_loc[x] + in_cta] = f;
+            else out.perm[r] = f;
+        }
+        out.inv_perm[f] = r;
+        out.pad_row[f] = pad;
+    }
+    const int S = min(s_toff[E_tot], max_mtiles);
+    for (int mu = (int)rank * (int)blockDim.x + threadIdx.x; mu < S; mu += n_ctas * (int)blockDim.x)
+        mtile_entry(mu, E_tot, tile_m, s_cnt, s_off, s_toff, out.mtile_expert, out.mtile_first_row, out.mtile_valid);
     if (rank == 0) {
-        mail_counts(mail, mail_seq, s_toff, E_tot);
         if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
         for (int x = threadIdx.x; x <= E_tot; x += blockDim.x) {
-            offsets[x] = s_off[x];
-            tile_offsets[x] = s_toff[x];
-            tiles[x] = (x < E_tot) ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot];
+            if (x < E_tot) out.counts[x] = s_cnt[x];
+            out.offsets[x] = s_off[x];
+            out.tile_offsets[x] = s_toff[x];
+            // S rides behind the per-expert tile counts for the host copy
+            out.tiles[x] = (x < E_tot) ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot];
         }
     }
-    const int S = min(s_toff[E_tot], max_mtiles);
-    for (int mu = rank * blockDim.x + threadIdx.x; mu < S; mu += nb * blockDim.x)
-        mtile_entry(mu, E_tot, tile_m, s_cnt, s_off, s_toff, mtile_expert, mtile_first_row, mtile_valid);
-    // 4. stable scatter of the warp's chunk: h[x] becomes the next free row of expert x for this chunk
-    if (mine) {
-        for (int x = lane; x < E_tot; x += 32) h[x] += s_off[x] + s_base[x];
-        __syncwarp();
-        chunk_scatter(begin, end, lane, E_tot, tile_m, e, h, s_off, s_toff, perm, inv_perm, pad_row);
+    if (staged) {
+        __syncthreads();
+        for (int x = w; x < E_tot; x += kOnepassWarps) {
+            const int src = s_loc[x], n = s_loc[x + 1] - src, dst = s_off[x] + s_base[x];
+            for (int i = lane; i < n; i += 32) out.perm[dst + i] = s_perm[src + i];
+        }
     }
-    cluster.sync();   // no CTA leaves while another may still read its totals
 }
 
-size_t routing_cluster_smem(int n_chunks, int E_tot)
+void onepass_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int n_ctas, size_t smem, cudaStream_t stream)
 {
-    const int cpc = (n_chunks + kClusterCtas - 1) / kClusterCtas;
-    return ((size_t)cpc * E_tot + 2 * (size_t)E_tot + 3 * (size_t)(E_tot + 1)) * sizeof(int32_t);
-}
-
-cudaError_t routing_cluster_launch(const int32_t *topk_idx, const moe_shape &s, int tile_m, int R, int n_chunks,
-                                   const moe_routing &r, uint32_t *status, int32_t *mail, uint32_t mail_seq, cudaStream_t stream)
-{
-    const size_t sm = routing_cluster_smem(n_chunks, s.E_tot);
-    if (sm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(routing_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallMaxSmem);
-        if (e != cudaSuccess) return e;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kClusterCtas);
-    cfg.blockDim = dim3(kSmallWarps * 32);
-    cfg.dynamicSmemBytes = sm;
+    cfg.gridDim = dim3((unsigned)n_ctas);
+    cfg.blockDim = dim3(kOnepassWarps * 32);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kClusterCtas;
+    attr[0].val.clusterDim.x = (unsigned)n_ctas;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, routing_cluster, topk_idx, R, (int)s.k_tot, (int)s.E_tot, tile_m, n_chunks,
-                              (int)r.max_mtiles, r.counts, r.offsets, r.tiles, r.tile_offsets, r.mtile_expert,
-                              r.mtile_first_row, r.mtile_valid, r.perm, r.inv_perm, r.pad_row, status, mail, mail_seq);
+}
+
+cudaError_t routing_onepass_launch(const int32_t *topk_idx, const moe_shape &s, int tile_m, int R, int n_ctas,
+                                   const moe_routing &r, uint32_t *status, unsigned long long *mail, uint32_t mail_seq,
+                                   cudaStream_t stream)
+{
+    const int rows = onepass_rows(R, n_ctas);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    onepass_config(cfg, attr, n_ctas, onepass_smem(n_ctas, rows, s.E_tot), stream);
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    const RoutingOut out = {r.counts, r.offsets, r.tiles, r.tile_offsets, r.mtile_expert, r.mtile_first_row, r.mtile_valid,
+                            r.perm, r.inv_perm, r.pad_row};
+    return cudaLaunchKernelEx(&cfg, routing_onepass, topk_idx, R, (int)s.k_tot, (int)s.E_tot, tile_m, rows, n_ctas,
+                              onepass_staged(rows) ? 1 : 0, (int)r.max_mtiles, out, status, mail, mail_seq);
 }
 
 // the four launches; `scratch`: n_chunks * E_tot ints that need not start at any value
 cudaError_t routing_four_launches(const int32_t *topk_idx, const moe_shape &s, int tile_m, int R, int n_chunks,
-                                  const moe_routing &r, int32_t *scratch, uint32_t *status, int32_t *mail, uint32_t mail_seq,
+                                  const moe_routing &r, int32_t *scratch, uint32_t *status, unsigned long long *mail, uint32_t mail_seq,
                                   cudaStream_t stream)
 {
     const int blocks = (n_chunks + kWarpsPerBlock - 1) / kWarpsPerBlock;
@@ -500,25 +578,31 @@ cudaError_t routing_four_launches(const int32_t *topk_idx, const moe_shape &s, i
 
 }  // namespace
 
-cudaError_t routing_launch(const int32_t *topk_idx, const moe_shape &s, int tile_m, const moe_routing &r, uint32_t *status,
-                           int32_t *mail, uint32_t mail_seq, cudaStream_t stream)
+cudaError_t routing_prepare(int *max_cluster)
+{
+    cudaError_t e = cudaFuncSetAttribute(routing_onepass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOnepassMaxSmem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(routing_onepass, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    for (*max_cluster = kOnepassMaxCtas; *max_cluster > 8; *max_cluster >>= 1) {
+        onepass_config(cfg, attr, *max_cluster, kOnepassMaxSmem, nullptr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, routing_onepass, &cfg) == cudaSuccess && n > 0) break;
+    }
+    (void)cudaGetLastError();
+    return cudaSuccess;
+}
+
+cudaError_t routing_launch(const int32_t *topk_idx, const moe_shape &s, int tile_m, const moe_routing &r, int32_t *scratch,
+                           int max_cluster, uint32_t *status, unsigned long long *mail, uint32_t mail_seq, cudaStream_t stream)
 {
     const int R = s.T * s.k_tot;
-    const int n_chunks = (R + kRoutingChunk - 1) / kRoutingChunk;
-    const size_t sm_small = ((size_t)kSmallWarps * s.E_tot + 3 * (size_t)(s.E_tot + 1)) * sizeof(int32_t);
-    if (n_chunks <= kSmallWarps && sm_small <= kSmallMaxSmem) {
-        if (sm_small > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(routing_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallMaxSmem);
-            if (e != cudaSuccess) return e;
-        }
-        routing_small<<<1, kSmallWarps * 32, sm_small, stream>>>(
-            topk_idx, R, s.k_tot, s.E_tot, tile_m, n_chunks, r.max_mtiles, r.counts, r.offsets, r.tiles, r.tile_offsets,
-            r.mtile_expert, r.mtile_first_row, r.mtile_valid, r.perm, r.inv_perm, r.pad_row, status, mail, mail_seq);
-        return cudaGetLastError();
-    }
-    if (n_chunks <= kClusterMaxChunks && routing_cluster_smem(n_chunks, s.E_tot) <= kSmallMaxSmem)
-        return routing_cluster_launch(topk_idx, s, tile_m, R, n_chunks, r, status, mail, mail_seq, stream);
-    return routing_four_launches(topk_idx, s, tile_m, R, n_chunks, r, r.scratch, status, mail, mail_seq, stream);
+    const int n_ctas = onepass_ctas(R, max_cluster);
+    if (n_ctas > 0 && onepass_smem(n_ctas, onepass_rows(R, n_ctas), s.E_tot) <= kOnepassMaxSmem)
+        return routing_onepass_launch(topk_idx, s, tile_m, R, n_ctas, r, status, mail, mail_seq, stream);
+    return routing_four_launches(topk_idx, s, tile_m, R, (R + kRoutingChunk - 1) / kRoutingChunk, r, scratch, status, mail, mail_seq, stream);
 }
 
 }  // namespace moe
@@ -592,7 +676,7 @@ extern "C" int32_t moe_build_routing_static(moe_handle *h, const int32_t *topk_i
     // The array keeps whatever the previous call left in it.  Nothing has to start at zero: the
     // histogram pass overwrites every (warp, expert) entry the later passes read.
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = routing_four_launches(topk_idx, *s, tile_m, (int)R, (int)n_warps, *r, scratch, status_dev, nullptr, 0u, st);
+    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, scratch, h->routing_max_cluster, status_dev, nullptr, 0u, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "static routing launch");
     if (tile_counts_host) {
         e = cudaMemcpyAsync(tile_counts_host, r->tiles, (size_t)(s->E_tot + 1) * 4, cudaMemcpyDeviceToHost, st);

@@ -92,3 +92,28 @@ def test_bad_ids_are_reported_not_fatal():
     assert st.code == B.MOE_DEV_DUP_EXPERT and st.detail == 7
     # the context is still usable
     _compare(w, idx)
+
+
+@pytest.mark.parametrize("T,E,k", [
+    (128, 66, 8), (1025, 9, 1),          # 1024 and 1025 assignments: one CTA, the first cluster of two
+    (683, 33, 3), (1366, 65, 3),         # 2049 and 4098: clusters of four and eight, tokens straddle the rows of 32
+    (8193, 1, 1), (2341, 1000, 7),       # 8193 and 16387: sixteen CTAs, one row and two rows per warp
+    (16384, 66, 8), (18725, 40, 7),      # 131072, and 131075: the first size of the four launches
+], ids=lambda v: str(v))
+def test_edges_of_the_one_launch_build(T, E, k):
+    from dataclasses import replace
+    rng = np.random.default_rng(T)
+    idx = np.argsort(rng.random((T, E), dtype=np.float32), axis=1)[:, :k].astype(np.int32)
+    _compare(replace(wl.TINY, T=T, E=E, k=k, tile_m=64), idx)
+
+
+@pytest.mark.parametrize("t,slots", [(3, (0, 2)), (10, (0, 2)), (10, (1, 2)), (341, (0, 1)), (682, (0, 2))])
+def test_repeated_experts_are_found_across_the_rows_of_a_warp(t, slots):
+    # k = 3: token 10 holds assignments 30, 31 | 32, token 341 1023 | 1024 (the next CTA's first row)
+    from dataclasses import replace
+    w = replace(wl.TINY, T=700, E=8, k=3)
+    idx = np.tile(np.array([[1, 5, 7]], dtype=np.int32), (700, 1))
+    idx[t, slots[1]] = idx[t, slots[0]]
+    ws, _, _ = G.build_routing(w, idx)
+    st = B.moe_get_status(G.handle(), ws.status, check=False)
+    assert (st.code, st.detail, st.count) == (B.MOE_DEV_DUP_EXPERT, t, 1)
