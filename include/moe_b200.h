@@ -180,8 +180,8 @@ typedef struct {
 
 /* Opens the library on CUDA device `device`; caches the SM count and the kernels'
  * residency (Section III-E: the SM count is cached at operator initialisation).  Also allocates the
- * handle's only memory outside the C++ heap: about 4 KB of pinned host memory that the GPU can address,
- * the mailbox through which the routing build hands the routed-tile counts to the whole-step calls
+ * handle's only memory outside the C++ heap: about 8 KB of pinned host memory that the GPU can address,
+ * the mailbox through which the routed-tile counts reach the host in the whole-step calls
  * (moe_layer, moe_post_router_layer); freed by moe_destroy.  No device memory is allocated.  [host] */
 int32_t moe_create(int32_t device, moe_handle **out);
 int32_t moe_destroy(moe_handle *h);
@@ -353,12 +353,15 @@ int32_t moe_clear_status(moe_handle *h, uint32_t *status_dev, void *stream);
  * E_tot + 1 ints, filled when the call returns; limits_or_null = NULL uses moe_query_occupancy's limits;
  * plan_out may be NULL.
  * Returns after the fused kernel has been launched (asynchronous on `stream`); the only host wait
- * inside is the one for the tile counts.  That wait is not a stream synchronisation: the routing kernel
- * that completes the counts stores them into the handle's pinned mailbox and then a sequence number;
- * the host polls that word (bounded: it gives up with MOE_ERR_CUDA when the stream finishes or fails
- * without the word, or after the handle's wait limit plus two seconds), copies the counts to
- * tile_counts_pinned, plans and launches while the routing build is still scattering, so that the
- * fused kernel is queued behind it without a gap (15 us per step on B200 against copy + synchronise).
+ * inside is the one for the tile counts.  That wait is not a stream synchronisation: a kernel of the step
+ * stores each count, with a sequence number beside it, into the handle's pinned mailbox; the host polls
+ * the words (bounded: it gives up with MOE_ERR_CUDA when the stream finishes or fails without them, or
+ * after the handle's wait limit plus two seconds), copies the counts to tile_counts_pinned and plans.
+ * The selector sees the counts through their sum S alone, so its picks for every S a routing of this
+ * shape can have are tabulated on the first call (kept in the handle, for the last 8 shapes); the fused
+ * kernel is launched at once and looks its communication-CTA count up by the S it reads on the device,
+ * and the host waits and plans beside it.  Where the picks cannot be tabulated (more than 256 possible S,
+ * tile-level readiness, picks that differ in their co-resident warps) the host waits and plans first.
  * If the mailbox could not be set up at moe_create the counts come by an asynchronous copy and a
  * stream synchronisation; tile_counts_pinned must then be pinned.  tile_counts_pinned = NULL selects the device-only-counts
  * path of Section III-E: no copy, no wait; the plan comes from plan_partition_estimate and the kernel

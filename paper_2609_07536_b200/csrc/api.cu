@@ -115,6 +115,7 @@ int32_t moe_create(int32_t device, moe_handle **out)
         return MOE_ERR_CUDA;
     }
     e = routing_prepare(&h->routing_max_cluster);
+    if (e == cudaSuccess) e = gemm1_prepare();
     if (e != cudaSuccess) {
         delete h;
         return MOE_ERR_CUDA;
@@ -148,6 +149,7 @@ int32_t moe_destroy(moe_handle *h)
 {
     if (h && h->counts_event) cudaEventDestroy(static_cast<cudaEvent_t>(h->counts_event));
     if (h && h->mail_host) cudaFreeHost(h->mail_host);
+    if (h) delete[] h->plan_tables;
     delete h;
     return MOE_OK;
 }
@@ -357,11 +359,11 @@ int32_t moe_build_routing(moe_handle *h, const int32_t *topk_idx, const moe_shap
 
 namespace {
 
-// Routing build of the whole-step calls.  With the handle's mailbox the kernel that finishes the counts stores
-// them into host memory itself and `*seq` is the number to wait for (wait_counts); without it, the plain
-// build with its copy, and `*seq` = 0.
+// Routing build of the whole-step calls.  With the handle's mailbox a kernel stores the counts into host memory and
+// `*seq` is the number to wait for (wait_counts): the build itself, or (`mail_later`) a launch behind it.  Without
+// the mailbox, the plain build with its copy, and `*seq` = 0.
 int32_t build_routing_mailed(moe_handle *h, const int32_t *topk_idx, const moe_shape *s, int32_t tile_m, const moe_routing *r,
-                             int32_t *tile_counts_host, uint32_t *status_dev, cudaStream_t st, uint32_t *seq)
+                             int32_t *tile_counts_host, bool mail_later, uint32_t *status_dev, cudaStream_t st, uint32_t *seq)
 {
     *seq = 0;
     if (!tile_counts_host || !h->mail_dev)
@@ -373,7 +375,7 @@ int32_t build_routing_mailed(moe_handle *h, const int32_t *topk_idx, const moe_s
     if (r->max_mtiles < max_mtiles_of(s, tile_m)) return MOE_ERR_SHAPE;
     if (const int32_t rc = require_handle_device(h, "moe_build_routing")) return rc;
     if (++h->mail_seq == 0u) h->mail_seq = 1u;
-    const cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev, h->mail_dev, h->mail_seq, st);
+    const cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev, mail_later ? nullptr : h->mail_dev, h->mail_seq, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "routing launch");
     *seq = h->mail_seq;
     return MOE_OK;
@@ -418,6 +420,60 @@ int32_t wait_counts(moe_handle *h, uint32_t seq, int32_t E_tot, int32_t *tile_co
     return MOE_OK;
 }
 
+// The tabulated selection for this shape, tile family and limits, made on the first use (0.5 us per entry, E_tot + 1
+// entries at most); nullptr where the launch has to wait for the counts instead: more m-tile counts than a table
+// holds, tile-level readiness (it depends on more than the sum of the counts), or picks that differ in what the
+// launch configuration fixes (grid, co-resident warps).
+const PlanTable *plan_table(moe_handle *h, const moe_shape *s, const moe_occupancy *occ, const moe_sm_limits *lim, const moe_rho *rho)
+{
+    for (int i = 0; i < h->n_plan_tables; ++i) {
+        const PlanTable &t = h->plan_tables[i];
+        if (t.tile_m == occ->tile_m && t.tile_n == occ->tile_n && memcmp(&t.shape, s, sizeof *s) == 0 &&
+            memcmp(&t.limits, lim, sizeof *lim) == 0)
+            return t.n > 0 ? &t : nullptr;
+    }
+    if (!h->plan_tables) {
+        h->plan_tables = new (std::nothrow) PlanTable[kPlanTables];
+        if (!h->plan_tables) return nullptr;
+    }
+    PlanTable &t = h->plan_tables[h->next_plan_table];
+    h->next_plan_table = (h->next_plan_table + 1) % kPlanTables;
+    if (h->n_plan_tables < kPlanTables) ++h->n_plan_tables;
+    t.shape = *s;
+    t.tile_m = occ->tile_m;
+    t.tile_n = occ->tile_n;
+    t.limits = *lim;
+    t.n = 0;
+    // an expert with rows has at most (rows - 1) / tile_m + 1 m-tiles
+    const int64_t R = (int64_t)s->T * s->k_tot, used = R < s->E_tot ? R : s->E_tot;
+    const int64_t first = ceil_div(R, occ->tile_m), last = (R - used) / occ->tile_m + used;
+    if (R < 1 || last - first + 1 > kPlanTableMax || occ->o_comp != 1 || occ->o_comm != 1 ||
+        (!lim->drain_help && lim->dep_model == MOE_DEP_TILE))
+        return nullptr;
+    const int slot = occ->comp_slot_sms;
+    for (int64_t S = first; S <= last; ++S) {
+        const int32_t count = (int32_t)S;
+        moe_plan p;
+        if (plan_partition(&count, 1, occ, lim, s, rho, &p) != MOE_OK) return nullptr;
+        if (S == first) t.plan = p;
+        const int c_slots = slot == 2 ? (p.comm_ctas + 1) & ~1 : p.comm_ctas, c0 = slot == 2 ? (t.plan.comm_ctas + 1) & ~1 : t.plan.comm_ctas;
+        if (p.comm_ctas < 1 || p.comm_ctas > 255 || p.co_warps != t.plan.co_warps || p.P != (lim->G - p.comm_ctas) / slot ||
+            c_slots + slot * p.P != c0 + slot * t.plan.P)
+            return nullptr;
+        t.C[S - first] = (uint8_t)p.comm_ctas;
+    }
+    t.first = (int32_t)first;
+    t.n = (int32_t)(last - first + 1);
+    return &t;
+}
+
+// moe_gemm2_combine with the launch's plan, or (`table`) with the plan looked up on the device by the m-tile count;
+// mail_seq != 0: this launch mails the counts
+int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
+                             const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
+                             const PlanTable *table, uint32_t mail_seq, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
+                             void *stream);
+
 }  // namespace
 
 extern "C" {
@@ -428,6 +484,18 @@ int32_t moe_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, c
                           void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream)
 {
     (void)topk_idx;
+    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, nullptr, 0u, out, y_ws, flags_ws, status_dev, stream);
+}
+
+}  // extern "C"
+
+namespace {
+
+int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
+                             const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
+                             const PlanTable *table, uint32_t mail_seq, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
+                             void *stream)
+{
     if (!h || !s || !occ || !r || !plan || !out || !status_dev) return MOE_ERR_NULL;
     if (!shape_ok(s)) return MOE_ERR_SHAPE;
     if (!tile_ok(occ->tile_m, occ->tile_n)) return MOE_ERR_UNSUPPORTED;
@@ -482,6 +550,19 @@ int32_t moe_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, c
     p.W_comp = (int32_t)Wc;
     p.S_dev = counts_on_device ? r->tiles + s->E_tot : nullptr;
     p.C = C; p.P = Pc; p.mode = mode; p.withhold = plan->debug_withhold_tile;
+    p.G = h->G;
+    p.slot_sms = slot_sms;
+    if (table) {
+        p.G = table->limits.G;
+        p.c_table_first = table->first;
+        p.c_table_n = table->n;
+        memcpy(p.c_table, table->C, (size_t)table->n);
+        if (mail_seq != 0u) {
+            p.mail = h->mail_dev;
+            p.mail_seq = mail_seq;
+            p.E_tot = s->E_tot;
+        }
+    }
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
     p.tok_blk = (int32_t)ceil_div(s->T, s->EP);
     p.tok_tiles_per_rank = (int32_t)ceil_div(p.tok_blk, kCommTileM);
@@ -597,6 +678,62 @@ int32_t moe_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, c
     return MOE_OK;
 }
 
+// What a whole-step call selects with.
+struct Selection {
+    moe_occupancy occ;
+    moe_sm_limits lim;
+    moe_rho rho;
+    const PlanTable *table;
+};
+int32_t selection_of(moe_handle *h, const moe_shape *s, int32_t tile_m, int32_t tile_n, const moe_sm_limits *limits_or_null,
+                     bool host_counts, Selection *sel)
+{
+    if (!shape_ok(s)) return MOE_ERR_SHAPE;
+    const int32_t rc = moe_query_occupancy(h, tile_m, tile_n, &sel->occ, &sel->lim, &sel->rho);
+    if (rc != MOE_OK) return rc;
+    if (limits_or_null) sel->lim = *limits_or_null;
+    sel->table = host_counts && h->mail_dev ? plan_table(h, s, &sel->occ, &sel->lim, &sel->rho) : nullptr;
+    return MOE_OK;
+}
+
+// What the whole-step calls do after the routing build (and GEMM1): select, launch, and have the counts on the host.
+// Where the selection is tabulated the launch goes out at once, queued behind its predecessor without a gap, and
+// the host waits for the counts and plans afterwards, beside the running kernel (step of the tiny configuration
+// 20.5 -> 16 us, of the DeepSeek shape at T = 16 76.7 -> 71); otherwise it waits first.  `mail_seq` != 0: this launch
+// mails the counts (table only).  `counts_event`: recorded behind the counts' copy, for a build without the mailbox
+// (seq = 0).
+int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
+                          const Selection &sel, const moe_routing *routing, uint32_t seq, uint32_t mail_seq,
+                          cudaEvent_t counts_event, int32_t *tile_counts, void *const *out, void *y_ws, uint32_t *flags_ws,
+                          uint32_t *status_dev, moe_plan *plan_out, void *ev_before, void *ev_after, cudaStream_t st)
+{
+    moe_plan plan;
+    int32_t rc = MOE_OK, n_mtiles = MOE_MTILES_ON_DEVICE;
+    auto counts_and_plan = [&]() -> int32_t {
+        const int32_t r = wait_counts(h, seq, s->E_tot, tile_counts, st, counts_event);
+        return r != MOE_OK ? r : plan_partition(tile_counts, s->E_tot, &sel.occ, &sel.lim, s, &sel.rho, &plan);
+    };
+    if (sel.table) {
+        plan = sel.table->plan;
+    } else if (tile_counts) {
+        if ((rc = counts_and_plan()) != MOE_OK) return rc;
+        n_mtiles = tile_counts[s->E_tot];
+    } else {
+        if ((rc = plan_partition_estimate(&sel.occ, &sel.lim, s, &sel.rho, &plan)) != MOE_OK) return rc;   // counts stay on the device
+    }
+    if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
+    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, sel.table, mail_seq, out, y_ws,
+                              flags_ws, status_dev, st);
+    if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
+    if (rc == MOE_OK && sel.table) rc = counts_and_plan();
+    if (plan_out && rc == MOE_OK) *plan_out = plan;
+    return rc;
+}
+
+}  // namespace
+
+extern "C" {
+
 int32_t moe_release_workspace(moe_handle *h, const uint32_t *flags_ws)
 {
     if (!h) return MOE_ERR_NULL;
@@ -634,32 +771,14 @@ int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int
 {
     if (!h || !s || !routing) return MOE_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    Selection sel;
+    int32_t rc = selection_of(h, s, tile_m, tile_n, limits_or_null, tile_counts_pinned != nullptr, &sel);
+    if (rc != MOE_OK) return rc;
     uint32_t seq = 0;
-    int32_t rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, status_dev, st, &seq);
+    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, sel.table != nullptr, status_dev, st, &seq);
     if (rc != MOE_OK) return rc;
-    if (tile_counts_pinned) {
-        // the counts reach the host while the routing build is still scattering: planning and the fused
-        // launch below are queued behind it without a gap
-        rc = wait_counts(h, seq, s->E_tot, tile_counts_pinned, st, nullptr);
-        if (rc != MOE_OK) return rc;
-    }
-    moe_occupancy occ;
-    moe_sm_limits lim;
-    moe_rho rho;
-    rc = moe_query_occupancy(h, tile_m, tile_n, &occ, &lim, &rho);
-    if (rc != MOE_OK) return rc;
-    if (limits_or_null) lim = *limits_or_null;
-    moe_plan plan;
-    rc = tile_counts_pinned ? plan_partition(tile_counts_pinned, s->E_tot, &occ, &lim, s, &rho, &plan)
-                            : plan_partition_estimate(&occ, &lim, s, &rho, &plan);   // counts stay on the device
-    if (rc != MOE_OK) return rc;
-    if (plan_out) *plan_out = plan;
-    if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
-    rc = moe_gemm2_combine(h, x_routed, W2, topk_idx, topk_w, s, &occ, routing,
-                           tile_counts_pinned ? tile_counts_pinned[s->E_tot] : MOE_MTILES_ON_DEVICE, &plan,
-                           out, y_ws, flags_ws, status_dev, st);
-    if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
-    return rc;
+    return select_and_launch(h, x_routed, W2, topk_w, s, sel, routing, seq, seq, nullptr, tile_counts_pinned, out, y_ws, flags_ws,
+                             status_dev, plan_out, ev_before, ev_after, st);
 }
 
 // ---- the post-router MoE layer on device-resident inputs (Section II-A: steps 1-3) -------------
@@ -672,37 +791,23 @@ int32_t moe_post_router_layer(moe_handle *h, const void *hidden, const void *W1,
 {
     if (!h || !s || !routing) return MOE_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    Selection sel;
+    int32_t rc = selection_of(h, s, tile_m, tile_n, limits_or_null, tile_counts_pinned != nullptr, &sel);
+    if (rc != MOE_OK) return rc;
+    const bool gemm1_mails = s->T > 0;
     uint32_t seq = 0;
-    int32_t rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, status_dev, st, &seq);
+    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, gemm1_mails, status_dev, st, &seq);
     if (rc != MOE_OK) return rc;
-    // GEMM1 reads the m-tile count on the device, so it is launched before the host waits for the counts:
-    // the wait and the planning are hidden behind it
-    if (tile_counts_pinned && seq == 0u && h->counts_event) cudaEventRecord(static_cast<cudaEvent_t>(h->counts_event), st);
-    rc = moe_gemm1_act(h, hidden, W1, s, tile_m, routing, MOE_MTILES_ON_DEVICE, h_routed_ws, x_routed_ws, status_dev, st);
+    // GEMM1 reads the m-tile count on the device, so it is launched before the host waits for the counts: the wait
+    // and the planning are hidden behind it.  Without the mailbox (seq = 0) the copy of the counts was queued right
+    // behind the routing kernels, before GEMM1: an event marks it.
+    cudaEvent_t counts_event = static_cast<cudaEvent_t>(h->counts_event);
+    if (tile_counts_pinned && seq == 0u && counts_event) cudaEventRecord(counts_event, st);
+    rc = launch_gemm1_act(h, hidden, W1, s, tile_m, routing, MOE_MTILES_ON_DEVICE, h_routed_ws, x_routed_ws, status_dev, seq, st);
     if (rc != MOE_OK) return rc;
-    moe_occupancy occ;
-    moe_sm_limits lim;
-    moe_rho rho;
-    rc = moe_query_occupancy(h, tile_m, tile_n, &occ, &lim, &rho);
-    if (rc != MOE_OK) return rc;
-    if (limits_or_null) lim = *limits_or_null;
-    moe_plan plan;
-    int32_t n_mtiles = MOE_MTILES_ON_DEVICE;
-    if (tile_counts_pinned) {
-        // the copy of the counts was queued right after the routing kernels, before GEMM1: wait for it alone
-        cudaEvent_t counts_ready = static_cast<cudaEvent_t>(h->counts_event);
-        if (seq == 0u && !counts_ready) return MOE_ERR_CUDA;
-        rc = wait_counts(h, seq, s->E_tot, tile_counts_pinned, st, counts_ready);
-        if (rc != MOE_OK) return rc;
-        rc = plan_partition(tile_counts_pinned, s->E_tot, &occ, &lim, s, &rho, &plan);
-        n_mtiles = tile_counts_pinned[s->E_tot];
-    } else {
-        rc = plan_partition_estimate(&occ, &lim, s, &rho, &plan);
-    }
-    if (rc != MOE_OK) return rc;
-    if (plan_out) *plan_out = plan;
-    return moe_gemm2_combine(h, x_routed_ws, W2, topk_idx, topk_w, s, &occ, routing, n_mtiles, &plan, out, y_ws,
-                             flags_ws, status_dev, st);
+    if (tile_counts_pinned && seq == 0u && !counts_event) return MOE_ERR_CUDA;
+    return select_and_launch(h, x_routed_ws, W2, topk_w, s, sel, routing, seq, 0u, counts_event, tile_counts_pinned, out, y_ws,
+                             flags_ws, status_dev, plan_out, nullptr, nullptr, st);
 }
 
 // ---- one-time service-rate characterisation (Eq. 13) ---------------------------------------

@@ -51,6 +51,9 @@ struct alignas(64) G1Params {
     int32_t sub_rows;              // rows of a piece that may be stored: min(tile_m, 128)
     int32_t I, NT;                 // intermediate size, n-tiles = ceil(I / 128)
     int32_t num_kb, last_ksteps;
+    unsigned long long *mail;      // != nullptr: the tile counts (S_dev - E_tot) are mailed to the host by this launch
+    uint32_t mail_seq;
+    int32_t E_tot;
 };
 
 struct G1Control {
@@ -97,9 +100,9 @@ __device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
     const int mu = piece / P.sub;
     const int half = piece - mu * P.sub;
     G1Tile t;
-    t.e = __ldg(&P.mtile_expert[mu]);
-    t.row0 = __ldg(&P.mtile_first_row[mu]) + half * kMmaM;
-    t.valid = max(0, min(P.sub_rows, __ldg(&P.mtile_valid[mu]) - half * kMmaM));
+    t.e = ld_chained(&P.mtile_expert[mu]);
+    t.row0 = ld_chained(&P.mtile_first_row[mu]) + half * kMmaM;
+    t.valid = max(0, min(P.sub_rows, ld_chained(&P.mtile_valid[mu]) - half * kMmaM));
     t.n0 = i_n * kG1TileN;
     return t;
 }
@@ -112,9 +115,11 @@ gather_rows(const uint4 *__restrict__ hidden, const int32_t *__restrict__ perm, 
             uint4 *__restrict__ h_routed)
 {
     const int r = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+    grid_dependency_wait();
+    grid_dependents_may_launch();
     if (r >= R) return;
     const int lane = threadIdx.x & 31;
-    const int t = __ldg(&perm[r]) / k_tot;
+    const int t = ld_chained(&perm[r]) / k_tot;
     const uint4 *src = hidden + (size_t)t * row_vec;
     uint4 *dst = h_routed + (size_t)r * row_vec;
     for (int c = lane; c < row_vec; c += 32) dst[c] = __ldg(&src[c]);
@@ -130,10 +135,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
     G1Control *ctl = reinterpret_cast<G1Control *>(ring + kStageBytesTotal);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int S = P.S_dev ? min(__ldg(P.S_dev), P.S) : P.S;
-    const int total_tiles = S * P.sub * P.NT;
     const int b = (int)blockIdx.x, stride = (int)gridDim.x;
-    const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kG1Stages; ++i) {
@@ -147,13 +149,21 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         ctl->abort = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        prefetch_tensormap(&P.tmA);
+        prefetch_tensormap(&P.tmB);
     }
     if (warp == 1) tmem_alloc(smem_u32(&ctl->tmem_base), kG1TmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
+    grid_dependency_wait();
+    const int S = P.S_dev ? min(ld_chained_uniform(P.S_dev), P.S) : P.S;
+    const int total_tiles = S * P.sub * P.NT;
+    const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
+    if (P.mail && b == 0 && warp == 3)
+        mail_counts(P.mail, P.mail_seq, P.E_tot, lane, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if (warp == 0 || warp == 2) {
         // ---------------- TMA producers
         const bool load_a = (warp == 0);
@@ -328,6 +338,11 @@ inline bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintp
 
 using namespace moe;
 
+cudaError_t moe::gemm1_prepare()
+{
+    return cudaFuncSetAttribute(moe_gemm1_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes());
+}
+
 extern "C" int32_t moe_gemm1_workspace_bytes(const moe_shape *s, size_t *h_routed_bytes)
 {
     if (!s || !h_routed_bytes) return MOE_ERR_NULL;
@@ -339,6 +354,13 @@ extern "C" int32_t moe_gemm1_workspace_bytes(const moe_shape *s, size_t *h_route
 extern "C" int32_t moe_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const moe_shape *s,
                                  int32_t tile_m, const moe_routing *r, int32_t n_mtiles, void *h_routed_ws,
                                  void *x_routed, uint32_t *status_dev, void *stream)
+{
+    return launch_gemm1_act(h, hidden, W1, s, tile_m, r, n_mtiles, h_routed_ws, x_routed, status_dev, 0u, stream);
+}
+
+int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const moe_shape *s, int32_t tile_m,
+                              const moe_routing *r, int32_t n_mtiles, void *h_routed_ws, void *x_routed, uint32_t *status_dev,
+                              uint32_t mail_seq, void *stream)
 {
     if (!h || !s || !r || !status_dev) return MOE_ERR_NULL;
     if (s->T < 0 || s->H < 64 || s->H % 16 != 0 || s->I < 16 || s->I % 16 != 0 || s->E_tot < 1 || s->k_tot < 1 ||
@@ -367,6 +389,11 @@ extern "C" int32_t moe_gemm1_act(moe_handle *h, const void *hidden, const void *
     p.status = status_dev;
     p.wait_ns = h->wait_ns;
     p.S = n_mtiles;
+    if (mail_seq != 0u && counts_on_device) {
+        p.mail = h->mail_dev;
+        p.mail_seq = mail_seq;
+        p.E_tot = s->E_tot;
+    }
     p.sub = tile_m == 256 ? 2 : 1;
     p.sub_rows = tile_m < kMmaM ? tile_m : kMmaM;
     p.I = s->I;
@@ -406,19 +433,22 @@ extern "C" int32_t moe_gemm1_act(moe_handle *h, const void *hidden, const void *
 
     // gather (the rows of a token are read k_tot times, from L2 after the first)
     const int row_vec = s->H * 2 / 16;
-    const unsigned gather_blocks = (unsigned)(((int64_t)R * 32 + 255) / 256);
-    gather_rows<<<gather_blocks, 256, 0, st>>>(static_cast<const uint4 *>(hidden), r->perm, R, s->k_tot, row_vec,
-                                               static_cast<uint4 *>(h_routed_ws));
-    cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1] = {chained_launch_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)(((int64_t)R * 32 + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gather_rows, static_cast<const uint4 *>(hidden), static_cast<const int32_t *>(r->perm), R,
+                                       (int)s->k_tot, row_vec, static_cast<uint4 *>(h_routed_ws));
     if (e != cudaSuccess) return cuda_fail(h, e, "gather_rows launch");
 
-    const size_t smem = g1_smem_bytes();
-    e = cudaFuncSetAttribute(moe_gemm1_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(h, e, "gemm1 shared memory attribute");
     const int64_t tiles_bound = (int64_t)n_mtiles * p.sub * p.NT;
-    const int grid = (int)(tiles_bound < h->G ? (tiles_bound > 0 ? tiles_bound : 1) : h->G);
-    moe_gemm1_act_kernel<<<grid, kThreads, smem, st>>>(p);
-    e = cudaGetLastError();
+    cfg.gridDim = dim3((unsigned)(tiles_bound < h->G ? (tiles_bound > 0 ? tiles_bound : 1) : h->G));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = g1_smem_bytes();
+    e = cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel, p);
     if (e != cudaSuccess) return cuda_fail(h, e, "gemm1 launch");
     return MOE_OK;
 }

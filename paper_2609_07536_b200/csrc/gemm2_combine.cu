@@ -180,6 +180,11 @@ __device__ __forceinline__ int epi_cols_per_group(int tn, int groups)
     return ((tn / 32 + groups - 1) / groups) * 32;
 }
 
+// What a launch's roles are divided by: compute tiles per split (Eq. 5), communication CTAs, compute slots.
+struct Part {
+    int W_comp, C, P;
+};
+
 struct Tile {
     int s, mu, p, i_n;
     int id;   // canonical tile number s * W_comp + (mu * TP + p) * NTs + i_n: indexes the readiness flags
@@ -364,11 +369,11 @@ __device__ __forceinline__ void store_accumulator_rows_staged(const FusedParams 
 // Epilogue, one warp: TMEM -> bf16 -> Y for the warp's TMEM lane quarter and column group of every tile of
 // this CTA, then the hand-over to the publisher warp.
 template <int TN, bool kPair>
-__device__ __forceinline__ void epilogue_role(const FusedParams &P, int W_comp, Control *ctl, uint8_t *aux, int b,
+__device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &pt, Control *ctl, uint8_t *aux, int b,
                                               uint32_t tmem_base, unsigned long long deadline, int rank)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int total_tiles = P.L * W_comp;
+    const int total_tiles = P.L * pt.W_comp;
     const int q4 = warp & 3;                   // TMEM lane quarter this warp may read
     const int grp = (warp - 4) >> 2;           // column group of the tile
     const int cols_per_group = epi_cols_per_group(TN, P.epi_warps >> 2);
@@ -382,23 +387,23 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, int W_comp, 
     int valid = 0, f_row = 0, valid_n = 0, first_n = 0;
     TL_DECL(long long tl_ew = 0, tl_ek = 0, tl_ep = 0, tl_q;)
     if (b < total_tiles) {
-        const int mu0 = decode_tile(b, P, W_comp).mu;
-        const int mu1 = decode_tile(min(b + P.P, total_tiles - 1), P, W_comp).mu;
-        valid = __ldg(&P.mtile_valid[mu0]);
-        const int first0 = __ldg(&P.mtile_first_row[mu0]);
-        valid_n = __ldg(&P.mtile_valid[mu1]);
-        first_n = __ldg(&P.mtile_first_row[mu1]);
-        if (row_in_tile < valid) f_row = __ldg(&P.perm[first0 + row_in_tile]);
+        const int mu0 = decode_tile(b, P, pt.W_comp).mu;
+        const int mu1 = decode_tile(min(b + pt.P, total_tiles - 1), P, pt.W_comp).mu;
+        valid = ld_chained(&P.mtile_valid[mu0]);
+        const int first0 = ld_chained(&P.mtile_first_row[mu0]);
+        valid_n = ld_chained(&P.mtile_valid[mu1]);
+        first_n = ld_chained(&P.mtile_first_row[mu1]);
+        if (row_in_tile < valid) f_row = ld_chained(&P.perm[first0 + row_in_tile]);
     }
     int it = 0;
-    for (int g = b; g < total_tiles; g += P.P, ++it) {
-        const Tile t = decode_tile(g, P, W_comp);
+    for (int g = b; g < total_tiles; g += pt.P, ++it) {
+        const Tile t = decode_tile(g, P, pt.W_comp);
         const int a = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
-        const int mu_nn = decode_tile(min(g + 2 * P.P, total_tiles - 1), P, W_comp).mu;
-        const int valid_nn = __ldg(&P.mtile_valid[mu_nn]);
-        const int first_nn = __ldg(&P.mtile_first_row[mu_nn]);
-        const int f_row_n = (row_in_tile < valid_n) ? __ldg(&P.perm[first_n + row_in_tile]) : 0;
+        const int mu_nn = decode_tile(min(g + 2 * pt.P, total_tiles - 1), P, pt.W_comp).mu;
+        const int valid_nn = ld_chained(&P.mtile_valid[mu_nn]);
+        const int first_nn = ld_chained(&P.mtile_first_row[mu_nn]);
+        const int f_row_n = (row_in_tile < valid_n) ? ld_chained(&P.perm[first_n + row_in_tile]) : 0;
         TL(tl_q = clock64());
         bool ok = wait_barrier(smem_u32(&ctl->tmem_full[a]), acc_phase, ctl, deadline, P.status, (uint32_t)g, 30u);
         TL(tl_ew += clock64() - tl_q; tl_q = clock64());
@@ -460,10 +465,10 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, int W_comp, 
 // the path of the epilogue warps, which go straight on to the next accumulator, and one fence covers every tile
 // whose epilogue has finished by then (up to kPubSlots).
 template <bool kPair>
-__device__ __forceinline__ void publisher_role(const FusedParams &P, int W_comp, Control *ctl, int b,
+__device__ __forceinline__ void publisher_role(const FusedParams &P, const Part &pt, Control *ctl, int b,
                                                unsigned long long deadline, int rank)
 {
-    const int total_tiles = P.L * W_comp;
+    const int total_tiles = P.L * pt.W_comp;
     if ((threadIdx.x & 31) == 0) {
         int it = 0;
         TL_DECL(long long tl_pw = 0, tl_pf = 0, tl_q;)
@@ -476,16 +481,16 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, int W_comp,
             // the following tiles too, as far as their epilogues are already over (waiting for more of them before
             // the fence was measured: no gain)
             int n = 1;
-            while (n < kPubSlots && g + n * P.P < total_tiles &&
+            while (n < kPubSlots && g + n * pt.P < total_tiles &&
                    mbar_test_wait(smem_u32(&ctl->epi_done[(it + n) & (kPubSlots - 1)]), (uint32_t)((it + n) / kPubSlots) & 1u))
                 ++n;
             fence_acq_rel_gpu();   // release: the epilogue warps' stores (observed through epi_done) come first
-            for (int j = 0; j < n; ++j, ++it, g += P.P) {
-                const Tile t = decode_tile(g, P, W_comp);
+            for (int j = 0; j < n; ++j, ++it, g += pt.P) {
+                const Tile t = decode_tile(g, P, pt.W_comp);
                 if (t.id != P.withhold) {
                     st_relaxed_u32(&P.flags[kPair ? 2 * t.id + rank : t.id], P.epoch);
 #if MOE_TIMELINE
-                    if (atomicAdd(&P.split_done[t.s], 1u) + 1u == (uint32_t)(W_comp * P.flag_parts) && P.timeline)
+                    if (atomicAdd(&P.split_done[t.s], 1u) + 1u == (uint32_t)(pt.W_comp * P.flag_parts) && P.timeline)
                         P.timeline[(size_t)gridDim.x * kTimelineSlots + t.s] = globaltimer_ns();
 #else
                     red_relaxed_add_u32(&P.split_done[t.s], 1u);
@@ -503,11 +508,11 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, int W_comp,
 // --------------------------------------------------------------------------- compute CTA
 
 template <int TN>
-__device__ void compute_cta(const FusedParams &P, int W_comp, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
+__device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
 {
     using C = Cfg<TN>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int total_tiles = P.L * W_comp;
+    const int total_tiles = P.L * pt.W_comp;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
     // setup: barriers (thread 0), TMEM allocation (warp 1)
@@ -546,13 +551,13 @@ __device__ void compute_cta(const FusedParams &P, int W_comp, uint8_t *ring, Con
             TL_DECL(long long tl_pw = 0, tl_q;)
             // the m-tile table entries of the NEXT tile are fetched while this tile's k-blocks are issued, so
             // that the two dependent global loads never stall the stream of copies at a tile boundary
-            Tile t = decode_tile(b, P, W_comp);
-            int e = __ldg(&P.mtile_expert[t.mu]);
-            int row0 = __ldg(&P.mtile_first_row[t.mu]);
-            for (int g = b; g < total_tiles && ok; g += P.P) {
-                const Tile t_next = decode_tile(min(g + P.P, total_tiles - 1), P, W_comp);
-                const int e_next = __ldg(&P.mtile_expert[t_next.mu]);
-                const int row0_next = __ldg(&P.mtile_first_row[t_next.mu]);
+            Tile t = decode_tile(b, P, pt.W_comp);
+            int e = ld_chained(&P.mtile_expert[t.mu]);
+            int row0 = ld_chained(&P.mtile_first_row[t.mu]);
+            for (int g = b; g < total_tiles && ok; g += pt.P) {
+                const Tile t_next = decode_tile(min(g + pt.P, total_tiles - 1), P, pt.W_comp);
+                const int e_next = ld_chained(&P.mtile_expert[t_next.mu]);
+                const int row0_next = ld_chained(&P.mtile_first_row[t_next.mu]);
                 const int n0 = t.s * P.split_w + t.i_n * TN;
                 int kx = t.p * P.K;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
@@ -609,7 +614,7 @@ __device__ void compute_cta(const FusedParams &P, int W_comp, uint8_t *ring, Con
             int it = 0;
             bool ok = true;
             TL_DECL(const long long tl_c0 = clock64(); long long tl_wf = 0, tl_wt = 0, tl_is = 0, tl_q;)
-            for (int g = b; g < total_tiles && ok; g += P.P, ++it) {
+            for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
                 const int a = it & 1;
                 const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
                 TL(tl_q = clock64());
@@ -664,9 +669,9 @@ __device__ void compute_cta(const FusedParams &P, int W_comp, uint8_t *ring, Con
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        epilogue_role<TN, false>(P, W_comp, ctl, aux, b, tmem_base, deadline, 0);
+        epilogue_role<TN, false>(P, pt, ctl, aux, b, tmem_base, deadline, 0);
     } else if (warp == 3) {
-        publisher_role<false>(P, W_comp, ctl, b, deadline, 0);
+        publisher_role<false>(P, pt, ctl, b, deadline, 0);
     }
     // ---------------- teardown
     tc_fence_before();
@@ -697,14 +702,14 @@ struct PairCfg {
     static constexpr int kTmemCols = 2 * kTileN;                        // two accumulator buffers
 };
 
-__device__ void compute_cta_pair(const FusedParams &P, int W_comp, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
+__device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
 {
     using C = PairCfg;
     constexpr int TN = C::kTileN;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader_cta = (rank == 0);
-    const int total_tiles = P.L * W_comp;
+    const int total_tiles = P.L * pt.W_comp;
     const int n_stages = P.pair_stages;   // 6, or 7 with the aux region as one more stage
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
@@ -744,13 +749,13 @@ __device__ void compute_cta_pair(const FusedParams &P, int W_comp, uint8_t *ring
             bool ok = true;
             TL_DECL(long long tl_pw = 0, tl_q;)
             // next tile's table entries are fetched one tile ahead (see compute_cta)
-            Tile t = decode_tile(b, P, W_comp);
-            int e = __ldg(&P.mtile_expert[t.mu]);
-            int row0 = __ldg(&P.mtile_first_row[t.mu]) + (int)rank * kMmaM;
-            for (int g = b; g < total_tiles && ok; g += P.P) {
-                const Tile t_next = decode_tile(min(g + P.P, total_tiles - 1), P, W_comp);
-                const int e_next = __ldg(&P.mtile_expert[t_next.mu]);
-                const int row0_next = __ldg(&P.mtile_first_row[t_next.mu]) + (int)rank * kMmaM;
+            Tile t = decode_tile(b, P, pt.W_comp);
+            int e = ld_chained(&P.mtile_expert[t.mu]);
+            int row0 = ld_chained(&P.mtile_first_row[t.mu]) + (int)rank * kMmaM;
+            for (int g = b; g < total_tiles && ok; g += pt.P) {
+                const Tile t_next = decode_tile(min(g + pt.P, total_tiles - 1), P, pt.W_comp);
+                const int e_next = ld_chained(&P.mtile_expert[t_next.mu]);
+                const int row0_next = ld_chained(&P.mtile_first_row[t_next.mu]) + (int)rank * kMmaM;
                 const int n0 = t.s * P.split_w + t.i_n * TN + (int)rank * (TN / 2);
                 int kx = t.p * P.K;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
@@ -813,7 +818,7 @@ __device__ void compute_cta_pair(const FusedParams &P, int W_comp, uint8_t *ring
             int it = 0;
             bool ok = true;
             TL_DECL(const long long tl_c0 = clock64(); long long tl_wf = 0, tl_wt = 0, tl_is = 0, tl_q; unsigned long long tl_late = 0;)
-            for (int g = b; g < total_tiles && ok; g += P.P, ++it) {
+            for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
                 const int a = it & 1;
                 const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
                 TL(tl_q = clock64());
@@ -874,9 +879,9 @@ __device__ void compute_cta_pair(const FusedParams &P, int W_comp, uint8_t *ring
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        epilogue_role<TN, true>(P, W_comp, ctl, aux, b, tmem_base, deadline, (int)rank);
+        epilogue_role<TN, true>(P, pt, ctl, aux, b, tmem_base, deadline, (int)rank);
     } else if (warp == 3) {
-        publisher_role<true>(P, W_comp, ctl, b, deadline, (int)rank);
+        publisher_role<true>(P, pt, ctl, b, deadline, (int)rank);
     }
     // ---------------- teardown: nobody leaves while its peer may still touch its memory (the co-resident
     // communication warps arrived on this cluster barrier right after the set-up one)
@@ -981,7 +986,7 @@ struct CommUnit {
 
 // `c`, `warp`: communication CTA and warp inside it (static map only).
 template <int TN>
-__device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const CommWarpRes res, int role, int c, int warp,
+__device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, const CommWarpRes res, int role, int c, int warp,
                           int tl_slot)
 {
     (void)tl_slot;   // index of the warp's record in a timeline build
@@ -1104,7 +1109,7 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
             uint32_t done = 0;
             if (lane == 0) done = ld_acquire_u32(&P.split_done[u.s]);
             done = __shfl_sync(0xffffffffu, done, 0);
-            if (done >= (uint32_t)(W_comp * P.flag_parts)) {
+            if (done >= (uint32_t)(pt.W_comp * P.flag_parts)) {
                 ready_mask |= 1u << u.s;
             } else {
                 // per tile: every (slot j, shard p, n-tile under this slab)
@@ -1117,12 +1122,12 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
                     const int tn = chk - qq * nt;
                     const int j = qq / P.TP;
                     const int p = qq - j * P.TP;
-                    const int row = __ldg(&P.pad_row[(size_t)u.t * P.k_tot + j]);
+                    const int row = ld_chained(&P.pad_row[(size_t)u.t * P.k_tot + j]);
                     if (row < 0 || row >= P.R_pad) continue;
                     const int mu = row / P.tile_m;
                     // a pair tile is published in two parts, one per CTA: the row's part is its 128-row half
                     const int part = (P.flag_parts == 2) ? ((row - mu * P.tile_m) >> 7) : 0;
-                    const int g = (u.s * W_comp + (mu * P.TP + p) * P.NTs + in0 + tn) * P.flag_parts + part;
+                    const int g = (u.s * pt.W_comp + (mu * P.TP + p) * P.NTs + in0 + tn) * P.flag_parts + part;
                     uint32_t spins = 0;
                     TL_DECL(const unsigned long long tl_f0 = globaltimer_ns();)
                     while (ld_acquire_u32(&P.flags[g]) != P.epoch) {
@@ -1192,8 +1197,8 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
         float nxt_w = 0.f;
         if (k < n_units && lane < P.k_tot) {
             const int tn = t0 + k / n_slabs;
-            nxt_row = __ldg(&P.pad_row[(size_t)tn * P.k_tot + lane]);
-            nxt_w = __ldg(&P.topk_w[(size_t)tn * P.k_tot + lane]);
+            nxt_row = ld_chained(&P.pad_row[(size_t)tn * P.k_tot + lane]);
+            nxt_w = ld_chained(&P.topk_w[(size_t)tn * P.k_tot + lane]);
         }
         for (; k < n_units; k += kCommWarps) {
             CommUnit u;
@@ -1208,8 +1213,8 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
             u.w = nxt_w;
             if (k + kCommWarps < n_units && lane < P.k_tot) {
                 const int tn = t0 + (k + kCommWarps) / n_slabs;
-                nxt_row = __ldg(&P.pad_row[(size_t)tn * P.k_tot + lane]);
-                nxt_w = __ldg(&P.topk_w[(size_t)tn * P.k_tot + lane]);
+                nxt_row = ld_chained(&P.pad_row[(size_t)tn * P.k_tot + lane]);
+                nxt_w = ld_chained(&P.topk_w[(size_t)tn * P.k_tot + lane]);
             }
             if (lane < P.k_tot) {
                 if (my_row >= P.R_pad) {
@@ -1237,8 +1242,8 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
         float nxt_w = 0.f;
         if (lane < P.k_tot) {
             const int tn = (int)(i0 / (uint32_t)P.comm_cols);
-            nxt_row = __ldg(&P.pad_row[(size_t)tn * P.k_tot + lane]);
-            nxt_w = __ldg(&P.topk_w[(size_t)tn * P.k_tot + lane]);
+            nxt_row = ld_chained(&P.pad_row[(size_t)tn * P.k_tot + lane]);
+            nxt_w = ld_chained(&P.topk_w[(size_t)tn * P.k_tot + lane]);
         }
         for (uint32_t item = i0; item < i1; ++item) {
             const int tok = (int)(item / (uint32_t)P.comm_cols);
@@ -1247,8 +1252,8 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
             float my_w = nxt_w;
             if (item + 1 < i1 && lane < P.k_tot) {
                 const int tn = (int)((item + 1) / (uint32_t)P.comm_cols);
-                nxt_row = __ldg(&P.pad_row[(size_t)tn * P.k_tot + lane]);
-                nxt_w = __ldg(&P.topk_w[(size_t)tn * P.k_tot + lane]);
+                nxt_row = ld_chained(&P.pad_row[(size_t)tn * P.k_tot + lane]);
+                nxt_w = ld_chained(&P.topk_w[(size_t)tn * P.k_tot + lane]);
             }
             if (lane < P.k_tot) {
                 if (my_row >= P.R_pad) {
@@ -1283,7 +1288,7 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
     if (role == kRoleStatic) {
         // the paper's static map: communication tile ct belongs to CTA ct mod C (Section III-A)
         for (int s = 0; s < P.L; ++s)
-            for (int ct = c; ct < P.comm_tiles; ct += P.C)
+            for (int ct = c; ct < P.comm_tiles; ct += pt.C)
                 if (!serve_tile(s, ct)) {
                     ctl->abort = 1u;
                     return;
@@ -1317,7 +1322,7 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
                     // token is complete before the split is: wait for the whole split, asleep most of the time.
                     uint32_t state = 0;   // 1: split complete, 2: split handed out already, 3: give up
                     if (lane == 0) {
-                        if (ld_acquire_u32(&P.split_done[s]) >= (uint32_t)(W_comp * P.flag_parts)) state = 1;
+                        if (ld_acquire_u32(&P.split_done[s]) >= (uint32_t)(pt.W_comp * P.flag_parts)) state = 1;
                         else {
                             const unsigned long long q = *reinterpret_cast<volatile unsigned long long *>(&P.queue[s]);
                             if ((uint32_t)q + (uint32_t)(q >> 32) >= n_items) state = 2;
@@ -1395,7 +1400,7 @@ __device__ void comm_warp(const FusedParams &P, int W_comp, Control *ctl, const 
 // The communication warps of a CTA whose only role is communication (dedicated communication CTA, or a
 // compute CTA that has run out of GEMM tiles): warps 0-11, stages in the operand ring.
 template <int TN>
-__device__ __forceinline__ void comm_cta(const FusedParams &P, int W_comp, uint8_t *ring, Control *ctl, uint8_t *aux, int role, int c)
+__device__ __forceinline__ void comm_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int role, int c)
 {
     const int warp = threadIdx.x >> 5;
     if (warp >= kCommWarps) return;
@@ -1405,19 +1410,19 @@ __device__ __forceinline__ void comm_cta(const FusedParams &P, int W_comp, uint8
     res.wq = (role == kRoleBack && P.co_warps > 0)
                  ? reinterpret_cast<float *>(aux + kCoWeightsOffset) + (kCoWarpsMax + warp) * kCoWeightFloats
                  : reinterpret_cast<float *>(aux) + warp * 256;
-    comm_warp<TN>(P, W_comp, ctl, res, role, c, warp, warp);
+    comm_warp<TN>(P, pt, ctl, res, role, c, warp, warp);
 }
 
 // Co-resident communication warp `cw` of a compute CTA: stages and weights in the aux region (free when
 // the epilogue stores straight from registers, which the host checks before it asks for such warps).
 template <int TN>
-__device__ __forceinline__ void co_resident_warp(const FusedParams &P, int W_comp, Control *ctl, uint8_t *aux, int cw)
+__device__ __forceinline__ void co_resident_warp(const FusedParams &P, const Part &pt, Control *ctl, uint8_t *aux, int cw)
 {
     CommWarpRes res;
     res.stages = aux + cw * kCommWarpBytes;
     res.full = &ctl->co_full[2 * cw];
     res.wq = reinterpret_cast<float *>(aux + kCoWeightsOffset) + cw * kCoWeightFloats;
-    comm_warp<TN>(P, W_comp, ctl, res, kRoleCoResident, 0, 0, cw);
+    comm_warp<TN>(P, pt, ctl, res, kRoleCoResident, 0, 0, cw);
 }
 
 // Co-resident warp number of warp 16..19.  The four warp schedulers of an SM take warps by number modulo
@@ -1443,11 +1448,22 @@ __device__ __forceinline__ void init_comm_barriers(Control *ctl)
 
 // --------------------------------------------------------------------------- kernel
 
-// Compute tiles per split of this launch (Eq. 5).  With the routed counts left on the device the m-tile
-// count is read from the routing workspace (the routing kernels ran earlier on the same stream).
-__device__ __forceinline__ int launch_w_comp(const FusedParams &P)
+// The launch's partition.  With the routed counts left on the device the m-tile count S is read from the routing
+// workspace (the routing kernel ran earlier on the same stream); with the selector's picks tabulated over S
+// (FusedParams::c_table) the communication-CTA count is looked up by it, so that no host wait lies between the
+// routing build and this launch.
+__device__ __forceinline__ Part launch_part(const FusedParams &P)
 {
-    return P.S_dev ? min(__ldg(P.S_dev), P.S) * P.TP * P.NTs : P.W_comp;
+    Part pt = {P.W_comp, P.C, P.P};
+    if (P.S_dev) {
+        const int S = ld_chained_uniform(P.S_dev);
+        pt.W_comp = min(S, P.S) * P.TP * P.NTs;
+        if (P.c_table_n > 0) {
+            pt.C = P.c_table[max(0, min(S - P.c_table_first, P.c_table_n - 1))];
+            pt.P = (P.G - pt.C) / P.slot_sms;
+        }
+    }
+    return pt;
 }
 
 template <int TN>
@@ -1460,26 +1476,33 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
     Control *ctl = reinterpret_cast<Control *>(ring + kStageBytesTotal);
     uint8_t *aux = reinterpret_cast<uint8_t *>(ring + kStageBytesTotal + ((sizeof(Control) + 127) & ~(size_t)127));
 
+    init_comm_barriers(ctl);
+    if (threadIdx.x == 32) {
+        prefetch_tensormap(&P.tmA);
+        prefetch_tensormap(&P.tmB);
+    }
+    grid_dependency_wait();
     if (blockIdx.x == 0 && threadIdx.x < (unsigned)P.L) {
         P.split_done_next[threadIdx.x] = 0u;
         P.queue_next[threadIdx.x] = 0ull;
     }
-    init_comm_barriers(ctl);
+    const Part pt = launch_part(P);
     __syncthreads();          // the only barrier all 20 warps share
-    TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < P.C ? 0u : 1u); });
+    TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < pt.C ? 0u : 1u); });
 
     const int warp = threadIdx.x >> 5;
-    const int W_comp = launch_w_comp(P);
-    if ((int)blockIdx.x < P.C) {
-        comm_cta<TN>(P, W_comp, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
+    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // an idle warp of communication CTA 0
+        mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
+    if ((int)blockIdx.x < pt.C) {
+        comm_cta<TN>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
     } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
-        if (co_warp_number(warp) < P.co_warps) co_resident_warp<TN>(P, W_comp, ctl, aux, co_warp_number(warp));
+        if (co_warp_number(warp) < P.co_warps) co_resident_warp<TN>(P, pt, ctl, aux, co_warp_number(warp));
         return;
     } else {
-        compute_cta<TN>(P, W_comp, ring, ctl, aux, (int)blockIdx.x - P.C);
+        compute_cta<TN>(P, pt, ring, ctl, aux, (int)blockIdx.x - pt.C);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         // out of GEMM tiles: help with the communication that is left (all TMA and TMEM traffic is over)
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !ctl->abort) comm_cta<TN>(P, W_comp, ring, ctl, aux, kRoleBack, 0);
+        if (P.drain_help && P.mode == MOE_MODE_FUSED && !ctl->abort) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleBack, 0);
     }
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
@@ -1500,36 +1523,43 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
     uint8_t *aux = seven ? ring + kStageBytesTotal
                          : reinterpret_cast<uint8_t *>(ring + kStageBytesTotal + ((sizeof(Control) + 127) & ~(size_t)127));
 
+    init_comm_barriers(ctl);
+    if (threadIdx.x == 32) {
+        prefetch_tensormap(&P.tmA);
+        prefetch_tensormap(&P.tmB);
+    }
+    grid_dependency_wait();
     if (blockIdx.x == 0 && threadIdx.x < (unsigned)P.L) {
         P.split_done_next[threadIdx.x] = 0u;
         P.queue_next[threadIdx.x] = 0ull;
     }
-    init_comm_barriers(ctl);
+    const Part pt = launch_part(P);
     __syncthreads();          // the only CTA-wide barrier all 20 warps share
-    TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < ((P.C + 1) & ~1) ? 0u : 1u); });
+    TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < ((pt.C + 1) & ~1) ? 0u : 1u); });
 
     const int warp = threadIdx.x >> 5;
-    const int c_even = (P.C + 1) & ~1;
-    const int W_comp = launch_w_comp(P);
-    if ((int)blockIdx.x < P.C) {
-        comm_cta<256>(P, W_comp, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
+    const int c_even = (pt.C + 1) & ~1;
+    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // an idle warp of communication CTA 0
+        mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
+    if ((int)blockIdx.x < pt.C) {
+        comm_cta<256>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
     } else if ((int)blockIdx.x < c_even) {
         // odd C: the last communication CTA's cluster-mate cannot compute (no partner).  With dynamic work
         // distribution it serves communication work as well; under the static map it has no tile list.
-        if (P.drain_help && P.mode == MOE_MODE_FUSED) comm_cta<256>(P, W_comp, ring, ctl, aux, kRoleFront, (int)blockIdx.x);
+        if (P.drain_help && P.mode == MOE_MODE_FUSED) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront, (int)blockIdx.x);
     } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
         // The compute warps of both CTAs meet at two cluster barriers (set-up and teardown), and a cluster
         // barrier counts every thread: these warps join the first, arrive at once on the second (they hold
         // nothing a peer could touch) and pick its completion up when their own work is done.
         cluster_sync_all();
         cluster_arrive();
-        if (co_warp_number(warp) < P.co_warps) co_resident_warp<256>(P, W_comp, ctl, aux, co_warp_number(warp));
+        if (co_warp_number(warp) < P.co_warps) co_resident_warp<256>(P, pt, ctl, aux, co_warp_number(warp));
         cluster_wait();
         return;
     } else {
-        compute_cta_pair(P, W_comp, ring, ctl, aux, ((int)blockIdx.x - c_even) >> 1);
+        compute_cta_pair(P, pt, ring, ctl, aux, ((int)blockIdx.x - c_even) >> 1);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !ctl->abort) comm_cta<256>(P, W_comp, ring, ctl, aux, kRoleBack, 0);
+        if (P.drain_help && P.mode == MOE_MODE_FUSED && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack, 0);
     }
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
@@ -1597,26 +1627,33 @@ cudaError_t pair_launch(const FusedParams &p, int grid, cudaStream_t stream)
     cfg.blockDim = dim3(kFusedThreads);
     cfg.dynamicSmemBytes = fused_smem_bytes(256);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0] = chained_launch_attribute();
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, moe_gemm2_combine_pair_kernel, p);
 }
 
 cudaError_t fused_launch(int tile_n, const FusedParams &p, int grid, cudaStream_t stream)
 {
-    const size_t sm = fused_smem_bytes(tile_n);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kFusedThreads);
+    cfg.dynamicSmemBytes = fused_smem_bytes(tile_n);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1] = {chained_launch_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     switch (tile_n) {
-    case 64: moe_gemm2_combine_kernel<64><<<grid, kFusedThreads, sm, stream>>>(p); break;
-    case 128: moe_gemm2_combine_kernel<128><<<grid, kFusedThreads, sm, stream>>>(p); break;
-    case 256: moe_gemm2_combine_kernel<256><<<grid, kFusedThreads, sm, stream>>>(p); break;
-    default: return cudaErrorInvalidValue;
+    case 64: return cudaLaunchKernelEx(&cfg, moe_gemm2_combine_kernel<64>, p);
+    case 128: return cudaLaunchKernelEx(&cfg, moe_gemm2_combine_kernel<128>, p);
+    case 256: return cudaLaunchKernelEx(&cfg, moe_gemm2_combine_kernel<256>, p);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace moe

@@ -6,6 +6,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <cstring>
 #include <unordered_map>
 
 #include "../../include/moe_b200.h"
@@ -22,6 +23,7 @@ constexpr int kStageBytesTotal = 192 * 1024;  // operand ring, all stages togeth
 constexpr int kCommTileM = 128;        // T_M^comm
 constexpr int kCommTileN = 1024;       // T_N^comm
 constexpr int kMailWords = 1024 + 1 + 31;   // the handle's count mailbox: one (count, sequence number) word per expert, then S
+constexpr int kPlanTableMax = 256;     // m-tile counts a tabulated selection may span (a shape has E_tot + 1 or fewer)
 constexpr int kRoutingChunk = 256;     // flat assignments handled by one warp while sorting
 constexpr uint64_t kDefaultWaitNs = 2000000000ull;
 constexpr int kTimelineSlots = 40;     // 64-bit words per CTA in a timeline buffer (timeline build only)
@@ -53,6 +55,12 @@ struct alignas(64) FusedParams {
     int32_t T, H, K, TP, EP, L, k_tot;
     int32_t S, tile_m, NTs, split_w, W_comp;
     int32_t C, P, mode, withhold;
+    unsigned long long *mail;           // != nullptr: the tile counts (S_dev - E_tot) are mailed to the host by this launch
+    uint32_t mail_seq;
+    int32_t E_tot;
+    int32_t G, slot_sms;                // c_table: SMs the partition is made of, SMs of one compute slot
+    int32_t c_table_first, c_table_n;   // c_table[i]: communication CTAs when S = c_table_first + i (0 entries: C and P above hold)
+    uint8_t c_table[kPlanTableMax];
     int32_t tok_blk, tok_tiles_per_rank, comm_cols, comm_tiles;
     int32_t num_kb, last_ksteps;
     int32_t drain_help;                 // compute CTAs serve communication tiles once their GEMM tiles are done
@@ -76,6 +84,17 @@ struct TensorMapKey {
     const void *x, *w2;
     int32_t T, k_tot, I, H, E_tot, box_n;
 };
+// The selector's pick for every m-tile count S that a routing of one shape can have: plan_partition depends on the
+// routed counts through their sum alone (but for tile-level readiness, which is not tabulated).
+struct PlanTable {
+    moe_shape shape;
+    int32_t tile_m, tile_n;
+    moe_sm_limits limits;
+    int32_t first, n;              // S = first .. first + n - 1; n = 0: not to be tabulated
+    moe_plan plan;                 // what all picks have in common, and the pick for `first`
+    uint8_t C[kPlanTableMax];
+};
+constexpr int kPlanTables = 8;     // shapes a handle keeps tabulated; the oldest goes first
 }  // namespace moe
 
 struct moe_handle {
@@ -103,9 +122,62 @@ struct moe_handle {
     CUtensorMap tmA, tmB;                               // last encoded operand tensor maps of the fused kernel ...
     moe::TensorMapKey tm_key = {};                      // ... and what they were encoded for
     bool tm_valid = false;
+    moe::PlanTable *plan_tables = nullptr;              // [kPlanTables], used as a ring
+    int n_plan_tables = 0, next_plan_table = 0;
 };
 
 namespace moe {
+
+// Every kernel of this library may be launched before its predecessor on the stream has finished: each waits for the
+// predecessor's writes (griddepcontrol.wait) before it touches global memory, so that the launch latencies and
+// prologues of a step's kernels lie beside the end of the kernel before.  Only the short kernels (routing, gather) let
+// their successor start early; behind the long ones it starts as they end.  CTAs that sit and wait on the SMs that a
+// long kernel leaves idle cost more than they save: whole step at T = 1 / 16 / 256 on the DeepSeek shape 73.2 / 72.4 /
+// 102.7 us with early starts everywhere, 68.2 / 69.7 / 99.1 as it is, 77.2 / 74.1 / 103.5 without chained launches.
+inline cudaLaunchAttribute chained_launch_attribute()
+{
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// (after the wait, so that everything before this kernel is complete when a successor starts)
+__device__ __forceinline__ void grid_dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Load of what a predecessor may have written: an ordinary load that stays behind the wait (a read-only __ldg may be moved)
+template <typename T>
+__device__ __forceinline__ T ld_chained(const T *p)
+{
+    static_assert(sizeof(T) == 4, "32-bit values");
+    uint32_t v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    T t;
+    memcpy(&t, &v, 4);
+    return t;
+}
+// The same for a count that every thread of a converged warp reads: the reduction makes the value warp-uniform for the
+// compiler as well, so that the loops it bounds keep their operands in uniform registers (the loop that issues the
+// MMAs is 5 % slower over a whole GEMM1 launch when it cannot)
+__device__ __forceinline__ int ld_chained_uniform(const int32_t *p)
+{
+    return (int)__reduce_max_sync(0xffffffffu, (unsigned)ld_chained(p));
+}
+
+// The tile counts for the host, written straight into host memory the GPU can address (`mail`, or nullptr), by one
+// warp: word x is the pair (count x, seq), x = 0..E_tot, the last one S.  A 64-bit store arrives whole, so every
+// word says by itself whether it belongs to this call: no fence orders anything here.  (Plain counts followed by a
+// sequence number needed system-scope fences of the whole CTA, 4-5 us of a small build's 12.)  A kernel is complete
+// only when these stores have crossed the bus, so they are left to the kernel behind the routing build where one
+// follows without waiting for the host.
+template <class Count>
+__device__ __forceinline__ void mail_counts(unsigned long long *mail, uint32_t seq, int E_tot, int lane, Count count)
+{
+    if (!mail) return;
+    for (int x = lane; x <= E_tot; x += 32)
+        *reinterpret_cast<volatile unsigned long long *>(mail + x) = ((unsigned long long)seq << 32) | (uint32_t)count(x);
+}
+#endif
 
 inline int tile_n_slot(int tile_n) { return tile_n == 64 ? 0 : tile_n == 128 ? 1 : tile_n == 256 ? 2 : -1; }
 
@@ -123,6 +195,11 @@ bool fused_timeline_build();   // the library was compiled with -DMOE_TIMELINE=1
 // CTA-pair kernel (256 x 256 tiles, clusters of two)
 cudaError_t pair_occupancy(int *blocks_per_sm, int *max_clusters);
 cudaError_t pair_launch(const FusedParams &p, int grid, cudaStream_t stream);
+// GEMM1 (gemm1_act.cu): once per device, kernel attributes
+cudaError_t gemm1_prepare();
+// moe_gemm1_act; mail_seq != 0: this launch mails the tile counts (with MOE_MTILES_ON_DEVICE)
+int32_t launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const moe_shape *s, int32_t tile_m, const moe_routing *r,
+                         int32_t n_mtiles, void *h_routed_ws, void *x_routed, uint32_t *status_dev, uint32_t mail_seq, void *stream);
 // routing kernels (routing.cu)
 // once per device: kernel attributes, and the largest cluster the one-launch build can run with
 cudaError_t routing_prepare(int *max_cluster);

@@ -25,14 +25,6 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kPerLane = kRoutingChunk / 32;   // assignments of a chunk held by one lane
 static_assert(kRoutingChunk % 32 == 0, "a chunk is a whole number of warp-wide rows");
 
-// The four launches of the large path are chained with programmatic stream serialization: a launch may be
-// set up while its predecessor still runs, and waits here, first thing, until the predecessor's writes are
-// visible.  Without that launch attribute this returns at once.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// lets the next kernel on the stream, if it was launched that way, be set up beside this one (after the wait above,
-// so that everything before this kernel is complete by then)
-__device__ __forceinline__ void grid_dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // launch `kernel` so that it may be set up before the previous kernel on the stream has finished
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
@@ -43,8 +35,7 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0] = chained_launch_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
@@ -71,7 +62,7 @@ __device__ __forceinline__ void chunk_load(const int32_t *__restrict__ topk_idx,
 #pragma unroll
     for (int i = 0; i < kPerLane; ++i) {
         const int f = begin + 32 * i + lane;
-        e[i] = f < end ? __ldg(topk_idx + f) : -1;
+        e[i] = f < end ? ld_chained(topk_idx + f) : -1;
     }
 }
 
@@ -152,19 +143,6 @@ __device__ __forceinline__ void expert_prefix(const int32_t *s_cnt, int32_t *s_o
     if (lane == 0) {
         s_off[E_tot] = off;
         s_toff[E_tot] = toff;
-    }
-}
-
-// The tile counts for the host, written straight into host memory the GPU can address (`mail`, or nullptr), by one
-// warp: word x is the pair (count x, seq), x = 0..E_tot, the last one S.  A 64-bit store arrives whole, so every
-// word says by itself whether it belongs to this call: no fence orders anything here.  (Plain counts followed by a
-// sequence number needed system-scope fences of the whole CTA, 4-5 us of a small build's 12.)
-__device__ __forceinline__ void mail_counts(unsigned long long *mail, uint32_t seq, const int32_t *s_toff, int E_tot, int lane)
-{
-    if (!mail) return;
-    for (int x = lane; x <= E_tot; x += 32) {
-        const uint32_t c = (uint32_t)((x < E_tot) ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot]);
-        *reinterpret_cast<volatile unsigned long long *>(mail + x) = ((unsigned long long)seq << 32) | c;
     }
 }
 
@@ -251,7 +229,8 @@ routing_finalize(int E_tot, int tile_m, int max_mtiles, const int32_t *__restric
     __syncthreads();
     if (threadIdx.x < 32) expert_prefix(s_cnt, s_off, s_toff, E_tot, tile_m, threadIdx.x);
     __syncthreads();
-    if (threadIdx.x < 32) mail_counts(mail, mail_seq, s_toff, E_tot, threadIdx.x);
+    if (threadIdx.x < 32)
+        mail_counts(mail, mail_seq, E_tot, threadIdx.x, [&](int x) { return x < E_tot ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot]; });
     if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
     for (int e = threadIdx.x; e <= E_tot; e += blockDim.x) {
         offsets[e] = s_off[e];
@@ -369,9 +348,9 @@ routing_onepass(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_to
 #pragma unroll
     for (int i = 0; i < kOnepassRows; ++i) {
         const int f = begin + 32 * i + lane;
-        e[i] = (i < rows && f < end) ? __ldg(topk_idx + f) : -1;
+        e[i] = (i < rows && f < end) ? ld_chained(topk_idx + f) : -1;
     }
-    if (begin > 0 && begin < end) before = __ldg(topk_idx + begin - 32 + lane);
+    if (begin > 0 && begin < end) before = ld_chained(topk_idx + begin - 32 + lane);
     uint16_t *h = hist + w * pitch;
     for (int x = lane; x < pitch / 2; x += 32) reinterpret_cast<uint32_t *>(h)[x] = 0u;
     __syncwarp();
@@ -483,7 +462,8 @@ routing_onepass(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_to
     __syncthreads();
 
     // ---- results
-    if (rank == 0 && w == kOnepassWarps - 1) mail_counts(mail, mail_seq, s_toff, E_tot, lane);
+    if (rank == 0 && w == kOnepassWarps - 1)
+        mail_counts(mail, mail_seq, E_tot, lane, [&](int x) { return x < E_tot ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot]; });
 #pragma unroll
     for (int i = 0; i < kOnepassRows; ++i) {
         const int f = begin + 32 * i + lane;
@@ -543,8 +523,7 @@ cudaError_t routing_onepass_launch(const int32_t *topk_idx, const moe_shape &s, 
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     onepass_config(cfg, attr, n_ctas, onepass_smem(n_ctas, rows, s.E_tot), stream);
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    attr[1] = chained_launch_attribute();
     cfg.numAttrs = 2;
     const RoutingOut out = {r.counts, r.offsets, r.tiles, r.tile_offsets, r.mtile_expert, r.mtile_first_row, r.mtile_valid,
                             r.perm, r.inv_perm, r.pad_row};
@@ -581,6 +560,9 @@ cudaError_t routing_four_launches(const int32_t *topk_idx, const moe_shape &s, i
 cudaError_t routing_prepare(int *max_cluster)
 {
     cudaError_t e = cudaFuncSetAttribute(routing_onepass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOnepassMaxSmem);
+    if (e != cudaSuccess) return e;
+    // the kernels before and behind it want all shared memory: no SM has to change its split between L1 and shared memory
+    e = cudaFuncSetAttribute(routing_onepass, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(routing_onepass, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

@@ -59,6 +59,11 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// pulls a tensor map that sits in kernel parameter space into the descriptor cache
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)map) : "memory");
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y)
 {
     asm volatile(

@@ -601,3 +601,45 @@ def test_random_small_shapes_with_co_resident_warps_against_the_oracle():
         _check_against_oracle(w, **kw)
         n_done += 1
     assert n_done >= 25
+
+
+@pytest.mark.parametrize("kw,limits", [
+    (dict(T=1, E=24, k=3), {}),                                            # fewer rows than experts
+    (dict(T=700, E=255, k=3), {}), (dict(T=700, E=300, k=3), {}),          # selection tabulated / more tile counts than a table holds
+    (dict(T=900, E=6, k=3, tile_m=256, tile_n=256, H=512), {}),            # CTA pairs
+    (dict(T=900, E=24, k=3), dict(force_comm_ctas=7)),
+    (dict(T=900, E=24, k=3), dict(drain_help=0)),                          # static map: communication CTAs own their tiles
+    (dict(T=900, E=24, k=3), dict(drain_help=0, dep_model=1)),             # tile-level readiness: not a function of the sum
+    (dict(T=900, E=24, k=3), dict(G=60)),
+], ids=str)
+def test_the_selection_of_the_whole_step_call_is_the_selector_s(kw, limits):
+    # where the picks are tabulated the launch looks its communication-CTA count up by the tile count on the device;
+    # the plan that comes back, the counts and the output are those of the three separate calls
+    h = G.handle()
+    base = dict(name="picks", H=256, I=64, tile_m=128, tile_n=128, EP=2, TP=1, L=2, routing="zipf", zipf_s=1.2)
+    base.update(kw)
+    w = replace(wl.TINY, **base)
+    x, W2 = wl.make_data(w)
+    xd, Wd = x.cuda(), W2.cuda()
+    ws = None
+    for seed in (3, 4):
+        idx, wt, _ = wl.make_routing(replace(w, routing_seed=seed))
+        ref_outs, _, ws, S, _ = G.run_layer(w, idx, wt, x, W2, ws=ws)
+        ref_outs = [o.copy() for o in ref_outs]
+        occ, lim, rho = B.moe_query_occupancy(h, w.tile_m, w.tile_n)
+        for k, v in limits.items():
+            setattr(lim, k, v)
+        want = B.plan_partition(ws.tile_counts[:w.E_tot].tolist(), occ, lim, ws.shape, rho)
+        for o in ws.out:
+            o.fill_(float("nan"))
+        ws.tile_counts.fill_(-7)
+        idx_d, wt_d = torch.from_numpy(idx).cuda(), torch.from_numpy(wt).cuda()
+        got = B.moe_layer(h, xd, Wd, idx_d, wt_d, ws, limits=lim)
+        assert int(ws.tile_counts[w.E_tot]) == S == int(ws.tile_counts[:w.E_tot].sum())
+        torch.cuda.synchronize()
+        assert B.moe_get_status(h, ws.status).code == 0
+        for f in ("comm_ctas", "R", "P", "W_comp", "W_comm", "delta", "pred_T_q", "co_warps", "drain_help"):
+            assert getattr(got, f) == getattr(want, f), f
+        own = [len(G.tokens_of_rank(w.T, w.EP, d)) for d in range(w.EP)]
+        for a, o, n in zip(ref_outs, ws.out, own):
+            assert np.array_equal(a[:n], o.float().cpu().numpy()[:n])
