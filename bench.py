@@ -614,8 +614,8 @@ def time_gemm1(h, dw, torch, n_warm=3, n_samples=9, cpu_rows=0):
     layer_us = statistics.median(a.elapsed_time(b) * 1e3 for a, b in lay)
     flops = 4.0 * w.R * w.H * w.I
     res = {"us": us, "tflops": flops / us / 1e6, "flops": flops,
-           "bytes_gather": 2.0 * w.R * w.H * 2, "launches": 2,
-           "post_router_layer_us": layer_us, "post_router_layer_launches": routing_launches(dw.shape.T * dw.shape.k_tot) + 3,
+           "launches": 1,
+           "post_router_layer_us": layer_us, "post_router_layer_launches": routing_launches(dw.shape.T * dw.shape.k_tot) + 2,
            "what": "gather + grouped GEMM1 (gate, up) + silu(gate) * up -> x_routed; timed alone (burst peak applies)"}
     if cpu_rows > 0:   # the oracle of this stage on a seeded sample of routed rows: parity check and CPU time
         import numpy as np

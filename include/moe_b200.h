@@ -383,9 +383,10 @@ int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int
  *   W1          [device] bf16 [E_tot, 2, I, H] (plane 0 gate, plane 1 up; H contiguous); I % 16 == 0
  *   routing     a routing workspace built by moe_build_routing with this tile_m; n_mtiles as for
  *               moe_gemm2_combine (MOE_MTILES_ON_DEVICE allowed)
- *   h_routed_ws [device] moe_gemm1_workspace_bytes() bytes: the gathered rows [R, H]
+ *   h_routed_ws [device] moe_gemm1_workspace_bytes() bytes: scratch for gathered rows (the kernel gathers while it
+ *               loads its operands and leaves it alone; still required)
  *   x_routed    [device] bf16 [R, I], 32-byte aligned, fully overwritten
- * Asynchronous on `stream` (one gather launch, one persistent tcgen05 launch); device-side problems go
+ * Asynchronous on `stream` (one persistent tcgen05 launch); device-side problems go
  * to the status word like in moe_gemm2_combine. */
 int32_t moe_gemm1_workspace_bytes(const moe_shape *shape, size_t *h_routed_bytes);
 int32_t moe_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const moe_shape *shape,

@@ -5,15 +5,26 @@
 // the input of GEMM2 + GatherRS.  The paper leaves this stage unchanged and does not name the
 // activation; SiLU gating is the reading taken.
 //
-// Two launches: gather_rows (one warp per routed row, 16-byte copies), then one persistent kernel,
-// one 512-thread CTA per SM, tile = 128 routed rows x 128 intermediate columns:
-//   warps 0, 2  TMA producers (one thread each): warp 0 the gathered rows (128 x 64 k), warp 2 the
-//               expert's 128 gate rows and 128 up rows of W1 for the same columns (two boxes that form
-//               one 256-row B operand), into four 48 KB stages, 128B swizzle;
-//   warp 1      issues tcgen05.mma (converged warp, elected lane; M = 128, N = 256, K = 16, bf16 -> fp32): accumulator
+// One persistent kernel, one 512-thread CTA per SM.  The gather is part of the operand loads: four loader warps know
+// the token of every row of the tile and copy each k-block of those rows straight from the hidden states into the
+// 128B-swizzled stage (16-byte cp.async, eight lanes per row).  A gather launch in front wrote and re-read the routed
+// rows, k_tot times the hidden states: 142 us and 1 GB of a 1280 us stage at 131072 rows of 2048 (now 1230 in all; Granite
+// shape, T = 4096: 120 -> 99 us).  (One TMA tile::gather4 copy per four rows does not keep up: 80 cycles each on an SM, 3660 us
+// for the stage.)  Rows past the end
+// of an expert's last tile are not fetched at all: nothing stored depends on them.
+//   tile_m <= 128: tile = 128 routed rows x 128 intermediate columns per CTA, four 48 KB stages;
+//   tile_m = 256 : tile = 256 rows x 128 columns per pair of CTAs (tcgen05 cta_group::2), seven 32 KB stages: CTA 0
+//                  holds rows 0..127 and loads the gate rows of W1, CTA 1 rows 128..255 and the up rows, so that a
+//                  k-block costs an SM 32 KB instead of 48.
+//   warp 0      TMA producer (one thread): the expert's 128 gate rows and 128 up rows of W1 for the same columns (64 k),
+//               which form one 256-row B operand;
+//   warps 12-15 loaders of the gathered rows; their copies arrive by themselves on the stage's `rows` barrier;
+//   warp 2      relay (one thread): waits for that barrier, makes the rows visible to the tensor core's proxy and
+//               arrives on the stage's full barrier (a fence in the issuing warp would cost every k-block its cycles);
+//   warp 1      issues tcgen05.mma (converged warp, elected lane; N = 256, K = 16, bf16 -> fp32): accumulator
 //               columns 0..127 are the gate projection, 128..255 the up projection of the same outputs;
 //               two accumulator buffers in TMEM;
-//   warps 4-15  epilogue: tcgen05.ld of 32 gate and the matching 32 up columns, silu(g) * u in fp32,
+//   warps 4-11  epilogue: tcgen05.ld of 32 gate and the matching 32 up columns, silu(g) * u in fp32,
 //               bf16, two 32-byte stores per row (x_routed rows are contiguous: no scatter here).
 // The n-tile index runs fastest in the tile sequence, so the CTAs of a wave share the gathered rows.
 // Every wait is bounded like in the fused kernel (status word, no trap).
@@ -29,26 +40,34 @@ namespace moe {
 namespace {
 
 constexpr int kG1TileN = 128;                                   // intermediate columns per tile
-constexpr int kG1ABytes = kMmaM * kBlockK * 2;                  // 16 KB
-constexpr int kG1BBytes = 2 * kG1TileN * kBlockK * 2;           // 32 KB: gate rows, then up rows
-constexpr int kG1StageBytes = kG1ABytes + kG1BBytes;            // 48 KB
-constexpr int kG1Stages = kStageBytesTotal / kG1StageBytes;     // 4
-constexpr int kG1EpiWarps = 12;
+constexpr int kG1EpiWarps = 8;          // warps 4..11: two column groups x four TMEM lane quarters
+constexpr int kG1LoadWarps = 4;         // warps 12..15
+constexpr int kG1RowsPerStep = 4 * kG1LoadWarps;   // rows that one copy instruction of all loader warps covers
 constexpr int kG1TmemCols = 512;                                // two 256-column accumulators
+constexpr int kG1MaxStages = 7;
+
+template <bool kPair>
+struct G1Cfg {
+    static constexpr int kABytes = kMmaM * kBlockK * 2;                              // 16 KB: this CTA's 128 rows
+    static constexpr int kBBytes = (kPair ? 1 : 2) * kG1TileN * kBlockK * 2;         // gate and up rows, or one of them
+    static constexpr int kStageBytes = kABytes + kBBytes;
+    static constexpr int kStages = kPair ? kG1MaxStages : 4;
+    static constexpr int kRingBytes = kStages * kStageBytes;
+};
 
 struct alignas(64) G1Params {
-    CUtensorMap tmA;   // h_routed [R, H]            box 64 x 128 rows
     CUtensorMap tmB;   // W1 as [E_tot * 2, I, H]    box 64 x 128 rows x 1 plane
     const int32_t *mtile_expert;
     const int32_t *mtile_first_row;
     const int32_t *mtile_valid;
+    const __nv_bfloat16 *hidden;   // [T, H]
+    const int32_t *perm;           // flat assignment of every routed row
     const int32_t *S_dev;          // != nullptr: the m-tile count is read here
     __nv_bfloat16 *x_routed;       // [R, I]
     uint32_t *status;
     unsigned long long wait_ns;
     int32_t S;                     // m-tiles of the routing workspace (or their bound with S_dev)
-    int32_t sub;                   // 128-row pieces per m-tile (1, or 2 for 256-row m-tiles)
-    int32_t sub_rows;              // rows of a piece that may be stored: min(tile_m, 128)
+    int32_t T, k_tot, H;
     int32_t I, NT;                 // intermediate size, n-tiles = ceil(I / 128)
     int32_t num_kb, last_ksteps;
     unsigned long long *mail;      // != nullptr: the tile counts (S_dev - E_tot) are mailed to the host by this launch
@@ -57,8 +76,9 @@ struct alignas(64) G1Params {
 };
 
 struct G1Control {
-    unsigned long long full[kG1Stages];
-    unsigned long long empty[kG1Stages];
+    unsigned long long full[kG1MaxStages];
+    unsigned long long empty[kG1MaxStages];
+    unsigned long long rows[kG1MaxStages];    // every loader thread's copies of the stage have landed
     unsigned long long tmem_full[2];
     unsigned long long tmem_empty[2];
     uint32_t tmem_base;
@@ -89,84 +109,96 @@ __device__ __forceinline__ bool g1_wait_warp(uint32_t bar, uint32_t parity, G1Co
     return __shfl_sync(0xffffffffu, ok, 0) != 0u;
 }
 
-struct G1Tile {
-    int e, row0, valid, n0;
-};
-// tile g of the sequence: (m-tile, 128-row piece) outer, n-tile inner
-__device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
+// silu(z) = z / (1 + exp(-z)).  The quotient as a product with the reciprocal, which one Newton-Raphson step
+// r (2 - d r) takes from the hardware's estimate to full precision: a third of the instructions of a division, which took
+// the epilogue warps more issue slots than the loaders and the MMA issuer beside them could spare.  (The bound keeps d
+// finite, where the step is defined; below it silu is under 1e-33.)
+__device__ __forceinline__ float silu(float z)
 {
-    const int piece = g / P.NT;
-    const int i_n = g - piece * P.NT;
-    const int mu = piece / P.sub;
-    const int half = piece - mu * P.sub;
-    G1Tile t;
-    t.e = ld_chained(&P.mtile_expert[mu]);
-    t.row0 = ld_chained(&P.mtile_first_row[mu]) + half * kMmaM;
-    t.valid = max(0, min(P.sub_rows, ld_chained(&P.mtile_valid[mu]) - half * kMmaM));
-    t.n0 = i_n * kG1TileN;
-    return t;
+    const float d = 1.0f + __expf(fminf(-z, 80.0f));
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    r = fmaf(r, fmaf(-d, r, 1.0f), r);
+    return z * r;
 }
 
-// --------------------------------------------------------------------------- gather
-
-// h_routed[r][:] = hidden[perm[r] / k_tot][:], one warp per routed row
-__global__ void __launch_bounds__(256)
-gather_rows(const uint4 *__restrict__ hidden, const int32_t *__restrict__ perm, int R, int k_tot, int row_vec,
-            uint4 *__restrict__ h_routed)
+struct G1Tile {
+    int e, row0, valid, n0;   // valid: rows of the whole m-tile (up to 256 for a pair tile)
+};
+// tile g of the sequence: m-tile outer, n-tile inner
+__device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
 {
-    const int r = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-    grid_dependency_wait();
-    grid_dependents_may_launch();
-    if (r >= R) return;
-    const int lane = threadIdx.x & 31;
-    const int t = ld_chained(&perm[r]) / k_tot;
-    const uint4 *src = hidden + (size_t)t * row_vec;
-    uint4 *dst = h_routed + (size_t)r * row_vec;
-    for (int c = lane; c < row_vec; c += 32) dst[c] = __ldg(&src[c]);
+    const int mu = g / P.NT;
+    G1Tile t;
+    t.e = ld_chained(&P.mtile_expert[mu]);
+    t.row0 = ld_chained(&P.mtile_first_row[mu]);
+    t.valid = ld_chained(&P.mtile_valid[mu]);
+    t.n0 = (g - mu * P.NT) * kG1TileN;
+    return t;
+}
+// rows of the m-tile that CTA `rank` of a pair holds
+__device__ __forceinline__ int g1_rows_of(int valid, uint32_t rank) { return max(0, min(kMmaM, valid - (int)rank * kMmaM)); }
+// flat assignments of the rows this loader thread copies (step i of the stage: row 16 i + `first`)
+__device__ __forceinline__ void g1_load_perm(const G1Params &P, const G1Tile &t, uint32_t rank, int first, int (&f)[kMmaM / kG1RowsPerStep])
+{
+    const int rows = g1_rows_of(t.valid, rank);
+#pragma unroll
+    for (int i = 0; i < kMmaM / kG1RowsPerStep; ++i) {
+        const int r = kG1RowsPerStep * i + first;
+        f[i] = r < rows ? ld_chained(&P.perm[t.row0 + (int)rank * kMmaM + r]) : -1;
+    }
 }
 
 // --------------------------------------------------------------------------- GEMM1 + activation
 
+template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
 {
+    using C = G1Cfg<kPair>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    G1Control *ctl = reinterpret_cast<G1Control *>(ring + kStageBytesTotal);
+    G1Control *ctl = reinterpret_cast<G1Control *>(ring + C::kRingBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = (int)blockIdx.x, stride = (int)gridDim.x;
+    const uint32_t rank = kPair ? cluster_ctarank() : 0u;
+    // tiles are dealt to the CTAs, or to the pairs
+    const int b = kPair ? (int)blockIdx.x >> 1 : (int)blockIdx.x, stride = kPair ? (int)gridDim.x >> 1 : (int)gridDim.x;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kG1Stages; ++i) {
-            mbar_init(smem_u32(&ctl->full[i]), 1);
+        for (int i = 0; i < C::kStages; ++i) {
+            mbar_init(smem_u32(&ctl->full[i]), kPair ? 3 : 2);   // the W1 producer and the relay of every CTA
             mbar_init(smem_u32(&ctl->empty[i]), 1);
+            mbar_init(smem_u32(&ctl->rows[i]), 32 * kG1LoadWarps);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
-            mbar_init(smem_u32(&ctl->tmem_empty[i]), kG1EpiWarps);
+            mbar_init(smem_u32(&ctl->tmem_empty[i]), (kPair ? 2 : 1) * kG1EpiWarps);
         }
         ctl->abort = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        prefetch_tensormap(&P.tmA);
         prefetch_tensormap(&P.tmB);
     }
-    if (warp == 1) tmem_alloc(smem_u32(&ctl->tmem_base), kG1TmemCols);
+    if (warp == 1) {
+        if (kPair) tmem_alloc_pair(smem_u32(&ctl->tmem_base), kG1TmemCols);
+        else tmem_alloc(smem_u32(&ctl->tmem_base), kG1TmemCols);
+    }
     tc_fence_before();
     __syncthreads();
+    if (kPair) cluster_sync_all();     // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     grid_dependency_wait();
     const int S = P.S_dev ? min(ld_chained_uniform(P.S_dev), P.S) : P.S;
-    const int total_tiles = S * P.sub * P.NT;
+    const int total_tiles = S * P.NT;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
-    if (P.mail && b == 0 && warp == 3)
+    if (P.mail && blockIdx.x == 0 && warp == 3)
         mail_counts(P.mail, P.mail_seq, P.E_tot, lane, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
-    if (warp == 0 || warp == 2) {
-        // ---------------- TMA producers
-        const bool load_a = (warp == 0);
+    if (warp == 0) {
+        // ---------------- W1 producer.  Pair: everything completes on the leader's full barrier, armed by the leader for both
+        // CTAs.
         if (lane == 0 && b < total_tiles) {
             int stage = 0;
             uint32_t phase = 0, armed = 0;
@@ -178,24 +210,24 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     ok = g1_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 50u);
                     if (!ok) break;
-                    const uint32_t full = smem_u32(&ctl->full[stage]);
-                    const uint32_t a_dst = smem_u32(ring + stage * kG1StageBytes);
-                    if (load_a) {
-                        mbar_arrive_expect_tx(full, (uint32_t)kG1StageBytes);
-                        tma_load_2d(a_dst, &P.tmA, full, kx, t.row0);
+                    const uint32_t own_full = smem_u32(&ctl->full[stage]);
+                    const uint32_t b_dst = smem_u32(ring + stage * C::kStageBytes) + C::kABytes;
+                    if (rank == 0) mbar_arrive_expect_tx(own_full, (kPair ? 2u : 1u) * (uint32_t)C::kBBytes);
+                    if (kPair) {   // gate rows, or up rows; the barrier lies at the same offset in the leader CTA (rank 0)
+                        tma_load_3d_pair(b_dst, &P.tmB, own_full & 0xFEFFFFFFu, kx, t.n0, 2 * t.e + (int)rank);
                     } else {
-                        tma_load_3d(a_dst + kG1ABytes, &P.tmB, full, kx, t.n0, 2 * t.e);                     // gate rows
-                        tma_load_3d(a_dst + kG1ABytes + kG1BBytes / 2, &P.tmB, full, kx, t.n0, 2 * t.e + 1); // up rows
+                        tma_load_3d(b_dst, &P.tmB, own_full, kx, t.n0, 2 * t.e);                       // gate rows
+                        tma_load_3d(b_dst + C::kBBytes / 2, &P.tmB, own_full, kx, t.n0, 2 * t.e + 1);  // up rows
                     }
                     armed |= 1u << stage;
-                    if (++stage == kG1Stages) { stage = 0; phase ^= 1u; }
+                    if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
                 }
                 t = t_next;
             }
-            if (!ok) {
+            if (!ok && rank == 0) {
                 // wind-down: let the copies already issued land before shared memory is released
                 const unsigned long long drain = globaltimer_ns() + 2000000ull;
-                for (int sidx = 0; sidx < kG1Stages; ++sidx) {
+                for (int sidx = 0; sidx < C::kStages; ++sidx) {
                     if (!(armed & (1u << sidx))) continue;
                     const uint32_t par = (sidx < stage) ? phase : (phase ^ 1u);
                     while (!mbar_try_wait(smem_u32(&ctl->full[sidx]), par) && globaltimer_ns() < drain) {}
@@ -203,15 +235,78 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             }
         }
         __syncwarp();
-    } else if (warp == 1) {
-        // ---------------- MMA issuer: the whole warp runs the loop, converged, and one elected lane issues.
-        // tcgen05.mma takes its descriptors and addresses from uniform registers, and the tensor pipe buffers
+    } else if (warp == 2) {
+        // ---------------- relay: rows landed -> visible to the tensor core's (async) proxy -> full barrier
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int g = b; g < total_tiles && ok; g += stride) {
+                for (int kb = 0; kb < P.num_kb; ++kb) {
+                    ok = g1_wait(smem_u32(&ctl->rows[stage]), phase, ctl, deadline, P.status, (uint32_t)g, 54u);
+                    if (!ok) break;
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    // (rank 1 relaxed: the copies have landed, and the fence is over when the next instruction issues; a
+                    // release at cluster scope takes ~1400 cycles, more than two k-blocks: 2550 us for the stage, 1230 so)
+                    if (rank != 0) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->full[stage]), 0u));
+                    else mbar_arrive(smem_u32(&ctl->full[stage]));
+                    if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp >= 4 + kG1EpiWarps) {
+        // ---------------- loaders: thread = one 16-byte column chunk of every 16th row
+        constexpr int kSteps = kMmaM / kG1RowsPerStep;
+        const int chunk = lane & 7, first = (warp - 4 - kG1EpiWarps) * 4 + (lane >> 3);
+        const uint32_t dst0 = (uint32_t)first * 128u + (uint32_t)((chunk ^ (first & 7)) << 4);   // 128B swizzle; 16 rows on: + 2048
+        if (b < total_tiles) {
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            G1Tile t_next = g1_decode(min(b + stride, total_tiles - 1), P);
+            int f[kSteps], f_next[kSteps];
+            g1_load_perm(P, g1_decode(b, P), rank, first, f);
+            for (int g = b; g < total_tiles && ok; g += stride) {
+                // fetched ahead: the table entries two tiles, the rows' assignments one tile
+                const G1Tile t_nn = g1_decode(min(g + 2 * stride, total_tiles - 1), P);
+                g1_load_perm(P, t_next, rank, first, f_next);
+                const __nv_bfloat16 *src[kSteps];
+#pragma unroll
+                for (int i = 0; i < kSteps; ++i)
+                    src[i] = f[i] >= 0 ? P.hidden + (size_t)min(f[i] / P.k_tot, P.T - 1) * (size_t)P.H + chunk * 8 : nullptr;
+                int left = P.H - chunk * 8;      // columns from this chunk on
+                for (int kb = 0; kb < P.num_kb; ++kb, left -= kBlockK) {
+                    ok = g1_wait_warp(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 55u);
+                    if (!ok) break;
+                    const uint32_t dst = smem_u32(ring + stage * C::kStageBytes) + dst0;
+                    if (left > 0) {              // (past the last column: no MMA reads it)
+#pragma unroll
+                        for (int i = 0; i < kSteps; ++i)
+                            if (src[i]) {
+                                cp_async_16(dst + (uint32_t)(i * kG1RowsPerStep * 128), src[i]);
+                                src[i] += kBlockK;
+                            }
+                    }
+                    cp_async_arrive(smem_u32(&ctl->rows[stage]));
+                    if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+                }
+                t_next = t_nn;
+#pragma unroll
+                for (int i = 0; i < kSteps; ++i) f[i] = f_next[i];
+            }
+            cp_async_wait_all();
+        }
+        __syncwarp();
+    } else if (warp == 1 && rank == 0) {
+        // ---------------- MMA issuer (pair: the leader CTA): the whole warp runs the loop, converged, and one elected lane
+        // issues.  tcgen05.mma takes its descriptors and addresses from uniform registers, and the tensor pipe buffers
         // little ahead of the MMA it executes: warp-uniform values in warp-uniform control flow spare a move per
         // operand and MMA, a whole k-block (four MMAs and the commit) is one statement with 32-bit descriptor
         // arithmetic, addresses advance by additions, the barrier's first look is the non-suspending test.
         {
-            constexpr uint32_t idesc = make_idesc(kMmaM, 2 * kG1TileN);
-            constexpr uint32_t kLoStage = (uint32_t)(kG1StageBytes >> 4), kLoB = (uint32_t)(kG1ABytes >> 4);
+            constexpr uint32_t idesc = make_idesc(kPair ? 2 * kMmaM : kMmaM, 2 * kG1TileN);
+            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoB = (uint32_t)(C::kABytes >> 4);
             const uint32_t lo0 = smem_desc_lo(smem_u32(ring));
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
             uint32_t a_lo = lo0, full_bar = full0, empty_bar = empty0;
@@ -236,19 +331,23 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     tc_fence_after();
                     if (elect_one_sync()) {
                         if (kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) {
-                            tc_kblock_bf16(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
+                            if (kPair) tc_kblock_bf16_pair(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
+                            else tc_kblock_bf16(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
                         } else {
                             const uint64_t a_desc = ((uint64_t)kSmemDescHi << 32) | a_lo, b_desc = a_desc + kLoB;
-                            for (int k = 0; k < P.last_ksteps; ++k)
-                                tc_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                            (k > 0 || kb > 0) ? 1u : 0u);
-                            tc_commit(empty_bar);
+                            for (int k = 0; k < P.last_ksteps; ++k) {
+                                const uint32_t acc = (k > 0 || kb > 0) ? 1u : 0u;
+                                if (kPair) tc_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
+                                else tc_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
+                            }
+                            if (kPair) tc_commit_pair(empty_bar);
+                            else tc_commit(empty_bar);
                         }
                     }
                     a_lo += kLoStage;
                     full_bar += 8u;
                     empty_bar += 8u;
-                    if (++stage == kG1Stages) {
+                    if (++stage == C::kStages) {
                         stage = 0;
                         phase ^= 1u;
                         a_lo = lo0;
@@ -257,17 +356,19 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     }
                 }
                 __syncwarp();
-                if (ok && elect_one_sync()) tc_commit(smem_u32(&ctl->tmem_full[a]));
+                if (ok && elect_one_sync()) {
+                    if (kPair) tc_commit_pair(smem_u32(&ctl->tmem_full[a]));
+                    else tc_commit(smem_u32(&ctl->tmem_full[a]));
+                }
             }
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + kG1EpiWarps) {
-        // ---------------- epilogue: four 32-column rounds per tile, dealt 2 / 1 / 1 to the column groups
+        // ---------------- epilogue: four 32-column rounds per tile, two per column group
         const int q4 = warp & 3;
         const int grp = (warp - 4) >> 2;
-        const int round0 = grp == 0 ? 0 : grp + 1;
-        const int n_rounds = grp == 0 ? 2 : 1;
-        const int row_in_tile = q4 * 32 + lane;
+        const int round0 = 2 * grp, n_rounds = 2;
+        const int row_in_tile = (int)rank * kMmaM + q4 * 32 + lane;
         int it = 0;
         for (int g = b; g < total_tiles; g += stride, ++it) {
             const G1Tile t = g1_decode(g, P);
@@ -291,7 +392,10 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     // everything this warp needs of the accumulator is in registers: hand the buffer back
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
+                    if (lane == 0) {
+                        if (kPair) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->tmem_empty[a]), 0u));   // the leader's barrier
+                        else mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
+                    }
                 }
                 if (row_ok) {
 #pragma unroll
@@ -302,9 +406,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                             for (int i = 0; i < 8; ++i) {
                                 const float g0 = __uint_as_float(gt[v * 16 + 2 * i]), g1 = __uint_as_float(gt[v * 16 + 2 * i + 1]);
                                 const float u0 = __uint_as_float(up[v * 16 + 2 * i]), u1 = __uint_as_float(up[v * 16 + 2 * i + 1]);
-                                // silu(z) * u = z / (1 + exp(-z)) * u
-                                const float x0 = g0 / (1.0f + __expf(-g0)) * u0;
-                                const float x1 = g1 / (1.0f + __expf(-g1)) * u1;
+                                const float x0 = silu(g0) * u0, x1 = silu(g1) * u1;
                                 __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
                                 w[i] = *reinterpret_cast<uint32_t *>(&h);
                             }
@@ -315,16 +417,20 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             }
         }
     }
-    // ---------------- teardown
+    // ---------------- teardown (pair: nobody leaves while its peer may still touch its memory)
     tc_fence_before();
     __syncthreads();
+    if (kPair) cluster_sync_all();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kG1TmemCols);
+        if (kPair) tmem_dealloc_pair(tmem_base, kG1TmemCols);
+        else tmem_dealloc(tmem_base, kG1TmemCols);
     }
 }
 
-size_t g1_smem_bytes() { return (size_t)kStageBytesTotal + 1024 + ((sizeof(G1Control) + 127) & ~(size_t)127); }
+template <bool kPair>
+constexpr size_t g1_smem_bytes() { return (size_t)G1Cfg<kPair>::kRingBytes + 1024 + ((sizeof(G1Control) + 127) & ~(size_t)127); }
+static_assert(g1_smem_bytes<true>() <= 227 * 1024, "GEMM1 pair stages exceed the shared memory of an SM");
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
@@ -340,7 +446,9 @@ using namespace moe;
 
 cudaError_t moe::gemm1_prepare()
 {
-    return cudaFuncSetAttribute(moe_gemm1_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes());
+    const cudaError_t e = cudaFuncSetAttribute(moe_gemm1_act_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<false>());
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(moe_gemm1_act_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<true>());
 }
 
 extern "C" int32_t moe_gemm1_workspace_bytes(const moe_shape *s, size_t *h_routed_bytes)
@@ -377,7 +485,6 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     if (n_mtiles < 0 || n_mtiles > r->max_mtiles) return MOE_ERR_SHAPE;
     if (const int32_t rc = moe::require_handle_device(h, "moe_gemm1_act")) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int R = s->T * s->k_tot;
 
     G1Params p;
     memset(&p, 0, sizeof p);
@@ -394,28 +501,18 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
         p.mail_seq = mail_seq;
         p.E_tot = s->E_tot;
     }
-    p.sub = tile_m == 256 ? 2 : 1;
-    p.sub_rows = tile_m < kMmaM ? tile_m : kMmaM;
+    p.perm = r->perm;
+    p.hidden = static_cast<const __nv_bfloat16 *>(hidden);
+    p.T = s->T;
+    p.H = s->H;
+    p.k_tot = s->k_tot;
     p.I = s->I;
     p.NT = (s->I + kG1TileN - 1) / kG1TileN;
     p.num_kb = (s->H + kBlockK - 1) / kBlockK;
     p.last_ksteps = (s->H - (p.num_kb - 1) * kBlockK) / kUmmaK;
-    if ((int64_t)n_mtiles * p.sub * p.NT >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
+    if ((int64_t)n_mtiles * p.NT >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
 
     EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(h->encode_tiled);
-    {
-        cuuint64_t dims[2] = {(cuuint64_t)s->H, (cuuint64_t)R};
-        cuuint64_t strides[1] = {(cuuint64_t)s->H * 2};
-        cuuint32_t box[2] = {(cuuint32_t)kBlockK, (cuuint32_t)kMmaM};
-        cuuint32_t es[2] = {1, 1};
-        CUresult cr = encode(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, h_routed_ws, dims, strides, box, es,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (cr != CUDA_SUCCESS) {
-            snprintf(h->err, sizeof h->err, "cuTensorMapEncodeTiled(h_routed) failed: %d", (int)cr);
-            return MOE_ERR_CUDA;
-        }
-    }
     {
         // W1 [E_tot][2][I][H] seen as [E_tot * 2 planes][I rows][H]: rows past I of a plane read zeros
         cuuint64_t dims[3] = {(cuuint64_t)s->H, (cuuint64_t)s->I, (cuuint64_t)s->E_tot * 2};
@@ -431,24 +528,23 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
         }
     }
 
-    // gather (the rows of a token are read k_tot times, from L2 after the first)
-    const int row_vec = s->H * 2 / 16;
+    const bool pair = tile_m == 256;
+    const int64_t tiles_bound = (int64_t)n_mtiles * p.NT;
+    const int slots = pair ? h->max_pairs : h->G;
+    const int used = (int)(tiles_bound < slots ? (tiles_bound > 0 ? tiles_bound : 1) : slots);
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1] = {chained_launch_attribute()};
+    cudaLaunchAttribute attr[2] = {chained_launch_attribute()};
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pair ? 2 : 1;
     cfg.stream = st;
-    cfg.gridDim = dim3((unsigned)(((int64_t)R * 32 + 255) / 256));
-    cfg.blockDim = dim3(256);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gather_rows, static_cast<const uint4 *>(hidden), static_cast<const int32_t *>(r->perm), R,
-                                       (int)s->k_tot, row_vec, static_cast<uint4 *>(h_routed_ws));
-    if (e != cudaSuccess) return cuda_fail(h, e, "gather_rows launch");
-
-    const int64_t tiles_bound = (int64_t)n_mtiles * p.sub * p.NT;
-    cfg.gridDim = dim3((unsigned)(tiles_bound < h->G ? (tiles_bound > 0 ? tiles_bound : 1) : h->G));
+    cfg.gridDim = dim3((unsigned)(pair ? 2 * used : used));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = g1_smem_bytes();
-    e = cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel, p);
+    cfg.dynamicSmemBytes = pair ? g1_smem_bytes<true>() : g1_smem_bytes<false>();
+    const cudaError_t e = pair ? cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<true>, p) : cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<false>, p);
     if (e != cudaSuccess) return cuda_fail(h, e, "gemm1 launch");
     return MOE_OK;
 }

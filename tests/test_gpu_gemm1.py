@@ -172,3 +172,22 @@ def test_random_small_shapes_against_the_oracle():
                     tile_m=tile_m, tile_n=256 if tile_m == 256 else 64, routing_seed=300 + case, data_seed=400 + case)
         w = replace(w, k=int(rng.integers(1, min(w.E, 3) + 1)))
         _check(w, counts_on_device=bool(rng.integers(2)))
+
+
+@pytest.mark.parametrize("tile_m", [64, 128, 256])
+@pytest.mark.parametrize("H,I", [(64, 16), (272, 208), (1024, 128)], ids=str)
+def test_row_gather_at_the_edges_of_the_m_tiles(tile_m, H, I):
+    # experts with 1, 3, 4, 5, 127 ... 257 rows: whole and partial groups of rows, m-tiles whose second half is empty,
+    # holds one row, is full; shapes with one k-block, a partial one, and more than the operand ring holds
+    counts = [1, 3, 4, 5, 127, 128, 129, 0, 255, 256, 257]
+    idx = np.repeat(np.arange(len(counts)), counts).astype(np.int32)
+    idx = np.random.default_rng(0).permutation(idx)[:, None].copy()
+    w = replace(wl.TINY, name="gather", T=len(idx), E=len(counts), k=1, H=H, I=I, tile_m=tile_m, tile_n=256 if tile_m == 256 else 64,
+                TP=1, EP=1, L=1, data_seed=5)
+    hidden, W1 = wl.make_gemm1_data(w)
+    x, _ = _run(w, idx, hidden, W1, counts_on_device=True)
+    r = rr.build_routing(idx, w.E_tot, w.tile_m)
+    ref = g1.gemm1_act(wl.bf16_bits(hidden), wl.bf16_bits(W1), idx, r["perm"], rows=np.arange(w.R, dtype=np.int32))
+    got = x.float().cpu().numpy()
+    assert not np.isnan(got).any()
+    assert np.all(np.abs(got - ref) <= _tolerance(ref)), float(np.max(np.abs(got - ref)))
