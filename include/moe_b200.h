@@ -92,10 +92,13 @@ typedef struct {
     int32_t selector_off;    /* != 0: use default_C */
     int32_t default_C;       /* the fixed count used when the selector is off */
     int32_t drain_help;      /* != 0: compute CTAs that run out of GEMM tiles serve the communication work
-                                that is left, and the work is handed out dynamically (warps pull token ranges
-                                from a queue per split) instead of by the static tile -> CTA map (an extension
+                                that is left, instead of the static tile -> CTA map (an extension
                                 of this library, not in the paper: with it the selector models the tail after
-                                the last compute wave as served by every SM);
+                                the last compute wave as served by every SM).  Large amounts of work, and all work when
+                                there are co-resident warps, are handed out dynamically (warps pull token ranges
+                                from a queue per split); of small amounts every warp takes an even share once the
+                                tiles are done, and a launch whose tiles fit the SMs at once runs with every SM
+                                computing;
                                 0: the paper's static partition and its recurrence exactly */
     int32_t co_warps_max;    /* upper end of the legal set {0..co_warps_max} of co-resident communication warps
                                 per compute CTA (0: a kernel family without them) */

@@ -538,13 +538,12 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     FusedParams p;
     memset(&p, 0, sizeof p);
     const int K = s->I / s->TP;
-    const int TN = occ->tile_n;
     p.T = s->T; p.H = s->H; p.K = K; p.TP = s->TP; p.EP = s->EP; p.L = s->L; p.k_tot = s->k_tot;
     p.S = n_mtiles;
     p.tile_m = occ->tile_m;
     p.flag_parts = pair ? 2 : 1;
     p.split_w = (int32_t)ceil_div(s->H, s->L);
-    p.NTs = (int32_t)ceil_div(p.split_w, TN);
+    p.NTs = (int32_t)ceil_div(p.split_w, occ->tile_n);
     const int64_t Wc = (int64_t)s->TP * n_mtiles * p.NTs;
     if (Wc * s->L * 2 >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
     p.W_comp = (int32_t)Wc;
@@ -609,6 +608,34 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     // Tile sequence: split-major (the paper's) whenever something consumes a split while the next one is
     // computed; m-tile-major across the splits (x is read from DRAM once) when nothing does
     p.tile_order = (plan->drain_help && p.co_warps == 0) ? 1 : 0;
+    const int64_t R = (int64_t)s->T * s->k_tot;
+    p.w2_once = R <= (int64_t)s->E_tot * kMmaM;    // at most one 128-row tile per expert on average
+    // Who serves what when the compute CTAs help: a queue per split, or, up to 32 units (of 8 KB) a warp, an even share for every
+    // warp once the tiles are done.  Hardly any token is complete before the last tiles are, so the queue's early start is
+    // worth little, while its atomics and its polling cost microseconds at the end (whole launch, queue -> even: DeepSeek shape
+    // T = 16 67 -> 58 us, 256 92 -> 76, 2048 149 -> 142; Granite shape T = 1003 40 -> 30, 4096 120 -> 107; Qwen shape T = 8192 240 ->
+    // 233); with more units the queue's balance wins (DeepSeek shape T = 16384, 74 units: 804 -> 815, 37 units: 719 -> 745).
+    // Co-resident warps draw on the queue; a launch with a withheld tile is about that tile's flag.
+    const int64_t units = (int64_t)s->T * s->L * ceil_div(p.split_w, p.slab_cols);
+    p.even = p.drain_help && p.co_warps == 0 && plan->debug_withhold_tile < 0 && units <= 32ll * 12 * h->G;
+    int TN = occ->tile_n, ctas_c = C, ctas_p = Pc;
+    if (p.even && !pair) {
+        // One wave: where every tile that this routing can have finds an SM of its own among the plan's, all of them compute (a
+        // communication CTA would have nothing to do until the only wave ends), on the narrowest tiles for which that holds
+        // (the time of a wave is the time to stream and store one tile: DeepSeek shape, T = 1, 19 -> 16 us).
+        const int64_t used = R < s->E_tot ? R : s->E_tot, bound = (R - used) / occ->tile_m + used;
+        const int64_t S_max = counts_on_device && bound < n_mtiles ? bound : n_mtiles;
+        for (int tn = 64; tn <= occ->tile_n; tn *= 2) {
+            if (S_max * s->TP * s->L * ceil_div(p.split_w, tn) > C + Pc) continue;
+            TN = tn;
+            p.NTs = (int32_t)ceil_div(p.split_w, TN);
+            p.W_comp = s->TP * n_mtiles * p.NTs;
+            p.C = ctas_c = 0;
+            p.P = ctas_p = C + Pc;
+            p.c_table_n = 0;
+            break;
+        }
+    }
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
@@ -632,15 +659,14 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     // tensor maps (Section II-A operands): x_routed [R, I] and W2 [E_tot, H, I], k contiguous.  Encoding the two
     // maps costs microseconds of host time between the wait for the tile counts and the launch: the handle
     // keeps the last pair and reuses it while buffers, sizes and tile family stay the same (a loop of steps).
-    const TensorMapKey key = {x_routed, W2, s->T, s->k_tot, s->I, s->H, s->E_tot, pair ? TN / 2 : TN};
+    const TensorMapKey key = {x_routed, W2, s->T, s->k_tot, s->I, s->H, s->E_tot, pair ? TN / 2 : TN, pair ? kMmaM : kXBoxRows};
     if (!h->tm_valid || memcmp(&h->tm_key, &key, sizeof key) != 0) {
         EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(h->encode_tiled);
-        const cuuint64_t R = (cuuint64_t)s->T * s->k_tot;
         h->tm_valid = false;
         {
-            cuuint64_t dims[2] = {(cuuint64_t)s->I, R};
+            cuuint64_t dims[2] = {(cuuint64_t)s->I, (cuuint64_t)R};
             cuuint64_t strides[1] = {(cuuint64_t)s->I * 2};
-            cuuint32_t box[2] = {(cuuint32_t)kBlockK, (cuuint32_t)kMmaM};
+            cuuint32_t box[2] = {(cuuint32_t)kBlockK, (cuuint32_t)(pair ? kMmaM : kXBoxRows)};
             cuuint32_t es[2] = {1, 1};
             CUresult cr = encode(&h->tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(x_routed), dims,
                                  strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -668,7 +694,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     }
     p.tmA = h->tmA;
     p.tmB = h->tmB;
-    const int grid = pair ? ((C + 1) & ~1) + 2 * Pc : C + Pc;
+    const int grid = pair ? ((C + 1) & ~1) + 2 * Pc : ctas_c + ctas_p;
     p.timeline = nullptr;
     if (h->timeline && h->timeline_bytes >= ((size_t)grid * kTimelineSlots + MOE_MAX_L) * sizeof(unsigned long long))
         p.timeline = h->timeline;

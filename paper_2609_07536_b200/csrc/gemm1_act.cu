@@ -70,6 +70,7 @@ struct alignas(64) G1Params {
     int32_t T, k_tot, H;
     int32_t I, NT;                 // intermediate size, n-tiles = ceil(I / 128)
     int32_t num_kb, last_ksteps;
+    int32_t w1_once;               // W1 is read (about) once: its lines go first when L2 needs room
     unsigned long long *mail;      // != nullptr: the tile counts (S_dev - E_tot) are mailed to the host by this launch
     uint32_t mail_seq;
     int32_t E_tot;
@@ -203,6 +204,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             int stage = 0;
             uint32_t phase = 0, armed = 0;
             bool ok = true;
+            const unsigned long long w_policy = P.w1_once ? l2_evict_first_policy() : l2_evict_normal_policy();
             G1Tile t = g1_decode(b, P);
             for (int g = b; g < total_tiles && ok; g += stride) {
                 const G1Tile t_next = g1_decode(min(g + stride, total_tiles - 1), P);   // fetched one tile ahead
@@ -216,8 +218,8 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     if (kPair) {   // gate rows, or up rows; the barrier lies at the same offset in the leader CTA (rank 0)
                         tma_load_3d_pair(b_dst, &P.tmB, own_full & 0xFEFFFFFFu, kx, t.n0, 2 * t.e + (int)rank);
                     } else {
-                        tma_load_3d(b_dst, &P.tmB, own_full, kx, t.n0, 2 * t.e);                       // gate rows
-                        tma_load_3d(b_dst + C::kBBytes / 2, &P.tmB, own_full, kx, t.n0, 2 * t.e + 1);  // up rows
+                        tma_load_3d_hint(b_dst, &P.tmB, own_full, kx, t.n0, 2 * t.e, w_policy);                       // gate rows
+                        tma_load_3d_hint(b_dst + C::kBBytes / 2, &P.tmB, own_full, kx, t.n0, 2 * t.e + 1, w_policy);  // up rows
                     }
                     armed |= 1u << stage;
                     if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
@@ -509,6 +511,7 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     p.I = s->I;
     p.NT = (s->I + kG1TileN - 1) / kG1TileN;
     p.num_kb = (s->H + kBlockK - 1) / kBlockK;
+    p.w1_once = (int64_t)s->T * s->k_tot <= (int64_t)s->E_tot * kMmaM;   // at most one 128-row tile per expert on average
     p.last_ksteps = (s->H - (p.num_kb - 1) * kBlockK) / kUmmaK;
     if ((int64_t)n_mtiles * p.NT >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
 

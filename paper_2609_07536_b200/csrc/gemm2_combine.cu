@@ -3,15 +3,16 @@
 //
 //   blockIdx <  C : communication CTA c (Section II-B: consumes published results; the same
 //                   C CTAs serve all splits in sequence; CTA c takes communication tiles
-//                   c, c+C, ... of a split -- or, with drain help, its warps pull token ranges
-//                   from a queue per split that former compute CTAs also serve).
+//                   c, c+C, ... of a split -- or, with drain help, its warps pull token ranges from a queue
+//                   per split, or take an even share of the units once the tiles are done; former compute
+//                   CTAs do the same).
 //   blockIdx >= C : compute CTA b = blockIdx - C (Section III-C: takes global tiles
 //                   b, b+P, b+2P, ... of the split-major sequence in which the expert
 //                   problems of one split are contiguous; m-tile-major across the splits when
 //                   the communication work is handed out dynamically).
 //
 // Compute CTA (warp-specialised; tile_m x tile_n with tile_m in {64, 128}):
-//   warps 0, 2  TMA producers (one thread each): warp 0 the x_routed tile (128 rows x 64 k), warp 2 the
+//   warps 0, 2  TMA producers (one thread each): warp 0 the x_routed tile (up to 128 rows x 64 k), warp 2 the
 //               W2 tile (tile_n rows x 64 k) of every k-block, into a ring of 128B-swizzled stages;
 //   warp 1      MMA issuer (the warp runs the loop converged, an elected lane issues; all operands warp-uniform):
 //               tcgen05.mma (M = 128, N = tile_n, K = 16, bf16 -> fp32) into one of two TMEM accumulator
@@ -395,23 +396,31 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
         first_n = ld_chained(&P.mtile_first_row[mu1]);
         if (row_in_tile < valid) f_row = ld_chained(&P.perm[first0 + row_in_tile]);
     }
-    int it = 0;
-    for (int g = b; g < total_tiles; g += pt.P, ++it) {
+    // Round -1 (one-CTA tiles: small launches, whose tail counts) is dry: the store path runs once without a tile while the first operands are on their way, on whatever the
+    // second accumulator buffer holds, so that its instructions are at hand when the first tile is done.
+    int it = (!kPair && P.even) ? -1 : 0;
+#pragma unroll 1
+    for (int g = b; g < total_tiles;) {
+        const bool dry = !kPair && it < 0;
         const Tile t = decode_tile(g, P, pt.W_comp);
         const int a = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
-        const int mu_nn = decode_tile(min(g + 2 * pt.P, total_tiles - 1), P, pt.W_comp).mu;
-        const int valid_nn = ld_chained(&P.mtile_valid[mu_nn]);
-        const int first_nn = ld_chained(&P.mtile_first_row[mu_nn]);
-        const int f_row_n = (row_in_tile < valid_n) ? ld_chained(&P.perm[first_n + row_in_tile]) : 0;
+        int valid_nn = valid_n, first_nn = first_n, f_row_n = 0;
+        bool ok = true;
+        if (!dry) {
+            const int mu_nn = decode_tile(min(g + 2 * pt.P, total_tiles - 1), P, pt.W_comp).mu;
+            valid_nn = ld_chained(&P.mtile_valid[mu_nn]);
+            first_nn = ld_chained(&P.mtile_first_row[mu_nn]);
+            if (row_in_tile < valid_n) f_row_n = ld_chained(&P.perm[first_n + row_in_tile]);
+        }
         TL(tl_q = clock64());
-        bool ok = wait_barrier(smem_u32(&ctl->tmem_full[a]), acc_phase, ctl, deadline, P.status, (uint32_t)g, 30u);
+        if (!dry) ok = wait_barrier(smem_u32(&ctl->tmem_full[a]), acc_phase, ctl, deadline, P.status, (uint32_t)g, 30u);
         TL(tl_ew += clock64() - tl_q; tl_q = clock64());
         if (ok) {
             tc_fence_after();
             const int n0 = t.s * P.split_w + t.i_n * TN;
             const int col_end = min(P.H, (t.s + 1) * P.split_w);
-            const bool row_ok = row_in_tile < valid;
+            const bool row_ok = !dry && row_in_tile < valid;
             // destination of this thread's row: the routed row belongs to flat assignment
             // f = (token, slot); Y is token-major so that the combine reads one contiguous block
             __nv_bfloat16 *ybase = Y;
@@ -423,7 +432,9 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
                 ybase = Y + ((size_t)tok * P.L + t.s) * (size_t)P.Q * (size_t)P.split_w;
             }
             const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * TN);
-            if (P.wide_store)
+            if (!dry && row_in_tile - lane >= valid) {
+                // none of the warp's 32 rows holds a token (small batches: most warps)
+            } else if (P.wide_store)
                 store_accumulator_rows_wide(P, taddr, col_first, n_cols, row_ok, ybase, q, n0, col_end, n0 - t.s * P.split_w);
             else if (P.slab_cols >= 32)
                 store_accumulator_rows_staged(P, taddr, col_first, n_cols, row_ok, ybase, q, n0, col_end,
@@ -431,6 +442,10 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
             else
                 store_accumulator_rows(P, taddr, col_first, n_cols, row_ok, ybase, q, n0, col_end, n0 - t.s * P.split_w);
             // the accumulator buffer (this CTA's half of it) may be overwritten by the MMA of the tile after next
+            if (dry) {
+                ++it;
+                continue;
+            }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
@@ -454,6 +469,8 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
         f_row = f_row_n;
         valid_n = valid_nn;
         first_n = first_nn;
+        g += pt.P;
+        ++it;
     }
     TL(if (warp == 4 && lane == 0) { tl_put(P, kTlEpiWait, (unsigned long long)tl_ew); tl_put(P, kTlEpiWork, (unsigned long long)tl_ek);
                                       tl_put(P, kTlEpiPubWait, (unsigned long long)tl_ep); });
@@ -488,7 +505,7 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, const Part 
             for (int j = 0; j < n; ++j, ++it, g += pt.P) {
                 const Tile t = decode_tile(g, P, pt.W_comp);
                 if (t.id != P.withhold) {
-                    st_relaxed_u32(&P.flags[kPair ? 2 * t.id + rank : t.id], P.epoch);
+                    if (!P.even) st_relaxed_u32(&P.flags[kPair ? 2 * t.id + rank : t.id], P.epoch);
 #if MOE_TIMELINE
                     if (atomicAdd(&P.split_done[t.s], 1u) + 1u == (uint32_t)(pt.W_comp * P.flag_parts) && P.timeline)
                         P.timeline[(size_t)gridDim.x * kTimelineSlots + t.s] = globaltimer_ns();
@@ -507,15 +524,13 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, const Part 
 
 // --------------------------------------------------------------------------- compute CTA
 
+// Barriers (thread 0) and TMEM (warp 1) of a compute CTA, before it is known that this CTA computes; a CTA-wide barrier of the
+// kernel makes them visible.
 template <int TN>
-__device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
+__device__ __forceinline__ void compute_setup(const FusedParams &P, Control *ctl)
 {
     using C = Cfg<TN>;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int total_tiles = P.L * pt.W_comp;
-    const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
-
-    // setup: barriers (thread 0), TMEM allocation (warp 1)
+    const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::kStages; ++i) {
             mbar_init(smem_u32(&ctl->full[i]), 1);
@@ -533,9 +548,15 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(&ctl->tmem_base), C::kTmemCols);
-    tc_fence_before();
-    sync_compute_warps(P);
-    tc_fence_after();
+}
+
+template <int TN>
+__device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
+{
+    using C = Cfg<TN>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int total_tiles = P.L * pt.W_comp;
+    const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
     const uint32_t tmem_base = ctl->tmem_base;
 
     if (warp == 0 || warp == 2) {
@@ -548,17 +569,23 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
             uint32_t phase = 0;
             uint32_t armed = 0;  // bit s: stage s was handed to the TMA unit at least once
             bool ok = true;
+            const unsigned long long w_policy = P.w2_once ? l2_evict_first_policy() : l2_evict_normal_policy();
             TL_DECL(long long tl_pw = 0, tl_q;)
             // the m-tile table entries of the NEXT tile are fetched while this tile's k-blocks are issued, so
             // that the two dependent global loads never stall the stream of copies at a tile boundary
             Tile t = decode_tile(b, P, pt.W_comp);
             int e = ld_chained(&P.mtile_expert[t.mu]);
             int row0 = ld_chained(&P.mtile_first_row[t.mu]);
+            int valid = ld_chained(&P.mtile_valid[t.mu]);
             for (int g = b; g < total_tiles && ok; g += pt.P) {
                 const Tile t_next = decode_tile(min(g + pt.P, total_tiles - 1), P, pt.W_comp);
                 const int e_next = ld_chained(&P.mtile_expert[t_next.mu]);
                 const int row0_next = ld_chained(&P.mtile_first_row[t_next.mu]);
+                const int valid_next = ld_chained(&P.mtile_valid[t_next.mu]);
                 const int n0 = t.s * P.split_w + t.i_n * TN;
+                // rows come in boxes of kXBoxRows: those past the end of the expert's last tile are not fetched, nothing stored
+                // depends on them
+                const int boxes = min((valid + kXBoxRows - 1) / kXBoxRows, kMmaM / kXBoxRows);
                 int kx = t.p * P.K;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     TL(tl_q = clock64());
@@ -569,10 +596,11 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                     const uint32_t a_dst = smem_u32(ring + stage * C::kStageBytes);
                     const bool skip_b = MOE_PROBE(kProbeSkipAllW2) || (MOE_PROBE(kProbeSkipOddW2) && (kb & 1));
                     if (load_a) {
-                        mbar_arrive_expect_tx(full, (uint32_t)C::kStageBytes);
-                        tma_load_2d(a_dst, &P.tmA, full, kx, row0);
+                        mbar_arrive_expect_tx(full, (uint32_t)(boxes * kXBoxRows * kBlockK * 2 + C::kBBytes));
+                        for (int i = 0; i < boxes; ++i)
+                            tma_load_2d(a_dst + (uint32_t)(i * kXBoxRows * kBlockK * 2), &P.tmA, full, kx, row0 + i * kXBoxRows);
                     } else if (!skip_b) {
-                        tma_load_3d(a_dst + C::kABytes, &P.tmB, full, kx, n0, e);
+                        tma_load_3d_hint(a_dst + C::kABytes, &P.tmB, full, kx, n0, e, w_policy);
                     } else {
                         // a probe that leaves the copy out completes its bytes by hand: this producer stays in
                         // the barrier's dependency chain, or the other one could lap it
@@ -584,6 +612,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                 t = t_next;
                 e = e_next;
                 row0 = row0_next;
+                valid = valid_next;
             }
             TL(if (load_a) tl_put(P, kTlProducerWait, (unsigned long long)tl_pw));
             if (!ok) {
@@ -933,6 +962,92 @@ __device__ __forceinline__ void fma_bf16x8(float (&acc)[8], const uint4 &v, floa
     }
 }
 
+// Reduces one unit that sits in shared memory at `stage_s`: the weighted sum of its Q rows in (j, p) order, one warp.  `w`:
+// lane j holds the weight of slot j (0: the slot has no source row); `wq`: room for Q floats; `orow`: where the unit's columns
+// of the token go.
+__device__ __forceinline__ void reduce_unit(const FusedParams &P, float w, bool all_valid, int ucols, int wslab, float *wq, uint32_t stage_s,
+                                            __nv_bfloat16 *orow)
+{
+    const int lane = threadIdx.x & 31;
+    const int n16 = ucols >> 3;
+    const uint32_t row_bytes = (uint32_t)wslab * 2u;
+    // per-row weights, read back as shared-memory broadcasts inside the unrolled loop
+    if (lane < P.k_tot)
+        for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w;
+    __syncwarp();
+    const uint32_t wq_s = smem_u32(wq);
+    if (all_valid && P.Q <= 16) {
+        // common case: every slot has a source row and the unit has at most 16 rows: weights stay in
+        // registers as packed pairs, rows are fetched eight at a time, two FMAs per instruction
+        unsigned long long ww[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const uint32_t wb = __float_as_uint(r < P.Q ? lds_f32(wq_s + (uint32_t)r * 4u) : 0.f);
+            ww[r] = pack_f32x2(wb, wb);
+        }
+        for (int c16 = lane; c16 < n16; c16 += 32) {
+            unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+            const uint32_t src = stage_s + (uint32_t)c16 * 16u;
+#pragma unroll
+            for (int r0 = 0; r0 < 16; r0 += 8) {
+                if (r0 < P.Q) {
+                    uint4 v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) v[i] = lds_v4(src + (uint32_t)min(r0 + i, P.Q - 1) * row_bytes);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) fma2_bf16x8(acc, v[i], ww[r0 + i]);   // rows past Q carry weight 0
+                }
+            }
+            float f[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) unpack_f32x2(acc[i], f[2 * i], f[2 * i + 1]);
+            uint4 pk;
+            __nv_bfloat162 h0 = __floats2bfloat162_rn(f[0], f[1]);
+            __nv_bfloat162 h1 = __floats2bfloat162_rn(f[2], f[3]);
+            __nv_bfloat162 h2 = __floats2bfloat162_rn(f[4], f[5]);
+            __nv_bfloat162 h3 = __floats2bfloat162_rn(f[6], f[7]);
+            pk.x = *reinterpret_cast<uint32_t *>(&h0);
+            pk.y = *reinterpret_cast<uint32_t *>(&h1);
+            pk.z = *reinterpret_cast<uint32_t *>(&h2);
+            pk.w = *reinterpret_cast<uint32_t *>(&h3);
+            __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), pk);
+        }
+    } else
+    for (int c16 = lane; c16 < ((n16 + 31) & ~31); c16 += 32) {
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        const uint32_t src = stage_s + (uint32_t)(c16 < n16 ? c16 : 0) * 16u;
+        for (int r0 = 0; r0 < P.Q; r0 += 8) {
+            uint4 v[8];
+            float w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int r = min(r0 + i, P.Q - 1);
+                v[i] = lds_v4(src + (uint32_t)r * row_bytes);
+                w[i] = lds_f32(wq_s + (uint32_t)r * 4u);
+                if (r0 + i >= P.Q) w[i] = 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                // a slot without a source row holds bytes nobody wrote: drop them
+                if (w[i] == 0.f) v[i] = make_uint4(0u, 0u, 0u, 0u);
+                fma_bf16x8(acc, v[i], w[i]);
+            }
+        }
+        if (c16 < n16) {
+            uint4 pk;
+            __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0], acc[1]);
+            __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[2], acc[3]);
+            __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[4], acc[5]);
+            __nv_bfloat162 h3 = __floats2bfloat162_rn(acc[6], acc[7]);
+            pk.x = *reinterpret_cast<uint32_t *>(&h0);
+            pk.y = *reinterpret_cast<uint32_t *>(&h1);
+            pk.z = *reinterpret_cast<uint32_t *>(&h2);
+            pk.w = *reinterpret_cast<uint32_t *>(&h3);
+            __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), pk);
+        }
+    }
+}
+
 // Communication warp.  Y is token-major: the k_tot * TP partial rows of one (token, split, column
 // slab) are one contiguous block (a "unit", at most 8 KB).  Every communication warp works on its own:
 // it owns two 8 KB stages of shared memory and one mbarrier per stage, fetches a unit with ONE bulk
@@ -1009,86 +1124,9 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
     auto consume = [&](const CommUnit &u, int st, uint32_t parity) -> bool {
         bool ok = wait_barrier(full_s + 8u * (uint32_t)st, parity, ctl, deadline2, P.status, (uint32_t)u.t, 43u);
         if (!ok) return false;
-        const int n16 = u.ucols >> 3;
-        const uint32_t row_bytes = (uint32_t)u.wslab * 2u;
-        // per-row weights, read back as shared-memory broadcasts inside the unrolled loop
-        if (lane < P.k_tot)
-            for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = u.w;
-        __syncwarp();
-        const uint32_t wq_s = smem_u32(wq);
-        const uint32_t stage_s = smem_u32(my_ring + st * kCommUnitBytes);
         __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(P.out[u.d]) +
                               (size_t)(u.t - u.d * P.tok_blk) * (size_t)P.H + u.s * P.split_w + (u.slab << P.slab_shift);
-        if (u.all_valid && P.Q <= 16) {
-            // common case: every slot has a source row and the unit has at most 16 rows: weights stay in
-            // registers as packed pairs, rows are fetched eight at a time, two FMAs per instruction
-            unsigned long long ww[16];
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const uint32_t wb = __float_as_uint(r < P.Q ? lds_f32(wq_s + (uint32_t)r * 4u) : 0.f);
-                ww[r] = pack_f32x2(wb, wb);
-            }
-            for (int c16 = lane; c16 < n16; c16 += 32) {
-                unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
-                const uint32_t src = stage_s + (uint32_t)c16 * 16u;
-#pragma unroll
-                for (int r0 = 0; r0 < 16; r0 += 8) {
-                    if (r0 < P.Q) {
-                        uint4 v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = lds_v4(src + (uint32_t)min(r0 + i, P.Q - 1) * row_bytes);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) fma2_bf16x8(acc, v[i], ww[r0 + i]);   // rows past Q carry weight 0
-                    }
-                }
-                float f[8];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) unpack_f32x2(acc[i], f[2 * i], f[2 * i + 1]);
-                uint4 pk;
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(f[0], f[1]);
-                __nv_bfloat162 h1 = __floats2bfloat162_rn(f[2], f[3]);
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(f[4], f[5]);
-                __nv_bfloat162 h3 = __floats2bfloat162_rn(f[6], f[7]);
-                pk.x = *reinterpret_cast<uint32_t *>(&h0);
-                pk.y = *reinterpret_cast<uint32_t *>(&h1);
-                pk.z = *reinterpret_cast<uint32_t *>(&h2);
-                pk.w = *reinterpret_cast<uint32_t *>(&h3);
-                __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), pk);
-            }
-        } else
-        for (int c16 = lane; c16 < ((n16 + 31) & ~31); c16 += 32) {
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const uint32_t src = stage_s + (uint32_t)(c16 < n16 ? c16 : 0) * 16u;
-            for (int r0 = 0; r0 < P.Q; r0 += 8) {
-                uint4 v[8];
-                float w[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = min(r0 + i, P.Q - 1);
-                    v[i] = lds_v4(src + (uint32_t)r * row_bytes);
-                    w[i] = lds_f32(wq_s + (uint32_t)r * 4u);
-                    if (r0 + i >= P.Q) w[i] = 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    // a slot without a source row holds bytes nobody wrote: drop them
-                    if (w[i] == 0.f) v[i] = make_uint4(0u, 0u, 0u, 0u);
-                    fma_bf16x8(acc, v[i], w[i]);
-                }
-            }
-            if (c16 < n16) {
-                uint4 pk;
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0], acc[1]);
-                __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[2], acc[3]);
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[4], acc[5]);
-                __nv_bfloat162 h3 = __floats2bfloat162_rn(acc[6], acc[7]);
-                pk.x = *reinterpret_cast<uint32_t *>(&h0);
-                pk.y = *reinterpret_cast<uint32_t *>(&h1);
-                pk.z = *reinterpret_cast<uint32_t *>(&h2);
-                pk.w = *reinterpret_cast<uint32_t *>(&h3);
-                __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), pk);
-            }
-        }
+        reduce_unit(P, u.w, u.all_valid, u.ucols, u.wslab, wq, smem_u32(my_ring + st * kCommUnitBytes), orow);
         __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
         TL(tl_last = globaltimer_ns(); if (tl_units == 0) tl_first = tl_last; ++tl_units; if (u.s < 4) ++tl_by_split[u.s]);
         return true;
@@ -1413,6 +1451,138 @@ __device__ __forceinline__ void comm_cta(const FusedParams &P, const Part &pt, u
     comm_warp<TN>(P, pt, ctl, res, role, c, warp, warp);
 }
 
+// Communication work of a launch with little of it (FusedParams::even): the units of all splits, dealt one by one over the
+// CTAs first, then over their warps 0-11, once all tiles are done.  Nothing is handed out and one thread of the CTA waits: the
+// queues' atomics and the polling of all warps on one word took longer than the work.  What is left of the tail is mostly
+// latency, instruction fetches among it (a launch runs this code once, from L2 at best): so the loop is short, one instance of
+// every step, rows four at a time.
+__device__ __forceinline__ void even_share(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp >= kCommWarps) return;
+    uint8_t *stages = ring + warp * kCommWarpBytes;
+    float *wq = reinterpret_cast<float *>(aux) + warp * 256;
+    const uint32_t full = smem_u32(&ctl->comm_full[2 * warp]), wq_s = smem_u32(wq);
+    const int n_slabs = (P.split_w + P.slab_cols - 1) >> P.slab_shift, per_split = P.T * n_slabs;
+    const int n_end = P.L * per_split, stride = kCommWarps * (int)gridDim.x;
+    int n = warp * (int)gridDim.x + (int)blockIdx.x;
+    const unsigned long long deadline = globaltimer_ns() + P.wait_ns, deadline2 = deadline + P.wait_ns / 4 + 1000000ull;
+    // routing of a unit's token, fetched one unit ahead: lane j, row and weight of slot j
+    int row = -1;
+    float w = 0.f;
+    const auto fetch_routing = [&]() {
+        row = -1;
+        w = 0.f;
+        if (n < n_end && lane < P.k_tot) {
+            const size_t f = (size_t)(n % per_split / n_slabs) * P.k_tot + lane;
+            row = ld_chained(&P.pad_row[f]);
+            w = ld_chained(&P.topk_w[f]);
+        }
+    };
+    fetch_routing();
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < P.L && !ctl->abort; ++s) {
+            uint32_t spins = 0;
+            while (ld_acquire_u32(&P.split_done[s]) < (uint32_t)(pt.W_comp * P.flag_parts)) {
+                if ((++spins & 31u) == 0u && globaltimer_ns() > deadline) {
+                    report(P.status, MOE_DEV_TIMEOUT, (uint32_t)s, 45u);
+                    ctl->abort = 1u;
+                    break;
+                }
+                __nanosleep(64);
+            }
+        }
+    }
+    asm volatile("bar.sync 2, %0;" ::"r"(32 * kCommWarps) : "memory");
+    if (__any_sync(0xffffffffu, ctl->abort != 0u)) return;
+    // rows published through ordinary stores are read by the copy engine next
+    asm volatile("fence.proxy.async;" ::: "memory");
+    const unsigned long long y_policy = l2_evict_first_policy();
+    const __nv_bfloat16 *Y = reinterpret_cast<const __nv_bfloat16 *>(P.Y);
+    // the unit in flight: issued one round ago
+    bool flying = false, all_valid = false;
+    int n16 = 0, row_bytes = 0, k = 0;
+    float w_f = 0.f;
+    __nv_bfloat16 *orow = nullptr;
+#pragma unroll 1
+    while (true) {
+        const bool have = n < n_end;
+        bool valid_n = false;
+        int n16_n = 0, row_bytes_n = 0;
+        float w_n = 0.f;
+        __nv_bfloat16 *orow_n = nullptr;
+        if (have) {
+            const int s = n / per_split, r = n - s * per_split, tok = r / n_slabs, c0 = (r - tok * n_slabs) << P.slab_shift;
+            const int split_cols = min(P.H, (s + 1) * P.split_w) - s * P.split_w, d = tok / P.tok_blk;
+            const int wslab = min(P.slab_cols, P.split_w - c0);            // layout pitch
+            n16_n = max(0, min(wslab, split_cols - c0)) >> 3;              // 16-byte chunks of real columns
+            row_bytes_n = wslab * 2;
+            if (lane < P.k_tot) {
+                if (row >= P.R_pad) {
+                    report(P.status, MOE_DEV_OOB, (uint32_t)row, 42u);
+                    row = -1;
+                }
+                if (row < 0) w = 0.f;
+            }
+            orow_n = reinterpret_cast<__nv_bfloat16 *>(P.out[d]) + (size_t)(tok - d * P.tok_blk) * (size_t)P.H + s * P.split_w + c0;
+            if (lane == 0) {
+                const uint32_t bytes = (uint32_t)(P.Q * row_bytes_n), bar = full + 8u * (uint32_t)(k & 1);
+                const __nv_bfloat16 *src = Y + (((size_t)tok * P.L + s) * (size_t)P.split_w + c0) * (size_t)P.Q;
+                mbar_arrive_expect_tx(bar, bytes);
+                bulk_load_once(smem_u32(stages + (k & 1) * kCommUnitBytes), src, bytes, bar, y_policy);   // Y is read once
+            }
+            w_n = w;
+            valid_n = __all_sync(0xffffffffu, lane >= P.k_tot || row >= 0);
+            ++k;
+            n += stride;
+            fetch_routing();
+        }
+        if (flying) {
+            const int prev = k - 1 - (have ? 1 : 0), st = prev & 1;
+            if (lane < P.k_tot)
+                for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w_f;
+            if (!wait_barrier(full + 8u * (uint32_t)st, (uint32_t)(prev >> 1) & 1u, ctl, deadline2, P.status, (uint32_t)n, 43u)) {
+                // (reported) the copy just issued must land before shared memory is released
+                const unsigned long long drain = globaltimer_ns() + 2000000ull;
+                while (have && !mbar_try_wait(full + 8u * (uint32_t)((k - 1) & 1), (uint32_t)((k - 1) >> 1) & 1u) && globaltimer_ns() < drain) {}
+                return;
+            }
+            __syncwarp();
+            const uint32_t stage_s = smem_u32(stages + st * kCommUnitBytes);
+#pragma unroll 1
+            for (int c16 = lane; c16 < n16; c16 += 32) {
+                unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+                uint32_t src = stage_s + (uint32_t)c16 * 16u;
+#pragma unroll 4
+                for (int q = 0; q < P.Q; ++q, src += (uint32_t)row_bytes) {
+                    uint4 v = lds_v4(src);
+                    const float wr = lds_f32(wq_s + (uint32_t)q * 4u);
+                    // a slot without a source row holds bytes nobody wrote: drop them
+                    if (!all_valid && wr == 0.f) v = make_uint4(0u, 0u, 0u, 0u);
+                    fma2_bf16x8(acc, v, pack_f32x2(__float_as_uint(wr), __float_as_uint(wr)));
+                }
+                uint32_t o[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float lo, hi;
+                    unpack_f32x2(acc[i], lo, hi);
+                    __nv_bfloat162 hh = __floats2bfloat162_rn(lo, hi);
+                    o[i] = *reinterpret_cast<uint32_t *>(&hh);
+                }
+                __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), make_uint4(o[0], o[1], o[2], o[3]));
+            }
+            __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
+        }
+        if (!have) break;
+        flying = true;
+        all_valid = valid_n;
+        n16 = n16_n;
+        row_bytes = row_bytes_n;
+        w_f = w_n;
+        orow = orow_n;
+    }
+}
+
 // Co-resident communication warp `cw` of a compute CTA: stages and weights in the aux region (free when
 // the epilogue stores straight from registers, which the host checks before it asks for such warps).
 template <int TN>
@@ -1475,9 +1645,12 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     Control *ctl = reinterpret_cast<Control *>(ring + kStageBytesTotal);
     uint8_t *aux = reinterpret_cast<uint8_t *>(ring + kStageBytesTotal + ((sizeof(Control) + 127) & ~(size_t)127));
+    const int warp = threadIdx.x >> 5;
 
+    // what does not depend on the predecessor is done before the wait for it: barriers, TMEM, tensor maps
     init_comm_barriers(ctl);
-    if (threadIdx.x == 32) {
+    if (P.P > 0) compute_setup<TN>(P, ctl);
+    if (threadIdx.x == 96) {
         prefetch_tensormap(&P.tmA);
         prefetch_tensormap(&P.tmB);
     }
@@ -1487,14 +1660,16 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
         P.queue_next[threadIdx.x] = 0ull;
     }
     const Part pt = launch_part(P);
+    tc_fence_before();
     __syncthreads();          // the only barrier all 20 warps share
+    tc_fence_after();
     TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < pt.C ? 0u : 1u); });
 
-    const int warp = threadIdx.x >> 5;
-    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // an idle warp of communication CTA 0
+    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // a warp that does not communicate
         mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if ((int)blockIdx.x < pt.C) {
-        comm_cta<TN>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
+        if (warp == 1 && P.P > 0) tmem_dealloc(ctl->tmem_base, Cfg<TN>::kTmemCols);
+        if (!P.even) comm_cta<TN>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
     } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
         if (co_warp_number(warp) < P.co_warps) co_resident_warp<TN>(P, pt, ctl, aux, co_warp_number(warp));
         return;
@@ -1502,8 +1677,9 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
         compute_cta<TN>(P, pt, ring, ctl, aux, (int)blockIdx.x - pt.C);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         // out of GEMM tiles: help with the communication that is left (all TMA and TMEM traffic is over)
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !ctl->abort) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleBack, 0);
+        if (P.drain_help && P.mode == MOE_MODE_FUSED && !P.even && !ctl->abort) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleBack, 0);
     }
+    if (P.even) even_share(P, pt, ring, ctl, aux);
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
 
@@ -1522,9 +1698,10 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
     Control *ctl = reinterpret_cast<Control *>(ring + kStageBytesTotal + (seven ? PairCfg::kStageBytes : 0));
     uint8_t *aux = seven ? ring + kStageBytesTotal
                          : reinterpret_cast<uint8_t *>(ring + kStageBytesTotal + ((sizeof(Control) + 127) & ~(size_t)127));
+    const int warp = threadIdx.x >> 5;
 
     init_comm_barriers(ctl);
-    if (threadIdx.x == 32) {
+    if (threadIdx.x == 96) {
         prefetch_tensormap(&P.tmA);
         prefetch_tensormap(&P.tmB);
     }
@@ -1537,16 +1714,15 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
     __syncthreads();          // the only CTA-wide barrier all 20 warps share
     TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < ((pt.C + 1) & ~1) ? 0u : 1u); });
 
-    const int warp = threadIdx.x >> 5;
     const int c_even = (pt.C + 1) & ~1;
-    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // an idle warp of communication CTA 0
+    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // a warp that does not communicate
         mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if ((int)blockIdx.x < pt.C) {
-        comm_cta<256>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
+        if (!P.even) comm_cta<256>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
     } else if ((int)blockIdx.x < c_even) {
         // odd C: the last communication CTA's cluster-mate cannot compute (no partner).  With dynamic work
         // distribution it serves communication work as well; under the static map it has no tile list.
-        if (P.drain_help && P.mode == MOE_MODE_FUSED) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront, (int)blockIdx.x);
+        if (P.drain_help && P.mode == MOE_MODE_FUSED && !P.even) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront, (int)blockIdx.x);
     } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
         // The compute warps of both CTAs meet at two cluster barriers (set-up and teardown), and a cluster
         // barrier counts every thread: these warps join the first, arrive at once on the second (they hold
@@ -1559,8 +1735,9 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
     } else {
         compute_cta_pair(P, pt, ring, ctl, aux, ((int)blockIdx.x - c_even) >> 1);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack, 0);
+        if (P.drain_help && P.mode == MOE_MODE_FUSED && !P.even && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack, 0);
     }
+    if (P.even) even_share(P, pt, ring, ctl, aux);
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
 

@@ -19,6 +19,7 @@ constexpr int kFusedThreads = kThreads + 32 * kCoWarpsMax;   // block size of th
 constexpr int kBlockK = 64;            // bf16 elements per k-block: one 128-byte swizzle row
 constexpr int kUmmaK = 16;             // K of one tcgen05.mma.kind::f16 instruction
 constexpr int kMmaM = 128;             // M of the MMA (tile_m = 64 stores the first 64 rows only)
+constexpr int kXBoxRows = 32;          // rows of one x_routed box of a one-CTA tile of the fused kernel
 constexpr int kStageBytesTotal = 192 * 1024;  // operand ring, all stages together
 constexpr int kCommTileM = 128;        // T_M^comm
 constexpr int kCommTileN = 1024;       // T_N^comm
@@ -62,6 +63,9 @@ struct alignas(64) FusedParams {
     int32_t c_table_first, c_table_n;   // c_table[i]: communication CTAs when S = c_table_first + i (0 entries: C and P above hold)
     uint8_t c_table[kPlanTableMax];
     int32_t tok_blk, tok_tiles_per_rank, comm_cols, comm_tiles;
+    int32_t even;                       // the communication work is dealt evenly to all warps once all tiles are done (no per-tile
+                                        // flags, no queue)
+    int32_t w2_once;                    // W2 is read (about) once: its lines go first when L2 needs room
     int32_t num_kb, last_ksteps;
     int32_t drain_help;                 // compute CTAs serve communication tiles once their GEMM tiles are done
     int32_t co_warps;                   // co-resident communication warps per compute CTA (0..2)
@@ -82,7 +86,7 @@ namespace moe {
 // what the two operand tensor maps of the fused kernel depend on
 struct TensorMapKey {
     const void *x, *w2;
-    int32_t T, k_tot, I, H, E_tot, box_n;
+    int32_t T, k_tot, I, H, E_tot, box_n, box_m;
 };
 // The selector's pick for every m-tile count S that a routing of one shape can have: plan_partition depends on the
 // routed counts through their sum alone (but for tile-level readiness, which is not tabulated).

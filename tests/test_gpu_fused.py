@@ -643,3 +643,33 @@ def test_the_selection_of_the_whole_step_call_is_the_selector_s(kw, limits):
         own = [len(G.tokens_of_rank(w.T, w.EP, d)) for d in range(w.EP)]
         for a, o, n in zip(ref_outs, ws.out, own):
             assert np.array_equal(a[:n], o.float().cpu().numpy()[:n])
+
+
+@pytest.mark.parametrize("kw", [
+    dict(T=1, E=9, k=3, H=208, I=80),                        # one wave of 64-column tiles, the last one partial
+    dict(T=1, E=40, k=8, H=1536, I=512, TP=2),               # one wave, tiles of the plan's CTAs filled by bound
+    dict(T=33, E=2, k=2, H=256, I=64, L=8, EP=8),            # 32-column splits, ranks without a token
+    dict(T=70, E=12, k=9, H=264, I=64, TP=2),                # 18 rows per unit, 16-byte stores, ragged width
+    dict(T=300, E=5, k=2, H=512, I=128, tile_m=64),          # 33, 64 and more rows in a 64-row tile: boxes of 32 rows
+    dict(T=600, E=3, k=2, H=1024, I=192, tile_m=256, L=2),   # CTA pairs
+], ids=str)
+def test_even_shares_at_the_edges(kw):
+    base = dict(name="even", routing_seed=5, data_seed=6, TP=1, EP=1, L=1, tile_m=128, tile_n=256, routing="zipf", zipf_s=1.2)
+    base.update(kw)
+    w = replace(wl.TINY, **base)
+    if -(-w.H // w.L) < 256 and w.tile_m != 256:
+        w = replace(w, tile_n=128 if -(-w.H // w.L) >= 128 else 64)
+    _check_against_oracle(w)
+    # a slot without an expert: reported, left out of its token's sum
+    idx, wt, _ = wl.make_routing(w)
+    x, W2 = wl.make_data(w)
+    bad = idx.copy()
+    bad[0, 1] = w.E_tot + 7
+    outs, _, ws, S, st = G.run_layer(w, bad, wt, x, W2, check_status=False)
+    assert st.code == B.MOE_DEV_OOB and st.count == 1
+    got = np.concatenate([o[:len(G.tokens_of_rank(w.T, w.EP, d))] for d, o in enumerate(outs)])
+    f = G.routing_to_numpy(ws, S)["inv_perm"].reshape(w.T, w.k_tot)
+    assert f[0, 1] == -1
+    xf, Wf = x.float().numpy(), W2.float().numpy()
+    want = sum(wt[0, j] * (Wf[bad[0, j]] @ xf[f[0, j]]) for j in range(w.k_tot) if j != 1)
+    assert np.max(np.abs(got[0] - want)) <= G.tolerance(want)
