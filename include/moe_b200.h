@@ -185,7 +185,8 @@ typedef struct {
  * residency (Section III-E: the SM count is cached at operator initialisation).  Also allocates the
  * handle's only memory outside the C++ heap: about 8 KB of pinned host memory that the GPU can address,
  * the mailbox through which the routed-tile counts reach the host in the whole-step calls
- * (moe_layer, moe_post_router_layer); freed by moe_destroy.  No device memory is allocated.  [host] */
+ * (moe_layer, moe_post_router_layer, moe_layer_host); freed by moe_destroy.  No device memory is allocated.
+ * [host] */
 int32_t moe_create(int32_t device, moe_handle **out);
 int32_t moe_destroy(moe_handle *h);
 /* Text of the last failing CUDA call on this handle ("" if none); owned by the handle. */
@@ -430,6 +431,8 @@ int32_t moe_calibrate_rho(moe_handle *h, const void *x_routed, const void *W2, c
  * topk_w from (pinned) host memory into `arena`, builds the routing, waits for the tile
  * counts, plans, launches the fused kernel and copies the EP output blocks back to
  * out_host (bf16 [T, H], token order).  W2 stays device resident (weights).  Synchronous.
+ * Larger x_routed are copied beside the GEMM on a stream that the handle makes on the first such call
+ * (with 64 KB of pinned host memory for the small inputs; moe_destroy frees both).
  * arena [device] of at least moe_host_arena_bytes(); plan_out may be NULL. */
 int32_t moe_host_arena_bytes(const moe_shape *shape, int32_t tile_m, int32_t tile_n, size_t *bytes);
 int32_t moe_layer_host(moe_handle *h, const void *x_routed_host, const int32_t *topk_idx_host,

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 from dataclasses import dataclass
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -251,7 +252,10 @@ def moe_build_routing_static(h, topk_idx, shape, tile_m, routing, tile_counts_ho
 def plan_partition(routed_tile_counts, occ, limits, shape, rho) -> moe_plan:
     """routed_tile_counts: host int32 sequence of ceil(M_e / T_M)."""
     n = len(routed_tile_counts)
-    arr = (C.c_int32 * n)(*[int(v) for v in routed_tile_counts])
+    try:     # (a list of ints at once: element by element took longer than the selection)
+        arr = (C.c_int32 * n).from_buffer(array("i", routed_tile_counts))
+    except TypeError:
+        arr = (C.c_int32 * n)(*[int(v) for v in routed_tile_counts])
     plan = moe_plan()
     _check(lib().plan_partition(arr, n, C.byref(occ), C.byref(limits), C.byref(shape), C.byref(rho),
                                 C.byref(plan)), "plan_partition")

@@ -32,6 +32,35 @@ int32_t require_handle_device(moe_handle *h, const char *who)
     return MOE_OK;
 }
 
+const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name)
+{
+    if (!h->maps && !(h->maps = new (std::nothrow) MapEntry[kMapEntries]())) return nullptr;
+    const uint64_t mixed = (reinterpret_cast<uintptr_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull;
+    MapEntry &m = h->maps[mixed >> 57];
+    static_assert(kMapEntries == 1 << (64 - 57), "the hash's upper bits index the table");
+    if (m.ptr == ptr && m.rows == rows && m.cols == cols && m.planes == planes && m.box_rows == box_rows) return &m.map;
+    typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
+                                      const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                      CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+    const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * (cuuint64_t)rows};
+    const cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)box_rows, 1}, es[3] = {1, 1, 1};
+    m.ptr = nullptr;
+    const CUresult cr = reinterpret_cast<EncodeTiledFn>(h->encode_tiled)(
+        &m.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, planes ? 3 : 2, const_cast<void *>(ptr), dims, strides, box, es,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (cr != CUDA_SUCCESS) {
+        snprintf(h->err, sizeof h->err, "cuTensorMapEncodeTiled(%s) failed: %d", name, (int)cr);
+        return nullptr;
+    }
+    m.rows = rows;
+    m.cols = cols;
+    m.planes = planes;
+    m.box_rows = box_rows;
+    m.ptr = ptr;
+    return &m.map;
+}
+
 namespace {
 
 inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -62,11 +91,6 @@ int32_t n_routing_warps(const moe_shape *s)
 {
     return (int32_t)ceil_div((int64_t)s->T * s->k_tot, kRoutingChunk);
 }
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
 
 }  // namespace
 }  // namespace moe
@@ -147,8 +171,13 @@ int32_t moe_create(int32_t device, moe_handle **out)
 
 int32_t moe_destroy(moe_handle *h)
 {
+    if (h && h->staging) cudaFreeHost(h->staging);
+    if (h && h->feed_stream) cudaStreamDestroy(h->feed_stream);
+    for (int i = 0; h && i < 2; ++i)
+        if (h->feed_events[i]) cudaEventDestroy(h->feed_events[i]);
     if (h && h->counts_event) cudaEventDestroy(static_cast<cudaEvent_t>(h->counts_event));
     if (h && h->mail_host) cudaFreeHost(h->mail_host);
+    if (h) delete[] h->maps;
     if (h) delete[] h->plan_tables;
     delete h;
     return MOE_OK;
@@ -471,7 +500,7 @@ const PlanTable *plan_table(moe_handle *h, const moe_shape *s, const moe_occupan
 // mail_seq != 0: this launch mails the counts
 int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                              const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
-                             const PlanTable *table, uint32_t mail_seq, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
+                             const PlanTable *table, uint32_t mail_seq, const RowFeed *feed, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
                              void *stream);
 
 }  // namespace
@@ -484,7 +513,7 @@ int32_t moe_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, c
                           void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream)
 {
     (void)topk_idx;
-    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, nullptr, 0u, out, y_ws, flags_ws, status_dev, stream);
+    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, nullptr, 0u, nullptr, out, y_ws, flags_ws, status_dev, stream);
 }
 
 }  // extern "C"
@@ -493,7 +522,7 @@ namespace {
 
 int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                              const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
-                             const PlanTable *table, uint32_t mail_seq, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
+                             const PlanTable *table, uint32_t mail_seq, const RowFeed *feed, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
                              void *stream)
 {
     if (!h || !s || !occ || !r || !plan || !out || !status_dev) return MOE_ERR_NULL;
@@ -564,15 +593,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     }
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
     p.tok_blk = (int32_t)ceil_div(s->T, s->EP);
-    p.tok_tiles_per_rank = (int32_t)ceil_div(p.tok_blk, kCommTileM);
     p.comm_cols = (int32_t)ceil_div(p.split_w, kCommTileN);
-    int64_t tok_tiles = 0;
-    for (int d = 0; d < s->EP; ++d) {
-        int64_t own = (int64_t)s->T - (int64_t)d * p.tok_blk;
-        if (own > p.tok_blk) own = p.tok_blk;
-        if (own > 0) tok_tiles += ceil_div(own, kCommTileM);
-    }
-    p.comm_tiles = (int32_t)(tok_tiles * p.comm_cols);
     p.num_kb = (int32_t)ceil_div(K, kBlockK);
     p.last_ksteps = (K - (p.num_kb - 1) * kBlockK) / kUmmaK;
     p.R_pad = (long long)occ->tile_m * n_mtiles;
@@ -595,6 +616,10 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
                     (reinterpret_cast<uintptr_t>(y_ws) & 31u) == 0) ? 1 : 0;
     p.status = status_dev;
     for (int d = 0; d < s->EP; ++d) p.out[d] = out[d];
+    if (feed) {
+        p.x_ready = feed->ready;
+        p.wait_ns += feed->extra_wait_ns;
+    }
     // Co-resident communication warps need the dynamic hand-out (they pull from the queues), the aux region
     // of shared memory (free only when the epilogue stores straight from registers) and units of at most 16
     // rows; where one of these does not hold the launch runs without them (same result, bit for bit).
@@ -656,44 +681,13 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.queue_next = reinterpret_cast<unsigned long long *>(flags_ws + 2 * MOE_MAX_L) + ((ep + 1u) & 1u) * MOE_MAX_L;
     p.flags = flags_ws + kSplitCounterWords;
 
-    // tensor maps (Section II-A operands): x_routed [R, I] and W2 [E_tot, H, I], k contiguous.  Encoding the two
-    // maps costs microseconds of host time between the wait for the tile counts and the launch: the handle
-    // keeps the last pair and reuses it while buffers, sizes and tile family stay the same (a loop of steps).
-    const TensorMapKey key = {x_routed, W2, s->T, s->k_tot, s->I, s->H, s->E_tot, pair ? TN / 2 : TN, pair ? kMmaM : kXBoxRows};
-    if (!h->tm_valid || memcmp(&h->tm_key, &key, sizeof key) != 0) {
-        EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(h->encode_tiled);
-        h->tm_valid = false;
-        {
-            cuuint64_t dims[2] = {(cuuint64_t)s->I, (cuuint64_t)R};
-            cuuint64_t strides[1] = {(cuuint64_t)s->I * 2};
-            cuuint32_t box[2] = {(cuuint32_t)kBlockK, (cuuint32_t)(pair ? kMmaM : kXBoxRows)};
-            cuuint32_t es[2] = {1, 1};
-            CUresult cr = encode(&h->tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(x_routed), dims,
-                                 strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (cr != CUDA_SUCCESS) {
-                snprintf(h->err, sizeof h->err, "cuTensorMapEncodeTiled(x_routed) failed: %d", (int)cr);
-                return MOE_ERR_CUDA;
-            }
-        }
-        {
-            cuuint64_t dims[3] = {(cuuint64_t)s->I, (cuuint64_t)s->H, (cuuint64_t)s->E_tot};
-            cuuint64_t strides[2] = {(cuuint64_t)s->I * 2, (cuuint64_t)s->H * s->I * 2};
-            cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)(pair ? TN / 2 : TN), 1};   // a pair CTA loads half the rows
-            cuuint32_t es[3] = {1, 1, 1};
-            CUresult cr = encode(&h->tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(W2), dims, strides,
-                                 box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (cr != CUDA_SUCCESS) {
-                snprintf(h->err, sizeof h->err, "cuTensorMapEncodeTiled(W2) failed: %d", (int)cr);
-                return MOE_ERR_CUDA;
-            }
-        }
-        h->tm_key = key;
-        h->tm_valid = true;
-    }
-    p.tmA = h->tmA;
-    p.tmB = h->tmB;
+    // operands (Section II-A): x_routed [R, I] and W2 [E_tot, H, I], k contiguous; a pair CTA loads half the n-tile's rows
+    const CUtensorMap *mA = operand_map(h, x_routed, 0, R, s->I, pair ? kMmaM : kXBoxRows, "x_routed");
+    if (!mA) return MOE_ERR_CUDA;
+    p.tmA = *mA;
+    const CUtensorMap *mB = operand_map(h, W2, s->E_tot, s->H, s->I, pair ? TN / 2 : TN, "W2");
+    if (!mB) return MOE_ERR_CUDA;
+    p.tmB = *mB;
     const int grid = pair ? ((C + 1) & ~1) + 2 * Pc : ctas_c + ctas_p;
     p.timeline = nullptr;
     if (h->timeline && h->timeline_bytes >= ((size_t)grid * kTimelineSlots + MOE_MAX_L) * sizeof(unsigned long long))
@@ -730,7 +724,7 @@ int32_t selection_of(moe_handle *h, const moe_shape *s, int32_t tile_m, int32_t 
 // (seq = 0).
 int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                           const Selection &sel, const moe_routing *routing, uint32_t seq, uint32_t mail_seq,
-                          cudaEvent_t counts_event, int32_t *tile_counts, void *const *out, void *y_ws, uint32_t *flags_ws,
+                          const RowFeed *feed, cudaEvent_t counts_event, int32_t *tile_counts, void *const *out, void *y_ws, uint32_t *flags_ws,
                           uint32_t *status_dev, moe_plan *plan_out, void *ev_before, void *ev_after, cudaStream_t st)
 {
     moe_plan plan;
@@ -748,7 +742,7 @@ int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, c
         if ((rc = plan_partition_estimate(&sel.occ, &sel.lim, s, &sel.rho, &plan)) != MOE_OK) return rc;   // counts stay on the device
     }
     if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
-    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, sel.table, mail_seq, out, y_ws,
+    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, sel.table, mail_seq, feed, out, y_ws,
                               flags_ws, status_dev, st);
     if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
     if (rc == MOE_OK && sel.table) rc = counts_and_plan();
@@ -772,8 +766,9 @@ int32_t moe_get_status(moe_handle *h, const uint32_t *status_dev, moe_status *ho
 {
     if (!h || !status_dev || !host) return MOE_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    uint32_t w[4];
-    cudaError_t e = cudaMemcpyAsync(w, status_dev, sizeof w, cudaMemcpyDeviceToHost, st);
+    // (through the mailbox's spare words: a copy to pageable memory is staged by the driver)
+    uint32_t on_stack[4], *w = h->mail_host ? reinterpret_cast<uint32_t *>(h->mail_host + kMailWords - 2) : on_stack;
+    cudaError_t e = cudaMemcpyAsync(w, status_dev, sizeof on_stack, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "status copy");
     host->code = w[0]; host->detail = w[1]; host->where = w[2]; host->count = w[3];
@@ -803,7 +798,7 @@ int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int
     uint32_t seq = 0;
     rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, sel.table != nullptr, status_dev, st, &seq);
     if (rc != MOE_OK) return rc;
-    return select_and_launch(h, x_routed, W2, topk_w, s, sel, routing, seq, seq, nullptr, tile_counts_pinned, out, y_ws, flags_ws,
+    return select_and_launch(h, x_routed, W2, topk_w, s, sel, routing, seq, seq, nullptr, nullptr, tile_counts_pinned, out, y_ws, flags_ws,
                              status_dev, plan_out, ev_before, ev_after, st);
 }
 
@@ -832,7 +827,7 @@ int32_t moe_post_router_layer(moe_handle *h, const void *hidden, const void *W1,
     rc = launch_gemm1_act(h, hidden, W1, s, tile_m, routing, MOE_MTILES_ON_DEVICE, h_routed_ws, x_routed_ws, status_dev, seq, st);
     if (rc != MOE_OK) return rc;
     if (tile_counts_pinned && seq == 0u && !counts_event) return MOE_ERR_CUDA;
-    return select_and_launch(h, x_routed_ws, W2, topk_w, s, sel, routing, seq, 0u, counts_event, tile_counts_pinned, out, y_ws,
+    return select_and_launch(h, x_routed_ws, W2, topk_w, s, sel, routing, seq, 0u, nullptr, counts_event, tile_counts_pinned, out, y_ws,
                              flags_ws, status_dev, plan_out, nullptr, nullptr, st);
 }
 
@@ -920,17 +915,45 @@ int32_t arena_layout(const moe_shape *s, int tile_m, int tile_n, ArenaLayout *a)
     if (rc != MOE_OK) return rc;
     const size_t R = (size_t)s->T * s->k_tot;
     auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    // idx, w, status and flags lie together: one copy brings the small inputs and the zeros (moe_layer_host)
     size_t off = 0;
     a->x = off; off += up(R * s->I * 2);
     a->idx = off; off += up(R * 4);
     a->w = off; off += up(R * 4);
+    a->status = off; off += up(16);
+    a->flags = off; off += up(a->flags_b);
     a->routing = off; off += up(a->routing_b);
     a->y = off; off += up(a->y_b);
-    a->flags = off; off += up(a->flags_b);
-    a->status = off; off += up(16);
     a->out = off; off += up((size_t)ceil_div(s->T, s->EP) * s->EP * s->H * 2);
     a->total = off;
     return MOE_OK;
+}
+constexpr size_t kFeedMinBytes = 2 << 20;    // x_routed from which the copies overlap the GEMM
+constexpr size_t kFeedLastBytes = 1 << 20;   // the last chunk holds this much or less
+typedef CUresult (*WriteValueFn)(CUstream, CUdeviceptr, cuuint32_t, unsigned int);
+// The stream and events of the overlapped copies, made on first use; false: not to be had, copy first instead.
+bool feed_ready(moe_handle *h)
+{
+    if (h->feed_stream) return true;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuStreamWriteValue32", &h->write_value, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess || !h->write_value) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    for (cudaEvent_t &ev : h->feed_events)
+        if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return false;
+    return cudaStreamCreateWithFlags(&h->feed_stream, cudaStreamNonBlocking) == cudaSuccess;
+}
+constexpr size_t kStagingBytes = 64 << 10;
+// The pinned buffer through which the small inputs go as one copy, made on first use.
+bool staging_ready(moe_handle *h)
+{
+    if (!h->staging && cudaHostAlloc(reinterpret_cast<void **>(&h->staging), kStagingBytes, cudaHostAllocPortable) != cudaSuccess) {
+        (void)cudaGetLastError();
+        h->staging = nullptr;
+    }
+    return h->staging != nullptr;
 }
 }  // namespace
 
@@ -960,50 +983,78 @@ int32_t moe_layer_host(moe_handle *h, const void *x_routed_host, const int32_t *
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *base = static_cast<char *>(arena);
     const size_t R = (size_t)s->T * s->k_tot;
-    cudaError_t e;
-    e = cudaMemcpyAsync(base + a.idx, topk_idx_host, R * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + a.status, 0, 16, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "idx copy");
+    Selection sel;
+    rc = selection_of(h, s, tile_m, tile_n, limits_or_null, true, &sel);
+    if (rc != MOE_OK) return rc;
+    if ((rc = require_handle_device(h, "moe_layer_host")) != MOE_OK) return rc;
     moe_routing rt;
     rc = moe_routing_view(base + a.routing, s, tile_m, &rt);
     if (rc != MOE_OK) return rc;
-    uint32_t *status = reinterpret_cast<uint32_t *>(base + a.status);
-    rc = moe_build_routing(h, reinterpret_cast<int32_t *>(base + a.idx), s, tile_m, &rt, tile_counts_pinned,
-                           status, st);
-    if (rc != MOE_OK) return rc;
-    cudaEvent_t counts_ready;
-    e = cudaEventCreateWithFlags(&counts_ready, cudaEventDisableTiming);
-    if (e != cudaSuccess) return cuda_fail(h, e, "event");
-    cudaEventRecord(counts_ready, st);
-    // the large copies overlap the wait for the counts
-    e = cudaMemcpyAsync(base + a.x, x_routed_host, R * s->I * 2, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base + a.w, topk_w_host, R * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + a.flags, 0, a.flags_b, st);
-    if (e == cudaSuccess) e = cudaEventSynchronize(counts_ready);
-    cudaEventDestroy(counts_ready);
-    if (e != cudaSuccess) return cuda_fail(h, e, "input copies");
+    uint32_t *status = reinterpret_cast<uint32_t *>(base + a.status), *ready = status + 16;   // (256 bytes lie there)
+    cudaError_t e;
+    const size_t small_b = a.flags + a.flags_b - a.idx;
+    if (small_b <= kStagingBytes && staging_ready(h)) {
+        // (the previous call on this handle has waited for its copy out of the staging buffer)
+        memset(h->staging, 0, small_b);
+        memcpy(h->staging, topk_idx_host, R * 4);
+        memcpy(h->staging + (a.w - a.idx), topk_w_host, R * 4);
+        e = cudaMemcpyAsync(base + a.idx, h->staging, small_b, cudaMemcpyHostToDevice, st);
+    } else {
+        e = cudaMemcpyAsync(base + a.idx, topk_idx_host, R * 4, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(base + a.w, topk_w_host, R * 4, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, a.flags + a.flags_b - a.status, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(h, e, "idx copy");
     h->epochs.erase(base + a.flags);  // the workspace was just cleared
-
-    moe_occupancy occ;
-    moe_sm_limits lim;
-    moe_rho rho;
-    rc = moe_query_occupancy(h, tile_m, tile_n, &occ, &lim, &rho);
-    if (rc != MOE_OK) return rc;
-    if (limits_or_null) lim = *limits_or_null;
-    moe_plan plan;
-    rc = plan_partition(tile_counts_pinned, s->E_tot, &occ, &lim, s, &rho, &plan);
-    if (rc != MOE_OK) return rc;
-    if (plan_out) *plan_out = plan;
+    // The rows of x_routed are most of the copies, and the GEMM takes them in order: from 2 MB on they come in chunks on a
+    // stream of the handle's, each with the rows so far written behind it, which the kernel's x producers wait for, so that the
+    // GEMM runs beside the copies.  A chunk costs the copy engine 7 us, so there are few: each brings 60 % of what is left,
+    // the last one 1 MB or less.
+    RowFeed feed = {nullptr, 0};
+    const size_t row_b = (size_t)s->I * 2, x_b = R * row_b;
+    const bool fed = x_b >= kFeedMinBytes && feed_ready(h);
+    // (nothing is left in flight on the way out: the caller's buffers and the handle's staging buffer are free again)
+    const auto fail = [&](int32_t code) {
+        cudaStreamSynchronize(st);
+        if (fed) cudaStreamSynchronize(h->feed_stream);
+        return code;
+    };
+    if (fed) {
+        feed.ready = ready;
+        feed.extra_wait_ns = x_b / 10;               // 10 GB/s: far below what a host link moves
+        e = cudaEventRecord(h->feed_events[0], st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->feed_stream, h->feed_events[0], 0);
+    } else {
+        e = cudaMemcpyAsync(base + a.x, x_routed_host, x_b, cudaMemcpyHostToDevice, st);
+    }
+    if (e != cudaSuccess) return fail(cuda_fail(h, e, "input copies"));
+    uint32_t seq = 0;
+    rc = build_routing_mailed(h, reinterpret_cast<int32_t *>(base + a.idx), s, tile_m, &rt, tile_counts_pinned, sel.table != nullptr,
+                              status, st, &seq);
+    if (rc != MOE_OK) return fail(rc);
+    for (size_t r = 0; fed && r < R && e == cudaSuccess;) {
+        size_t rows = R - r;
+        if (rows * row_b > kFeedLastBytes) rows = (rows * 3 + 4) / 5;
+        e = cudaMemcpyAsync(base + a.x + r * row_b, static_cast<const char *>(x_routed_host) + r * row_b, rows * row_b,
+                            cudaMemcpyHostToDevice, h->feed_stream);
+        r += rows;
+        if (e == cudaSuccess && reinterpret_cast<WriteValueFn>(h->write_value)(h->feed_stream, (CUdeviceptr)(uintptr_t)ready, (cuuint32_t)r, 0) != CUDA_SUCCESS)
+            e = cudaErrorUnknown;
+    }
+    if (fed && e == cudaSuccess) e = cudaEventRecord(h->feed_events[1], h->feed_stream);
+    if (e != cudaSuccess) return fail(cuda_fail(h, e, "input copies"));
     void *outs[MOE_MAX_EP];
     const size_t blk = (size_t)ceil_div(s->T, s->EP);
     for (int d = 0; d < s->EP; ++d) outs[d] = base + a.out + (size_t)d * blk * s->H * 2;
-    rc = moe_gemm2_combine(h, base + a.x, W2_dev, nullptr, reinterpret_cast<float *>(base + a.w), s, &occ, &rt,
-                           tile_counts_pinned[s->E_tot], &plan, outs, base + a.y,
-                           reinterpret_cast<uint32_t *>(base + a.flags), status, st);
-    if (rc != MOE_OK) return rc;
+    rc = select_and_launch(h, base + a.x, W2_dev, reinterpret_cast<float *>(base + a.w), s, sel, &rt, seq, sel.table ? seq : 0u,
+                           fed ? &feed : nullptr, nullptr, tile_counts_pinned, outs, base + a.y,
+                           reinterpret_cast<uint32_t *>(base + a.flags), status, plan_out, nullptr, nullptr, st);
+    if (rc != MOE_OK) return fail(rc);
+    // whatever the kernel needed of the rows, their copies are over before the caller has its buffers back
+    if (fed) e = cudaStreamWaitEvent(st, h->feed_events[1], 0);
     // rank d owns tokens [d*blk, (d+1)*blk): the EP blocks are contiguous in token order
-    e = cudaMemcpyAsync(out_host, base + a.out, (size_t)s->T * s->H * 2, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "output copy");
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, base + a.out, (size_t)s->T * s->H * 2, cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return fail(cuda_fail(h, e, "output copy"));
     moe_status hs;
     return moe_get_status(h, status, &hs, st);
 }

@@ -434,11 +434,6 @@ template <bool kPair>
 constexpr size_t g1_smem_bytes() { return (size_t)G1Cfg<kPair>::kRingBytes + 1024 + ((sizeof(G1Control) + 127) & ~(size_t)127); }
 static_assert(g1_smem_bytes<true>() <= 227 * 1024, "GEMM1 pair stages exceed the shared memory of an SM");
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-
 inline bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
 }  // namespace
@@ -515,21 +510,10 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     p.last_ksteps = (s->H - (p.num_kb - 1) * kBlockK) / kUmmaK;
     if ((int64_t)n_mtiles * p.NT >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
 
-    EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(h->encode_tiled);
-    {
-        // W1 [E_tot][2][I][H] seen as [E_tot * 2 planes][I rows][H]: rows past I of a plane read zeros
-        cuuint64_t dims[3] = {(cuuint64_t)s->H, (cuuint64_t)s->I, (cuuint64_t)s->E_tot * 2};
-        cuuint64_t strides[2] = {(cuuint64_t)s->H * 2, (cuuint64_t)s->H * 2 * (cuuint64_t)s->I};
-        cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)kG1TileN, 1};
-        cuuint32_t es[3] = {1, 1, 1};
-        CUresult cr = encode(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(W1), dims, strides, box, es,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (cr != CUDA_SUCCESS) {
-            snprintf(h->err, sizeof h->err, "cuTensorMapEncodeTiled(W1) failed: %d", (int)cr);
-            return MOE_ERR_CUDA;
-        }
-    }
+    // W1 [E_tot][2][I][H] seen as [E_tot * 2 planes][I rows][H]: rows past I of a plane read zeros
+    const CUtensorMap *mB = operand_map(h, W1, 2 * s->E_tot, s->I, s->H, kG1TileN, "W1");
+    if (!mB) return MOE_ERR_CUDA;
+    p.tmB = *mB;
 
     const bool pair = tile_m == 256;
     const int64_t tiles_bound = (int64_t)n_mtiles * p.NT;

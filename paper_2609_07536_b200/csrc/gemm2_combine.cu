@@ -2,10 +2,9 @@
 // role by blockIdx.
 //
 //   blockIdx <  C : communication CTA c (Section II-B: consumes published results; the same
-//                   C CTAs serve all splits in sequence; CTA c takes communication tiles
-//                   c, c+C, ... of a split -- or, with drain help, its warps pull token ranges from a queue
-//                   per split, or take an even share of the units once the tiles are done; former compute
-//                   CTAs do the same).
+//                   C CTAs serve all splits in sequence, its warps an even share of every split's
+//                   units -- or, with drain help, all CTAs serve once their tiles are done, by even
+//                   shares, or from a queue of token ranges per split).
 //   blockIdx >= C : compute CTA b = blockIdx - C (Section III-C: takes global tiles
 //                   b, b+P, b+2P, ... of the split-major sequence in which the expert
 //                   problems of one split are contiguous; m-tile-major across the splits when
@@ -216,6 +215,28 @@ __device__ __forceinline__ Tile decode_tile(int g, const FusedParams &P, int W_c
         t.id = t.s * W_comp + r * P.NTs + t.i_n;
     }
     return t;
+}
+
+// x_routed that is still being copied in (FusedParams::x_ready): waits until the rows up to `last_row` have arrived.  One
+// thread; `seen`: rows known to have arrived.  The copies were issued before this launch, so the wait ends on its own.
+__device__ __forceinline__ bool wait_rows(const FusedParams &P, int last_row, uint32_t &seen, Control *ctl, unsigned long long deadline)
+{
+    const uint32_t need = (uint32_t)last_row + 1u;
+    if (seen >= need) return true;
+    uint32_t spins = 0;
+    while ((seen = ld_acquire_sys_u32(P.x_ready)) < need) {
+        __nanosleep(200);
+        if ((++spins & 15u) == 0u) {
+            if (ctl->abort) return false;
+            if (globaltimer_ns() > deadline) {
+                ctl->abort = 1u;
+                report(P.status, MOE_DEV_TIMEOUT, (uint32_t)last_row, 46u);
+                return false;
+            }
+        }
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");   // read next by TMA
+    return true;
 }
 
 // --------------------------------------------------------------------------- epilogue helper
@@ -569,6 +590,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
             uint32_t phase = 0;
             uint32_t armed = 0;  // bit s: stage s was handed to the TMA unit at least once
             bool ok = true;
+            uint32_t seen = 0;
             const unsigned long long w_policy = P.w2_once ? l2_evict_first_policy() : l2_evict_normal_policy();
             TL_DECL(long long tl_pw = 0, tl_q;)
             // the m-tile table entries of the NEXT tile are fetched while this tile's k-blocks are issued, so
@@ -586,6 +608,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                 // rows come in boxes of kXBoxRows: those past the end of the expert's last tile are not fetched, nothing stored
                 // depends on them
                 const int boxes = min((valid + kXBoxRows - 1) / kXBoxRows, kMmaM / kXBoxRows);
+                if (load_a && P.x_ready && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
                 int kx = t.p * P.K;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     TL(tl_q = clock64());
@@ -781,11 +804,16 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
             Tile t = decode_tile(b, P, pt.W_comp);
             int e = ld_chained(&P.mtile_expert[t.mu]);
             int row0 = ld_chained(&P.mtile_first_row[t.mu]) + (int)rank * kMmaM;
+            uint32_t seen = 0;
             for (int g = b; g < total_tiles && ok; g += pt.P) {
                 const Tile t_next = decode_tile(min(g + pt.P, total_tiles - 1), P, pt.W_comp);
                 const int e_next = ld_chained(&P.mtile_expert[t_next.mu]);
                 const int row0_next = ld_chained(&P.mtile_first_row[t_next.mu]) + (int)rank * kMmaM;
                 const int n0 = t.s * P.split_w + t.i_n * TN + (int)rank * (TN / 2);
+                if (load_a && P.x_ready) {
+                    const int last = ld_chained(&P.mtile_first_row[t.mu]) + ld_chained(&P.mtile_valid[t.mu]) - 1;
+                    if (!(ok = wait_rows(P, last, seen, ctl, deadline))) break;
+                }
                 int kx = t.p * P.K;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     const uint32_t own_full = smem_u32(&ctl->full[stage]);
@@ -1057,8 +1085,6 @@ __device__ __forceinline__ void reduce_unit(const FusedParams &P, float w, bool 
 // overlap across the warps of an SM.
 //
 // Who runs it (role):
-//   kRoleStatic      warp w of communication CTA c, static map: units w, w+12, ... of the communication
-//                    tiles c, c+C, ... of every split (the paper's map);
 //   kRoleFront       warp of a communication CTA, dynamic hand-out: ranges from the front of the
 //                    per-split queues, split 0 first; a unit waits for the tiles under it (flags);
 //   kRoleBack        warp of a compute CTA whose GEMM tiles are done (drain help): ranges from the back,
@@ -1083,7 +1109,7 @@ static_assert(PairCfg::kStageBytes + ((sizeof(Control) + 127) & ~(size_t)127) <=
 static_assert(kCoWeightsOffset + (kCoWarpsMax + kCommWarps) * kCoWeightFloats * 4 <= kAuxBytes,
               "co-resident stages and weights exceed the aux region");
 
-enum { kRoleStatic = 0, kRoleFront = 1, kRoleBack = 2, kRoleCoResident = 3 };
+enum { kRoleFront = 1, kRoleBack = 2, kRoleCoResident = 3 };
 
 // what one communication warp owns
 struct CommWarpRes {
@@ -1099,10 +1125,8 @@ struct CommUnit {
     bool all_valid;   // every slot of the token has a source row
 };
 
-// `c`, `warp`: communication CTA and warp inside it (static map only).
 template <int TN>
-__device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, const CommWarpRes res, int role, int c, int warp,
-                          int tl_slot)
+__device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, const CommWarpRes res, int role, int tl_slot)
 {
     (void)tl_slot;   // index of the warp's record in a timeline build
     const int lane = threadIdx.x & 31;
@@ -1132,7 +1156,6 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
         return true;
     };
 
-    int unit = 0;            // running unit number of this CTA
     int n_mine = 0;          // units this warp has issued so far: stage n_mine & 1, parity (n_mine >> 1) & 1
     CommUnit prev;
     prev.live = false;
@@ -1212,65 +1235,6 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
         return true;
     };
 
-    // serve communication tile ct of split s; false when this warp had to give up (reported)
-    auto serve_tile = [&](int s, int ct) -> bool {
-        const int split_c0 = s * P.split_w;
-        const int split_c1 = min(P.H, split_c0 + P.split_w);
-        const int tok_tile = ct / P.comm_cols;
-        const int col_tile = ct - tok_tile * P.comm_cols;
-        const int d = tok_tile / P.tok_tiles_per_rank;
-        const int ti = tok_tile - d * P.tok_tiles_per_rank;
-        const int t0 = d * P.tok_blk + ti * kCommTileM;
-        const int t1 = min(min(P.T, (d + 1) * P.tok_blk), t0 + kCommTileM);
-        const int c0 = split_c0 + col_tile * kCommTileN;
-        const int c1 = min(split_c1, c0 + kCommTileN);
-        if (t0 >= t1 || c0 >= c1) return true;
-        const int slab0 = (c0 - split_c0) >> P.slab_shift;
-        const int n_slabs = ((c1 - split_c0 + P.slab_cols - 1) >> P.slab_shift) - slab0;
-        const int n_units = (t1 - t0) * n_slabs;
-        // first unit of this tile that belongs to this warp
-        int k = (warp - unit % kCommWarps + kCommWarps) % kCommWarps;
-        // routing of a unit's token is fetched one unit ahead, off the per-unit critical path
-        int nxt_row = -1;
-        float nxt_w = 0.f;
-        if (k < n_units && lane < P.k_tot) {
-            const int tn = t0 + k / n_slabs;
-            nxt_row = ld_chained(&P.pad_row[(size_t)tn * P.k_tot + lane]);
-            nxt_w = ld_chained(&P.topk_w[(size_t)tn * P.k_tot + lane]);
-        }
-        for (; k < n_units; k += kCommWarps) {
-            CommUnit u;
-            u.t = t0 + k / n_slabs;
-            u.slab = slab0 + k % n_slabs;
-            u.d = d;
-            u.s = s;
-            u.wslab = min(P.slab_cols, P.split_w - (u.slab << P.slab_shift));            // layout pitch
-            u.ucols = min(u.wslab, split_c1 - split_c0 - (u.slab << P.slab_shift));       // real columns
-            u.live = true;
-            int my_row = nxt_row;
-            u.w = nxt_w;
-            if (k + kCommWarps < n_units && lane < P.k_tot) {
-                const int tn = t0 + (k + kCommWarps) / n_slabs;
-                nxt_row = ld_chained(&P.pad_row[(size_t)tn * P.k_tot + lane]);
-                nxt_w = ld_chained(&P.topk_w[(size_t)tn * P.k_tot + lane]);
-            }
-            if (lane < P.k_tot) {
-                if (my_row >= P.R_pad) {
-                    report(P.status, MOE_DEV_OOB, (uint32_t)my_row, 42u);
-                    my_row = -1;
-                }
-                if (my_row < 0) u.w = 0.f;
-            }
-            u.all_valid = __all_sync(0xffffffffu, lane >= P.k_tot || my_row >= 0);
-            if (!unit_step(u)) {
-                unit += n_units;
-                return false;
-            }
-        }
-        unit += n_units;
-        return true;
-    };
-
     // serve items [i0, i1) of split s on this warp alone.  An item is one token x one communication
     // column tile (token-major numbering); its units are the column slabs of that tile.
     auto serve_items = [&](int s, uint32_t i0, uint32_t i1) -> bool {
@@ -1323,15 +1287,7 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
         return true;
     };
 
-    if (role == kRoleStatic) {
-        // the paper's static map: communication tile ct belongs to CTA ct mod C (Section III-A)
-        for (int s = 0; s < P.L; ++s)
-            for (int ct = c; ct < P.comm_tiles; ct += pt.C)
-                if (!serve_tile(s, ct)) {
-                    ctl->abort = 1u;
-                    return;
-                }
-    } else {
+    {
         // Dynamic hand-out, to warps.  Every split has a two-ended queue of its items in one 64-bit word
         // (low half: items taken from the front, high half: from the back).  Warps of the communication
         // CTAs and co-resident warps take from the front, split 0 first; warps of compute CTAs that have
@@ -1438,7 +1394,7 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
 // The communication warps of a CTA whose only role is communication (dedicated communication CTA, or a
 // compute CTA that has run out of GEMM tiles): warps 0-11, stages in the operand ring.
 template <int TN>
-__device__ __forceinline__ void comm_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int role, int c)
+__device__ __forceinline__ void comm_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int role)
 {
     const int warp = threadIdx.x >> 5;
     if (warp >= kCommWarps) return;
@@ -1448,138 +1404,175 @@ __device__ __forceinline__ void comm_cta(const FusedParams &P, const Part &pt, u
     res.wq = (role == kRoleBack && P.co_warps > 0)
                  ? reinterpret_cast<float *>(aux + kCoWeightsOffset) + (kCoWarpsMax + warp) * kCoWeightFloats
                  : reinterpret_cast<float *>(aux) + warp * 256;
-    comm_warp<TN>(P, pt, ctl, res, role, c, warp, warp);
+    comm_warp<TN>(P, pt, ctl, res, role, warp);
 }
 
-// Communication work of a launch with little of it (FusedParams::even): the units of all splits, dealt one by one over the
-// CTAs first, then over their warps 0-11, once all tiles are done.  Nothing is handed out and one thread of the CTA waits: the
-// queues' atomics and the polling of all warps on one word took longer than the work.  What is left of the tail is mostly
-// latency, instruction fetches among it (a launch runs this code once, from L2 at best): so the loop is short, one instance of
-// every step, rows four at a time.
-__device__ __forceinline__ void even_share(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux)
+// Communication work by shares: the units of a split, dealt one by one over the serving CTAs first, then over their warps
+// 0-11, once the tiles under them are done: all CTAs when the compute CTAs help (FusedParams::even: once for all splits), the
+// communication CTAs under the static partition (split after split).  Nothing is handed out and one thread of the CTA waits:
+// the queues' atomics and the polling of all warps on one word took longer than the work of a small launch; and with whole
+// communication tiles per CTA (the paper's map) CTAs have no work where tiles are few (DeepSeek shape, T = 2048, EP = 4, static:
+// 16 tiles a split, so that 32 CTAs took as long as 16, 218 us; 167 us by units).  What is left of a small launch's tail is
+// mostly latency, instruction fetches among it (it runs this code once, from L2 at best): so the loop is short, one instance of
+// every step.  (Rows read straight into registers by 20 warps, eight loads ahead, instead of by one bulk copy per unit into
+// shared memory: 46 GB/s a CTA instead of 56.)
+// `c` of `n_ctas` serving CTAs.
+constexpr int kRowsAhead = 4;   // rows of a unit fetched from shared memory together
+__device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int c, int n_ctas)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp >= kCommWarps) return;
     uint8_t *stages = ring + warp * kCommWarpBytes;
-    float *wq = reinterpret_cast<float *>(aux) + warp * 256;
+    float *wq = reinterpret_cast<float *>(aux) + warp * 256;      // weights of the unit's rows
     const uint32_t full = smem_u32(&ctl->comm_full[2 * warp]), wq_s = smem_u32(wq);
-    const int n_slabs = (P.split_w + P.slab_cols - 1) >> P.slab_shift, per_split = P.T * n_slabs;
-    const int n_end = P.L * per_split, stride = kCommWarps * (int)gridDim.x;
-    int n = warp * (int)gridDim.x + (int)blockIdx.x;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns, deadline2 = deadline + P.wait_ns / 4 + 1000000ull;
-    // routing of a unit's token, fetched one unit ahead: lane j, row and weight of slot j
-    int row = -1;
-    float w = 0.f;
-    const auto fetch_routing = [&]() {
-        row = -1;
-        w = 0.f;
-        if (n < n_end && lane < P.k_tot) {
-            const size_t f = (size_t)(n % per_split / n_slabs) * P.k_tot + lane;
-            row = ld_chained(&P.pad_row[f]);
-            w = ld_chained(&P.topk_w[f]);
-        }
-    };
-    fetch_routing();
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < P.L && !ctl->abort; ++s) {
-            uint32_t spins = 0;
-            while (ld_acquire_u32(&P.split_done[s]) < (uint32_t)(pt.W_comp * P.flag_parts)) {
-                if ((++spins & 31u) == 0u && globaltimer_ns() > deadline) {
-                    report(P.status, MOE_DEV_TIMEOUT, (uint32_t)s, 45u);
-                    ctl->abort = 1u;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-    }
-    asm volatile("bar.sync 2, %0;" ::"r"(32 * kCommWarps) : "memory");
-    if (__any_sync(0xffffffffu, ctl->abort != 0u)) return;
-    // rows published through ordinary stores are read by the copy engine next
-    asm volatile("fence.proxy.async;" ::: "memory");
     const unsigned long long y_policy = l2_evict_first_policy();
     const __nv_bfloat16 *Y = reinterpret_cast<const __nv_bfloat16 *>(P.Y);
-    // the unit in flight: issued one round ago
-    bool flying = false, all_valid = false;
-    int n16 = 0, row_bytes = 0, k = 0;
-    float w_f = 0.f;
-    __nv_bfloat16 *orow = nullptr;
+    // unit n of a split: token n / n_slabs, column slab n % n_slabs; this warp's next one is `workers` on
+    const int n_slabs = (P.split_w + P.slab_cols - 1) >> P.slab_shift, workers = kCommWarps * n_ctas;
+    const int step_tok = workers / n_slabs, step_slab = workers - step_tok * n_slabs;
+    int k = 0;                // copies issued so far: stage k & 1, parity (k >> 1) & 1
 #pragma unroll 1
-    while (true) {
-        const bool have = n < n_end;
-        bool valid_n = false;
-        int n16_n = 0, row_bytes_n = 0;
-        float w_n = 0.f;
-        __nv_bfloat16 *orow_n = nullptr;
-        if (have) {
-            const int s = n / per_split, r = n - s * per_split, tok = r / n_slabs, c0 = (r - tok * n_slabs) << P.slab_shift;
-            const int split_cols = min(P.H, (s + 1) * P.split_w) - s * P.split_w, d = tok / P.tok_blk;
-            const int wslab = min(P.slab_cols, P.split_w - c0);            // layout pitch
-            n16_n = max(0, min(wslab, split_cols - c0)) >> 3;              // 16-byte chunks of real columns
-            row_bytes_n = wslab * 2;
-            if (lane < P.k_tot) {
-                if (row >= P.R_pad) {
-                    report(P.status, MOE_DEV_OOB, (uint32_t)row, 42u);
-                    row = -1;
-                }
-                if (row < 0) w = 0.f;
-            }
-            orow_n = reinterpret_cast<__nv_bfloat16 *>(P.out[d]) + (size_t)(tok - d * P.tok_blk) * (size_t)P.H + s * P.split_w + c0;
-            if (lane == 0) {
-                const uint32_t bytes = (uint32_t)(P.Q * row_bytes_n), bar = full + 8u * (uint32_t)(k & 1);
-                const __nv_bfloat16 *src = Y + (((size_t)tok * P.L + s) * (size_t)P.split_w + c0) * (size_t)P.Q;
-                mbar_arrive_expect_tx(bar, bytes);
-                bulk_load_once(smem_u32(stages + (k & 1) * kCommUnitBytes), src, bytes, bar, y_policy);   // Y is read once
-            }
-            w_n = w;
-            valid_n = __all_sync(0xffffffffu, lane >= P.k_tot || row >= 0);
-            ++k;
-            n += stride;
-            fetch_routing();
+    for (int s = 0; s < P.L; ++s) {
+        int n = warp * n_ctas + c;
+        if (P.even && s > 0) {     // the deal goes on where the split before ended
+            n -= (int)((long long)s * P.T * n_slabs % workers);
+            if (n < 0) n += workers;
         }
-        if (flying) {
-            const int prev = k - 1 - (have ? 1 : 0), st = prev & 1;
-            if (lane < P.k_tot)
-                for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w_f;
-            if (!wait_barrier(full + 8u * (uint32_t)st, (uint32_t)(prev >> 1) & 1u, ctl, deadline2, P.status, (uint32_t)n, 43u)) {
-                // (reported) the copy just issued must land before shared memory is released
-                const unsigned long long drain = globaltimer_ns() + 2000000ull;
-                while (have && !mbar_try_wait(full + 8u * (uint32_t)((k - 1) & 1), (uint32_t)((k - 1) >> 1) & 1u) && globaltimer_ns() < drain) {}
-                return;
+        int tok = n / n_slabs, slab = n - tok * n_slabs, d = 0;
+        // routing of a unit's token, fetched one unit ahead: lane j, row and weight of slot j
+        int row = -1;
+        float w = 0.f;
+        const auto fetch_routing = [&]() {
+            row = -1;
+            w = 0.f;
+            if (tok < P.T && lane < P.k_tot) {
+                row = ld_chained(&P.pad_row[(size_t)tok * P.k_tot + lane]);
+                w = ld_chained(&P.topk_w[(size_t)tok * P.k_tot + lane]);
             }
-            __syncwarp();
-            const uint32_t stage_s = smem_u32(stages + st * kCommUnitBytes);
-#pragma unroll 1
-            for (int c16 = lane; c16 < n16; c16 += 32) {
-                unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
-                uint32_t src = stage_s + (uint32_t)c16 * 16u;
-#pragma unroll 4
-                for (int q = 0; q < P.Q; ++q, src += (uint32_t)row_bytes) {
-                    uint4 v = lds_v4(src);
-                    const float wr = lds_f32(wq_s + (uint32_t)q * 4u);
-                    // a slot without a source row holds bytes nobody wrote: drop them
-                    if (!all_valid && wr == 0.f) v = make_uint4(0u, 0u, 0u, 0u);
-                    fma2_bf16x8(acc, v, pack_f32x2(__float_as_uint(wr), __float_as_uint(wr)));
+        };
+        fetch_routing();
+        if (P.mode != MOE_MODE_COMBINE_ONLY && (s == 0 || !P.even)) {
+            if (threadIdx.x == 0) {
+                for (int sw = s; sw < (P.even ? P.L : s + 1) && !ctl->abort; ++sw) {
+                    uint32_t spins = 0;
+                    while (ld_acquire_u32(&P.split_done[sw]) < (uint32_t)(pt.W_comp * P.flag_parts)) {
+                        if ((++spins & 31u) == 0u && globaltimer_ns() > deadline) {
+                            report(P.status, MOE_DEV_TIMEOUT, (uint32_t)sw, 45u);
+                            ctl->abort = 1u;
+                            break;
+                        }
+                        __nanosleep(64);
+                    }
                 }
-                uint32_t o[4];
+            }
+            asm volatile("bar.sync 2, %0;" ::"r"(32 * kCommWarps) : "memory");
+            // rows published through ordinary stores are read by the copy engine next
+            asm volatile("fence.proxy.async;" ::: "memory");
+        }
+        // (a warp that gives up keeps coming to the barriers)
+        if (__any_sync(0xffffffffu, ctl->abort != 0u)) continue;
+        // the unit in flight: issued one round ago
+        bool flying = false, all_valid = false;
+        int n16 = 0, row_bytes = 0;
+        float w_f = 0.f;
+        __nv_bfloat16 *orow = nullptr;
+#pragma unroll 1
+        while (true) {
+            const bool have = tok < P.T;
+            bool valid_n = false;
+            int n16_n = 0, row_bytes_n = 0;
+            float w_n = 0.f;
+            __nv_bfloat16 *orow_n = nullptr;
+            if (have) {
+                const int c0 = slab << P.slab_shift, split_cols = min(P.H, (s + 1) * P.split_w) - s * P.split_w;
+                const int wslab = min(P.slab_cols, P.split_w - c0);            // layout pitch
+                n16_n = max(0, min(wslab, split_cols - c0)) >> 3;              // 16-byte chunks of real columns
+                row_bytes_n = wslab * 2;
+                while (tok >= (d + 1) * P.tok_blk) ++d;                        // owning rank
+                if (lane < P.k_tot) {
+                    if (row >= P.R_pad) {
+                        report(P.status, MOE_DEV_OOB, (uint32_t)row, 42u);
+                        row = -1;
+                    }
+                    if (row < 0) w = 0.f;
+                }
+                orow_n = reinterpret_cast<__nv_bfloat16 *>(P.out[d]) + (size_t)(tok - d * P.tok_blk) * (size_t)P.H + s * P.split_w + c0;
+                if (lane == 0) {
+                    const uint32_t bytes = (uint32_t)(P.Q * row_bytes_n), bar = full + 8u * (uint32_t)(k & 1);
+                    const __nv_bfloat16 *src = Y + (((size_t)tok * P.L + s) * (size_t)P.split_w + c0) * (size_t)P.Q;
+                    mbar_arrive_expect_tx(bar, bytes);
+                    bulk_load_once(smem_u32(stages + (k & 1) * kCommUnitBytes), src, bytes, bar, y_policy);   // Y is read once
+                }
+                w_n = w;
+                valid_n = __all_sync(0xffffffffu, lane >= P.k_tot || row >= 0);
+                ++k;
+                tok += step_tok;
+                slab += step_slab;
+                if (slab >= n_slabs) {
+                    slab -= n_slabs;
+                    ++tok;
+                }
+                fetch_routing();
+            }
+            if (flying) {
+                const int prev = k - 1 - (have ? 1 : 0), st = prev & 1;
+                if (lane < P.k_tot)
+                    for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w_f;
+                if (!wait_barrier(full + 8u * (uint32_t)st, (uint32_t)(prev >> 1) & 1u, ctl, deadline2, P.status, (uint32_t)tok, 43u)) {
+                    // (reported) the copy just issued must land before shared memory is released
+                    const unsigned long long drain = globaltimer_ns() + 2000000ull;
+                    while (have && !mbar_try_wait(full + 8u * (uint32_t)((k - 1) & 1), (uint32_t)((k - 1) >> 1) & 1u) && globaltimer_ns() < drain) {}
+                    break;
+                }
+                __syncwarp();
+                const uint32_t stage_s = smem_u32(stages + st * kCommUnitBytes);
+#pragma unroll 1
+                for (int c16 = lane; c16 < n16; c16 += 32) {
+                    unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+                    uint32_t src = stage_s + (uint32_t)c16 * 16u, wsrc = wq_s;
+#pragma unroll 1
+                    for (int q = 0; q < P.Q; q += kRowsAhead, wsrc += 4u * kRowsAhead) {
+                        uint4 v[kRowsAhead];
+                        float wr[kRowsAhead];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float lo, hi;
-                    unpack_f32x2(acc[i], lo, hi);
-                    __nv_bfloat162 hh = __floats2bfloat162_rn(lo, hi);
-                    o[i] = *reinterpret_cast<uint32_t *>(&hh);
+                        for (int i = 0; i < kRowsAhead; ++i, src += (uint32_t)row_bytes)
+                            v[i] = q + i < P.Q ? lds_v4(src) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                        for (int i = 0; i < kRowsAhead; i += 4) {
+                            const uint4 w4 = lds_v4(wsrc + 4u * i);
+                            wr[i] = __uint_as_float(w4.x);
+                            wr[i + 1] = __uint_as_float(w4.y);
+                            wr[i + 2] = __uint_as_float(w4.z);
+                            wr[i + 3] = __uint_as_float(w4.w);
+                        }
+#pragma unroll
+                        for (int i = 0; i < kRowsAhead; ++i) {
+                            // a slot without a source row holds bytes nobody wrote, and there is no row past Q: nothing is added
+                            if ((!all_valid && wr[i] == 0.f) || q + i >= P.Q) v[i] = make_uint4(0u, 0u, 0u, 0u), wr[i] = 0.f;
+                            fma2_bf16x8(acc, v[i], pack_f32x2(__float_as_uint(wr[i]), __float_as_uint(wr[i])));
+                        }
+                    }
+                    uint32_t o[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float lo, hi;
+                        unpack_f32x2(acc[i], lo, hi);
+                        __nv_bfloat162 hh = __floats2bfloat162_rn(lo, hi);
+                        o[i] = *reinterpret_cast<uint32_t *>(&hh);
+                    }
+                    __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), make_uint4(o[0], o[1], o[2], o[3]));
                 }
-                __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), make_uint4(o[0], o[1], o[2], o[3]));
+                __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
             }
-            __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
+            if (!have) break;
+            flying = true;
+            all_valid = valid_n;
+            n16 = n16_n;
+            row_bytes = row_bytes_n;
+            w_f = w_n;
+            orow = orow_n;
         }
-        if (!have) break;
-        flying = true;
-        all_valid = valid_n;
-        n16 = n16_n;
-        row_bytes = row_bytes_n;
-        w_f = w_n;
-        orow = orow_n;
     }
 }
 
@@ -1592,7 +1585,7 @@ __device__ __forceinline__ void co_resident_warp(const FusedParams &P, const Par
     res.stages = aux + cw * kCommWarpBytes;
     res.full = &ctl->co_full[2 * cw];
     res.wq = reinterpret_cast<float *>(aux + kCoWeightsOffset) + cw * kCoWeightFloats;
-    comm_warp<TN>(P, pt, ctl, res, kRoleCoResident, 0, 0, cw);
+    comm_warp<TN>(P, pt, ctl, res, kRoleCoResident, cw);
 }
 
 // Co-resident warp number of warp 16..19.  The four warp schedulers of an SM take warps by number modulo
@@ -1665,11 +1658,12 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
     tc_fence_after();
     TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < pt.C ? 0u : 1u); });
 
-    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // a warp that does not communicate
+    const bool queued = P.drain_help && !P.even;           // (drain help is a matter of fused launches)
+    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)
         mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if ((int)blockIdx.x < pt.C) {
         if (warp == 1 && P.P > 0) tmem_dealloc(ctl->tmem_base, Cfg<TN>::kTmemCols);
-        if (!P.even) comm_cta<TN>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
+        if (queued) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleFront);
     } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
         if (co_warp_number(warp) < P.co_warps) co_resident_warp<TN>(P, pt, ctl, aux, co_warp_number(warp));
         return;
@@ -1677,9 +1671,9 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
         compute_cta<TN>(P, pt, ring, ctl, aux, (int)blockIdx.x - pt.C);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         // out of GEMM tiles: help with the communication that is left (all TMA and TMEM traffic is over)
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !P.even && !ctl->abort) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleBack, 0);
+        if (queued && !ctl->abort) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleBack);
     }
-    if (P.even) even_share(P, pt, ring, ctl, aux);
+    if (P.even || (!queued && (int)blockIdx.x < pt.C)) serve_shares(P, pt, ring, ctl, aux, (int)blockIdx.x, P.even ? (int)gridDim.x : pt.C);
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
 
@@ -1715,14 +1709,15 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
     TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < ((pt.C + 1) & ~1) ? 0u : 1u); });
 
     const int c_even = (pt.C + 1) & ~1;
-    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)   // a warp that does not communicate
+    const bool queued = P.drain_help && !P.even;           // (drain help is a matter of fused launches)
+    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)
         mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if ((int)blockIdx.x < pt.C) {
-        if (!P.even) comm_cta<256>(P, pt, ring, ctl, aux, P.drain_help ? kRoleFront : kRoleStatic, (int)blockIdx.x);
+        if (queued) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront);
     } else if ((int)blockIdx.x < c_even) {
         // odd C: the last communication CTA's cluster-mate cannot compute (no partner).  With dynamic work
         // distribution it serves communication work as well; under the static map it has no tile list.
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !P.even) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront, (int)blockIdx.x);
+        if (queued) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront);
     } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
         // The compute warps of both CTAs meet at two cluster barriers (set-up and teardown), and a cluster
         // barrier counts every thread: these warps join the first, arrive at once on the second (they hold
@@ -1735,9 +1730,9 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
     } else {
         compute_cta_pair(P, pt, ring, ctl, aux, ((int)blockIdx.x - c_even) >> 1);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
-        if (P.drain_help && P.mode == MOE_MODE_FUSED && !P.even && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack, 0);
+        if (queued && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack);
     }
-    if (P.even) even_share(P, pt, ring, ctl, aux);
+    if (P.even || (!queued && (int)blockIdx.x < pt.C)) serve_shares(P, pt, ring, ctl, aux, (int)blockIdx.x, P.even ? (int)gridDim.x : pt.C);
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
 

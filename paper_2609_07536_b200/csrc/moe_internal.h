@@ -62,9 +62,10 @@ struct alignas(64) FusedParams {
     int32_t G, slot_sms;                // c_table: SMs the partition is made of, SMs of one compute slot
     int32_t c_table_first, c_table_n;   // c_table[i]: communication CTAs when S = c_table_first + i (0 entries: C and P above hold)
     uint8_t c_table[kPlanTableMax];
-    int32_t tok_blk, tok_tiles_per_rank, comm_cols, comm_tiles;
+    int32_t tok_blk, comm_cols;
     int32_t even;                       // the communication work is dealt evenly to all warps once all tiles are done (no per-tile
                                         // flags, no queue)
+    const uint32_t *x_ready;            // != nullptr: x_routed is still being copied in; the rows that have arrived
     int32_t w2_once;                    // W2 is read (about) once: its lines go first when L2 needs room
     int32_t num_kb, last_ksteps;
     int32_t drain_help;                 // compute CTAs serve communication tiles once their GEMM tiles are done
@@ -83,10 +84,20 @@ struct alignas(64) FusedParams {
 }  // namespace moe
 
 namespace moe {
-// what the two operand tensor maps of the fused kernel depend on
-struct TensorMapKey {
-    const void *x, *w2;
-    int32_t T, k_tot, I, H, E_tot, box_n, box_m;
+// An operand tensor map (bf16, k contiguous, 64 x box_rows boxes, 128B swizzle) and what it was encoded for: [rows, cols], or
+// [planes, rows, cols].  Encoding one costs a microsecond of host time per launch: the handle keeps the maps of the operands that
+// it has seen (a model's layers, the buffers of a loop of steps) in a small direct-mapped table.
+struct alignas(64) MapEntry {
+    CUtensorMap map;
+    const void *ptr;
+    int64_t rows;
+    int32_t cols, planes, box_rows;
+};
+constexpr int kMapEntries = 128;
+// x_routed of a launch that starts while the rows are still being copied in (host-buffer entry point)
+struct RowFeed {
+    const uint32_t *ready;         // [device] rows that have arrived, written behind each copy
+    uint64_t extra_wait_ns;        // what the copies may add to the kernel's wait limit
 };
 // The selector's pick for every m-tile count S that a routing of one shape can have: plan_partition depends on the
 // routed counts through their sum alone (but for tile-level readiness, which is not tabulated).
@@ -119,13 +130,15 @@ struct moe_handle {
     unsigned long long *mail_host = nullptr;
     unsigned long long *mail_dev = nullptr;             // the same memory as the GPU addresses it
     uint32_t mail_seq = 0;
+    char *staging = nullptr;                            // host-buffer entry point: pinned, the small inputs on their way to the GPU
+    cudaStream_t feed_stream = nullptr;                 // host-buffer entry point: copies x_routed in beside the caller's stream ...
+    cudaEvent_t feed_events[2] = {nullptr, nullptr};    // ... from the first event on, up to the second
+    void *write_value = nullptr;                        // cuStreamWriteValue32
     void *counts_event = nullptr;                       // cudaEvent_t: "the tile counts have reached the host"
     unsigned long long *timeline = nullptr;             // timeline build: where the next fused launch records
     size_t timeline_bytes = 0;
     uint32_t probe = 0;                                 // timeline build: moe_set_probe bits for the next launches
-    CUtensorMap tmA, tmB;                               // last encoded operand tensor maps of the fused kernel ...
-    moe::TensorMapKey tm_key = {};                      // ... and what they were encoded for
-    bool tm_valid = false;
+    moe::MapEntry *maps = nullptr;                      // [kMapEntries], by a hash of the operand's address
     moe::PlanTable *plan_tables = nullptr;              // [kPlanTables], used as a ring
     int n_plan_tables = 0, next_plan_table = 0;
 };
@@ -190,6 +203,8 @@ int32_t cuda_fail(moe_handle *h, cudaError_t e, const char *what);
 // message in the handle) otherwise.  Every launching entry point checks it: kernels run on the
 // current device, the buffers and the cached residency belong to the handle's.
 int32_t require_handle_device(moe_handle *h, const char *who);
+// the tensor map of an operand (planes = 0: two dimensions); nullptr, with a message in the handle, when it cannot be encoded
+const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name);
 // fused kernel (gemm2_combine.cu)
 size_t fused_smem_bytes(int tile_n);
 cudaError_t fused_occupancy(int tile_n, int *blocks_per_sm);

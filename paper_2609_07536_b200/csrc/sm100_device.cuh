@@ -367,6 +367,13 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+// ... of a word that the copy engine or the stream writes
+__device__ __forceinline__ uint32_t ld_acquire_sys_u32(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.sys.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 // Release fence at GPU scope for a flag published with a relaxed store afterwards.  Lighter than
 // __threadfence(), which is a sequentially consistent fence.
 __device__ __forceinline__ void fence_acq_rel_gpu()

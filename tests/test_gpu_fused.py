@@ -673,3 +673,33 @@ def test_even_shares_at_the_edges(kw):
     xf, Wf = x.float().numpy(), W2.float().numpy()
     want = sum(wt[0, j] * (Wf[bad[0, j]] @ xf[f[0, j]]) for j in range(w.k_tot) if j != 1)
     assert np.max(np.abs(got[0] - want)) <= G.tolerance(want)
+
+
+@pytest.mark.parametrize("kw", [
+    dict(T=700, tile_m=256, tile_n=256),         # CTA pairs, rows in 10 chunks
+    dict(T=90, tile_m=128, tile_n=256),          # under the size that is copied in chunks
+    dict(T=3000, tile_m=128, tile_n=128),        # the most chunks, more tile counts than the selection tabulates
+], ids=str)
+@pytest.mark.parametrize("pinned", [True, False], ids=["pinned", "pageable"])
+def test_host_buffers_copied_in_beside_the_gemm(kw, pinned):
+    h = G.handle()
+    w = replace(wl.GRANITE, name="hostfeed", **kw)
+    if w.T == 3000:
+        w = replace(w, E=300, k=3)
+    idx, wt, _ = wl.make_routing(w)
+    x, W2 = wl.make_data(w)
+    dev, plan, ws, S, st = G.run_layer(w, idx, wt, x, W2)
+    shape = G.shape_of(w)
+    nbytes = B.moe_host_arena_bytes(shape, w.tile_m, w.tile_n)
+    arena = torch.full((nbytes + 256,), 255, dtype=torch.uint8, device="cuda")      # (NaNs wherever nothing was copied yet)
+    off = (-arena.data_ptr()) % 256
+    host = lambda t: t.pin_memory() if pinned else t
+    xh, ih, wh = host(x), host(torch.from_numpy(idx)), host(torch.from_numpy(wt))
+    counts = torch.zeros(w.E_tot + 1, dtype=torch.int32).pin_memory()
+    Wd = W2.cuda()
+    cat = np.concatenate([o[:len(G.tokens_of_rank(w.T, w.EP, d))] for d, o in enumerate(dev)])
+    for _ in range(2):
+        out_h = host(torch.full((w.T, w.H), float("nan"), dtype=torch.bfloat16))
+        p2 = B.moe_layer_host(h, xh, ih, wh, Wd, shape, w.tile_m, w.tile_n, None, arena.data_ptr() + off, nbytes, counts, out_h)
+        assert (p2.comm_ctas, p2.P) == (plan.comm_ctas, plan.P) and int(counts[w.E_tot]) == S
+        assert np.array_equal(out_h.float().numpy(), cat)
