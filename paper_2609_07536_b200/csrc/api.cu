@@ -256,15 +256,16 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n, moe_o
         // One-time service-rate characterisation of this kernel family on B200 (Eq. 13), one constant per
         // GEMM tile shape (Section III-E: every kernel choice brings its own).  Reference run: DeepSeek-V2-
         // Lite shape, T = 4096, uniform routing, TP = 2, EP = 2, L = 2, K = 704; each role alone on its
-        // share of the SMs at C = 32: time per communication wave / time per compute wave.
-        //   128x256: 70.8 us / 5.88 us ; 256x256 (CTA pair): 71.0 / 4.75 ; 128x128: 70.6 / 3.97
+        // share of the SMs at C = 32: time per communication wave (of 32-row tiles: the work is dealt out in units, so
+        // that whole 128-row tiles per CTA would make the selector see waves that are not there) / time per compute wave.
+        //   128x256: 19.7 us / 6.47 us ; 256x256 (CTA pair): 19.5 / 4.68 ; 128x128: 18.8 / 5.43
         rho->K_ref = 704;
         rho->tile_m_ref = tile_m;
         rho->tile_n_ref = tile_n;
-        if (tile_m == 256) rho->rho_ref = 14.96;
-        else if (tile_n == 256) rho->rho_ref = 12.04;
-        else if (tile_n == 128) rho->rho_ref = 17.80;
-        else rho->rho_ref = 17.80 * 2.0;          // 64-wide tiles: Eq. 14 tile-area scaling from 128x128
+        if (tile_m == 256) rho->rho_ref = 4.17;
+        else if (tile_n == 256) rho->rho_ref = 3.04;
+        else if (tile_n == 128) rho->rho_ref = 3.46;
+        else rho->rho_ref = 3.46 * 2.0;          // 64-wide tiles: Eq. 14 tile-area scaling from 128x128
         if (tile_m == 64) rho->rho_ref *= 1.0;     // a 64-row tile still occupies a 128-row MMA: same wave time
         if (tile_n == 64) { rho->tile_n_ref = 64; }
         rho->D_ref = 2;
@@ -277,7 +278,7 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n, moe_o
         //   a co-resident warp beside a running GEMM serves 2.6-2.8 GB/s (2.2 times slower than a dedicated warp)
         //   and each one stretches the compute wave by 1.25 % (683 -> 704 -> 714 us of GEMM phase for w = 0, 1, 2,
         //   of which 2 % is the split-major tile order that w > 0 needs when L > 1: x is read once per split).
-        //   the dynamic hand-out gives out single tokens of a communication tile (T_M^comm pieces per tile).
+        //   the work is given out in single tokens of a communication tile (T_M^comm pieces per tile).
         rho->comm_warps_per_cta = 12;
         rho->comm_quanta_per_tile = kCommTileM;
         rho->reserved0 = 0;

@@ -21,7 +21,7 @@ constexpr int kUmmaK = 16;             // K of one tcgen05.mma.kind::f16 instruc
 constexpr int kMmaM = 128;             // M of the MMA (tile_m = 64 stores the first 64 rows only)
 constexpr int kXBoxRows = 32;          // rows of one x_routed box of a one-CTA tile of the fused kernel
 constexpr int kStageBytesTotal = 192 * 1024;  // operand ring, all stages together
-constexpr int kCommTileM = 128;        // T_M^comm
+constexpr int kCommTileM = 32;         // T_M^comm: the piece in which the selector counts communication work (a CTA's units are 8 KB)
 constexpr int kCommTileN = 1024;       // T_N^comm
 constexpr int kMailWords = 1024 + 1 + 31;   // the handle's count mailbox: one (count, sequence number) word per expert, then S
 constexpr int kPlanTableMax = 256;     // m-tile counts a tabulated selection may span (a shape has E_tot + 1 or fewer)
