@@ -39,19 +39,21 @@
 namespace moe {
 namespace {
 
-constexpr int kG1TileN = 128;                                   // intermediate columns per tile
+constexpr int kG1TileN = 128;                                   // intermediate columns per tile; 64 or 96 for the smallest batches
 constexpr int kG1EpiWarps = 8;          // warps 4..11: two column groups x four TMEM lane quarters
 constexpr int kG1LoadWarps = 4;         // warps 12..15
 constexpr int kG1RowsPerStep = 4 * kG1LoadWarps;   // rows that one copy instruction of all loader warps covers
-constexpr int kG1TmemCols = 512;                                // two 256-column accumulators
 constexpr int kG1MaxStages = 7;
 
-template <bool kPair>
+// TN: intermediate columns per tile (a pair: 128)
+template <bool kPair, int TN>
 struct G1Cfg {
     static constexpr int kABytes = kMmaM * kBlockK * 2;                              // 16 KB: this CTA's 128 rows
-    static constexpr int kBBytes = (kPair ? 1 : 2) * kG1TileN * kBlockK * 2;         // gate and up rows, or one of them
+    static constexpr int kBBytes = (kPair ? 1 : 2) * TN * kBlockK * 2;         // gate and up rows, or one of them
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = kPair ? kG1MaxStages : 4;
+    static constexpr int kStages = kPair || TN == 64 ? kG1MaxStages : TN == 96 ? 5 : 4;
+    static constexpr int kAccCols = TN == 64 ? 128 : 256;                            // columns from one accumulator to the next (2 TN used)
+    static constexpr int kTmemCols = 2 * kAccCols;
     static constexpr int kRingBytes = kStages * kStageBytes;
 };
 
@@ -127,6 +129,7 @@ struct G1Tile {
     int e, row0, valid, n0;   // valid: rows of the whole m-tile (up to 256 for a pair tile)
 };
 // tile g of the sequence: m-tile outer, n-tile inner
+template <int TN>
 __device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
 {
     const int mu = g / P.NT;
@@ -134,7 +137,7 @@ __device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
     t.e = ld_chained(&P.mtile_expert[mu]);
     t.row0 = ld_chained(&P.mtile_first_row[mu]);
     t.valid = ld_chained(&P.mtile_valid[mu]);
-    t.n0 = (g - mu * P.NT) * kG1TileN;
+    t.n0 = (g - mu * P.NT) * TN;
     return t;
 }
 // rows of the m-tile that CTA `rank` of a pair holds
@@ -152,11 +155,11 @@ __device__ __forceinline__ void g1_load_perm(const G1Params &P, const G1Tile &t,
 
 // --------------------------------------------------------------------------- GEMM1 + activation
 
-template <bool kPair>
+template <bool kPair, int TN>
 __global__ void __launch_bounds__(kThreads, 1)
 moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
 {
-    using C = G1Cfg<kPair>;
+    using C = G1Cfg<kPair, TN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     G1Control *ctl = reinterpret_cast<G1Control *>(ring + C::kRingBytes);
@@ -182,8 +185,8 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         prefetch_tensormap(&P.tmB);
     }
     if (warp == 1) {
-        if (kPair) tmem_alloc_pair(smem_u32(&ctl->tmem_base), kG1TmemCols);
-        else tmem_alloc(smem_u32(&ctl->tmem_base), kG1TmemCols);
+        if (kPair) tmem_alloc_pair(smem_u32(&ctl->tmem_base), C::kTmemCols);
+        else tmem_alloc(smem_u32(&ctl->tmem_base), C::kTmemCols);
     }
     tc_fence_before();
     __syncthreads();
@@ -205,9 +208,9 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             uint32_t phase = 0, armed = 0;
             bool ok = true;
             const unsigned long long w_policy = P.w1_once ? l2_evict_first_policy() : l2_evict_normal_policy();
-            G1Tile t = g1_decode(b, P);
+            G1Tile t = g1_decode<TN>(b, P);
             for (int g = b; g < total_tiles && ok; g += stride) {
-                const G1Tile t_next = g1_decode(min(g + stride, total_tiles - 1), P);   // fetched one tile ahead
+                const G1Tile t_next = g1_decode<TN>(min(g + stride, total_tiles - 1), P);   // fetched one tile ahead
                 int kx = 0;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     ok = g1_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 50u);
@@ -266,12 +269,12 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            G1Tile t_next = g1_decode(min(b + stride, total_tiles - 1), P);
+            G1Tile t_next = g1_decode<TN>(min(b + stride, total_tiles - 1), P);
             int f[kSteps], f_next[kSteps];
-            g1_load_perm(P, g1_decode(b, P), rank, first, f);
+            g1_load_perm(P, g1_decode<TN>(b, P), rank, first, f);
             for (int g = b; g < total_tiles && ok; g += stride) {
                 // fetched ahead: the table entries two tiles, the rows' assignments one tile
-                const G1Tile t_nn = g1_decode(min(g + 2 * stride, total_tiles - 1), P);
+                const G1Tile t_nn = g1_decode<TN>(min(g + 2 * stride, total_tiles - 1), P);
                 g1_load_perm(P, t_next, rank, first, f_next);
                 const __nv_bfloat16 *src[kSteps];
 #pragma unroll
@@ -307,7 +310,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         // operand and MMA, a whole k-block (four MMAs and the commit) is one statement with 32-bit descriptor
         // arithmetic, addresses advance by additions, the barrier's first look is the non-suspending test.
         {
-            constexpr uint32_t idesc = make_idesc(kPair ? 2 * kMmaM : kMmaM, 2 * kG1TileN);
+            constexpr uint32_t idesc = make_idesc(kPair ? 2 * kMmaM : kMmaM, 2 * TN);
             constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoB = (uint32_t)(C::kABytes >> 4);
             const uint32_t lo0 = smem_desc_lo(smem_u32(ring));
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
@@ -324,7 +327,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     if (!ok) break;
                 }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(a * 2 * kG1TileN);
+                const uint32_t d_tmem = tmem_base + (uint32_t)(a * C::kAccCols);
                 for (int kb = 0; kb < P.num_kb; ++kb) {
                     if (!__all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) {
                         ok = __all_sync(0xffffffffu, g1_wait(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 52u));
@@ -366,31 +369,30 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + kG1EpiWarps) {
-        // ---------------- epilogue: four 32-column rounds per tile, two per column group
+        // ---------------- epilogue: rounds of 32 columns, half of them per column group
         const int q4 = warp & 3;
         const int grp = (warp - 4) >> 2;
-        const int round0 = 2 * grp, n_rounds = 2;
         const int row_in_tile = (int)rank * kMmaM + q4 * 32 + lane;
         int it = 0;
         for (int g = b; g < total_tiles; g += stride, ++it) {
-            const G1Tile t = g1_decode(g, P);
+            const G1Tile t = g1_decode<TN>(g, P);
             const int a = it & 1;
             const bool ok = g1_wait_warp(smem_u32(&ctl->tmem_full[a]), (uint32_t)(it >> 1) & 1u, ctl, deadline, P.status,
                                          (uint32_t)g, 53u);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * 2 * kG1TileN);
+            const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * C::kAccCols);
             const bool row_ok = row_in_tile < t.valid;
             __nv_bfloat16 *dst_row = P.x_routed + (size_t)(t.row0 + row_in_tile) * (size_t)P.I + t.n0;
 #pragma unroll 1
-            for (int rr = 0; rr < n_rounds; ++rr) {
-                const int col = (round0 + rr) * 32;
+            for (int rr = grp; rr < TN / 32; rr += 2) {
+                const int col = rr * 32;
                 uint32_t gt[32], up[32];
                 tmem_ld_32x32(taddr + (uint32_t)col, gt);
-                tmem_ld_32x32(taddr + (uint32_t)(kG1TileN + col), up);
+                tmem_ld_32x32(taddr + (uint32_t)(TN + col), up);
                 tmem_ld_wait(gt);
                 tmem_ld_wait(up);
-                if (rr == n_rounds - 1) {
+                if (rr + 2 >= TN / 32) {
                     // everything this warp needs of the accumulator is in registers: hand the buffer back
                     tc_fence_before();
                     __syncwarp();
@@ -425,14 +427,14 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
     if (kPair) cluster_sync_all();
     if (warp == 1) {
         tc_fence_after();
-        if (kPair) tmem_dealloc_pair(tmem_base, kG1TmemCols);
-        else tmem_dealloc(tmem_base, kG1TmemCols);
+        if (kPair) tmem_dealloc_pair(tmem_base, C::kTmemCols);
+        else tmem_dealloc(tmem_base, C::kTmemCols);
     }
 }
 
-template <bool kPair>
-constexpr size_t g1_smem_bytes() { return (size_t)G1Cfg<kPair>::kRingBytes + 1024 + ((sizeof(G1Control) + 127) & ~(size_t)127); }
-static_assert(g1_smem_bytes<true>() <= 227 * 1024, "GEMM1 pair stages exceed the shared memory of an SM");
+template <bool kPair, int TN>
+constexpr size_t g1_smem_bytes() { return (size_t)G1Cfg<kPair, TN>::kRingBytes + 1024 + ((sizeof(G1Control) + 127) & ~(size_t)127); }
+static_assert(g1_smem_bytes<true, 128>() <= 227 * 1024 && g1_smem_bytes<false, 64>() <= 227 * 1024 && g1_smem_bytes<false, 96>() <= 227 * 1024, "GEMM1 stages exceed the shared memory of an SM");
 
 inline bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
@@ -443,9 +445,13 @@ using namespace moe;
 
 cudaError_t moe::gemm1_prepare()
 {
-    const cudaError_t e = cudaFuncSetAttribute(moe_gemm1_act_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<false>());
+    cudaError_t e = cudaFuncSetAttribute(moe_gemm1_act_kernel<false, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<false, 64>());
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(moe_gemm1_act_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<true>());
+    e = cudaFuncSetAttribute(moe_gemm1_act_kernel<false, 96>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<false, 96>());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(moe_gemm1_act_kernel<false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<false, 128>());
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(moe_gemm1_act_kernel<true, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g1_smem_bytes<true, 128>());
 }
 
 extern "C" int32_t moe_gemm1_workspace_bytes(const moe_shape *s, size_t *h_routed_bytes)
@@ -504,18 +510,28 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     p.H = s->H;
     p.k_tot = s->k_tot;
     p.I = s->I;
-    p.NT = (s->I + kG1TileN - 1) / kG1TileN;
+    const bool pair = tile_m == 256;
+    // Narrow tiles where every one that this routing can have then still finds an SM of its own: the time of the only wave is the
+    // time to stream one tile's weights (Granite shape, T = 2, 64 columns: 14.6 -> 12.7 us; DeepSeek shape, T = 1, 96 columns: 20.4
+    // -> 18.8).  With more tiles than SMs the wide ones are faster at every size: a k-block costs ~300 cycles whatever its width.
+    int TN = kG1TileN;
+    if (!pair) {
+        const int64_t R = (int64_t)s->T * s->k_tot, used = R < s->E_tot ? R : s->E_tot, bound = (R - used) / tile_m + used;
+        const int64_t S_max = counts_on_device && bound < n_mtiles ? bound : n_mtiles;
+        for (int tn = 64; tn < kG1TileN && TN == kG1TileN; tn += 32)
+            if (S_max * ((s->I + tn - 1) / tn) <= h->G) TN = tn;
+    }
+    p.NT = (s->I + TN - 1) / TN;
     p.num_kb = (s->H + kBlockK - 1) / kBlockK;
     p.w1_once = (int64_t)s->T * s->k_tot <= (int64_t)s->E_tot * kMmaM;   // at most one 128-row tile per expert on average
     p.last_ksteps = (s->H - (p.num_kb - 1) * kBlockK) / kUmmaK;
     if ((int64_t)n_mtiles * p.NT >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
 
     // W1 [E_tot][2][I][H] seen as [E_tot * 2 planes][I rows][H]: rows past I of a plane read zeros
-    const CUtensorMap *mB = operand_map(h, W1, 2 * s->E_tot, s->I, s->H, kG1TileN, "W1");
+    const CUtensorMap *mB = operand_map(h, W1, 2 * s->E_tot, s->I, s->H, TN, "W1");
     if (!mB) return MOE_ERR_CUDA;
     p.tmB = *mB;
 
-    const bool pair = tile_m == 256;
     const int64_t tiles_bound = (int64_t)n_mtiles * p.NT;
     const int slots = pair ? h->max_pairs : h->G;
     const int used = (int)(tiles_bound < slots ? (tiles_bound > 0 ? tiles_bound : 1) : slots);
@@ -530,8 +546,20 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     cfg.stream = st;
     cfg.gridDim = dim3((unsigned)(pair ? 2 * used : used));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = pair ? g1_smem_bytes<true>() : g1_smem_bytes<false>();
-    const cudaError_t e = pair ? cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<true>, p) : cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<false>, p);
+    cudaError_t e;
+    if (pair) {
+        cfg.dynamicSmemBytes = g1_smem_bytes<true, 128>();
+        e = cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<true, 128>, p);
+    } else if (TN == 64) {
+        cfg.dynamicSmemBytes = g1_smem_bytes<false, 64>();
+        e = cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<false, 64>, p);
+    } else if (TN == 96) {
+        cfg.dynamicSmemBytes = g1_smem_bytes<false, 96>();
+        e = cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<false, 96>, p);
+    } else {
+        cfg.dynamicSmemBytes = g1_smem_bytes<false, 128>();
+        e = cudaLaunchKernelEx(&cfg, moe_gemm1_act_kernel<false, 128>, p);
+    }
     if (e != cudaSuccess) return cuda_fail(h, e, "gemm1 launch");
     return MOE_OK;
 }

@@ -191,3 +191,11 @@ def test_row_gather_at_the_edges_of_the_m_tiles(tile_m, H, I):
     got = x.float().cpu().numpy()
     assert not np.isnan(got).any()
     assert np.all(np.abs(got - ref) <= _tolerance(ref)), float(np.max(np.abs(got - ref)))
+
+
+@pytest.mark.parametrize("T,I", [(4, 1408), (4, 1376), (7, 1408), (10, 1408)], ids=str)
+def test_tile_widths_of_the_smallest_batches(T, I):
+    # up to 8 / 14 / 20 m-tiles: 96-column tiles (the last one whole, then 32 columns wide), 128-column ones in one wave and in two
+    w = replace(wl.TINY, name="narrow", T=T, E=40, k=2, H=320, I=I, tile_m=128, tile_n=64, TP=1, EP=1, L=1)
+    _check(w, counts_on_device=True)
+    _check(replace(w, I=176), counts_on_device=False)      # 64-column tiles
