@@ -357,9 +357,13 @@ def all_traffic_bytes(w, x_passes=1):
             2 * w.T * w.L * w.k_tot * w.TP * (-(-w.H // w.L)) * 2 + w.T * w.H * 2)
 
 
-def routing_launches(R):
-    """Launches of one routing build: one (a single cluster) up to 131072 assignments, four (histogram, column scan,
-    finalize, scatter) beyond."""
+def routing_launches(w):
+    """Launches of one routing build of a whole-step call: none up to 2048 assignments on one-CTA tiles (the next kernel builds
+    the routing itself; up to 640 experts, up to 512 in front of GEMM1), one (a single cluster) up to 131072 assignments, four
+    (histogram, column scan, finalize, scatter) beyond."""
+    R = w.T * w.k_tot
+    if R <= 2048 and w.tile_m <= 128 and w.E_tot <= 512:
+        return 0
     return 1 if R <= 131072 else 4
 
 
@@ -615,7 +619,7 @@ def time_gemm1(h, dw, torch, n_warm=3, n_samples=9, cpu_rows=0):
     flops = 4.0 * w.R * w.H * w.I
     res = {"us": us, "tflops": flops / us / 1e6, "flops": flops,
            "launches": 1,
-           "post_router_layer_us": layer_us, "post_router_layer_launches": routing_launches(dw.shape.T * dw.shape.k_tot) + 2,
+           "post_router_layer_us": layer_us, "post_router_layer_launches": routing_launches(w) + 2,
            "what": "gather + grouped GEMM1 (gate, up) + silu(gate) * up -> x_routed; timed alone (burst peak applies)"}
     if cpu_rows > 0:   # the oracle of this stage on a seeded sample of routed rows: parity check and CPU time
         import numpy as np
@@ -1019,7 +1023,7 @@ def main():
             "roofline": roofline,
             "e2e": {"value": job_value(e2e_us, world), "unit": "us/layer", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "steps": Ke},
-            "gpu_launches": (routing_launches(w.T * w.k_tot) + 1) * K,
+            "gpu_launches": (routing_launches(w) + 1) * K,
             "clocks": clocks,
             "paper_context": {"hardware": "4xA100-SXM4-40GB", "mean_regret": 0.0322, "solver_us": 0.157,
                               "geomean_speedup_over_comet": 2.528},

@@ -371,7 +371,9 @@ int32_t moe_clear_status(moe_handle *h, uint32_t *status_dev, void *stream);
  * path of Section III-E: no copy, no wait; the plan comes from plan_partition_estimate and the kernel
  * reads the tile count on the device (the whole call is then asynchronous; it is not meant for graph replay: the launch epoch that marks
  * this launch's flags is a kernel argument set by the host on every call).  ev_before / ev_after: optional cudaEvent_t handles (NULL = none)
- * recorded on `stream` right before and right after the fused launch, for timing it. */
+ * recorded on `stream` right before and right after the fused launch, for timing it.
+ * Batches of up to 2048 assignments on one-CTA tiles take a single launch: the fused kernel (in moe_post_router_layer: GEMM1)
+ * builds the routing itself, into the same arrays. */
 int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int32_t *topk_idx,
                   const float *topk_w, const moe_shape *shape, int32_t tile_m, int32_t tile_n,
                   const moe_sm_limits *limits_or_null, const moe_routing *routing,

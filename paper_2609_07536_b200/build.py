@@ -19,7 +19,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmoe_b200.so")
 TIMELINE_LIB = os.path.join(HERE, "libmoe_b200_timeline.so")
 SOURCES = ["api.cu", "routing.cu", "gemm2_combine.cu", "gemm1_act.cu", "solver.cpp"]
-HEADERS = [os.path.join(CSRC, "moe_internal.h"), os.path.join(CSRC, "sm100_device.cuh"),
+HEADERS = [os.path.join(CSRC, "moe_internal.h"), os.path.join(CSRC, "sm100_device.cuh"), os.path.join(CSRC, "routing_device.cuh"),
            os.path.join(os.path.dirname(HERE), "include", "moe_b200.h")]
 
 

@@ -390,13 +390,14 @@ int32_t moe_build_routing(moe_handle *h, const int32_t *topk_idx, const moe_shap
 namespace {
 
 // Routing build of the whole-step calls.  With the handle's mailbox a kernel stores the counts into host memory and
-// `*seq` is the number to wait for (wait_counts): the build itself, or (`mail_later`) a launch behind it.  Without
-// the mailbox, the plain build with its copy, and `*seq` = 0.
+// `*seq` is the number to wait for (wait_counts): the build itself, or (`mail_later`) a launch behind it, which may also build the
+// routing (`launch_builds`: nothing is launched here).  Without the mailbox, the plain build with its copy, and `*seq` = 0.
 int32_t build_routing_mailed(moe_handle *h, const int32_t *topk_idx, const moe_shape *s, int32_t tile_m, const moe_routing *r,
-                             int32_t *tile_counts_host, bool mail_later, uint32_t *status_dev, cudaStream_t st, uint32_t *seq)
+                             int32_t *tile_counts_host, bool mail_later, bool launch_builds, uint32_t *status_dev, cudaStream_t st,
+                             uint32_t *seq)
 {
     *seq = 0;
-    if (!tile_counts_host || !h->mail_dev)
+    if ((!tile_counts_host || !h->mail_dev) && !launch_builds)
         return moe_build_routing(h, topk_idx, s, tile_m, r, tile_counts_host, status_dev, st);
     if (!s || !r || !status_dev) return MOE_ERR_NULL;
     if (!shape_ok(s)) return MOE_ERR_SHAPE;
@@ -405,9 +406,12 @@ int32_t build_routing_mailed(moe_handle *h, const int32_t *topk_idx, const moe_s
     if (r->max_mtiles < max_mtiles_of(s, tile_m)) return MOE_ERR_SHAPE;
     if (const int32_t rc = require_handle_device(h, "moe_build_routing")) return rc;
     if (++h->mail_seq == 0u) h->mail_seq = 1u;
-    const cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev, mail_later ? nullptr : h->mail_dev, h->mail_seq, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "routing launch");
-    *seq = h->mail_seq;
+    if (!launch_builds) {
+        const cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev,
+                                             mail_later ? nullptr : h->mail_dev, h->mail_seq, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "routing launch");
+    }
+    *seq = tile_counts_host ? h->mail_seq : 0u;
     return MOE_OK;
 }
 
@@ -498,11 +502,11 @@ const PlanTable *plan_table(moe_handle *h, const moe_shape *s, const moe_occupan
 }
 
 // moe_gemm2_combine with the launch's plan, or (`table`) with the plan looked up on the device by the m-tile count;
-// mail_seq != 0: this launch mails the counts
+// mail_seq != 0: this launch mails the counts; topk_idx != nullptr: it builds the routing first (m-tile count on the device)
 int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                              const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
-                             const PlanTable *table, uint32_t mail_seq, const RowFeed *feed, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
-                             void *stream);
+                             const PlanTable *table, uint32_t mail_seq, const int32_t *topk_idx, const RowFeed *feed,
+                             void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream);
 
 }  // namespace
 
@@ -514,7 +518,7 @@ int32_t moe_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, c
                           void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream)
 {
     (void)topk_idx;
-    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, nullptr, 0u, nullptr, out, y_ws, flags_ws, status_dev, stream);
+    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, nullptr, 0u, nullptr, nullptr, out, y_ws, flags_ws, status_dev, stream);
 }
 
 }  // extern "C"
@@ -523,8 +527,8 @@ namespace {
 
 int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                              const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
-                             const PlanTable *table, uint32_t mail_seq, const RowFeed *feed, void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev,
-                             void *stream)
+                             const PlanTable *table, uint32_t mail_seq, const int32_t *topk_idx, const RowFeed *feed,
+                             void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream)
 {
     if (!h || !s || !occ || !r || !plan || !out || !status_dev) return MOE_ERR_NULL;
     if (!shape_ok(s)) return MOE_ERR_SHAPE;
@@ -581,6 +585,8 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.C = C; p.P = Pc; p.mode = mode; p.withhold = plan->debug_withhold_tile;
     p.G = h->G;
     p.slot_sms = slot_sms;
+    p.E_tot = s->E_tot;
+    if (topk_idx) p.routing = {topk_idx, routing_out(*r), s->T * s->k_tot, r->max_mtiles};
     if (table) {
         p.G = table->limits.G;
         p.c_table_first = table->first;
@@ -589,7 +595,6 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
         if (mail_seq != 0u) {
             p.mail = h->mail_dev;
             p.mail_seq = mail_seq;
-            p.E_tot = s->E_tot;
         }
     }
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
@@ -725,8 +730,8 @@ int32_t selection_of(moe_handle *h, const moe_shape *s, int32_t tile_m, int32_t 
 // (seq = 0).
 int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                           const Selection &sel, const moe_routing *routing, uint32_t seq, uint32_t mail_seq,
-                          const RowFeed *feed, cudaEvent_t counts_event, int32_t *tile_counts, void *const *out, void *y_ws, uint32_t *flags_ws,
-                          uint32_t *status_dev, moe_plan *plan_out, void *ev_before, void *ev_after, cudaStream_t st)
+                          const int32_t *topk_idx, const RowFeed *feed, cudaEvent_t counts_event, int32_t *tile_counts,
+                          void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, moe_plan *plan_out, void *ev_before, void *ev_after, cudaStream_t st)
 {
     moe_plan plan;
     int32_t rc = MOE_OK, n_mtiles = MOE_MTILES_ON_DEVICE;
@@ -743,7 +748,7 @@ int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, c
         if ((rc = plan_partition_estimate(&sel.occ, &sel.lim, s, &sel.rho, &plan)) != MOE_OK) return rc;   // counts stay on the device
     }
     if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
-    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, sel.table, mail_seq, feed, out, y_ws,
+    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, sel.table, mail_seq, topk_idx, feed, out, y_ws,
                               flags_ws, status_dev, st);
     if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
     if (rc == MOE_OK && sel.table) rc = counts_and_plan();
@@ -797,10 +802,11 @@ int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int
     int32_t rc = selection_of(h, s, tile_m, tile_n, limits_or_null, tile_counts_pinned != nullptr, &sel);
     if (rc != MOE_OK) return rc;
     uint32_t seq = 0;
-    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, sel.table != nullptr, status_dev, st, &seq);
+    const bool inlined = routing_inline_ok(*s, tile_m, kFusedThreads) && (sel.table || !tile_counts_pinned);
+    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, sel.table != nullptr, inlined, status_dev, st, &seq);
     if (rc != MOE_OK) return rc;
-    return select_and_launch(h, x_routed, W2, topk_w, s, sel, routing, seq, seq, nullptr, nullptr, tile_counts_pinned, out, y_ws, flags_ws,
-                             status_dev, plan_out, ev_before, ev_after, st);
+    return select_and_launch(h, x_routed, W2, topk_w, s, sel, routing, seq, seq, inlined ? topk_idx : nullptr, nullptr, nullptr, tile_counts_pinned, out, y_ws,
+                             flags_ws, status_dev, plan_out, ev_before, ev_after, st);
 }
 
 // ---- the post-router MoE layer on device-resident inputs (Section II-A: steps 1-3) -------------
@@ -817,18 +823,20 @@ int32_t moe_post_router_layer(moe_handle *h, const void *hidden, const void *W1,
     int32_t rc = selection_of(h, s, tile_m, tile_n, limits_or_null, tile_counts_pinned != nullptr, &sel);
     if (rc != MOE_OK) return rc;
     const bool gemm1_mails = s->T > 0;
+    const bool inlined = routing_inline_ok(*s, tile_m, kThreads) && (h->mail_dev || !tile_counts_pinned);
     uint32_t seq = 0;
-    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, gemm1_mails, status_dev, st, &seq);
+    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, gemm1_mails, inlined, status_dev, st, &seq);
     if (rc != MOE_OK) return rc;
     // GEMM1 reads the m-tile count on the device, so it is launched before the host waits for the counts: the wait
     // and the planning are hidden behind it.  Without the mailbox (seq = 0) the copy of the counts was queued right
     // behind the routing kernels, before GEMM1: an event marks it.
     cudaEvent_t counts_event = static_cast<cudaEvent_t>(h->counts_event);
     if (tile_counts_pinned && seq == 0u && counts_event) cudaEventRecord(counts_event, st);
-    rc = launch_gemm1_act(h, hidden, W1, s, tile_m, routing, MOE_MTILES_ON_DEVICE, h_routed_ws, x_routed_ws, status_dev, seq, st);
+    rc = launch_gemm1_act(h, hidden, W1, inlined ? topk_idx : nullptr, s, tile_m, routing, MOE_MTILES_ON_DEVICE, h_routed_ws, x_routed_ws,
+                          status_dev, seq, st);
     if (rc != MOE_OK) return rc;
     if (tile_counts_pinned && seq == 0u && !counts_event) return MOE_ERR_CUDA;
-    return select_and_launch(h, x_routed_ws, W2, topk_w, s, sel, routing, seq, 0u, nullptr, counts_event, tile_counts_pinned, out, y_ws,
+    return select_and_launch(h, x_routed_ws, W2, topk_w, s, sel, routing, seq, 0u, nullptr, nullptr, counts_event, tile_counts_pinned, out, y_ws,
                              flags_ws, status_dev, plan_out, nullptr, nullptr, st);
 }
 
@@ -1030,8 +1038,9 @@ int32_t moe_layer_host(moe_handle *h, const void *x_routed_host, const int32_t *
     }
     if (e != cudaSuccess) return fail(cuda_fail(h, e, "input copies"));
     uint32_t seq = 0;
-    rc = build_routing_mailed(h, reinterpret_cast<int32_t *>(base + a.idx), s, tile_m, &rt, tile_counts_pinned, sel.table != nullptr,
-                              status, st, &seq);
+    int32_t *const idx = reinterpret_cast<int32_t *>(base + a.idx);
+    const bool inlined = routing_inline_ok(*s, tile_m, kFusedThreads) && (sel.table || !tile_counts_pinned);
+    rc = build_routing_mailed(h, idx, s, tile_m, &rt, tile_counts_pinned, sel.table != nullptr, inlined, status, st, &seq);
     if (rc != MOE_OK) return fail(rc);
     for (size_t r = 0; fed && r < R && e == cudaSuccess;) {
         size_t rows = R - r;
@@ -1048,7 +1057,7 @@ int32_t moe_layer_host(moe_handle *h, const void *x_routed_host, const int32_t *
     const size_t blk = (size_t)ceil_div(s->T, s->EP);
     for (int d = 0; d < s->EP; ++d) outs[d] = base + a.out + (size_t)d * blk * s->H * 2;
     rc = select_and_launch(h, base + a.x, W2_dev, reinterpret_cast<float *>(base + a.w), s, sel, &rt, seq, sel.table ? seq : 0u,
-                           fed ? &feed : nullptr, nullptr, tile_counts_pinned, outs, base + a.y,
+                           inlined ? idx : nullptr, fed ? &feed : nullptr, nullptr, tile_counts_pinned, outs, base + a.y,
                            reinterpret_cast<uint32_t *>(base + a.flags), status, plan_out, nullptr, nullptr, st);
     if (rc != MOE_OK) return fail(rc);
     // whatever the kernel needed of the rows, their copies are over before the caller has its buffers back

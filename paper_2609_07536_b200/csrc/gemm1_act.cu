@@ -34,6 +34,7 @@
 #include <cstring>
 
 #include "moe_internal.h"
+#include "routing_device.cuh"
 #include "sm100_device.cuh"
 
 namespace moe {
@@ -65,6 +66,8 @@ struct alignas(64) G1Params {
     const __nv_bfloat16 *hidden;   // [T, H]
     const int32_t *perm;           // flat assignment of every routed row
     const int32_t *S_dev;          // != nullptr: the m-tile count is read here
+    InlineRouting routing;         // topk_idx != nullptr: this launch builds the routing first (one-CTA tiles)
+    int32_t tile_m;
     __nv_bfloat16 *x_routed;       // [R, I]
     uint32_t *status;
     unsigned long long wait_ns;
@@ -194,6 +197,8 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     grid_dependency_wait();
+    if (!kPair && P.routing.topk_idx)
+        routing_inline<kThreads / 32, false>(P.routing, P.k_tot, P.E_tot, P.tile_m, P.status, reinterpret_cast<int32_t *>(ring));
     const int S = P.S_dev ? min(ld_chained_uniform(P.S_dev), P.S) : P.S;
     const int total_tiles = S * P.NT;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
@@ -466,11 +471,11 @@ extern "C" int32_t moe_gemm1_act(moe_handle *h, const void *hidden, const void *
                                  int32_t tile_m, const moe_routing *r, int32_t n_mtiles, void *h_routed_ws,
                                  void *x_routed, uint32_t *status_dev, void *stream)
 {
-    return launch_gemm1_act(h, hidden, W1, s, tile_m, r, n_mtiles, h_routed_ws, x_routed, status_dev, 0u, stream);
+    return launch_gemm1_act(h, hidden, W1, nullptr, s, tile_m, r, n_mtiles, h_routed_ws, x_routed, status_dev, 0u, stream);
 }
 
-int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const moe_shape *s, int32_t tile_m,
-                              const moe_routing *r, int32_t n_mtiles, void *h_routed_ws, void *x_routed, uint32_t *status_dev,
+int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const int32_t *topk_idx, const moe_shape *s,
+                              int32_t tile_m, const moe_routing *r, int32_t n_mtiles, void *h_routed_ws, void *x_routed, uint32_t *status_dev,
                               uint32_t mail_seq, void *stream)
 {
     if (!h || !s || !r || !status_dev) return MOE_ERR_NULL;
@@ -502,8 +507,10 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     if (mail_seq != 0u && counts_on_device) {
         p.mail = h->mail_dev;
         p.mail_seq = mail_seq;
-        p.E_tot = s->E_tot;
     }
+    p.E_tot = s->E_tot;
+    p.tile_m = tile_m;
+    if (topk_idx) p.routing = {topk_idx, routing_out(*r), s->T * s->k_tot, r->max_mtiles};
     p.perm = r->perm;
     p.hidden = static_cast<const __nv_bfloat16 *>(hidden);
     p.T = s->T;

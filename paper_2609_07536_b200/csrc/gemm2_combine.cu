@@ -42,6 +42,7 @@
 #include <cuda_bf16.h>
 
 #include "moe_internal.h"
+#include "routing_device.cuh"
 #include "sm100_device.cuh"
 
 // Timeline build (-DMOE_TIMELINE=1, a separate library): the kernels record per-CTA time stamps and cycle
@@ -1648,6 +1649,8 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
         prefetch_tensormap(&P.tmB);
     }
     grid_dependency_wait();
+    if (P.routing.topk_idx)
+        routing_inline<kFusedThreads / 32, true>(P.routing, P.k_tot, P.E_tot, P.tile_m, P.status, reinterpret_cast<int32_t *>(ring));
     if (blockIdx.x == 0 && threadIdx.x < (unsigned)P.L) {
         P.split_done_next[threadIdx.x] = 0u;
         P.queue_next[threadIdx.x] = 0ull;

@@ -29,6 +29,19 @@ constexpr int kRoutingChunk = 256;     // flat assignments handled by one warp w
 constexpr uint64_t kDefaultWaitNs = 2000000000ull;
 constexpr int kTimelineSlots = 40;     // 64-bit words per CTA in a timeline buffer (timeline build only)
 
+// the routing arrays as the kernels write them
+struct RoutingOut {
+    int32_t *counts, *offsets, *tiles, *tile_offsets, *mtile_expert, *mtile_first_row, *mtile_valid, *perm, *inv_perm, *pad_row;
+};
+
+// routing build inside a kernel that uses it (topk_idx = nullptr: the arrays are there already)
+struct InlineRouting {
+    const int32_t *topk_idx;
+    RoutingOut out;
+    int32_t R, max_mtiles;
+};
+constexpr int kInlineMaxR = 2048;      // assignments up to which a kernel builds the routing itself: four rows of 32 per warp of 16 warps
+
 // Parameters of one fused launch.  Passed by value (__grid_constant__): the two tensor maps
 // must sit in kernel parameter space, 64-byte aligned.
 struct alignas(64) FusedParams {
@@ -37,6 +50,7 @@ struct alignas(64) FusedParams {
     const int32_t *mtile_expert;
     const int32_t *mtile_first_row;
     const int32_t *mtile_valid;
+    InlineRouting routing;         // topk_idx != nullptr: this launch builds the routing first
     const int32_t *S_dev;          // != nullptr: the m-tile count is read here by the kernel (S and W_comp below are unset)
     const int32_t *pad_row;
     const int32_t *perm;
@@ -216,9 +230,19 @@ cudaError_t pair_occupancy(int *blocks_per_sm, int *max_clusters);
 cudaError_t pair_launch(const FusedParams &p, int grid, cudaStream_t stream);
 // GEMM1 (gemm1_act.cu): once per device, kernel attributes
 cudaError_t gemm1_prepare();
-// moe_gemm1_act; mail_seq != 0: this launch mails the tile counts (with MOE_MTILES_ON_DEVICE)
-int32_t launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const moe_shape *s, int32_t tile_m, const moe_routing *r,
-                         int32_t n_mtiles, void *h_routed_ws, void *x_routed, uint32_t *status_dev, uint32_t mail_seq, void *stream);
+// moe_gemm1_act; mail_seq != 0: this launch mails the tile counts (with MOE_MTILES_ON_DEVICE); topk_idx != nullptr: it builds the
+// routing first
+int32_t launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1, const int32_t *topk_idx, const moe_shape *s, int32_t tile_m,
+                         const moe_routing *r, int32_t n_mtiles, void *h_routed_ws, void *x_routed, uint32_t *status_dev, uint32_t mail_seq, void *stream);
+inline RoutingOut routing_out(const moe_routing &r)
+{
+    return {r.counts, r.offsets, r.tiles, r.tile_offsets, r.mtile_expert, r.mtile_first_row, r.mtile_valid, r.perm, r.inv_perm, r.pad_row};
+}
+// whether a kernel of `threads` threads on one-CTA tiles may build this batch's routing itself
+inline bool routing_inline_ok(const moe_shape &s, int tile_m, int threads)
+{
+    return s.T > 0 && tile_m <= 128 && (int64_t)s.T * s.k_tot <= kInlineMaxR && s.E_tot <= threads;
+}
 // routing kernels (routing.cu)
 // once per device: kernel attributes, and the largest cluster the one-launch build can run with
 cudaError_t routing_prepare(int *max_cluster);

@@ -4,7 +4,8 @@
 // ceil(M_e / T_M) tiles along the token dimension; Eq. 16: their sum S.
 // The routed rows are the flat assignments f = t * k_tot + j in a *stable* order by expert.
 //
-// Two launch shapes, the same outputs bit for bit:
+// Two launch shapes here, the same outputs bit for bit (a whole-step call on a small batch has neither: the kernel that uses
+// the routing builds it itself, routing_device.cuh):
 //   routing_onepass  up to 131072 assignments: one launch of one cluster of 1 to 16 CTAs; the ids stay in
 //                    registers from the histogram to the scatter, the per-expert totals of the CTAs cross
 //                    through distributed shared memory;
@@ -17,6 +18,7 @@
 //                    match_any gives each lane its rank among equal experts -> stable.
 
 #include "moe_internal.h"
+#include "routing_device.cuh"
 
 namespace moe {
 namespace {
@@ -39,15 +41,6 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
-__device__ __forceinline__ void report(uint32_t *status, uint32_t code, uint32_t detail, uint32_t where)
-{
-    if (atomicCAS(&status[0], 0u, code) == 0u) {
-        status[1] = detail;
-        status[2] = where;
-    }
-    atomicAdd(&status[3], 1u);
 }
 
 // ---- the three steps every path runs on a chunk, one warp per chunk --------------------------------------
@@ -76,14 +69,14 @@ __device__ __forceinline__ void chunk_hist(const int32_t *__restrict__ topk_idx,
         const int f = begin + 32 * i + lane;
         if (f >= end) continue;
         if (e[i] < 0 || e[i] >= E_tot) {
-            report(status, MOE_DEV_OOB, (uint32_t)f, 1u);
+            routing_report(status, MOE_DEV_OOB, (uint32_t)f, 1u);
             continue;
         }
         atomicAdd(&h[e[i]], 1);
         // the same expert twice inside one token?
         const int t = f / k_tot, j = f - t * k_tot;
         for (int jj = 0; jj < j; ++jj)
-            if (__ldg(topk_idx + t * k_tot + jj) == e[i]) report(status, MOE_DEV_DUP_EXPERT, (uint32_t)t, 1u);
+            if (__ldg(topk_idx + t * k_tot + jj) == e[i]) routing_report(status, MOE_DEV_DUP_EXPERT, (uint32_t)t, 1u);
     }
 }
 
@@ -144,22 +137,6 @@ __device__ __forceinline__ void expert_prefix(const int32_t *s_cnt, int32_t *s_o
         s_off[E_tot] = off;
         s_toff[E_tot] = toff;
     }
-}
-
-// m-tile table entry mu: the expert is found by bisection in the tile prefix
-__device__ __forceinline__ void mtile_entry(int mu, int E_tot, int tile_m, const int32_t *s_cnt, const int32_t *s_off,
-                                            const int32_t *s_toff, int32_t *__restrict__ mtile_expert,
-                                            int32_t *__restrict__ mtile_first_row, int32_t *__restrict__ mtile_valid)
-{
-    int lo = 0, hi = E_tot - 1;          // largest e with tile_offsets[e] <= mu
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_toff[mid] <= mu) lo = mid; else hi = mid - 1;
-    }
-    const int e = lo, i = mu - s_toff[e];
-    mtile_expert[mu] = e;
-    mtile_first_row[mu] = s_off[e] + i * tile_m;
-    mtile_valid[mu] = min(tile_m, s_cnt[e] - i * tile_m);
 }
 
 // ---- large batches: four launches over the whole GPU -------------------------------------------------------
@@ -231,7 +208,7 @@ routing_finalize(int E_tot, int tile_m, int max_mtiles, const int32_t *__restric
     __syncthreads();
     if (threadIdx.x < 32)
         mail_counts(mail, mail_seq, E_tot, threadIdx.x, [&](int x) { return x < E_tot ? s_toff[x + 1] - s_toff[x] : s_toff[E_tot]; });
-    if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
+    if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) routing_report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
     for (int e = threadIdx.x; e <= E_tot; e += blockDim.x) {
         offsets[e] = s_off[e];
         tile_offsets[e] = s_toff[e];
@@ -290,13 +267,6 @@ constexpr int kOnepassRows = 8;
 constexpr int kOnepassMaxCtas = 16;
 constexpr size_t kOnepassMaxSmem = 200 * 1024;
 
-struct RoutingOut {
-    int32_t *counts, *offsets, *tiles, *tile_offsets, *mtile_expert, *mtile_first_row, *mtile_valid, *perm, *inv_perm, *pad_row;
-};
-
-// counter row of a warp: 16-bit (a CTA holds at most 8192 assignments), its pitch an odd number of 32-bit words,
-// so that the 32 counters of one expert lie in 32 banks
-__host__ __device__ constexpr int onepass_pitch(int E_tot) { return 2 * (((E_tot + 1) / 2) | 1); }
 // CTAs for R assignments (0: too many for one launch): one more row per warp lengthens the chain by ~1 us, a cluster
 // of 2 to 16 costs 0.7 us over a single CTA whatever its size: as many CTAs as it takes to keep one row per warp
 int onepass_ctas(int R, int max_cluster)
@@ -342,59 +312,10 @@ routing_onepass(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_to
     grid_dependency_wait();
     grid_dependents_may_launch();
 
-    // ---- ids of the warp's chunk, and the 32 before it (a token may straddle the boundary)
     const int begin = min(R, ((int)rank * kOnepassWarps + w) * rows * 32), end = min(R, begin + rows * 32);
-    int e[kOnepassRows], before = -1;
-#pragma unroll
-    for (int i = 0; i < kOnepassRows; ++i) {
-        const int f = begin + 32 * i + lane;
-        e[i] = (i < rows && f < end) ? ld_chained(topk_idx + f) : -1;
-    }
-    if (begin > 0 && begin < end) before = ld_chained(topk_idx + begin - 32 + lane);
+    int e[kOnepassRows], rk[kOnepassRows];
     uint16_t *h = hist + w * pitch;
-    for (int x = lane; x < pitch / 2; x += 32) reinterpret_cast<uint32_t *>(h)[x] = 0u;
-    __syncwarp();
-
-    // ---- ranks inside the chunk; bad ids are reported and left out, repeated experts reported and kept
-    int rk[kOnepassRows];
-    int j = (begin + lane) % k_tot, m0 = begin % k_tot;             // slot of this lane's assignment, of the row's first
-    const int step = 32 % k_tot, id_bits = E_tot > 1 ? 32 - __clz(E_tot - 1) : 0;
-#pragma unroll
-    for (int i = 0; i < kOnepassRows; ++i) {
-        rk[i] = 0;
-        if (i >= rows || begin + 32 * i >= end) break;              // warp-uniform
-        const int f = begin + 32 * i + lane;
-        const bool ok = e[i] >= 0 && e[i] < E_tot;
-        if (f < end && !ok) report(status, MOE_DEV_OOB, (uint32_t)f, 1u);
-        // lanes with the same expert, bit by bit of the id (match_any takes ~80 cycles of the SM per row when the
-        // ids differ; these votes take a quarter of that at 66 experts)
-        uint32_t same = __ballot_sync(0xffffffffu, ok);
-        for (int b = 0; b < id_bits; ++b) {
-            const bool bit = (e[i] >> b) & 1;
-            const uint32_t m = __ballot_sync(0xffffffffu, bit);
-            same &= bit ? m : ~m;
-        }
-        const uint32_t lower = same & ((1u << lane) - 1u);
-        const int base = ok ? (int)h[e[i]] : 0;
-        __syncwarp();
-        if (ok && lower == 0u) h[e[i]] = (uint16_t)(base + __popc(same));
-        __syncwarp();
-        rk[i] = base + __popc(lower);
-        // the same expert twice inside one token: among the lanes of this row, then in the row before
-        const int in_row = min(j, lane);
-        int twice = ok ? __popc(lower & (((1u << in_row) - 1u) << (lane - in_row))) : 0;
-        for (int d = 1; d <= m0; ++d) {
-            const int v = __shfl_sync(0xffffffffu, before, 32 - d);
-            if (ok && j - lane >= d && v == e[i]) ++twice;
-        }
-        for (; twice > 0; --twice) report(status, MOE_DEV_DUP_EXPERT, (uint32_t)(f / k_tot), 1u);
-        before = e[i];
-        j += step;
-        if (j >= k_tot) j -= k_tot;
-        m0 += step;
-        if (m0 >= k_tot) m0 -= k_tot;
-        if (!ok) e[i] = -1;
-    }
+    rank_chunk(topk_idx, begin, end, rows, k_tot, E_tot, pitch, h, e, rk, status);
     __syncthreads();
 
     // ---- thread x, expert x: exclusive prefix of the warps' counts; this CTA's total, pushed to every CTA; rows in the
@@ -483,7 +404,7 @@ routing_onepass(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_to
     for (int mu = (int)rank * (int)blockDim.x + threadIdx.x; mu < S; mu += n_ctas * (int)blockDim.x)
         mtile_entry(mu, E_tot, tile_m, s_cnt, s_off, s_toff, out.mtile_expert, out.mtile_first_row, out.mtile_valid);
     if (rank == 0) {
-        if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
+        if (threadIdx.x == 0 && s_toff[E_tot] > max_mtiles) routing_report(status, MOE_DEV_OOB, (uint32_t)s_toff[E_tot], 2u);
         for (int x = threadIdx.x; x <= E_tot; x += blockDim.x) {
             if (x < E_tot) out.counts[x] = s_cnt[x];
             out.offsets[x] = s_off[x];
@@ -525,8 +446,7 @@ cudaError_t routing_onepass_launch(const int32_t *topk_idx, const moe_shape &s, 
     onepass_config(cfg, attr, n_ctas, onepass_smem(n_ctas, rows, s.E_tot), stream);
     attr[1] = chained_launch_attribute();
     cfg.numAttrs = 2;
-    const RoutingOut out = {r.counts, r.offsets, r.tiles, r.tile_offsets, r.mtile_expert, r.mtile_first_row, r.mtile_valid,
-                            r.perm, r.inv_perm, r.pad_row};
+    const RoutingOut out = routing_out(r);
     return cudaLaunchKernelEx(&cfg, routing_onepass, topk_idx, R, (int)s.k_tot, (int)s.E_tot, tile_m, rows, n_ctas,
                               onepass_staged(rows) ? 1 : 0, (int)r.max_mtiles, out, status, mail, mail_seq);
 }

@@ -117,3 +117,53 @@ def test_repeated_experts_are_found_across_the_rows_of_a_warp(t, slots):
     ws, _, _ = G.build_routing(w, idx)
     st = B.moe_get_status(G.handle(), ws.status, check=False)
     assert (st.code, st.detail, st.count) == (B.MOE_DEV_DUP_EXPERT, t, 1)
+
+
+@pytest.mark.parametrize("T,E,k", [
+    (1, 1, 1), (11, 3, 3),                  # less than one row of 32, a row and a bit
+    (682, 33, 3), (683, 33, 3),             # 2046 assignments, and 2049: built by a launch of its own
+    (256, 512, 8), (256, 513, 8),           # 2048, at and above the expert limit of GEMM1
+    (200, 640, 7), (200, 641, 7),           # at and above that of the fused kernel
+], ids=lambda v: str(v))
+@pytest.mark.parametrize("entry", ["layer", "post_router"])
+def test_routing_built_by_the_kernel_that_uses_it(entry, T, E, k):
+    from dataclasses import replace
+    h = G.handle()
+    w = replace(wl.TINY, T=T, E=E, k=k, H=128, I=64, tile_m=64, tile_n=128, TP=1, EP=1, L=1)
+    rng = np.random.default_rng(T + E)
+    idx = np.argsort(rng.random((T, E), dtype=np.float32), axis=1)[:, :k].astype(np.int32)
+    x = torch.zeros(T * k, 64, dtype=torch.bfloat16, device="cuda")
+    hidden = torch.ones(T, 128, dtype=torch.bfloat16, device="cuda")
+    W1, W2 = (torch.zeros(E, *s, dtype=torch.bfloat16, device="cuda") for s in ((2, 64, 128), (128, 64)))
+    wt = torch.ones(T, k, device="cuda")
+    ws = B.alloc_workspace(G.shape_of(w), w.tile_m, w.tile_n)
+    hr = torch.empty(B.moe_gemm1_workspace_bytes(ws.shape), dtype=torch.uint8, device="cuda")
+
+    def run(ids, on_device):
+        ws.routing_ws.fill_(0x77)
+        ws.tile_counts.fill_(-7)
+        B.moe_clear_status(h, ws.status)
+        d = torch.from_numpy(np.ascontiguousarray(ids)).cuda()
+        if entry == "layer":
+            B.moe_layer(h, x, W2, d, wt, ws, counts_on_device=on_device)
+        else:
+            B.moe_post_router_layer(h, hidden, W1, W2, d, wt, ws, hr, x, counts_on_device=on_device)
+        torch.cuda.synchronize()
+        return B.moe_get_status(h, ws.status, check=False)
+
+    ref = rr.build_routing(idx, E, w.tile_m)
+    for on_device in (False, True):
+        assert run(idx, on_device).code == 0
+        got = G.routing_to_numpy(ws, ref["S"])
+        for key in KEYS:
+            assert np.array_equal(got[key], ref[key]), (key, on_device)
+        assert on_device or ws.tile_counts.tolist() == ref["tiles"].tolist() + [ref["S"]]
+    bad = idx.copy()
+    bad[T // 2, k - 1] = E
+    st = run(bad, False)                    # reported once, whatever the number of CTAs
+    assert (st.code, st.detail, st.count) == (B.MOE_DEV_OOB, T // 2 * k + k - 1, 1)
+    if k > 1:
+        dup = idx.copy()
+        dup[T // 2, k - 1] = dup[T // 2, 0]
+        st = run(dup, False)
+        assert (st.code, st.detail, st.count) == (B.MOE_DEV_DUP_EXPERT, T // 2, 1)
