@@ -254,8 +254,8 @@ int32_t moe_routing_view(void *routing_ws, const moe_shape *shape, int32_t tile_
  * Section II-A (token-expert assignments), Eq. 5 (ceil(M_e / T_M) tiles per expert), Eq. 16
  * (their sum).  Stable sort of the flat assignments f = t * k_tot + j by expert.
  * topk_idx [device] int32 [T, k_tot]; tile_counts_host [host, pinned] receives
- * tiles[0..E_tot) followed by S (E_tot + 1 ints) by an asynchronous copy: synchronise the
- * stream before reading it.  Bad expert ids / repeated experts are reported in status_dev. */
+ * tiles[0..E_tot) followed by S (E_tot + 1 ints) from the build itself, or by an asynchronous copy where
+ * the GPU cannot address it: synchronise the stream before reading it.  Bad expert ids / repeated experts are reported in status_dev. */
 int32_t moe_build_routing(moe_handle *h, const int32_t *topk_idx, const moe_shape *shape,
                           int32_t tile_m, const moe_routing *routing,
                           int32_t *tile_counts_host, uint32_t *status_dev, void *stream);

@@ -376,9 +376,11 @@ int32_t moe_build_routing(moe_handle *h, const int32_t *topk_idx, const moe_shap
     if (r->max_mtiles < max_mtiles_of(s, tile_m)) return MOE_ERR_SHAPE;
     if (const int32_t rc = require_handle_device(h, "moe_build_routing")) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev, nullptr, 0u, st);
+    int32_t *const direct = host_writable(tile_counts_host);
+    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, r->scratch, h->routing_max_cluster, status_dev,
+                                   reinterpret_cast<unsigned long long *>(direct), 0u, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "routing launch");
-    if (tile_counts_host) {
+    if (tile_counts_host && !direct) {
         e = cudaMemcpyAsync(tile_counts_host, r->tiles, (size_t)(s->E_tot + 1) * 4, cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "tile counts copy");
     }

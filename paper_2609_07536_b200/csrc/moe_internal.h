@@ -200,11 +200,16 @@ __device__ __forceinline__ int ld_chained_uniform(const int32_t *p)
 // word says by itself whether it belongs to this call: no fence orders anything here.  (Plain counts followed by a
 // sequence number needed system-scope fences of the whole CTA, 4-5 us of a small build's 12.)  A kernel is complete
 // only when these stores have crossed the bus, so they are left to the kernel behind the routing build where one
-// follows without waiting for the host.
+// follows without waiting for the host.  seq = 0: `mail` is a plain array of E_tot + 1 counts, for a caller that synchronises
+// with the stream.
 template <class Count>
 __device__ __forceinline__ void mail_counts(unsigned long long *mail, uint32_t seq, int E_tot, int lane, Count count)
 {
     if (!mail) return;
+    if (seq == 0u) {
+        for (int x = lane; x <= E_tot; x += 32) reinterpret_cast<volatile int32_t *>(mail)[x] = count(x);
+        return;
+    }
     for (int x = lane; x <= E_tot; x += 32)
         *reinterpret_cast<volatile unsigned long long *>(mail + x) = ((unsigned long long)seq << 32) | (uint32_t)count(x);
 }
@@ -244,9 +249,11 @@ inline bool routing_inline_ok(const moe_shape &s, int tile_m, int threads)
     return s.T > 0 && tile_m <= 128 && (int64_t)s.T * s.k_tot <= kInlineMaxR && s.E_tot <= threads;
 }
 // routing kernels (routing.cu)
+// the address under which a kernel can write the caller's tile_counts_host itself (pinned memory), nullptr: it takes a copy
+int32_t *host_writable(int32_t *tile_counts_host);
 // once per device: kernel attributes, and the largest cluster the one-launch build can run with
 cudaError_t routing_prepare(int *max_cluster);
-// mail / mail_seq: see moe_handle::mail_host (nullptr: the counts are not mailed); `scratch`: ceil(R / 256) * E_tot ints
+// mail / mail_seq: see mail_counts (nullptr: the counts are not mailed); `scratch`: ceil(R / 256) * E_tot ints
 // for the sizes that take more than one launch, any contents
 cudaError_t routing_launch(const int32_t *topk_idx, const moe_shape &s, int tile_m, const moe_routing &r, int32_t *scratch,
                            int max_cluster, uint32_t *status, unsigned long long *mail, uint32_t mail_seq, cudaStream_t stream);

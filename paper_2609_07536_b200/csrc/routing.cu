@@ -497,6 +497,19 @@ cudaError_t routing_prepare(int *max_cluster)
     return cudaSuccess;
 }
 
+// A copy of the counts behind the build takes 9 us of the stream for a few hundred bytes (its hand-over, then the copy); stores
+// of the build's last warp take one.
+int32_t *host_writable(int32_t *tile_counts_host)
+{
+    cudaPointerAttributes a;
+    if (!tile_counts_host) return nullptr;
+    if (cudaPointerGetAttributes(&a, tile_counts_host) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? static_cast<int32_t *>(a.devicePointer) : nullptr;
+}
+
 cudaError_t routing_launch(const int32_t *topk_idx, const moe_shape &s, int tile_m, const moe_routing &r, int32_t *scratch,
                            int max_cluster, uint32_t *status, unsigned long long *mail, uint32_t mail_seq, cudaStream_t stream)
 {
@@ -578,9 +591,11 @@ extern "C" int32_t moe_build_routing_static(moe_handle *h, const int32_t *topk_i
     // The array keeps whatever the previous call left in it.  Nothing has to start at zero: the
     // histogram pass overwrites every (warp, expert) entry the later passes read.
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, scratch, h->routing_max_cluster, status_dev, nullptr, 0u, st);
+    int32_t *const direct = host_writable(tile_counts_host);
+    cudaError_t e = routing_launch(topk_idx, *s, tile_m, *r, scratch, h->routing_max_cluster, status_dev,
+                                   reinterpret_cast<unsigned long long *>(direct), 0u, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "static routing launch");
-    if (tile_counts_host) {
+    if (tile_counts_host && !direct) {
         e = cudaMemcpyAsync(tile_counts_host, r->tiles, (size_t)(s->E_tot + 1) * 4, cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "tile counts copy");
     }

@@ -167,3 +167,18 @@ def test_routing_built_by_the_kernel_that_uses_it(entry, T, E, k):
         dup[T // 2, k - 1] = dup[T // 2, 0]
         st = run(dup, False)
         assert (st.code, st.detail, st.count) == (B.MOE_DEV_DUP_EXPERT, T // 2, 1)
+
+
+@pytest.mark.parametrize("T,E,k", [(5, 33, 2), (40000, 40, 4)], ids=["one_launch", "four_launches"])
+@pytest.mark.parametrize("pinned", [True, False], ids=["pinned", "pageable"])
+def test_counts_reach_any_host_memory(T, E, k, pinned):
+    from dataclasses import replace
+    w = replace(wl.TINY, T=T, E=E, k=k, tile_m=128)
+    idx = np.argsort(np.random.default_rng(5).random((T, E), dtype=np.float32), axis=1)[:, :k].astype(np.int32)
+    ref = rr.build_routing(idx, E, w.tile_m)
+    ws = B.alloc_workspace(G.shape_of(w), w.tile_m, w.tile_n)
+    host = torch.full((E + 3,), -7, dtype=torch.int32)
+    host = host.pin_memory() if pinned else host
+    ws.tile_counts = host[1:E + 2]
+    G.build_routing(w, idx, ws)
+    assert host.tolist() == [-7] + ref["tiles"].tolist() + [ref["S"], -7]
