@@ -441,13 +441,14 @@ def run_decode(h, args, device, peaks):
         rows.append(quick_config(h, replace(w, tile_m=tm, tile_n=tn), device, peaks, steps=max(20, args.steps), warm=max(3, args.warmup),
                                  counts_on_device_too=True))
     main = rows[2]   # T = 256
-    w = replace(wl.DSV2L, name="dsv2lite_decode", T=main["T"])
+    tm, tn = (int(v) for v in main["tile"].split("x"))
+    w = replace(wl.DSV2L, name="dsv2lite_decode", T=main["T"], tile_m=tm, tile_n=tn)
     idx, wt, info = wl.make_routing(w)
     print(json.dumps({
         "metric": METRIC, "value": main["step_us"], "unit": "us/layer", "n_gpus": 1, "steps": main["steps"],
         "warmup": max(3, args.warmup), "ms_per_step": main["step_us"] / 1e3, "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
-        "config": dict(config_of(replace(w, tile_m=int(main["tile"].split("x")[0]), tile_n=int(main["tile"].split("x")[1])), info, 1),
+        "config": dict(config_of(w, info, 1),
                        T_list=list(DECODE_T), value_is_for_T=main["T"]),
         "roofline": {"bound": "hbm", "achieved": all_traffic_bytes(w) / main["fused_kernel_us"] / 1e3, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": main["frac_of_all_traffic_bound"], "traffic": None,
@@ -456,7 +457,7 @@ def run_decode(h, args, device, peaks):
                                     "(FLOPs or combine bytes) does not bound these launches",
                      "kernel": "moe_gemm2_combine_kernel", "kernel_us": main["fused_kernel_us"]},
         "decode": rows, "cpu_baseline": None, "e2e": None,
-        "gpu_launches": 2 * main["steps"],      # one routing launch (single-CTA build at these sizes) + the fused launch
+        "gpu_launches": (routing_launches(w) + 1) * main["steps"],
     }))
 
 

@@ -372,6 +372,8 @@ int32_t moe_clear_status(moe_handle *h, uint32_t *status_dev, void *stream);
  * reads the tile count on the device (the whole call is then asynchronous; it is not meant for graph replay: the launch epoch that marks
  * this launch's flags is a kernel argument set by the host on every call).  ev_before / ev_after: optional cudaEvent_t handles (NULL = none)
  * recorded on `stream` right before and right after the fused launch, for timing it.
+ * Where the combine is dealt out evenly after the GEMM (drain help, up to 32 units of 8 KB per warp) and limits ask for no
+ * particular C, the kernel divides its CTAs by whole waves of its tiles; plan_out still holds the selector's pick.
  * Batches of up to 2048 assignments on one-CTA tiles take a single launch: the fused kernel (in moe_post_router_layer: GEMM1)
  * builds the routing itself, into the same arrays. */
 int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int32_t *topk_idx,

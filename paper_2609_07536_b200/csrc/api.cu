@@ -504,10 +504,10 @@ const PlanTable *plan_table(moe_handle *h, const moe_shape *s, const moe_occupan
 }
 
 // moe_gemm2_combine with the launch's plan, or (`table`) with the plan looked up on the device by the m-tile count;
-// mail_seq != 0: this launch mails the counts; topk_idx != nullptr: it builds the routing first (m-tile count on the device)
+// own_division: an even launch may divide its CTAs itself; mail_seq != 0: this launch mails the counts; topk_idx != nullptr: it builds the routing first (m-tile count on the device)
 int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                              const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
-                             const PlanTable *table, uint32_t mail_seq, const int32_t *topk_idx, const RowFeed *feed,
+                             bool own_division, const PlanTable *table, uint32_t mail_seq, const int32_t *topk_idx, const RowFeed *feed,
                              void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream);
 
 }  // namespace
@@ -520,7 +520,7 @@ int32_t moe_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, c
                           void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream)
 {
     (void)topk_idx;
-    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, nullptr, 0u, nullptr, nullptr, out, y_ws, flags_ws, status_dev, stream);
+    return launch_gemm2_combine(h, x_routed, W2, topk_w, s, occ, r, n_mtiles, plan, false, nullptr, 0u, nullptr, nullptr, out, y_ws, flags_ws, status_dev, stream);
 }
 
 }  // extern "C"
@@ -529,7 +529,7 @@ namespace {
 
 int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                              const moe_occupancy *occ, const moe_routing *r, int32_t n_mtiles, const moe_plan *plan,
-                             const PlanTable *table, uint32_t mail_seq, const int32_t *topk_idx, const RowFeed *feed,
+                             bool own_division, const PlanTable *table, uint32_t mail_seq, const int32_t *topk_idx, const RowFeed *feed,
                              void *const *out, void *y_ws, uint32_t *flags_ws, uint32_t *status_dev, void *stream)
 {
     if (!h || !s || !occ || !r || !plan || !out || !status_dev) return MOE_ERR_NULL;
@@ -652,6 +652,15 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     const int64_t units = (int64_t)s->T * s->L * ceil_div(p.split_w, p.slab_cols);
     p.even = p.drain_help && p.co_warps == 0 && plan->debug_withhold_tile < 0 && units <= 32ll * 12 * h->G;
     int TN = occ->tile_n, ctas_c = C, ctas_p = Pc;
+    // In a whole-step call with no C asked for, such a launch divides its CTAs by itself, from the m-tile count that it reads
+    // (launch_part): the plan's C is taken for communication beside the GEMM, of which there is none, and on counts left on
+    // the device it comes from an estimate, which costs up to a wave.
+    p.balance = p.even && own_division;
+    if (p.balance) {
+        p.C = ctas_c = 0;                                        // slots to divide: all of the plan's
+        p.P = ctas_p = pair ? Pc + (C + 1) / 2 : Pc + C;
+        p.c_table_n = 0;
+    }
     if (p.even && !pair) {
         // One wave: where every tile that this routing can have finds an SM of its own among the plan's, all of them compute (a
         // communication CTA would have nothing to do until the only wave ends), on the narrowest tiles for which that holds
@@ -696,7 +705,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     const CUtensorMap *mB = operand_map(h, W2, s->E_tot, s->H, s->I, pair ? TN / 2 : TN, "W2");
     if (!mB) return MOE_ERR_CUDA;
     p.tmB = *mB;
-    const int grid = pair ? ((C + 1) & ~1) + 2 * Pc : ctas_c + ctas_p;
+    const int grid = pair ? ((ctas_c + 1) & ~1) + 2 * ctas_p : ctas_c + ctas_p;
     p.timeline = nullptr;
     if (h->timeline && h->timeline_bytes >= ((size_t)grid * kTimelineSlots + MOE_MAX_L) * sizeof(unsigned long long))
         p.timeline = h->timeline;
@@ -750,7 +759,8 @@ int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, c
         if ((rc = plan_partition_estimate(&sel.occ, &sel.lim, s, &sel.rho, &plan)) != MOE_OK) return rc;   // counts stay on the device
     }
     if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
-    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, sel.table, mail_seq, topk_idx, feed, out, y_ws,
+    const bool own_division = sel.lim.force_comm_ctas <= 0 && !sel.lim.selector_off;
+    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, own_division, sel.table, mail_seq, topk_idx, feed, out, y_ws,
                               flags_ws, status_dev, st);
     if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
     if (rc == MOE_OK && sel.table) rc = counts_and_plan();

@@ -1627,6 +1627,16 @@ __device__ __forceinline__ Part launch_part(const FusedParams &P)
             pt.P = (P.G - pt.C) / P.slot_sms;
         }
     }
+    if (P.balance) {
+        // As many waves as all slots need, over as few slots as then suffice: the same number of tiles on each but the last
+        // few.  The CTAs left over only serve their share of the combine; with them computing too the same waves take longer
+        // (DeepSeek shape T = 128: 78.5 -> 74.6 us whole step, Qwen shape T = 512 74.3 -> 70.7).  Against the plan's C, with counts
+        // on the device: DeepSeek shape T = 16 63.1 -> 57.2, T = 300 85.2 -> 77.1, T = 1024 120.9 -> 116.3; with counts on the
+        // host: Granite shape T = 4096 89.1 -> 85.4, Qwen shape T = 8192 235.4 -> 233.1, others equal.
+        const int tiles = pt.W_comp * P.L, waves = max(1, (tiles + P.P - 1) / P.P);
+        pt.P = max(1, (tiles + waves - 1) / waves);
+        pt.C = (P.P - pt.P) * P.slot_sms;
+    }
     return pt;
 }
 

@@ -79,6 +79,7 @@ struct alignas(64) FusedParams {
     int32_t tok_blk, comm_cols;
     int32_t even;                       // the communication work is dealt evenly to all warps once all tiles are done (no per-tile
                                         // flags, no queue)
+    int32_t balance;                    // (even) P counts all compute slots; the kernel divides them by whole waves of its tiles
     const uint32_t *x_ready;            // != nullptr: x_routed is still being copied in; the rows that have arrived
     int32_t w2_once;                    // W2 is read (about) once: its lines go first when L2 needs room
     int32_t num_kb, last_ksteps;

@@ -703,3 +703,28 @@ def test_host_buffers_copied_in_beside_the_gemm(kw, pinned):
         p2 = B.moe_layer_host(h, xh, ih, wh, Wd, shape, w.tile_m, w.tile_n, None, arena.data_ptr() + off, nbytes, counts, out_h)
         assert (p2.comm_ctas, p2.P) == (plan.comm_ctas, plan.P) and int(counts[w.E_tot]) == S
         assert np.array_equal(out_h.float().numpy(), cat)
+
+
+@pytest.mark.parametrize("E", [36, 37, 38, 74, 75], ids=lambda e: f"{e}_mtiles")
+@pytest.mark.parametrize("tile,H", [((128, 64), 256), ((256, 256), 512)], ids=["one_cta", "pair"])
+def test_whole_step_launch_divided_by_whole_waves(tile, H, E):
+    # E m-tiles of 4 one-CTA tiles (148 SMs) or 2 pair tiles (74 pairs): under one wave, one, just over one, two, just over two;
+    # bit for bit what a launch with a given partition computes, with the counts on the host and on the device
+    h = G.handle()
+    w = replace(wl.TINY, name="waves", T=4 * E, E=E, k=2, H=H, I=128, tile_m=tile[0], tile_n=tile[1], TP=1, EP=2, L=1)
+    _, wt, _ = wl.make_routing(w)
+    t = np.arange(w.T)
+    idx = np.stack([t % E, (t + 1) % E], axis=1).astype(np.int32)
+    x, W2 = wl.make_data(w)
+    ref_outs, _, ws, S, _ = G.run_layer(w, idx, wt, x, W2, force_C=3)
+    assert S == E
+    ref_outs = [o.copy() for o in ref_outs]
+    xd, Wd, idx_d, wt_d = x.cuda(), W2.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(wt).cuda()
+    for on_device in (False, True):
+        for o in ws.out:
+            o.fill_(float("nan"))
+        B.moe_layer(h, xd, Wd, idx_d, wt_d, ws, counts_on_device=on_device)
+        torch.cuda.synchronize()
+        assert B.moe_get_status(h, ws.status).code == 0
+        for a, o in zip(ref_outs, ws.out):
+            assert np.array_equal(a, o.float().cpu().numpy(), equal_nan=True), on_device
