@@ -199,3 +199,12 @@ def test_tile_widths_of_the_smallest_batches(T, I):
     w = replace(wl.TINY, name="narrow", T=T, E=40, k=2, H=320, I=I, tile_m=128, tile_n=64, TP=1, EP=1, L=1)
     _check(w, counts_on_device=True)
     _check(replace(w, I=176), counts_on_device=False)      # 64-column tiles
+
+
+@pytest.mark.parametrize("tile_m,E", [(128, 148), (128, 149), (128, 296), (128, 297), (256, 73), (256, 74), (256, 75), (256, 149)], ids=str)
+def test_tiles_dealt_by_whole_waves(tile_m, E):
+    # one m-tile per expert, one tile each: a wave of 148 CTAs (74 pairs), one tile more, two waves, one more
+    w = replace(wl.TINY, name="waves", T=8 * E, E=E, k=2, H=256, I=128, tile_m=tile_m, tile_n=256, TP=1, EP=1, L=1)
+    idx, _, _ = wl.make_routing(w)
+    assert rr.build_routing(idx, E, tile_m)["S"] == E
+    _check(w, n_rows=200, counts_on_device=True)
