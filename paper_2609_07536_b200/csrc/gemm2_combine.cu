@@ -1745,6 +1745,9 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         if (queued && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack);
     }
+    // The next kernel on the stream may be placed while the shares are served: a following step's routing build, and GEMM1 behind
+    // it, then start 2-3 us earlier (whole layer, Granite shape T = 1003 86.5 -> 84.1 us).  (One-CTA tiles: 0 to +0.4 us, not done.)
+    if (P.even) grid_dependents_may_launch();
     if (P.even || (!queued && (int)blockIdx.x < pt.C)) serve_shares(P, pt, ring, ctl, aux, (int)blockIdx.x, P.even ? (int)gridDim.x : pt.C);
     TL(if (threadIdx.x == 0) tl_put(P, kTlCtaEnd, globaltimer_ns()));
 }
