@@ -198,7 +198,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
     const uint32_t tmem_base = ctl->tmem_base;
     grid_dependency_wait();
     if (!kPair && P.routing.topk_idx)
-        routing_inline<kThreads / 32, false>(P.routing, P.k_tot, P.E_tot, P.tile_m, P.status, reinterpret_cast<int32_t *>(ring));
+        routing_inline<kThreads / 32, false>(P.routing, P.k_tot, P.E_tot, P.tile_m, P.status, P.mail, P.mail_seq, reinterpret_cast<int32_t *>(ring));
     const int S = P.S_dev ? min(ld_chained_uniform(P.S_dev), P.S) : P.S;
     const int total_tiles = S * P.NT;
     {
@@ -211,7 +211,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
     }
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
-    if (P.mail && blockIdx.x == 0 && warp == 3)
+    if (P.mail && (kPair || !P.routing.topk_idx) && blockIdx.x == 0 && warp == 3)
         mail_counts(P.mail, P.mail_seq, P.E_tot, lane, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if (warp == 0) {
         // ---------------- W1 producer.  Pair: everything completes on the leader's full barrier, armed by the leader for both

@@ -1660,7 +1660,7 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
     }
     grid_dependency_wait();
     if (P.routing.topk_idx)
-        routing_inline<kFusedThreads / 32, true>(P.routing, P.k_tot, P.E_tot, P.tile_m, P.status, reinterpret_cast<int32_t *>(ring));
+        routing_inline<kFusedThreads / 32, true>(P.routing, P.k_tot, P.E_tot, P.tile_m, P.status, P.mail, P.mail_seq, reinterpret_cast<int32_t *>(ring));
     if (blockIdx.x == 0 && threadIdx.x < (unsigned)P.L) {
         P.split_done_next[threadIdx.x] = 0u;
         P.queue_next[threadIdx.x] = 0ull;
@@ -1672,7 +1672,7 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
     TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < pt.C ? 0u : 1u); });
 
     const bool queued = P.drain_help && !P.even;           // (drain help is a matter of fused launches)
-    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)
+    if (P.mail && !P.routing.topk_idx && blockIdx.x == 0 && warp == kCommWarps)
         mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
     if ((int)blockIdx.x < pt.C) {
         if (warp == 1 && P.P > 0) tmem_dealloc(ctl->tmem_base, Cfg<TN>::kTmemCols);

@@ -108,7 +108,8 @@ __device__ __forceinline__ void rank_chunk(const int32_t *__restrict__ topk_idx,
 // `sm`: shared memory, which bulk copies of the CTA may write afterwards.  Every thread comes here; behind it the arrays may be read.
 constexpr int kInlineRows = 4;
 template <int kWarps, bool kCombines>
-__device__ __forceinline__ void routing_inline(const InlineRouting &p, int k_tot, int E_tot, int tile_m, uint32_t *status_dev, int32_t *sm)
+__device__ __forceinline__ void routing_inline(const InlineRouting &p, int k_tot, int E_tot, int tile_m, uint32_t *status_dev,
+                                               unsigned long long *mail, uint32_t mail_seq, int32_t *sm)
 {
     const bool first = blockIdx.x == 0;
     uint32_t *status = first ? status_dev : nullptr;
@@ -159,6 +160,10 @@ __device__ __forceinline__ void routing_inline(const InlineRouting &p, int k_tot
         }
     }
     __syncthreads();
+    // the counts leave for the host before anything else: in a loop of the smallest steps it is what prepares the next one (tiny shape
+    // T = 256: 13.6 -> 12.6 us against mailing them once the arrays are written)
+    if (first && w == kWarps - 1)
+        mail_counts(mail, mail_seq, E_tot, lane, [&](int y) { return y < E_tot ? s_toff[y + 1] - s_toff[y] : s_toff[E_tot]; });
 #pragma unroll
     for (int i = 0; i < kInlineRows; ++i) {
         const int f = begin + 32 * i + lane;
