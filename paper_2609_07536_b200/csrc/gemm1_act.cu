@@ -24,8 +24,8 @@
 //   warp 1      issues tcgen05.mma (converged warp, elected lane; N = 256, K = 16, bf16 -> fp32): accumulator
 //               columns 0..127 are the gate projection, 128..255 the up projection of the same outputs;
 //               two accumulator buffers in TMEM;
-//   warps 4-11  epilogue: tcgen05.ld of 32 gate and the matching 32 up columns, silu(g) * u in fp32,
-//               bf16, two 32-byte stores per row (x_routed rows are contiguous: no scatter here).
+//   warps 4-11  epilogue: tcgen05.ld of 16 gate and the matching 16 up columns, silu(g) * u in fp32,
+//               bf16, one 32-byte store per row (x_routed rows are contiguous: no scatter here).
 // The n-tile index runs fastest in the tile sequence, so the CTAs of a wave share the gathered rows.
 // Every wait is bounded like in the fused kernel (status word, no trap).
 
@@ -115,18 +115,8 @@ __device__ __forceinline__ bool g1_wait_warp(uint32_t bar, uint32_t parity, G1Co
     return __shfl_sync(0xffffffffu, ok, 0) != 0u;
 }
 
-// silu(z) = z / (1 + exp(-z)).  The quotient as a product with the reciprocal, which one Newton-Raphson step
-// r (2 - d r) takes from the hardware's estimate to full precision: a third of the instructions of a division, which took
-// the epilogue warps more issue slots than the loaders and the MMA issuer beside them could spare.  (The bound keeps d
-// finite, where the step is defined; below it silu is under 1e-33.)
-__device__ __forceinline__ float silu(float z)
-{
-    const float d = 1.0f + __expf(fminf(-z, 80.0f));
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    r = fmaf(r, fmaf(-d, r, 1.0f), r);
-    return z * r;
-}
+// silu(z) = z / silu_divisor(z).  The quotient is the division operator's, correctly rounded: what is left of the error is __expf's.
+__device__ __forceinline__ float silu_divisor(float z) { return 1.0f + __expf(-z); }
 
 struct G1Tile {
     int e, row0, valid, n0;   // valid: rows of the whole m-tile (up to 256 for a pair tile)
@@ -382,7 +372,10 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + kG1EpiWarps) {
-        // ---------------- epilogue: rounds of 32 columns, half of them per column group
+        // ---------------- epilogue: rounds of 16 columns (one 32-byte store per row), a contiguous half of the tile per column
+        // group.  Every division is a branch (its slow path), so a lane's divisions run one after the other: where a launch is
+        // one wave, that chain is its tail, and it is split evenly over the groups and holds nothing but the divisions (whole layer,
+        // DeepSeek shape, T = 1: 43.3 us in rounds of 32 columns with exponentials and divisions mixed, 41.3 so).
         const int q4 = warp & 3;
         const int grp = (warp - 4) >> 2;
         const int row_in_tile = (int)rank * kMmaM + q4 * 32 + lane;
@@ -398,14 +391,13 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             const bool row_ok = row_in_tile < t.valid;
             __nv_bfloat16 *dst_row = P.x_routed + (size_t)(t.row0 + row_in_tile) * (size_t)P.I + t.n0;
 #pragma unroll 1
-            for (int rr = grp; rr < TN / 32; rr += 2) {
-                const int col = rr * 32;
-                uint32_t gt[32], up[32];
-                tmem_ld_32x32(taddr + (uint32_t)col, gt);
-                tmem_ld_32x32(taddr + (uint32_t)(TN + col), up);
+            for (int col = grp * (TN / 2); col < (grp + 1) * (TN / 2); col += 16) {
+                uint32_t gt[16], up[16];
+                tmem_ld_32x16(taddr + (uint32_t)col, gt);
+                tmem_ld_32x16(taddr + (uint32_t)(TN + col), up);
                 tmem_ld_wait(gt);
                 tmem_ld_wait(up);
-                if (rr + 2 >= TN / 32) {
+                if (col + 16 == (grp + 1) * (TN / 2)) {
                     // everything this warp needs of the accumulator is in registers: hand the buffer back
                     tc_fence_before();
                     __syncwarp();
@@ -414,22 +406,19 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                         else mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
                     }
                 }
-                if (row_ok) {
+                if (row_ok && t.n0 + col < P.I) {
+                    float x[16], d[16];
 #pragma unroll
-                    for (int v = 0; v < 2; ++v) {
-                        if (t.n0 + col + v * 16 < P.I) {
-                            uint32_t w[8];
+                    for (int i = 0; i < 16; ++i) d[i] = silu_divisor(__uint_as_float(gt[i]));
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float g0 = __uint_as_float(gt[v * 16 + 2 * i]), g1 = __uint_as_float(gt[v * 16 + 2 * i + 1]);
-                                const float u0 = __uint_as_float(up[v * 16 + 2 * i]), u1 = __uint_as_float(up[v * 16 + 2 * i + 1]);
-                                const float x0 = silu(g0) * u0, x1 = silu(g1) * u1;
-                                __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-                                w[i] = *reinterpret_cast<uint32_t *>(&h);
-                            }
-                            st_global_v8(dst_row + col + v * 16, w);
-                        }
+                    for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(gt[i]) / d[i];
+                    uint32_t w[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * i] * __uint_as_float(up[2 * i]), x[2 * i + 1] * __uint_as_float(up[2 * i + 1]));
+                        w[i] = *reinterpret_cast<uint32_t *>(&h);
                     }
+                    st_global_v8(dst_row + col, w);
                 }
             }
         }

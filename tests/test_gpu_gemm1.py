@@ -93,6 +93,30 @@ def test_same_bits_for_every_m_tile_size():
         assert np.array_equal(base, bits), tm
 
 
+@pytest.mark.parametrize("tile_m", [64, 128, 256])
+def test_activation_over_its_whole_range(tile_m):
+    # one-hot hidden states and unit up rows make g a stored bf16 number and the product silu(g) itself.  The fp32 value
+    # may be off by __expf's documented 2 + floor(1.173 |g|) ulp, half an ulp each for the sum and the quotient, and one for
+    # the reference's own rounding; the stored bf16 is then the rounding of a number in that interval.
+    T, H, I = 64, 64, 128
+    w = replace(wl.TINY, name="g1silu", T=T, E=1, k=1, n_shared=0, H=H, I=I, TP=1, EP=1, L=1, tile_m=tile_m, tile_n=256 if tile_m == 256 else 64)
+    exps, mants = np.arange(-22, 10), np.arange(128)          # 2^-22 .. 1020, both signs, all mantissas
+    mag = (2.0 ** exps[:, None] * (1.0 + mants[None, :] / 128.0)).ravel()
+    g = np.concatenate([mag, -mag])
+    assert g.size == T * I
+    W1 = torch.ones((1, 2, I, H), dtype=torch.bfloat16)
+    W1[0, 0] = torch.from_numpy(g.reshape(T, I).T.copy()).to(torch.bfloat16)
+    hidden = torch.eye(T, H, dtype=torch.bfloat16)
+    x, _ = _run(w, np.zeros((T, 1), np.int32), hidden, W1)
+    got = x.float().cpu().numpy().astype(np.float64).ravel()
+    ref = g / (1.0 + np.exp(-np.maximum(g, -700.0)))
+    delta = (4.0 + np.floor(1.173 * np.abs(g))) * 2.0 ** -23
+    lo, hi = (torch.from_numpy(ref * (1.0 + sgn * delta)).to(torch.float32).to(torch.bfloat16).double().numpy() for sgn in (-1.0, 1.0))
+    far = g < -88.0                                           # exp(-g) overflows fp32 there: -0, for results under 1e-36
+    assert np.all((got >= np.minimum(lo, hi))[~far]) and np.all((got <= np.maximum(lo, hi))[~far])
+    assert np.all(np.abs(got[far]) <= 1e-36)
+
+
 def test_output_feeds_the_down_projection():
     # GEMM1's x_routed goes straight into GEMM2 + combine; the layer's output matches the oracle's GEMM2
     # evaluated on the very bits GEMM1 produced
