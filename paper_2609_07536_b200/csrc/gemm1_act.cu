@@ -20,7 +20,8 @@
 //               which form one 256-row B operand;
 //   warps 12-15 loaders of the gathered rows; their copies arrive by themselves on the stage's `rows` barrier;
 //   warp 2      relay (one thread): waits for that barrier, makes the rows visible to the tensor core's proxy and
-//               arrives on the stage's full barrier (a fence in the issuing warp would cost every k-block its cycles);
+//               arrives on the stage's full barrier (a fence in the issuing warp would cost every k-block its cycles).  Pair: the
+//               other CTA's relay hands its rows to the leader's, which arrives for both;
 //   warp 1      issues tcgen05.mma (converged warp, elected lane; N = 256, K = 16, bf16 -> fp32): accumulator
 //               columns 0..127 are the gate projection, 128..255 the up projection of the same outputs;
 //               two accumulator buffers in TMEM;
@@ -85,17 +86,19 @@ struct G1Control {
     unsigned long long full[kG1MaxStages];
     unsigned long long empty[kG1MaxStages];
     unsigned long long rows[kG1MaxStages];    // every loader thread's copies of the stage have landed
+    unsigned long long peer_rows[kG1MaxStages];   // leader of a pair: the other CTA's rows of the stage, handed over by its relay
     unsigned long long tmem_full[2];
     unsigned long long tmem_empty[2];
     uint32_t tmem_base;
     volatile uint32_t abort;
 };
 
+template <bool kCluster = false>   // kCluster: what the other CTA of the pair released
 __device__ __forceinline__ bool g1_wait(uint32_t bar, uint32_t parity, G1Control *ctl, unsigned long long deadline,
                                         uint32_t *status, uint32_t detail, uint32_t where)
 {
     uint32_t spins = 0;
-    while (!mbar_try_wait(bar, parity)) {
+    while (!(kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity))) {
         if ((++spins & 63u) == 0u) {
             if (ctl->abort) return false;
             if (globaltimer_ns() > deadline) {
@@ -164,9 +167,10 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::kStages; ++i) {
-            mbar_init(smem_u32(&ctl->full[i]), kPair ? 3 : 2);   // the W1 producer and the relay of every CTA
+            mbar_init(smem_u32(&ctl->full[i]), 2);               // the W1 producer and the relay of this CTA
             mbar_init(smem_u32(&ctl->empty[i]), 1);
             mbar_init(smem_u32(&ctl->rows[i]), 32 * kG1LoadWarps);
+            mbar_init(smem_u32(&ctl->peer_rows[i]), 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
@@ -244,7 +248,10 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         }
         __syncwarp();
     } else if (warp == 2) {
-        // ---------------- relay: rows landed -> visible to the tensor core's (async) proxy -> full barrier
+        // ---------------- relay: rows landed -> visible to the tensor core's (async) proxy -> full barrier.  Pair: the other CTA's
+        // relay hands its rows to the leader's, release to acquire at cluster scope, and that one arrives for both.  (With an
+        // unrestricted release: 1500-1900 cycles later per stage, stage alone, Granite shape T = 1003 46 -> 57 us, Qwen shape
+        // T = 2880 159 -> 190.)
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
@@ -254,10 +261,13 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     ok = g1_wait(smem_u32(&ctl->rows[stage]), phase, ctl, deadline, P.status, (uint32_t)g, 54u);
                     if (!ok) break;
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    // (rank 1 relaxed: the copies have landed, and the fence is over when the next instruction issues; a
-                    // release at cluster scope takes ~1400 cycles, more than two k-blocks: 2550 us for the stage, 1230 so)
-                    if (rank != 0) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->full[stage]), 0u));
-                    else mbar_arrive(smem_u32(&ctl->full[stage]));
+                    if (rank != 0) {
+                        mbar_arrive_cluster_release_shared(mapa_u32(smem_u32(&ctl->peer_rows[stage]), 0u));
+                    } else {
+                        if (kPair) ok = g1_wait<true>(smem_u32(&ctl->peer_rows[stage]), phase, ctl, deadline, P.status, (uint32_t)g, 56u);
+                        if (!ok) break;
+                        mbar_arrive(smem_u32(&ctl->full[stage]));
+                    }
                     if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
                 }
             }

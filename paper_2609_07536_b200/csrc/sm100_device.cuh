@@ -173,6 +173,26 @@ __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_add
 {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// Hand-over of shared memory between the CTAs of a cluster: arrival on the other CTA's barrier, and the wait for it there.
+// The release covers shared memory alone, which is what is handed over: the unrestricted one also waits for the SM's
+// global traffic, 1500-1900 cycles beside a GEMM.
+__device__ __forceinline__ void mbar_arrive_cluster_release_shared(uint32_t cluster_addr)
+{
+    asm volatile("fence.release.sync_restrict::shared::cta.cluster;\n\t"
+                 "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 // 16-byte asynchronous copy global -> shared, past L1; a thread's earlier copies arrive on a barrier when they have landed
 // (the barrier's count includes these arrivals)
 __device__ __forceinline__ void cp_async_16(uint32_t dst, const void *src)

@@ -100,3 +100,19 @@ def test_header_is_plain_c():
     res = subprocess.run([gcc, "-std=c99", "-Wall", "-Werror", "-fsyntax-only", "-x", "c", header],
                          capture_output=True, text=True)
     assert res.returncode == 0, res.stderr
+
+
+def test_relaxed_cluster_arrivals_only_hand_tmem_back():
+    # A relaxed arrival orders no memory.  In another CTA's barrier it may only stand for TMEM reads, which the tcgen05
+    # fence right before it orders; rows in shared memory cross with a release and an acquire at cluster scope.
+    csrc = os.path.join(ROOT, "paper_2609_07536_b200", "csrc")
+    uses = 0
+    for name in ("gemm1_act.cu", "gemm2_combine.cu"):
+        lines = open(os.path.join(csrc, name)).read().splitlines()
+        for i, line in enumerate(lines):
+            if "mbar_arrive_cluster_relaxed(" in line:
+                uses += 1
+                assert "tmem_empty" in line and any("tc_fence_before()" in v for v in lines[i - 5:i]), (name, i + 1, line)
+    assert uses == 2
+    gemm1 = open(os.path.join(csrc, "gemm1_act.cu")).read()
+    assert "mbar_arrive_cluster_release_shared(" in gemm1 and "mbar_try_wait_cluster(" in gemm1

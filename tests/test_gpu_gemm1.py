@@ -93,6 +93,18 @@ def test_same_bits_for_every_m_tile_size():
         assert np.array_equal(base, bits), tm
 
 
+@pytest.mark.parametrize("H", [64, 128, 272, 448, 2048])      # 1, 2, 5, 7, 32 k-blocks a tile: seven stages
+def test_pair_hand_over_repeats_the_same_bits(H):
+    # more tiles than pairs, so that the stages wrap inside and across tiles
+    w = replace(wl.TINY, name="g1pair", T=1030, E=4, k=2, H=H, I=2048, TP=1, EP=1, L=1, tile_m=128, tile_n=64)
+    idx, _, _ = wl.make_routing(w)
+    hidden, W1 = wl.make_gemm1_data(w)
+    base, _ = _run(w, idx, hidden, W1)
+    for _ in range(3):
+        x, _ = _run(replace(w, tile_m=256, tile_n=256), idx, hidden, W1)
+        assert torch.equal(x.view(torch.int16), base.view(torch.int16))
+
+
 @pytest.mark.parametrize("tile_m", [64, 128, 256])
 def test_activation_over_its_whole_range(tile_m):
     # one-hot hidden states and unit up rows make g a stored bf16 number and the product silu(g) itself.  The fp32 value
