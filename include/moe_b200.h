@@ -361,19 +361,21 @@ int32_t moe_clear_status(moe_handle *h, uint32_t *status_dev, void *stream);
  * stores each count, with a sequence number beside it, into the handle's pinned mailbox; the host polls
  * the words (bounded: it gives up with MOE_ERR_CUDA when the stream finishes or fails without them, or
  * after the handle's wait limit plus two seconds), copies the counts to tile_counts_pinned and plans.
- * The selector sees the counts through their sum S alone, so its picks for every S a routing of this
- * shape can have are tabulated on the first call (kept in the handle, for the last 8 shapes); the fused
- * kernel is launched at once and looks its communication-CTA count up by the S it reads on the device,
- * and the host waits and plans beside it.  Where the picks cannot be tabulated (more than 256 possible S,
- * tile-level readiness, picks that differ in their co-resident warps) the host waits and plans first.
+ * Where the combine is dealt out evenly after the GEMM (drain help, up to 32 units of 8 KB per warp), limits ask for no
+ * particular C and no co-resident warp can be picked, the kernel divides its CTAs by whole waves of the tiles it counts on the
+ * device, whatever the selection: it is launched at once, at every batch size from the first call on, and the host waits and
+ * plans beside it; plan_out holds the selector's pick (the division launched: waves = ceil(tiles / slots), with
+ * ceil(tiles / waves) of the slots computing).  Other launches need the pick.  The selector sees the counts through their sum S
+ * alone: the first two calls with a shape and limits wait for the counts, the second tabulates the picks for every S that a
+ * routing of the shape can have, behind its launch, and from then on (for the 8 selections used last) the kernel is launched
+ * at once and looks its C up.  Where the picks cannot be tabulated (more than 256 possible S, tile-level readiness, picks
+ * that differ in their co-resident warps) the host always waits and plans first.
  * If the mailbox could not be set up at moe_create the counts come by an asynchronous copy and a
  * stream synchronisation; tile_counts_pinned must then be pinned.  tile_counts_pinned = NULL selects the device-only-counts
  * path of Section III-E: no copy, no wait; the plan comes from plan_partition_estimate and the kernel
  * reads the tile count on the device (the whole call is then asynchronous; it is not meant for graph replay: the launch epoch that marks
  * this launch's flags is a kernel argument set by the host on every call).  ev_before / ev_after: optional cudaEvent_t handles (NULL = none)
  * recorded on `stream` right before and right after the fused launch, for timing it.
- * Where the combine is dealt out evenly after the GEMM (drain help, up to 32 units of 8 KB per warp) and limits ask for no
- * particular C, the kernel divides its CTAs by whole waves of its tiles; plan_out still holds the selector's pick.
  * Batches of up to 2048 assignments on one-CTA tiles take a single launch: the fused kernel (in moe_post_router_layer: GEMM1)
  * builds the routing itself, into the same arrays. */
 int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int32_t *topk_idx,

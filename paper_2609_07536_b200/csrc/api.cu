@@ -456,51 +456,103 @@ int32_t wait_counts(moe_handle *h, uint32_t seq, int32_t E_tot, int32_t *tile_co
     return MOE_OK;
 }
 
-// The tabulated selection for this shape, tile family and limits, made on the first use (0.5 us per entry, E_tot + 1
-// entries at most); nullptr where the launch has to wait for the counts instead: more m-tile counts than a table
-// holds, tile-level readiness (it depends on more than the sum of the counts), or picks that differ in what the
-// launch configuration fixes (grid, co-resident warps).
-const PlanTable *plan_table(moe_handle *h, const moe_shape *s, const moe_occupancy *occ, const moe_sm_limits *lim, const moe_rho *rho)
+// The most m-tiles that a routing of this shape can have: an expert with rows has at most (rows - 1) / tile_m + 1.
+int64_t most_mtiles(const moe_shape *s, int tile_m)
 {
-    for (int i = 0; i < h->n_plan_tables; ++i) {
-        const PlanTable &t = h->plan_tables[i];
-        if (t.tile_m == occ->tile_m && t.tile_n == occ->tile_n && memcmp(&t.shape, s, sizeof *s) == 0 &&
-            memcmp(&t.limits, lim, sizeof *lim) == 0)
-            return t.n > 0 ? &t : nullptr;
-    }
-    if (!h->plan_tables) {
-        h->plan_tables = new (std::nothrow) PlanTable[kPlanTables];
-        if (!h->plan_tables) return nullptr;
-    }
-    PlanTable &t = h->plan_tables[h->next_plan_table];
-    h->next_plan_table = (h->next_plan_table + 1) % kPlanTables;
-    if (h->n_plan_tables < kPlanTables) ++h->n_plan_tables;
-    t.shape = *s;
-    t.tile_m = occ->tile_m;
-    t.tile_n = occ->tile_n;
-    t.limits = *lim;
-    t.n = 0;
-    // an expert with rows has at most (rows - 1) / tile_m + 1 m-tiles
     const int64_t R = (int64_t)s->T * s->k_tot, used = R < s->E_tot ? R : s->E_tot;
-    const int64_t first = ceil_div(R, occ->tile_m), last = (R - used) / occ->tile_m + used;
+    return (R - used) / tile_m + used;
+}
+// column slab of one unit: the largest power of two with Q * columns * 2 <= 8 KB, at most 1024
+int slab_shift_of(const moe_shape *s)
+{
+    int sh = 10;
+    while (sh > 3 && ((int64_t)s->k_tot * s->TP << sh) * 2 > 8192) --sh;
+    return sh;
+}
+// Who serves what when the compute CTAs help: a queue per split, or, up to 32 units (of 8 KB) a warp, an even share for every
+// warp once the tiles are done.  Hardly any token is complete before the last tiles are, so the queue's early start is
+// worth little, while its atomics and its polling cost microseconds at the end (whole launch, queue -> even: DeepSeek shape
+// T = 16 67 -> 58 us, 256 92 -> 76, 2048 149 -> 142; Granite shape T = 1003 40 -> 30, 4096 120 -> 107; Qwen shape T = 8192 240 ->
+// 233); with more units the queue's balance wins (DeepSeek shape T = 16384, 74 units: 804 -> 815, 37 units: 719 -> 745).
+bool few_units(const moe_handle *h, const moe_shape *s)
+{
+    const int64_t split_w = ceil_div(s->H, s->L);
+    return (int64_t)s->T * s->L * ceil_div(split_w, 1 << slab_shift_of(s)) <= 32ll * 12 * h->G;
+}
+
+// Whether a whole-step launch with these limits divides its CTAs by itself whatever the counts turn out to be (even shares, no C
+// asked for, no co-resident warps): such a launch needs no selection, and goes out before the counts are on the host, at a
+// batch size that was never seen before as well (32 sizes in turn, 15 us a step as with repeated ones; 52 when the picks for all
+// counts had to be tabulated first).
+bool divides_itself(const moe_handle *h, const moe_shape *s, const moe_occupancy *occ, const moe_sm_limits *lim)
+{
+    if (!lim->drain_help || lim->force_comm_ctas > 0 || lim->selector_off || lim->C_max < 1 || s->T < 1 || !few_units(h, s)) return false;
+    const int slot = occ->comp_slot_sms;
+    if (occ->o_comp != 1 || occ->o_comm != 1 || lim->G <= slot || lim->G > (slot == 2 ? 2 * h->max_pairs : h->G)) return false;   // (else: what the launch says to the plan)
+    const int64_t NTs = ceil_div(ceil_div(s->H, s->L), occ->tile_n);
+    if ((int64_t)s->TP * max_mtiles_of(s, occ->tile_m) * NTs * s->L >= (int64_t)1 << 30) return false;     // (too many tiles: the wait knows better)
+    const int32_t w_top = lim->force_co_warps >= 0 && lim->force_co_warps < lim->co_warps_max ? lim->force_co_warps : lim->co_warps_max;
+    if (w_top < 1) return true;
+    if (lim->force_co_warps >= 0) return false;
+    // the selector tries co-resident warps from co_min_waves waves on, with C up to C_co_max
+    const int32_t C_most = lim->C_co_max < lim->C_max ? lim->C_co_max : lim->C_max;
+    if (C_most < 1) return true;
+    const int64_t P_least = (lim->G - C_most) / slot, tiles = (int64_t)s->L * s->TP * most_mtiles(s, occ->tile_m) * NTs;
+    return P_least >= 1 && ceil_div(tiles, P_least) < lim->co_min_waves;
+}
+
+// What the handle knows of the selection for this shape, tile family and limits: the table where one is made (n > 0), else an
+// entry to make it in (nullptr: the allocation failed).  The entry used longest ago goes first.
+PlanTable *plan_table(moe_handle *h, const moe_shape *s, const moe_occupancy *occ, const moe_sm_limits *lim)
+{
+    if (!h->plan_tables && !(h->plan_tables = new (std::nothrow) PlanTable[kPlanTables]())) return nullptr;
+    PlanTable *old = &h->plan_tables[0];
+    for (int i = 0; i < kPlanTables; ++i) {
+        PlanTable &t = h->plan_tables[i];
+        if (t.last_use && t.tile_m == occ->tile_m && t.tile_n == occ->tile_n && memcmp(&t.shape, s, sizeof *s) == 0 &&
+            memcmp(&t.limits, lim, sizeof *lim) == 0) {
+            t.last_use = ++h->plan_table_uses;
+            t.again = true;
+            return &t;
+        }
+        if (t.last_use < old->last_use) old = &t;
+    }
+    old->shape = *s;
+    old->tile_m = occ->tile_m;
+    old->tile_n = occ->tile_n;
+    old->limits = *lim;
+    old->n = -1;
+    old->again = false;
+    old->last_use = ++h->plan_table_uses;
+    return old;
+}
+
+// Tabulates the selection for every m-tile count of the shape (0.5 us each, 17-43 us in all); n = 0 where the launch has to wait for
+// the counts: more m-tile counts than a table holds, tile-level readiness (it depends on more than the sum of the counts),
+// or picks that differ in what the launch configuration fixes (grid, co-resident warps).
+void tabulate(PlanTable &t, const moe_occupancy *occ, const moe_rho *rho)
+{
+    t.n = 0;
+    const moe_shape *s = &t.shape;
+    const moe_sm_limits *lim = &t.limits;
+    const int64_t R = (int64_t)s->T * s->k_tot, first = ceil_div(R, occ->tile_m), last = most_mtiles(s, occ->tile_m);
     if (R < 1 || last - first + 1 > kPlanTableMax || occ->o_comp != 1 || occ->o_comm != 1 ||
         (!lim->drain_help && lim->dep_model == MOE_DEP_TILE))
-        return nullptr;
+        return;
     const int slot = occ->comp_slot_sms;
     for (int64_t S = first; S <= last; ++S) {
         const int32_t count = (int32_t)S;
         moe_plan p;
-        if (plan_partition(&count, 1, occ, lim, s, rho, &p) != MOE_OK) return nullptr;
+        if (plan_partition(&count, 1, occ, lim, s, rho, &p) != MOE_OK) return;
         if (S == first) t.plan = p;
         const int c_slots = slot == 2 ? (p.comm_ctas + 1) & ~1 : p.comm_ctas, c0 = slot == 2 ? (t.plan.comm_ctas + 1) & ~1 : t.plan.comm_ctas;
         if (p.comm_ctas < 1 || p.comm_ctas > 255 || p.co_warps != t.plan.co_warps || p.P != (lim->G - p.comm_ctas) / slot ||
             c_slots + slot * p.P != c0 + slot * t.plan.P)
-            return nullptr;
+            return;
         t.C[S - first] = (uint8_t)p.comm_ctas;
     }
     t.first = (int32_t)first;
     t.n = (int32_t)(last - first + 1);
-    return &t;
 }
 
 // moe_gemm2_combine with the launch's plan, or (`table`) with the plan looked up on the device by the m-tile count;
@@ -594,10 +646,10 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
         p.c_table_first = table->first;
         p.c_table_n = table->n;
         memcpy(p.c_table, table->C, (size_t)table->n);
-        if (mail_seq != 0u) {
-            p.mail = h->mail_dev;
-            p.mail_seq = mail_seq;
-        }
+    }
+    if (mail_seq != 0u) {
+        p.mail = h->mail_dev;
+        p.mail_seq = mail_seq;
     }
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
     p.tok_blk = (int32_t)ceil_div(s->T, s->EP);
@@ -612,12 +664,8 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.pad_row = r->pad_row;
     p.perm = r->perm;
     p.Q = s->k_tot * s->TP;
-    {   // column slab of one unit: the largest power of two with Q * slab_cols * 2 <= 8 KB, at most 1024
-        int sh = 10;
-        while (sh > 3 && ((int64_t)p.Q << sh) * 2 > 8192) --sh;
-        p.slab_shift = sh;
-        p.slab_cols = 1 << sh;
-    }
+    p.slab_shift = slab_shift_of(s);
+    p.slab_cols = 1 << p.slab_shift;
     p.topk_w = topk_w;
     p.Y = y_ws;
     p.wide_store = (p.slab_cols >= 32 && p.split_w % 16 == 0 && s->H % 16 == 0 &&
@@ -643,14 +691,9 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.tile_order = (plan->drain_help && p.co_warps == 0) ? 1 : 0;
     const int64_t R = (int64_t)s->T * s->k_tot;
     p.w2_once = R <= (int64_t)s->E_tot * kMmaM;    // at most one 128-row tile per expert on average
-    // Who serves what when the compute CTAs help: a queue per split, or, up to 32 units (of 8 KB) a warp, an even share for every
-    // warp once the tiles are done.  Hardly any token is complete before the last tiles are, so the queue's early start is
-    // worth little, while its atomics and its polling cost microseconds at the end (whole launch, queue -> even: DeepSeek shape
-    // T = 16 67 -> 58 us, 256 92 -> 76, 2048 149 -> 142; Granite shape T = 1003 40 -> 30, 4096 120 -> 107; Qwen shape T = 8192 240 ->
-    // 233); with more units the queue's balance wins (DeepSeek shape T = 16384, 74 units: 804 -> 815, 37 units: 719 -> 745).
-    // Co-resident warps draw on the queue; a launch with a withheld tile is about that tile's flag.
-    const int64_t units = (int64_t)s->T * s->L * ceil_div(p.split_w, p.slab_cols);
-    p.even = p.drain_help && p.co_warps == 0 && plan->debug_withhold_tile < 0 && units <= 32ll * 12 * h->G;
+    // Even shares or the queue (few_units).  Co-resident warps draw on the queue; a launch with a withheld tile is about that
+    // tile's flag.
+    p.even = p.drain_help && p.co_warps == 0 && plan->debug_withhold_tile < 0 && few_units(h, s);
     int TN = occ->tile_n, ctas_c = C, ctas_p = Pc;
     // In a whole-step call with no C asked for, such a launch divides its CTAs by itself, from the m-tile count that it reads
     // (launch_part): the plan's C is taken for communication beside the GEMM, of which there is none, and on counts left on
@@ -665,8 +708,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
         // One wave: where every tile that this routing can have finds an SM of its own among the plan's, all of them compute (a
         // communication CTA would have nothing to do until the only wave ends), on the narrowest tiles for which that holds
         // (the time of a wave is the time to stream and store one tile: DeepSeek shape, T = 1, 19 -> 16 us).
-        const int64_t used = R < s->E_tot ? R : s->E_tot, bound = (R - used) / occ->tile_m + used;
-        const int64_t S_max = counts_on_device && bound < n_mtiles ? bound : n_mtiles;
+        const int64_t bound = most_mtiles(s, occ->tile_m), S_max = counts_on_device && bound < n_mtiles ? bound : n_mtiles;
         for (int tn = 64; tn <= occ->tile_n; tn *= 2) {
             if (S_max * s->TP * s->L * ceil_div(p.split_w, tn) > C + Pc) continue;
             TN = tn;
@@ -720,7 +762,10 @@ struct Selection {
     moe_occupancy occ;
     moe_sm_limits lim;
     moe_rho rho;
-    const PlanTable *table;
+    bool divides;          // divides_itself, with the counts on the host wanted
+    PlanTable *table;      // else, with the counts on the host wanted: plan_table
+    // whether the fused launch goes out before the counts are on the host
+    bool launch_first() const { return divides || (table && table->n > 0); }
 };
 int32_t selection_of(moe_handle *h, const moe_shape *s, int32_t tile_m, int32_t tile_n, const moe_sm_limits *limits_or_null,
                      bool host_counts, Selection *sel)
@@ -729,15 +774,17 @@ int32_t selection_of(moe_handle *h, const moe_shape *s, int32_t tile_m, int32_t 
     const int32_t rc = moe_query_occupancy(h, tile_m, tile_n, &sel->occ, &sel->lim, &sel->rho);
     if (rc != MOE_OK) return rc;
     if (limits_or_null) sel->lim = *limits_or_null;
-    sel->table = host_counts && h->mail_dev ? plan_table(h, s, &sel->occ, &sel->lim, &sel->rho) : nullptr;
+    const bool mailed = host_counts && h->mail_dev;
+    sel->divides = mailed && divides_itself(h, s, &sel->occ, &sel->lim);
+    sel->table = mailed && !sel->divides ? plan_table(h, s, &sel->occ, &sel->lim) : nullptr;
     return MOE_OK;
 }
 
 // What the whole-step calls do after the routing build (and GEMM1): select, launch, and have the counts on the host.
-// Where the selection is tabulated the launch goes out at once, queued behind its predecessor without a gap, and
-// the host waits for the counts and plans afterwards, beside the running kernel (step of the tiny configuration
-// 20.5 -> 16 us, of the DeepSeek shape at T = 16 76.7 -> 71); otherwise it waits first.  `mail_seq` != 0: this launch
-// mails the counts (table only).  `counts_event`: recorded behind the counts' copy, for a build without the mailbox
+// Where the launch divides its CTAs by itself, or the selection is tabulated, it goes out at once, queued behind its
+// predecessor without a gap, and the host waits for the counts and plans afterwards, beside the running kernel (step of the
+// tiny configuration 20.5 -> 16 us, of the DeepSeek shape at T = 16 76.7 -> 71); otherwise it waits first, and from a
+// selection's second call on makes the table behind the launch.  `mail_seq` != 0: a launch that goes out first mails the counts.  `counts_event`: recorded behind the counts' copy, for a build without the mailbox
 // (seq = 0).
 int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, const float *topk_w, const moe_shape *s,
                           const Selection &sel, const moe_routing *routing, uint32_t seq, uint32_t mail_seq,
@@ -750,8 +797,18 @@ int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, c
         const int32_t r = wait_counts(h, seq, s->E_tot, tile_counts, st, counts_event);
         return r != MOE_OK ? r : plan_partition(tile_counts, s->E_tot, &sel.occ, &sel.lim, s, &sel.rho, &plan);
     };
-    if (sel.table) {
-        plan = sel.table->plan;
+    const bool first = sel.launch_first();
+    const PlanTable *table = first && !sel.divides ? sel.table : nullptr;
+    if (sel.divides) {
+        const int slot = sel.occ.comp_slot_sms;         // (the launch divides all of G, whatever C is)
+        memset(&plan, 0, sizeof plan);
+        plan.comm_ctas = plan.R = 1;
+        plan.P = (sel.lim.G - 1) / slot;
+        plan.mode = MOE_MODE_FUSED;
+        plan.debug_withhold_tile = -1;
+        plan.drain_help = 1;
+    } else if (table) {
+        plan = table->plan;
     } else if (tile_counts) {
         if ((rc = counts_and_plan()) != MOE_OK) return rc;
         n_mtiles = tile_counts[s->E_tot];
@@ -760,10 +817,11 @@ int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, c
     }
     if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
     const bool own_division = sel.lim.force_comm_ctas <= 0 && !sel.lim.selector_off;
-    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, own_division, sel.table, mail_seq, topk_idx, feed, out, y_ws,
+    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, own_division, table, first ? mail_seq : 0u, topk_idx, feed, out, y_ws,
                               flags_ws, status_dev, st);
     if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
-    if (rc == MOE_OK && sel.table) rc = counts_and_plan();
+    if (rc == MOE_OK && first) rc = counts_and_plan();
+    else if (rc == MOE_OK && sel.table && sel.table->again && sel.table->n < 0) tabulate(*sel.table, &sel.occ, &sel.rho);
     if (plan_out && rc == MOE_OK) *plan_out = plan;
     return rc;
 }
@@ -814,8 +872,8 @@ int32_t moe_layer(moe_handle *h, const void *x_routed, const void *W2, const int
     int32_t rc = selection_of(h, s, tile_m, tile_n, limits_or_null, tile_counts_pinned != nullptr, &sel);
     if (rc != MOE_OK) return rc;
     uint32_t seq = 0;
-    const bool inlined = routing_inline_ok(*s, tile_m, kFusedThreads) && (sel.table || !tile_counts_pinned);
-    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, sel.table != nullptr, inlined, status_dev, st, &seq);
+    const bool inlined = routing_inline_ok(*s, tile_m, kFusedThreads) && (sel.launch_first() || !tile_counts_pinned);
+    rc = build_routing_mailed(h, topk_idx, s, tile_m, routing, tile_counts_pinned, sel.launch_first(), inlined, status_dev, st, &seq);
     if (rc != MOE_OK) return rc;
     return select_and_launch(h, x_routed, W2, topk_w, s, sel, routing, seq, seq, inlined ? topk_idx : nullptr, nullptr, nullptr, tile_counts_pinned, out, y_ws,
                              flags_ws, status_dev, plan_out, ev_before, ev_after, st);
@@ -1051,8 +1109,8 @@ int32_t moe_layer_host(moe_handle *h, const void *x_routed_host, const int32_t *
     if (e != cudaSuccess) return fail(cuda_fail(h, e, "input copies"));
     uint32_t seq = 0;
     int32_t *const idx = reinterpret_cast<int32_t *>(base + a.idx);
-    const bool inlined = routing_inline_ok(*s, tile_m, kFusedThreads) && (sel.table || !tile_counts_pinned);
-    rc = build_routing_mailed(h, idx, s, tile_m, &rt, tile_counts_pinned, sel.table != nullptr, inlined, status, st, &seq);
+    const bool inlined = routing_inline_ok(*s, tile_m, kFusedThreads) && (sel.launch_first() || !tile_counts_pinned);
+    rc = build_routing_mailed(h, idx, s, tile_m, &rt, tile_counts_pinned, sel.launch_first(), inlined, status, st, &seq);
     if (rc != MOE_OK) return fail(rc);
     for (size_t r = 0; fed && r < R && e == cudaSuccess;) {
         size_t rows = R - r;
@@ -1068,7 +1126,7 @@ int32_t moe_layer_host(moe_handle *h, const void *x_routed_host, const int32_t *
     void *outs[MOE_MAX_EP];
     const size_t blk = (size_t)ceil_div(s->T, s->EP);
     for (int d = 0; d < s->EP; ++d) outs[d] = base + a.out + (size_t)d * blk * s->H * 2;
-    rc = select_and_launch(h, base + a.x, W2_dev, reinterpret_cast<float *>(base + a.w), s, sel, &rt, seq, sel.table ? seq : 0u,
+    rc = select_and_launch(h, base + a.x, W2_dev, reinterpret_cast<float *>(base + a.w), s, sel, &rt, seq, seq,
                            inlined ? idx : nullptr, fed ? &feed : nullptr, nullptr, tile_counts_pinned, outs, base + a.y,
                            reinterpret_cast<uint32_t *>(base + a.flags), status, plan_out, nullptr, nullptr, st);
     if (rc != MOE_OK) return fail(rc);

@@ -120,11 +120,13 @@ struct PlanTable {
     moe_shape shape;
     int32_t tile_m, tile_n;
     moe_sm_limits limits;
-    int32_t first, n;              // S = first .. first + n - 1; n = 0: not to be tabulated
+    int32_t first, n;              // S = first .. first + n - 1; n = 0: not to be tabulated; n < 0: not made yet
+    bool again;                    // not the first call with this selection: worth tabulating
+    uint64_t last_use;             // number of the last call with it (0: entry unused)
     moe_plan plan;                 // what all picks have in common, and the pick for `first`
     uint8_t C[kPlanTableMax];
 };
-constexpr int kPlanTables = 8;     // shapes a handle keeps tabulated; the oldest goes first
+constexpr int kPlanTables = 8;     // selections a handle keeps tabulated; the one used longest ago goes first
 }  // namespace moe
 
 struct moe_handle {
@@ -154,8 +156,8 @@ struct moe_handle {
     size_t timeline_bytes = 0;
     uint32_t probe = 0;                                 // timeline build: moe_set_probe bits for the next launches
     moe::MapEntry *maps = nullptr;                      // [kMapEntries], by a hash of the operand's address
-    moe::PlanTable *plan_tables = nullptr;              // [kPlanTables], used as a ring
-    int n_plan_tables = 0, next_plan_table = 0;
+    moe::PlanTable *plan_tables = nullptr;              // [kPlanTables]
+    uint64_t plan_table_uses = 0;
 };
 
 namespace moe {
