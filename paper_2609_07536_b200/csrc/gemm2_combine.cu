@@ -41,6 +41,8 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "moe_internal.h"
 #include "routing_device.cuh"
 #include "sm100_device.cuh"
@@ -981,100 +983,67 @@ __device__ __forceinline__ void fma2_bf16x8(unsigned long long (&acc)[4], const 
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i] = ffma2(pack_f32x2(u[i] << 16, u[i] & 0xFFFF0000u), ww, acc[i]);
 }
-__device__ __forceinline__ void fma_bf16x8(float (&acc)[8], const uint4 &v, float w)
-{
-    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        acc[2 * i + 0] = fmaf(w, __uint_as_float(u[i] << 16), acc[2 * i + 0]);
-        acc[2 * i + 1] = fmaf(w, __uint_as_float(u[i] & 0xFFFF0000u), acc[2 * i + 1]);
-    }
-}
 
-// Reduces one unit that sits in shared memory at `stage_s`: the weighted sum of its Q rows in (j, p) order, one warp.  `w`:
-// lane j holds the weight of slot j (0: the slot has no source row); `wq`: room for Q floats; `orow`: where the unit's columns
-// of the token go.
-__device__ __forceinline__ void reduce_unit(const FusedParams &P, float w, bool all_valid, int ucols, int wslab, float *wq, uint32_t stage_s,
+// The weights of a unit's rows, read back as shared-memory broadcasts.  `w`: lane j holds the weight of slot j (0: the slot has
+// no source row); `wq`: room for Q floats, rounded up to the rows that reduce_unit takes together.
+__device__ __forceinline__ void put_row_weights(const FusedParams &P, float w, float *wq)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane < P.k_tot)
+        for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w;
+}
+// Reduces one unit that sits in shared memory at `stage_s`: the weighted sum of its Q rows in (j, p) order, one warp.  all_valid:
+// every slot has a source row; `orow`: where the unit's columns of the token go; kAhead: rows fetched from shared memory together.
+template <int kAhead>
+__device__ __forceinline__ void reduce_unit(const FusedParams &P, bool all_valid, int n16, int row_bytes, const float *wq, uint32_t stage_s,
                                             __nv_bfloat16 *orow)
 {
     const int lane = threadIdx.x & 31;
-    const int n16 = ucols >> 3;
-    const uint32_t row_bytes = (uint32_t)wslab * 2u;
-    // per-row weights, read back as shared-memory broadcasts inside the unrolled loop
-    if (lane < P.k_tot)
-        for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w;
-    __syncwarp();
+    __syncwarp();   // the weights
     const uint32_t wq_s = smem_u32(wq);
-    if (all_valid && P.Q <= 16) {
-        // common case: every slot has a source row and the unit has at most 16 rows: weights stay in
-        // registers as packed pairs, rows are fetched eight at a time, two FMAs per instruction
-        unsigned long long ww[16];
+#pragma unroll 1
+    for (int c16 = lane; c16 < n16; c16 += 32) {
+        unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+        uint32_t src = stage_s + (uint32_t)c16 * 16u, wsrc = wq_s;
+        const auto add_rows = [&](int q, auto whole_group) {
+            constexpr bool whole = decltype(whole_group)::value;
+            uint4 v[kAhead];
+            float wr[kAhead];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            const uint32_t wb = __float_as_uint(r < P.Q ? lds_f32(wq_s + (uint32_t)r * 4u) : 0.f);
-            ww[r] = pack_f32x2(wb, wb);
-        }
-        for (int c16 = lane; c16 < n16; c16 += 32) {
-            unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
-            const uint32_t src = stage_s + (uint32_t)c16 * 16u;
+            for (int i = 0; i < kAhead; ++i, src += (uint32_t)row_bytes)
+                v[i] = whole || q + i < P.Q ? lds_v4(src) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int r0 = 0; r0 < 16; r0 += 8) {
-                if (r0 < P.Q) {
-                    uint4 v[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) v[i] = lds_v4(src + (uint32_t)min(r0 + i, P.Q - 1) * row_bytes);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) fma2_bf16x8(acc, v[i], ww[r0 + i]);   // rows past Q carry weight 0
-                }
-            }
-            float f[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) unpack_f32x2(acc[i], f[2 * i], f[2 * i + 1]);
-            uint4 pk;
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(f[0], f[1]);
-            __nv_bfloat162 h1 = __floats2bfloat162_rn(f[2], f[3]);
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(f[4], f[5]);
-            __nv_bfloat162 h3 = __floats2bfloat162_rn(f[6], f[7]);
-            pk.x = *reinterpret_cast<uint32_t *>(&h0);
-            pk.y = *reinterpret_cast<uint32_t *>(&h1);
-            pk.z = *reinterpret_cast<uint32_t *>(&h2);
-            pk.w = *reinterpret_cast<uint32_t *>(&h3);
-            __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), pk);
-        }
-    } else
-    for (int c16 = lane; c16 < ((n16 + 31) & ~31); c16 += 32) {
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        const uint32_t src = stage_s + (uint32_t)(c16 < n16 ? c16 : 0) * 16u;
-        for (int r0 = 0; r0 < P.Q; r0 += 8) {
-            uint4 v[8];
-            float w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int r = min(r0 + i, P.Q - 1);
-                v[i] = lds_v4(src + (uint32_t)r * row_bytes);
-                w[i] = lds_f32(wq_s + (uint32_t)r * 4u);
-                if (r0 + i >= P.Q) w[i] = 0.f;
+            for (int i = 0; i < kAhead; i += 4) {
+                const uint4 w4 = lds_v4(wsrc + 4u * i);
+                wr[i] = __uint_as_float(w4.x);
+                wr[i + 1] = __uint_as_float(w4.y);
+                wr[i + 2] = __uint_as_float(w4.z);
+                wr[i + 3] = __uint_as_float(w4.w);
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                // a slot without a source row holds bytes nobody wrote: drop them
-                if (w[i] == 0.f) v[i] = make_uint4(0u, 0u, 0u, 0u);
-                fma_bf16x8(acc, v[i], w[i]);
+            for (int i = 0; i < kAhead; ++i) {
+                // a slot without a source row holds bytes nobody wrote, and there is no row past Q: nothing is added
+                if (!whole && ((!all_valid && wr[i] == 0.f) || q + i >= P.Q)) v[i] = make_uint4(0u, 0u, 0u, 0u), wr[i] = 0.f;
+                fma2_bf16x8(acc, v[i], pack_f32x2(__float_as_uint(wr[i]), __float_as_uint(wr[i])));
             }
+        };
+#pragma unroll 1
+        for (int q = 0; q < P.Q; q += kAhead, wsrc += 4u * kAhead) {
+            // (long launches spare the checks of whole groups; short ones the second instance of the code)
+            if (kAhead == 8 && all_valid && q + kAhead <= P.Q) add_rows(q, std::true_type{});
+            else add_rows(q, std::false_type{});
         }
-        if (c16 < n16) {
-            uint4 pk;
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0], acc[1]);
-            __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[2], acc[3]);
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[4], acc[5]);
-            __nv_bfloat162 h3 = __floats2bfloat162_rn(acc[6], acc[7]);
-            pk.x = *reinterpret_cast<uint32_t *>(&h0);
-            pk.y = *reinterpret_cast<uint32_t *>(&h1);
-            pk.z = *reinterpret_cast<uint32_t *>(&h2);
-            pk.w = *reinterpret_cast<uint32_t *>(&h3);
-            __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), pk);
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float lo, hi;
+            unpack_f32x2(acc[i], lo, hi);
+            __nv_bfloat162 hh = __floats2bfloat162_rn(lo, hi);
+            o[i] = *reinterpret_cast<uint32_t *>(&hh);
         }
+        __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), make_uint4(o[0], o[1], o[2], o[3]));
     }
+    __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
 }
 
 // Communication warp.  Y is token-major: the k_tot * TP partial rows of one (token, split, column
@@ -1151,8 +1120,8 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
         if (!ok) return false;
         __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(P.out[u.d]) +
                               (size_t)(u.t - u.d * P.tok_blk) * (size_t)P.H + u.s * P.split_w + (u.slab << P.slab_shift);
-        reduce_unit(P, u.w, u.all_valid, u.ucols, u.wslab, wq, smem_u32(my_ring + st * kCommUnitBytes), orow);
-        __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
+        put_row_weights(P, u.w, wq);
+        reduce_unit<8>(P, u.all_valid, u.ucols >> 3, u.wslab * 2, wq, smem_u32(my_ring + st * kCommUnitBytes), orow);
         TL(tl_last = globaltimer_ns(); if (tl_units == 0) tl_first = tl_last; ++tl_units; if (u.s < 4) ++tl_by_split[u.s]);
         return true;
     };
@@ -1425,7 +1394,7 @@ __device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &p
     if (warp >= kCommWarps) return;
     uint8_t *stages = ring + warp * kCommWarpBytes;
     float *wq = reinterpret_cast<float *>(aux) + warp * 256;      // weights of the unit's rows
-    const uint32_t full = smem_u32(&ctl->comm_full[2 * warp]), wq_s = smem_u32(wq);
+    const uint32_t full = smem_u32(&ctl->comm_full[2 * warp]);
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns, deadline2 = deadline + P.wait_ns / 4 + 1000000ull;
     const unsigned long long y_policy = l2_evict_first_policy();
     const __nv_bfloat16 *Y = reinterpret_cast<const __nv_bfloat16 *>(P.Y);
@@ -1518,53 +1487,14 @@ __device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &p
             }
             if (flying) {
                 const int prev = k - 1 - (have ? 1 : 0), st = prev & 1;
-                if (lane < P.k_tot)
-                    for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w_f;
+                put_row_weights(P, w_f, wq);
                 if (!wait_barrier(full + 8u * (uint32_t)st, (uint32_t)(prev >> 1) & 1u, ctl, deadline2, P.status, (uint32_t)tok, 43u)) {
                     // (reported) the copy just issued must land before shared memory is released
                     const unsigned long long drain = globaltimer_ns() + 2000000ull;
                     while (have && !mbar_try_wait(full + 8u * (uint32_t)((k - 1) & 1), (uint32_t)((k - 1) >> 1) & 1u) && globaltimer_ns() < drain) {}
                     break;
                 }
-                __syncwarp();
-                const uint32_t stage_s = smem_u32(stages + st * kCommUnitBytes);
-#pragma unroll 1
-                for (int c16 = lane; c16 < n16; c16 += 32) {
-                    unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
-                    uint32_t src = stage_s + (uint32_t)c16 * 16u, wsrc = wq_s;
-#pragma unroll 1
-                    for (int q = 0; q < P.Q; q += kRowsAhead, wsrc += 4u * kRowsAhead) {
-                        uint4 v[kRowsAhead];
-                        float wr[kRowsAhead];
-#pragma unroll
-                        for (int i = 0; i < kRowsAhead; ++i, src += (uint32_t)row_bytes)
-                            v[i] = q + i < P.Q ? lds_v4(src) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                        for (int i = 0; i < kRowsAhead; i += 4) {
-                            const uint4 w4 = lds_v4(wsrc + 4u * i);
-                            wr[i] = __uint_as_float(w4.x);
-                            wr[i + 1] = __uint_as_float(w4.y);
-                            wr[i + 2] = __uint_as_float(w4.z);
-                            wr[i + 3] = __uint_as_float(w4.w);
-                        }
-#pragma unroll
-                        for (int i = 0; i < kRowsAhead; ++i) {
-                            // a slot without a source row holds bytes nobody wrote, and there is no row past Q: nothing is added
-                            if ((!all_valid && wr[i] == 0.f) || q + i >= P.Q) v[i] = make_uint4(0u, 0u, 0u, 0u), wr[i] = 0.f;
-                            fma2_bf16x8(acc, v[i], pack_f32x2(__float_as_uint(wr[i]), __float_as_uint(wr[i])));
-                        }
-                    }
-                    uint32_t o[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float lo, hi;
-                        unpack_f32x2(acc[i], lo, hi);
-                        __nv_bfloat162 hh = __floats2bfloat162_rn(lo, hi);
-                        o[i] = *reinterpret_cast<uint32_t *>(&hh);
-                    }
-                    __stcs(reinterpret_cast<uint4 *>(orow + c16 * 8), make_uint4(o[0], o[1], o[2], o[3]));
-                }
-                __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
+                reduce_unit<kRowsAhead>(P, all_valid, n16, row_bytes, wq, smem_u32(stages + st * kCommUnitBytes), orow);
             }
             if (!have) break;
             flying = true;

@@ -807,3 +807,27 @@ def test_tabulated_selection_from_the_first_call_to_the_third(kw, limits):
         for a, o, n in zip(ref, outs, own):
             assert np.array_equal(a[:n], o.float().cpu().numpy()), step
     B.moe_destroy(h)
+
+
+@pytest.mark.parametrize("k,n_shared", [(3, 0), (2, 2), (9, 0)])       # Q = 3, 4, 9 rows a unit: short of a multiple of four or eight, and not
+def test_an_infinity_stays_one_on_every_route(k, n_shared):
+    # a partial result over the bf16 range: its token's column is infinite (not NaN) whether the units are dealt evenly, drawn from
+    # the queue or served by the communication CTAs, and nothing else changes
+    w = replace(wl.TINY, name="inf", T=200, E=12, k=k, n_shared=n_shared, H=256, I=64, TP=1, EP=1, L=1, tile_m=128, tile_n=128)
+    idx, wt, _ = wl.make_routing(w)
+    x, W2 = wl.make_data(w)
+    r = rr.build_routing(idx, w.E_tot, w.tile_m)
+    tok, col = 17, 40
+    for j in (0, w.k_tot - 1):                          # the unit's first row, and its last
+        xj, Wj = x.clone(), W2.clone()
+        xj[int(r["inv_perm"].reshape(w.T, w.k_tot)[tok, j])] = 3e38
+        Wj[int(idx[tok, j])].zero_()
+        Wj[int(idx[tok, j]), col] = 1.0
+        base = None
+        for kw in (dict(), dict(co_warps=2), dict(drain_help=0)):
+            outs, _, _, _, st = G.run_layer(w, idx, np.abs(wt) + 0.125, xj, Wj, **kw)
+            got = np.concatenate(outs)[:w.T]
+            assert st.code == 0 and got[tok, col] == np.inf
+            assert np.isfinite(np.delete(got[tok], col)).all()
+            base = got if base is None else base
+            assert np.array_equal(base, got), kw
