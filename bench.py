@@ -351,10 +351,34 @@ def calibrate(h, device, C_ref=32, tile=(128, 256)):
 
 # ----------------------------------------------------------------------------- other workloads, briefly
 
-def all_traffic_bytes(w, x_passes=1):
-    """Every byte one launch has to move through HBM: x (once per pass), W2, Y written and read back, out."""
-    return (w.R * w.I * 2 * x_passes + w.E_tot * w.H * w.I * 2 +
+def all_traffic_bytes(w, idx, x_passes=1):
+    """Every byte one launch has to move through HBM: x (once per pass), W2 of the experts that some token chose, Y written and
+    read back, out."""
+    import numpy as np
+    return (w.R * w.I * 2 * x_passes + len(np.unique(idx)) * w.H * w.I * 2 +
             2 * w.T * w.L * w.k_tot * w.TP * (-(-w.H // w.L)) * 2 + w.T * w.H * 2)
+
+
+def launched_division(w, lim, plan, S):
+    """The division of the CTAs that a moe_layer call launches, from the tile count S: the plan's, or, where the combine is dealt
+    out evenly and no C is asked for, whole waves of the tiles over all slots (moe_layer in moe_b200.h), on one-CTA tiles on the
+    narrowest ones that are a single wave.  comm_ctas: CTAs (of `P` compute slots' neighbours) that only combine."""
+    split_w, slot = -(-w.H // w.L), 2 if w.tile_m == 256 else 1
+    slab = 1024
+    while slab > 8 and w.k_tot * w.TP * slab * 2 > 8192:
+        slab //= 2
+    units = w.T * w.L * -(-split_w // slab)
+    if not lim.drain_help or lim.force_comm_ctas > 0 or lim.selector_off or plan.co_warps or units > 32 * 12 * lim.G:
+        return {"comm_ctas": plan.comm_ctas, "P": plan.P, "by": "plan"}
+    slots, tn = lim.G // slot, w.tile_n
+    if slot == 1:
+        used = min(w.R, w.E_tot)
+        S_max = (w.R - used) // w.tile_m + used
+        tn = next((n for n in (64, 128, 256) if n <= w.tile_n and S_max * w.TP * w.L * -(-split_w // n) <= slots), w.tile_n)
+    tiles = S * w.TP * w.L * -(-split_w // tn)
+    waves = max(1, -(-tiles // slots))
+    P = max(1, -(-tiles // waves))
+    return {"comm_ctas": (slots - P) * slot, "P": P, "tile_n": tn, "waves": waves, "by": "whole waves of the tiles"}
 
 
 def routing_launches(w):
@@ -394,10 +418,11 @@ def quick_config(h, w, device, peaks, steps=30, warm=5, counts_on_device_too=Fal
     step_us = t0.elapsed_time(t1) * 1e3 / steps
     t_flops = dw.flops / peaks["bf16_tflops"] / 1e6
     t_comb = dw.combine_bytes / peaks["hbm_gbs"] / 1e3
-    t_all = all_traffic_bytes(w) / peaks["hbm_gbs"] / 1e3
+    t_all = all_traffic_bytes(w, dw.idx) / peaks["hbm_gbs"] / 1e3
     roof = max(t_flops, t_comb)
     out = {"workload": w.name, "T": w.T, "tile": f"{w.tile_m}x{w.tile_n}", "L": w.L, "steps": steps,
-           "plan": {"comm_ctas": plan.comm_ctas, "P": plan.P, "co_warps": plan.co_warps},
+           "plan": {"comm_ctas": plan.comm_ctas, "P": plan.P, "co_warps": plan.co_warps},      # the selector's pick
+           "launched": launched_division(w, lim, plan, int(dw.ws.tile_counts[w.E_tot])),
            "step_us": step_us, "fused_kernel_us": fused, "tflops": dw.flops / fused / 1e6,
            "roofline_us": roof, "roofline_bound": "tensor" if t_flops >= t_comb else "hbm", "roofline_frac": roof / fused,
            "hbm_all_traffic_us": t_all, "frac_of_all_traffic_bound": t_all / fused,
@@ -450,10 +475,10 @@ def run_decode(h, args, device, peaks):
         "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
         "config": dict(config_of(w, info, 1),
                        T_list=list(DECODE_T), value_is_for_T=main["T"]),
-        "roofline": {"bound": "hbm", "achieved": all_traffic_bytes(w) / main["fused_kernel_us"] / 1e3, "peak": peaks["hbm_gbs"],
+        "roofline": {"bound": "hbm", "achieved": all_traffic_bytes(w, idx) / main["fused_kernel_us"] / 1e3, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": main["frac_of_all_traffic_bound"], "traffic": None,
-                     "peak_source": peaks["source"] + ": copy bandwidth; bytes = ALL HBM traffic of a launch (x, W2, Y written "
-                                    "and read back, out): at decode sizes the weights dominate, the headline roofline "
+                     "peak_source": peaks["source"] + ": copy bandwidth; bytes = ALL HBM traffic of a launch (x, W2 of the chosen experts, Y "
+                                    "written and read back, out): at decode sizes the weights dominate, the headline roofline "
                                     "(FLOPs or combine bytes) does not bound these launches",
                      "kernel": "moe_gemm2_combine_kernel", "kernel_us": main["fused_kernel_us"]},
         "decode": rows, "cpu_baseline": None, "e2e": None,
@@ -933,6 +958,7 @@ def main():
         extra["combine_only"] = {"us": comb_only, "gbs": dw.combine_bytes / comb_only / 1e3,
                                  "frac_of_hbm_peak": dw.combine_bytes / comb_only / 1e3 / peaks["hbm_gbs"], "C": lim_all}
         # ---- selector regret on this workload: every feasible C timed
+        # (of moe_gemm2_combine, which launches the plan it is given; moe_layer does so where "launched" says by "plan")
         if not args.no_regret:
             extra["regret"] = regret_of_workload(step, torch, counts, lim, (plan.comm_ctas, plan.co_warps), n_warm=1, n_samples=5)
             # the paper's static partition on the same workload: its pick, its sweep, its regret
@@ -1001,10 +1027,9 @@ def main():
             "frac_of_sustained_peak": (ach / tf_sust) if tensor_bound else None,
             "sustained_peak": tf_sust if tensor_bound else None,
         }
-        # DRAM read + write bytes of one fused launch from the ncu capture summarised in
-        # profiles/fused_gemm2_combine_dsv2lite_ncu.md (same workload, same launch configuration)
+        # DRAM read + write bytes of one fused launch from an ncu capture (same workload, same launch configuration)
         x_passes = 1 if (args.drain_help and plan.co_warps == 0) else w.L   # m-tile-major order reads x once, split-major once per split
-        all_bytes = all_traffic_bytes(w, x_passes)
+        all_bytes = all_traffic_bytes(w, dw.idx, x_passes)
         # every byte the launch has to move through HBM (x, W2, Y written and read back, out): not part of the
         # headline roofline, but the real bound at small T, where every expert's weights are read for a few rows
         roofline["hbm_all_traffic_us"] = all_bytes / peaks["hbm_gbs"] / 1e3
@@ -1018,7 +1043,8 @@ def main():
             "config": config_of(w, dw.info, world),
             "plan": {"comm_ctas": plan.comm_ctas, "R": plan.R, "P": plan.P, "W_comp": plan.W_comp,
                      "W_comm": plan.W_comm, "rho": plan.rho_q / 2 ** 20, "drain_help": plan.drain_help,
-                     "co_warps": plan.co_warps},
+                     "co_warps": plan.co_warps},                                                # the selector's pick
+            "launched": launched_division(w, lim, plan, counts[w.E_tot]),
             "fused_kernel_us": fused_med, "tflops": dw.flops / fused_med / 1e6,
             "wall_ms_per_step": wall * 1e3 / K,
             "roofline": roofline,
