@@ -8,8 +8,8 @@
 // One persistent kernel, one 512-thread CTA per SM.  The gather is part of the operand loads: four loader warps know
 // the token of every row of the tile and copy each k-block of those rows straight from the hidden states into the
 // 128B-swizzled stage (16-byte cp.async, eight lanes per row).  A gather launch in front wrote and re-read the routed
-// rows, k_tot times the hidden states: 142 us and 1 GB of a 1280 us stage at 131072 rows of 2048 (now 1230 in all; Granite
-// shape, T = 4096: 120 -> 99 us).  (One TMA tile::gather4 copy per four rows does not keep up: 80 cycles each on an SM, 3660 us
+// rows, k_tot times the hidden states: 142 us and 1 GB of a 1280 us stage at 131072 rows of 2048 (now 1260 in all; Granite
+// shape, T = 4096: 120 -> 98 us).  (One TMA tile::gather4 copy per four rows does not keep up: 80 cycles each on an SM, 3660 us
 // for the stage.)  Rows past the end
 // of an expert's last tile are not fetched at all: nothing stored depends on them.
 //   tile_m <= 128: tile = 128 routed rows x 128 intermediate columns per CTA, four 48 KB stages;
@@ -21,7 +21,7 @@
 //   warps 12-15 loaders of the gathered rows; their copies arrive by themselves on the stage's `rows` barrier;
 //   warp 2      relay (one thread): waits for that barrier, makes the rows visible to the tensor core's proxy and
 //               arrives on the stage's full barrier (a fence in the issuing warp would cost every k-block its cycles).  Pair: the
-//               other CTA's relay hands its rows to the leader's, which arrives for both;
+//               other CTA's relay arrives on the leader's barrier;
 //   warp 1      issues tcgen05.mma (converged warp, elected lane; N = 256, K = 16, bf16 -> fp32): accumulator
 //               columns 0..127 are the gate projection, 128..255 the up projection of the same outputs;
 //               two accumulator buffers in TMEM;
@@ -60,7 +60,7 @@ struct G1Cfg {
 };
 
 struct alignas(64) G1Params {
-    CUtensorMap tmB;   // W1 as [E_tot * 2, I, H]    box 64 x 128 rows x 1 plane
+    CUtensorMap tmB;   // W1 as [E_tot * 2, I, H]    box 64 x tile columns (128, 96 or 64) x 1 plane
     const int32_t *mtile_expert;
     const int32_t *mtile_first_row;
     const int32_t *mtile_valid;
@@ -74,7 +74,7 @@ struct alignas(64) G1Params {
     unsigned long long wait_ns;
     int32_t S;                     // m-tiles of the routing workspace (or their bound with S_dev)
     int32_t T, k_tot, H;
-    int32_t I, NT;                 // intermediate size, n-tiles = ceil(I / 128)
+    int32_t I, NT;                 // intermediate size, n-tiles = ceil(I / tile columns)
     int32_t num_kb, last_ksteps;
     int32_t w1_once;               // W1 is read (about) once: its lines go first when L2 needs room
     unsigned long long *mail;      // != nullptr: the tile counts (S_dev - E_tot) are mailed to the host by this launch
@@ -86,7 +86,6 @@ struct G1Control {
     unsigned long long full[kG1MaxStages];
     unsigned long long empty[kG1MaxStages];
     unsigned long long rows[kG1MaxStages];    // every loader thread's copies of the stage have landed
-    unsigned long long peer_rows[kG1MaxStages];   // leader of a pair: the other CTA's rows of the stage, handed over by its relay
     unsigned long long tmem_full[2];
     unsigned long long tmem_empty[2];
     uint32_t tmem_base;
@@ -167,10 +166,9 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::kStages; ++i) {
-            mbar_init(smem_u32(&ctl->full[i]), 2);               // the W1 producer and the relay of this CTA
+            mbar_init(smem_u32(&ctl->full[i]), kPair ? 3 : 2);   // the W1 producer and the relay of every CTA
             mbar_init(smem_u32(&ctl->empty[i]), 1);
             mbar_init(smem_u32(&ctl->rows[i]), 32 * kG1LoadWarps);
-            mbar_init(smem_u32(&ctl->peer_rows[i]), 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
@@ -249,9 +247,9 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         __syncwarp();
     } else if (warp == 2) {
         // ---------------- relay: rows landed -> visible to the tensor core's (async) proxy -> full barrier.  Pair: the other CTA's
-        // relay hands its rows to the leader's, release to acquire at cluster scope, and that one arrives for both.  (With an
-        // unrestricted release: 1500-1900 cycles later per stage, stage alone, Granite shape T = 1003 46 -> 57 us, Qwen shape
-        // T = 2880 159 -> 190.)
+        // relay hands its rows to the leader's MMA issuer, release to acquire at cluster scope.  (With an unrestricted
+        // release: 1500-1900 cycles later per stage, stage alone, Granite shape T = 1003 46 -> 57 us, Qwen shape T = 2880
+        // 159 -> 190.  By way of the leader's relay, one barrier more: whole layer, DeepSeek shape T = 16384, +0.5 %.)
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
@@ -261,13 +259,8 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     ok = g1_wait(smem_u32(&ctl->rows[stage]), phase, ctl, deadline, P.status, (uint32_t)g, 54u);
                     if (!ok) break;
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    if (rank != 0) {
-                        mbar_arrive_cluster_release_shared(mapa_u32(smem_u32(&ctl->peer_rows[stage]), 0u));
-                    } else {
-                        if (kPair) ok = g1_wait<true>(smem_u32(&ctl->peer_rows[stage]), phase, ctl, deadline, P.status, (uint32_t)g, 56u);
-                        if (!ok) break;
-                        mbar_arrive(smem_u32(&ctl->full[stage]));
-                    }
+                    if (rank != 0) mbar_arrive_cluster_release_shared(mapa_u32(smem_u32(&ctl->full[stage]), 0u));
+                    else mbar_arrive(smem_u32(&ctl->full[stage]));
                     if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
                 }
             }
@@ -342,8 +335,8 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(a * C::kAccCols);
                 for (int kb = 0; kb < P.num_kb; ++kb) {
-                    if (!__all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) {
-                        ok = __all_sync(0xffffffffu, g1_wait(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 52u));
+                    if (!__all_sync(0xffffffffu, kPair ? mbar_test_wait_cluster(full_bar, phase) : mbar_test_wait(full_bar, phase))) {
+                        ok = __all_sync(0xffffffffu, g1_wait<kPair>(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 52u));
                         if (!ok) break;
                     }
                     tc_fence_after();
