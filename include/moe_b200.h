@@ -111,8 +111,8 @@ typedef struct {
                                 phase is at least this many waves long, ceil(L * W_comp / P(C)) >= co_min_waves (a
                                 one-time characterisation: on short launches their start-up costs more than they can
                                 overlap; moe_query_occupancy returns INT32_MAX for the 256-row CTA-pair tiles, where
-                                a co-resident warp costs the seventh operand stage and never paid); a forced w is not
-                                subject to it */
+                                a co-resident warp costs the seventh operand stage and does not pay in a loop of equal
+                                steps); a forced w is not subject to it */
 } moe_sm_limits;
 
 /* Relative wave service rate (Eq. 13-15). */

@@ -247,9 +247,11 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n, moe_o
         limits->dep_model = MOE_DEP_SPLIT;
         // Lower end of the co-resident family's legal set (one-time sweep).  One-CTA tiles: below 24 compute waves
         // co-resident warps lost 2-5 % (T = 1024: 19 waves; T = 2048: 37).  CTA-pair tiles: a co-resident warp takes
-        // the shared memory of the seventh operand stage, and with seven stages for w = 0 the best w > 0 candidate
-        // never beat the best w = 0 one at any size of the sweep (1.00-1.05 of it): the family is not offered (a
-        // forced w is still honoured).
+        // the shared memory of the seventh operand stage.  In a loop of equal steps w = 0 is the fastest at every size
+        // (w = 0 / 1 / 2, 20 steps: T = 8192 425 / 433 / 429 us, 16384 783 / 802 / 793, 32768 1516 / 1541 / 1521; 400 steps, where
+        // the power cap sets the clock: 496 / 503 / 502, 902 / 914 / 911, 1718 / 1743 / 1743); only between launches of other
+        // candidates (the sweep) was w = 2 ahead, by up to 3 % from T = 16384 on.  The family is not offered (a forced w is
+        // still honoured).
         limits->co_min_waves = (tile_m == 256) ? INT32_MAX : 24;
     }
     if (rho) {
@@ -297,10 +299,13 @@ int32_t moe_select_tile(moe_handle *h, const moe_shape *s, int32_t *tile_m, int3
     // Conventional kernel dispatch (Section III-E: it runs before the resource manager and hands it the tile
     // shape and residency of the kernel it chose).  Widest n-tile the split holds; rows: the 256-row CTA-pair
     // tile moves a third less operand traffic per FLOP but pads every expert's last tile to 256 rows and needs
-    // two co-scheduled SMs, so it pays once an expert fills most of one such tile on average (measured on the
-    // DeepSeek-V2-Lite shape, fused kernel, 128x256 against 256x256: 78 / 100 us at T = 16, 128 / 132 at 1024
-    // (124 rows per expert), 172 / 160 at 2048 (248 rows), 257 / 243 at 4096, 466 / 423 at 8192, 885 / 791 at
-    // 16384; Qwen shape (546 rows per expert) 265 / 242, Granite shape (819 rows, K = 256) 134 / 131).
+    // two co-scheduled SMs, so it pays once an expert fills most of one such tile on average.  Measured, whole fused step and
+    // whole layer, 128 x 256 against 256 x 256, us, at 128 / 192 / 256 / 512 rows per expert:
+    //   Granite shape  step 53/54  59/59  67/65  93/89    layer  80/87   99/90  105/103  143/142
+    //   Qwen shape     step 117/115  143/129  170/146  273/237    layer  232/251  309/282  368/337  587/565
+    //   DeepSeek shape step 136/135  149/145  195/177  357/319    layer  267/312  322/330  418/400  789/779
+    // From 192 on the pair is at most 3 % behind for a layer (DeepSeek shape, 192 and 224), up to 10 % ahead; at 160 and below
+    // 128-row tiles are at most 4 % behind for a step, up to a quarter ahead for a layer.
     const int64_t split_w = ceil_div(s->H, s->L);
     const int32_t tn = split_w >= 256 ? 256 : split_w >= 128 ? 128 : 64;
     const int64_t rows_per_expert = (int64_t)s->T * s->k_tot / s->E_tot;

@@ -45,8 +45,8 @@ constexpr int kInlineMaxR = 2048;      // assignments up to which a kernel build
 // Parameters of one fused launch.  Passed by value (__grid_constant__): the two tensor maps
 // must sit in kernel parameter space, 64-byte aligned.
 struct alignas(64) FusedParams {
-    CUtensorMap tmA;   // x_routed [R, I]      box 64 x 128 rows, 128B swizzle
-    CUtensorMap tmB;   // W2 [E_tot, H, I]     box 64 x tile_n x 1, 128B swizzle
+    CUtensorMap tmA;   // x_routed [R, I]      box 64 x 32 rows (one-CTA tiles) or 128 (pair), 128B swizzle
+    CUtensorMap tmB;   // W2 [E_tot, H, I]     box 64 x tile_n rows (a pair's CTA: half of them) x 1, 128B swizzle
     const int32_t *mtile_expert;
     const int32_t *mtile_first_row;
     const int32_t *mtile_valid;
@@ -164,10 +164,11 @@ namespace moe {
 
 // Every kernel of this library may be launched before its predecessor on the stream has finished: each waits for the
 // predecessor's writes (griddepcontrol.wait) before it touches global memory, so that the launch latencies and
-// prologues of a step's kernels lie beside the end of the kernel before.  Only the short kernels (routing, gather) let
-// their successor start early; behind the long ones it starts as they end.  CTAs that sit and wait on the SMs that a
-// long kernel leaves idle cost more than they save: whole step at T = 1 / 16 / 256 on the DeepSeek shape 73.2 / 72.4 /
-// 102.7 us with early starts everywhere, 68.2 / 69.7 / 99.1 as it is, 77.2 / 74.1 / 103.5 without chained launches.
+// prologues of a step's kernels lie beside the end of the kernel before.  The routing kernels let their successor start
+// early, and the pair kernel does once it serves its shares of the combine; behind the other long ones it starts as they
+// end.  CTAs that sit and wait on the SMs that a long kernel leaves idle cost more than they save: whole step at T = 1 / 16 /
+// 256 on the DeepSeek shape 73.2 / 72.4 / 102.7 us with early starts everywhere, 68.2 / 69.7 / 99.1 from the short kernels
+// alone, 77.2 / 74.1 / 103.5 without chained launches (measured when the routing build was a launch of its own at these sizes).
 inline cudaLaunchAttribute chained_launch_attribute()
 {
     cudaLaunchAttribute a = {};
