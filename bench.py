@@ -45,7 +45,7 @@ def load_peaks():
 def config_of(w, info, world):
     """The `config` object of the JSON line: the same dict in the main arm and in the reference arm."""
     x_mb, w2_mb = w.R * w.I * 2 / 1e6, w.E_tot * w.H * w.I * 2 / 1e6
-    y_mb = w.T * w.L * w.k_tot * w.TP * (-(-w.H // w.L)) * 2 / 1e6
+    y_mb = w.T * w.L * w.k_tot * (-(-w.H // w.L)) * 2 / 1e6
     return {"workload": w.name, "T": w.T, "H": w.H, "I": w.I, "E": w.E, "k": w.k,
             "n_shared": w.n_shared, "TP": w.TP, "EP": w.EP, "tile": f"{w.tile_m}x{w.tile_n}",
             "L": w.L, "routing": f"{w.routing} s={w.zipf_s}", "r_expert": info["r_expert"],
@@ -171,7 +171,7 @@ class DeviceWorkload:
         self.shape = B.make_shape(w.T, w.H, w.I, w.E_tot, w.k_tot, w.TP, w.EP, w.L)
         self.ws = B.alloc_workspace(self.shape, w.tile_m, w.tile_n, device=device)
         self.flops = 2.0 * w.R * w.I * w.H
-        self.combine_bytes = w.TP * w.R * w.H * 2 + w.T * w.H * 2 + w.R * 8
+        self.combine_bytes = w.R * w.H * 2 + w.T * w.H * 2 + w.R * 8   # (the K-shards are summed in the GEMM's accumulators)
 
 
 def make_stepper(h, dw, limits_override=None):
@@ -356,7 +356,7 @@ def all_traffic_bytes(w, idx, x_passes=1):
     read back, out."""
     import numpy as np
     return (w.R * w.I * 2 * x_passes + len(np.unique(idx)) * w.H * w.I * 2 +
-            2 * w.T * w.L * w.k_tot * w.TP * (-(-w.H // w.L)) * 2 + w.T * w.H * 2)
+            2 * w.T * w.L * w.k_tot * (-(-w.H // w.L)) * 2 + w.T * w.H * 2)
 
 
 def launched_division(w, lim, plan, S):
@@ -365,7 +365,7 @@ def launched_division(w, lim, plan, S):
     narrowest ones that are a single wave.  comm_ctas: CTAs (of `P` compute slots' neighbours) that only combine."""
     split_w, slot = -(-w.H // w.L), 2 if w.tile_m == 256 else 1
     slab = 1024
-    while slab > 8 and w.k_tot * w.TP * slab * 2 > 8192:
+    while slab > 8 and w.k_tot * slab * 2 > 8192:
         slab //= 2
     units = w.T * w.L * -(-split_w // slab)
     if not lim.drain_help or lim.force_comm_ctas > 0 or lim.selector_off or plan.co_warps or units > 32 * 12 * lim.G:
@@ -374,8 +374,8 @@ def launched_division(w, lim, plan, S):
     if slot == 1:
         used = min(w.R, w.E_tot)
         S_max = (w.R - used) // w.tile_m + used
-        tn = next((n for n in (64, 128, 256) if n <= w.tile_n and S_max * w.TP * w.L * -(-split_w // n) <= slots), w.tile_n)
-    tiles = S * w.TP * w.L * -(-split_w // tn)
+        tn = next((n for n in (64, 128, 256) if n <= w.tile_n and S_max * w.L * -(-split_w // n) <= slots), w.tile_n)
+    tiles = S * w.L * -(-split_w // tn)
     waves = max(1, -(-tiles // slots))
     P = max(1, -(-tiles // waves))
     return {"comm_ctas": (slots - P) * slot, "P": P, "tile_n": tn, "waves": waves, "by": "whole waves of the tiles"}
@@ -512,7 +512,7 @@ def gemm_only_mma_record(h, dw, step, occ, lim):
     comp = rec[rec[:, TL["tiles"]] > 0]
     if not comp.size:
         return None
-    kb = comp[:, TL["tiles"]] * (-(-(w.I // w.TP) // 64))
+    kb = comp[:, TL["tiles"]] * (-(-w.I // 64))
     med = lambda v: float(np.median(v))
     return {"cycles_per_kblock": med(comp[:, TL["mma_cycles"]] / kb), "waiting_for_operands": med(comp[:, TL["wait_operand"]] / kb),
             "issuing": med(comp[:, TL["issue"]] / kb), "waiting_for_accumulator_buffer": med(comp[:, TL["wait_tmem"]] / kb),
@@ -553,8 +553,7 @@ def run_timeline(h, dw, step, occ, lim, args):
         return {"min": float((v.min() - t0) / 1e3), "median": float((np.median(v) - t0) / 1e3),
                 "max": float((v.max() - t0) / 1e3)} if v.size else None
 
-    K = w.I // w.TP
-    num_kb = -(-K // 64)
+    num_kb = -(-w.I // 64)
     kb = comp[:, TL["tiles"]] * num_kb
     per_kb = lambda slot: float(np.median(comp[:, TL[slot]] / kb)) if comp.size else None
     out = {
@@ -578,7 +577,7 @@ def run_timeline(h, dw, step, occ, lim, args):
         # the SM clock the launch really ran at: cycles of the MMA thread's loop over the time it took
         "sm_clock_ghz_during_gemm": float(np.median(comp[:, TL["mma_cycles"]] / np.maximum(1.0, comp[:, TL["mma_end"]] - comp[:, TL["begin"]]))) if comp.size else None,
     }
-    Q = w.k_tot * w.TP
+    Q = w.k_tot
     slab = 1024
     while slab > 8 and Q * slab * 2 > 8192:
         slab //= 2
@@ -976,10 +975,10 @@ def main():
         if not args.no_cpu_baseline:
             extra["cpu_baseline"], _ = cpu_baseline(w, dw.idx, dw.wt, dw.x_cpu, dw.W2_cpu)
         # ---- context: the library GEMM (cuBLAS through torch.matmul) on a dense problem with the same FLOPs and the
-        # same contraction length K = I / TP: [R * TP, K] x [K, H].  Not part of the operator: it says what a dense
+        # same contraction length I: [R, I] x [I, H].  Not part of the operator: it says what a dense
         # GEMM without routing, padding, scattered stores and flags reaches at this K on this GPU.
-        a_ = torch.randn((w.R * w.TP, w.I // w.TP), device=device, dtype=torch.bfloat16)
-        b_ = torch.randn((w.H, w.I // w.TP), device=device, dtype=torch.bfloat16)
+        a_ = torch.randn((w.R, w.I), device=device, dtype=torch.bfloat16)
+        b_ = torch.randn((w.H, w.I), device=device, dtype=torch.bfloat16)
         evs = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(9)]
         for _ in range(2):
             c_ = a_ @ b_.t()
@@ -988,7 +987,7 @@ def main():
         torch.cuda.synchronize()
         cub = statistics.median(ea.elapsed_time(eb) * 1e3 for ea, eb in evs)
         extra["context_cublas_same_flops"] = {
-            "shape": [w.R * w.TP, w.H, w.I // w.TP], "us": cub, "tflops": dw.flops / cub / 1e6,
+            "shape": [w.R, w.H, w.I], "us": cub, "tflops": dw.flops / cub / 1e6,
             "gemm_only_over_cublas": cub / extra["gemm_only"]["us"],
             "what": "torch.matmul (cuBLAS) on a dense bf16 GEMM of the same FLOPs and K, timed alone; context, not a target"}
         del a_, b_, c_

@@ -20,7 +20,8 @@
  *  - bf16 tensors are passed as void*; layouts are row-major with the last index contiguous.
  *
  * Symbols: T tokens (paper M), H hidden size (paper N), I expert intermediate size,
- * TP emulated tensor-parallel shards (split-K partials, paper g), K = I / TP (paper K),
+ * TP emulated tensor-parallel shards (K-shards of I / TP columns, paper g), K = I / TP (paper K); the selector
+ * counts a tile per shard, the launch adds the shards' products in the accumulator of one tile over all of I,
  * EP emulated destination ranks (paper D), E_tot experts (routed + shared), k_tot experts per
  * token, R = T * k_tot routed rows, L pipeline splits along H, S = sum_e ceil(M_e / T_M).
  */
@@ -151,7 +152,7 @@ typedef struct {
     int64_t pred_T_q;    /* T(C*) in compute-wave units, scaled by 2^20 */
     int64_t rho_q;       /* rho scaled by 2^20 and rounded to nearest */
     int32_t mode;        /* MOE_MODE_* (plan_partition writes MOE_MODE_FUSED) */
-    int32_t debug_withhold_tile; /* test hook: global tile whose readiness is never raised; -1 = none */
+    int32_t debug_withhold_tile; /* test hook: global tile (split, m-tile, K-shard, n-tile) whose readiness is never raised; -1 = none */
     int32_t drain_help;  /* copied from moe_sm_limits: compute CTAs help with the communication tail */
     int32_t co_warps;    /* co-resident communication warps per compute CTA (Section III-B with communication
                             work sharing the SM of a compute CTA instead of reserving one): they serve split s
@@ -241,7 +242,7 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n,
 int32_t moe_select_tile(moe_handle *h, const moe_shape *shape, int32_t *tile_m, int32_t *tile_n);
 
 /* Sizes of the caller-allocated workspaces [bytes]: routing arrays, the tile-padded GEMM2
- * output Y (bf16, token-major: [T][L][k_tot * TP][ceil(H/L)]), readiness flags + split counters +
+ * output Y (bf16, token-major: [T][L][k_tot][ceil(H/L)], with room for TP times as much), readiness flags + split counters +
  * work queues (must be zero-filled once before first use and not shared between handles), status
  * (16 bytes). */
 int32_t moe_workspace_bytes(const moe_shape *shape, int32_t tile_m, int32_t tile_n,

@@ -467,11 +467,11 @@ int64_t most_mtiles(const moe_shape *s, int tile_m)
     const int64_t R = (int64_t)s->T * s->k_tot, used = R < s->E_tot ? R : s->E_tot;
     return (R - used) / tile_m + used;
 }
-// column slab of one unit: the largest power of two with Q * columns * 2 <= 8 KB, at most 1024
+// column slab of one unit: the largest power of two with k_tot * columns * 2 <= 8 KB, at most 1024
 int slab_shift_of(const moe_shape *s)
 {
     int sh = 10;
-    while (sh > 3 && ((int64_t)s->k_tot * s->TP << sh) * 2 > 8192) --sh;
+    while (sh > 3 && ((int64_t)s->k_tot << sh) * 2 > 8192) --sh;
     return sh;
 }
 // Who serves what when the compute CTAs help: a queue per split, or, up to 32 units (of 8 KB) a warp, an even share for every
@@ -630,18 +630,20 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
 
     FusedParams p;
     memset(&p, 0, sizeof p);
-    const int K = s->I / s->TP;
-    p.T = s->T; p.H = s->H; p.K = K; p.TP = s->TP; p.EP = s->EP; p.L = s->L; p.k_tot = s->k_tot;
+    // the sum over the K-shards is taken in the accumulators: a tile runs over all of I, whatever TP is
+    p.T = s->T; p.H = s->H; p.EP = s->EP; p.L = s->L; p.k_tot = s->k_tot;
     p.S = n_mtiles;
     p.tile_m = occ->tile_m;
     p.flag_parts = pair ? 2 : 1;
     p.split_w = (int32_t)ceil_div(s->H, s->L);
     p.NTs = (int32_t)ceil_div(p.split_w, occ->tile_n);
-    const int64_t Wc = (int64_t)s->TP * n_mtiles * p.NTs;
-    if (Wc * s->L * 2 >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
+    const int64_t Wc = (int64_t)n_mtiles * p.NTs;
+    if (Wc * s->TP * s->L * 2 >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
     p.W_comp = (int32_t)Wc;
     p.S_dev = counts_on_device ? r->tiles + s->E_tot : nullptr;
-    p.C = C; p.P = Pc; p.mode = mode; p.withhold = plan->debug_withhold_tile;
+    p.C = C; p.P = Pc; p.mode = mode;
+    // (the plan counts a tile per K-shard: split, m-tile, shard, n-tile)
+    p.withhold = plan->debug_withhold_tile < 0 ? -1 : plan->debug_withhold_tile / (s->TP * p.NTs) * p.NTs + plan->debug_withhold_tile % p.NTs;
     p.G = h->G;
     p.slot_sms = slot_sms;
     p.E_tot = s->E_tot;
@@ -659,8 +661,8 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
     p.tok_blk = (int32_t)ceil_div(s->T, s->EP);
     p.comm_cols = (int32_t)ceil_div(p.split_w, kCommTileN);
-    p.num_kb = (int32_t)ceil_div(K, kBlockK);
-    p.last_ksteps = (K - (p.num_kb - 1) * kBlockK) / kUmmaK;
+    p.num_kb = (int32_t)ceil_div(s->I, kBlockK);
+    p.last_ksteps = (s->I - (p.num_kb - 1) * kBlockK) / kUmmaK;
     p.R_pad = (long long)occ->tile_m * n_mtiles;
     p.wait_ns = h->wait_ns;
     p.mtile_expert = r->mtile_expert;
@@ -668,7 +670,6 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.mtile_valid = r->mtile_valid;
     p.pad_row = r->pad_row;
     p.perm = r->perm;
-    p.Q = s->k_tot * s->TP;
     p.slab_shift = slab_shift_of(s);
     p.slab_cols = 1 << p.slab_shift;
     p.topk_w = topk_w;
@@ -685,7 +686,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     // of shared memory (free only when the epilogue stores straight from registers) and units of at most 16
     // rows; where one of these does not hold the launch runs without them (same result, bit for bit).
     p.co_warps = plan->co_warps < fused_co_warps_max() ? plan->co_warps : fused_co_warps_max();
-    if (!p.drain_help || !p.wide_store || p.Q > 16) p.co_warps = 0;
+    if (!p.drain_help || !p.wide_store || s->k_tot > 16) p.co_warps = 0;
     // warps 16-19 of a compute CTA: co-resident communication warps, or -- when none is asked for -- a fourth
     // epilogue column group (a third less epilogue work per warp: what bounds tiles with a short K)
     p.epi_warps = (p.co_warps == 0 && p.wide_store) ? 16 : 12;
@@ -715,10 +716,10 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
         // (the time of a wave is the time to stream and store one tile: DeepSeek shape, T = 1, 19 -> 16 us).
         const int64_t bound = most_mtiles(s, occ->tile_m), S_max = counts_on_device && bound < n_mtiles ? bound : n_mtiles;
         for (int tn = 64; tn <= occ->tile_n; tn *= 2) {
-            if (S_max * s->TP * s->L * ceil_div(p.split_w, tn) > C + Pc) continue;
+            if (S_max * s->L * ceil_div(p.split_w, tn) > C + Pc) continue;
             TN = tn;
             p.NTs = (int32_t)ceil_div(p.split_w, TN);
-            p.W_comp = s->TP * n_mtiles * p.NTs;
+            p.W_comp = n_mtiles * p.NTs;
             p.C = ctas_c = 0;
             p.P = ctas_p = C + Pc;
             p.c_table_n = 0;

@@ -23,12 +23,17 @@
 // Compute CTA pair (256 x 256 tiles): the same roles in both CTAs of a cluster of two; one
 //   tcgen05.mma.cta_group::2 spans both SMs, each CTA loads only its own operand halves; six operand
 //   stages, seven when the aux region of shared memory is free while the GEMM runs.
-// Y is token-major: the epilogue scatters each accumulator row to its (token, slot, shard) place, so
-//   that the k_tot * TP partial rows of one (token, split, column slab) form one contiguous block.
+// Y is token-major: the epilogue scatters each accumulator row to its (token, slot) place, so
+//   that the k_tot rows of one (token, split, column slab) form one contiguous block.  The sum over the tensor-parallel
+//   K-shards (Section II-A: each rank's partial product, here all on one GPU) is taken in the accumulator, in fp32: a tile runs over
+//   all of I.  With a tile and a bf16 row of Y per shard, each partial was rounded, stored, read back and added by the combine:
+//   TP times the Y traffic and the epilogue stores.  Whole step at TP = 2, us, a tile per shard -> now: Granite shape T = 4096
+//   130 -> 96, Qwen shape T = 8192 287 -> 249, DeepSeek shape T = 256 88 -> 82 and T = 16384 943 -> 836; three calls with the static
+//   partition, DeepSeek shape T = 2048 207 -> 178.  Y holds a row per assignment, rounded once instead of once per shard.
 // Communication CTA (12 independent warps): a warp fetches such a block with one bulk asynchronous
 //   copy into its own double-buffered shared-memory stage (the readiness of the producing tiles is
 //   checked first: split counter, else per-tile flags with ld.acquire.gpu; bounded), sums the rows in
-//   fp32 in (j, p) order with the token's weights and stores bf16 into the owning rank's buffer.
+//   fp32 in slot order with the token's weights and stores bf16 into the owning rank's buffer.
 // Co-resident communication warps (Section III-B with o_comm > 1 in spirit: communication work that
 //   shares an SM with a compute CTA instead of reserving one): a compute CTA may carry extra warps
 //   (of 16-19; two have stages) that run the same per-unit pipeline on stages of their own, take work from
@@ -189,33 +194,29 @@ struct Part {
 };
 
 struct Tile {
-    int s, mu, p, i_n;
-    int id;   // canonical tile number s * W_comp + (mu * TP + p) * NTs + i_n: indexes the readiness flags
+    int s, mu, i_n;
+    int id;   // canonical tile number s * W_comp + mu * NTs + i_n: indexes the readiness flags
 };
 // Tile g of the processing sequence.  Split-major (Section III-C: all tiles of split s precede those of
 // s + 1; inside a split the expert problems are contiguous), or, when the work is handed out dynamically
 // and nothing waits for an early split (drain help), m-tile-major: the n-tiles of ALL splits of one
-// (m-tile, K-shard) are adjacent, so that the x rows are read from DRAM once instead of once per split.
+// m-tile are adjacent, so that the x rows are read from DRAM once instead of once per split.
 __device__ __forceinline__ Tile decode_tile(int g, const FusedParams &P, int W_comp)
 {
     Tile t;
     if (P.tile_order == 0) {
         t.s = g / W_comp;
         const int idx = g - t.s * W_comp;
-        const int r = idx / P.NTs;
-        t.i_n = idx - r * P.NTs;
-        t.mu = r / P.TP;
-        t.p = r - t.mu * P.TP;
+        t.mu = idx / P.NTs;
+        t.i_n = idx - t.mu * P.NTs;
         t.id = g;
     } else {
         const int per_m = P.L * P.NTs;
-        const int r = g / per_m;
-        const int j = g - r * per_m;
+        t.mu = g / per_m;
+        const int j = g - t.mu * per_m;
         t.s = j / P.NTs;
         t.i_n = j - t.s * P.NTs;
-        t.mu = r / P.TP;
-        t.p = r - t.mu * P.TP;
-        t.id = t.s * W_comp + r * P.NTs + t.i_n;
+        t.id = t.s * W_comp + t.mu * P.NTs + t.i_n;
     }
     return t;
 }
@@ -246,7 +247,7 @@ __device__ __forceinline__ bool wait_rows(const FusedParams &P, int last_row, ui
 
 // One thread = one accumulator row (TMEM lane).  Reads COLS fp32 columns starting at `col_first` of
 // the accumulator at `taddr`, rounds to bf16 and writes them to the row's place in the token-major Y:
-// slab = column slab inside the split, q = row of the unit (slot j, shard p).
+// slab = column slab inside the split, q = row of the unit (slot j).
 __device__ __forceinline__ void store_accumulator_rows(const FusedParams &P, uint32_t taddr, int col_first, int n_cols, bool row_ok,
                                                        __nv_bfloat16 *ybase, int q, int n0, int col_end, int cis0)
 {
@@ -274,7 +275,7 @@ __device__ __forceinline__ void store_accumulator_rows(const FusedParams &P, uin
                     pk.y = *reinterpret_cast<uint32_t *>(&h1);
                     pk.z = *reinterpret_cast<uint32_t *>(&h2);
                     pk.w = *reinterpret_cast<uint32_t *>(&h3);
-                    *reinterpret_cast<uint4 *>(ybase + ((size_t)slab * P.Q << P.slab_shift) + (size_t)q * wslab + cin) = pk;
+                    *reinterpret_cast<uint4 *>(ybase + ((size_t)slab * P.k_tot << P.slab_shift) + (size_t)q * wslab + cin) = pk;
                 }
             }
         }
@@ -297,7 +298,7 @@ __device__ __forceinline__ void emit_wide_joined(const FusedParams &P, const uin
     const int cis = cis0 + col;
     const int slab = cis >> P.slab_shift;
     const int wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
-    __nv_bfloat16 *dst = ybase + ((size_t)slab * P.Q << P.slab_shift) + (size_t)q * wslab + (cis & (P.slab_cols - 1));
+    __nv_bfloat16 *dst = ybase + ((size_t)slab * P.k_tot << P.slab_shift) + (size_t)q * wslab + (cis & (P.slab_cols - 1));
     if (!row_ok || MOE_PROBE(kProbeSkipYStores)) dst = nullptr;
     uint32_t w[16];
 #pragma unroll
@@ -358,7 +359,7 @@ __device__ __forceinline__ void store_accumulator_rows_staged(const FusedParams 
         const int cis = cis0 + col;
         const int slab = cis >> P.slab_shift;
         const int wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
-        stg->rowptr[lane] = row_ok ? (unsigned long long)(ybase + ((size_t)slab * P.Q << P.slab_shift) + (size_t)q * wslab +
+        stg->rowptr[lane] = row_ok ? (unsigned long long)(ybase + ((size_t)slab * P.k_tot << P.slab_shift) + (size_t)q * wslab +
                                                           (cis & (P.slab_cols - 1)))
                                    : 0ull;
         tmem_ld_wait(r);
@@ -452,8 +453,8 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
             if (row_ok) {
                 const int f = f_row;
                 const int tok = f / P.k_tot;
-                q = (f - tok * P.k_tot) * P.TP + t.p;
-                ybase = Y + ((size_t)tok * P.L + t.s) * (size_t)P.Q * (size_t)P.split_w;
+                q = f - tok * P.k_tot;
+                ybase = Y + ((size_t)tok * P.L + t.s) * (size_t)P.k_tot * (size_t)P.split_w;
             }
             const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * TN);
             if (!dry && row_in_tile - lane >= valid) {
@@ -612,7 +613,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                 // depends on them
                 const int boxes = min((valid + kXBoxRows - 1) / kXBoxRows, kMmaM / kXBoxRows);
                 if (load_a && P.x_ready && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
-                int kx = t.p * P.K;
+                int kx = 0;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     TL(tl_q = clock64());
                     ok = wait_barrier_1t(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 10u);
@@ -817,7 +818,7 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
                     const int last = ld_chained(&P.mtile_first_row[t.mu]) + ld_chained(&P.mtile_valid[t.mu]) - 1;
                     if (!(ok = wait_rows(P, last, seen, ctl, deadline))) break;
                 }
-                int kx = t.p * P.K;
+                int kx = 0;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     const uint32_t own_full = smem_u32(&ctl->full[stage]);
                     TL(tl_q = clock64());
@@ -985,14 +986,13 @@ __device__ __forceinline__ void fma2_bf16x8(unsigned long long (&acc)[4], const 
 }
 
 // The weights of a unit's rows, read back as shared-memory broadcasts.  `w`: lane j holds the weight of slot j (0: the slot has
-// no source row); `wq`: room for Q floats, rounded up to the rows that reduce_unit takes together.
+// no source row); `wq`: room for k_tot floats, rounded up to the rows that reduce_unit takes together.
 __device__ __forceinline__ void put_row_weights(const FusedParams &P, float w, float *wq)
 {
     const int lane = threadIdx.x & 31;
-    if (lane < P.k_tot)
-        for (int p = 0; p < P.TP; ++p) wq[lane * P.TP + p] = w;
+    if (lane < P.k_tot) wq[lane] = w;
 }
-// Reduces one unit that sits in shared memory at `stage_s`: the weighted sum of its Q rows in (j, p) order, one warp.  all_valid:
+// Reduces one unit that sits in shared memory at `stage_s`: the weighted sum of its k_tot rows in slot order, one warp.  all_valid:
 // every slot has a source row; `orow`: where the unit's columns of the token go; kAhead: rows fetched from shared memory together.
 template <int kAhead>
 __device__ __forceinline__ void reduce_unit(const FusedParams &P, bool all_valid, int n16, int row_bytes, const float *wq, uint32_t stage_s,
@@ -1011,7 +1011,7 @@ __device__ __forceinline__ void reduce_unit(const FusedParams &P, bool all_valid
             float wr[kAhead];
 #pragma unroll
             for (int i = 0; i < kAhead; ++i, src += (uint32_t)row_bytes)
-                v[i] = whole || q + i < P.Q ? lds_v4(src) : make_uint4(0u, 0u, 0u, 0u);
+                v[i] = whole || q + i < P.k_tot ? lds_v4(src) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int i = 0; i < kAhead; i += 4) {
                 const uint4 w4 = lds_v4(wsrc + 4u * i);
@@ -1022,15 +1022,15 @@ __device__ __forceinline__ void reduce_unit(const FusedParams &P, bool all_valid
             }
 #pragma unroll
             for (int i = 0; i < kAhead; ++i) {
-                // a slot without a source row holds bytes nobody wrote, and there is no row past Q: nothing is added
-                if (!whole && ((!all_valid && wr[i] == 0.f) || q + i >= P.Q)) v[i] = make_uint4(0u, 0u, 0u, 0u), wr[i] = 0.f;
+                // a slot without a source row holds bytes nobody wrote, and there is no row past the last slot: nothing is added
+                if (!whole && ((!all_valid && wr[i] == 0.f) || q + i >= P.k_tot)) v[i] = make_uint4(0u, 0u, 0u, 0u), wr[i] = 0.f;
                 fma2_bf16x8(acc, v[i], pack_f32x2(__float_as_uint(wr[i]), __float_as_uint(wr[i])));
             }
         };
 #pragma unroll 1
-        for (int q = 0; q < P.Q; q += kAhead, wsrc += 4u * kAhead) {
+        for (int q = 0; q < P.k_tot; q += kAhead, wsrc += 4u * kAhead) {
             // (long launches spare the checks of whole groups; short ones the second instance of the code)
-            if (kAhead == 8 && all_valid && q + kAhead <= P.Q) add_rows(q, std::true_type{});
+            if (kAhead == 8 && all_valid && q + kAhead <= P.k_tot) add_rows(q, std::true_type{});
             else add_rows(q, std::false_type{});
         }
         uint32_t o[4];
@@ -1046,11 +1046,11 @@ __device__ __forceinline__ void reduce_unit(const FusedParams &P, bool all_valid
     __syncwarp();   // all lanes are done with the stage (and with wq) before either is reused
 }
 
-// Communication warp.  Y is token-major: the k_tot * TP partial rows of one (token, split, column
+// Communication warp.  Y is token-major: the k_tot rows of one (token, split, column
 // slab) are one contiguous block (a "unit", at most 8 KB).  Every communication warp works on its own:
 // it owns two 8 KB stages of shared memory and one mbarrier per stage, fetches a unit with ONE bulk
 // asynchronous copy (global -> shared), and while that copy is in flight it reduces the previous unit
-// in fp32 in (j, p) order with the token's weights and stores the bf16 result into the owning rank's
+// in fp32 in slot order with the token's weights and stores the bf16 result into the owning rank's
 // buffer.  No warp waits on another one: the issue latency of the copies and the memory latency
 // overlap across the warps of an SM.
 //
@@ -1070,7 +1070,7 @@ static_assert(kCommWarps * kCommWarpBytes <= kStageBytesTotal, "communication st
 // Co-resident communication warps live in the aux region, which the epilogue leaves alone when it
 // stores straight from registers: two warps' stages (32 KB), then the per-row weights in compact
 // 16-float slots -- four for co-resident warps, twelve for the CTA's own warps once they turn to
-// communication (their usual 256-float slots would overlap the co-resident stages).  Needs Q <= 16.
+// communication (their usual 256-float slots would overlap the co-resident stages).  Needs k_tot <= 16.
 constexpr int kCoWarpsAux = 2;          // co-resident warps whose stages fit the aux region
 constexpr int kCoWeightFloats = 16;
 constexpr int kCoWeightsOffset = kCoWarpsAux * kCommWarpBytes;
@@ -1085,7 +1085,7 @@ enum { kRoleFront = 1, kRoleBack = 2, kRoleCoResident = 3 };
 struct CommWarpRes {
     uint8_t *stages;              // 2 x kCommUnitBytes
     unsigned long long *full;     // 2 mbarriers (initialised with count 1 at kernel start)
-    float *wq;                    // room for Q floats
+    float *wq;                    // room for k_tot floats
 };
 
 struct CommUnit {
@@ -1143,22 +1143,20 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
             if (done >= (uint32_t)(pt.W_comp * P.flag_parts)) {
                 ready_mask |= 1u << u.s;
             } else {
-                // per tile: every (slot j, shard p, n-tile under this slab)
+                // per tile: every (slot j, n-tile under this slab)
                 const int cs0 = u.slab << P.slab_shift;
                 const int in0 = cs0 / TN;
                 const int nt = (cs0 + u.ucols - 1) / TN - in0 + 1;
                 bool failed = false;
-                for (int chk = lane; chk < P.Q * nt && !failed; chk += 32) {
-                    const int qq = chk / nt;
-                    const int tn = chk - qq * nt;
-                    const int j = qq / P.TP;
-                    const int p = qq - j * P.TP;
+                for (int chk = lane; chk < P.k_tot * nt && !failed; chk += 32) {
+                    const int j = chk / nt;
+                    const int tn = chk - j * nt;
                     const int row = ld_chained(&P.pad_row[(size_t)u.t * P.k_tot + j]);
                     if (row < 0 || row >= P.R_pad) continue;
                     const int mu = row / P.tile_m;
                     // a pair tile is published in two parts, one per CTA: the row's part is its 128-row half
                     const int part = (P.flag_parts == 2) ? ((row - mu * P.tile_m) >> 7) : 0;
-                    const int g = (u.s * pt.W_comp + (mu * P.TP + p) * P.NTs + in0 + tn) * P.flag_parts + part;
+                    const int g = (u.s * pt.W_comp + mu * P.NTs + in0 + tn) * P.flag_parts + part;
                     uint32_t spins = 0;
                     TL_DECL(const unsigned long long tl_f0 = globaltimer_ns();)
                     while (ld_acquire_u32(&P.flags[g]) != P.epoch) {
@@ -1186,9 +1184,9 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
         const int st = n_mine & 1;
         if (lane == 0) {
             const uint32_t full = full_s + 8u * (uint32_t)st;
-            const uint32_t bytes = (uint32_t)(P.Q * u.wslab) * 2u;
-            const __nv_bfloat16 *src = Y + ((size_t)u.t * P.L + u.s) * (size_t)P.Q * (size_t)P.split_w +
-                                       ((size_t)u.slab * P.Q << P.slab_shift);
+            const uint32_t bytes = (uint32_t)(P.k_tot * u.wslab) * 2u;
+            const __nv_bfloat16 *src = Y + ((size_t)u.t * P.L + u.s) * (size_t)P.k_tot * (size_t)P.split_w +
+                                       ((size_t)u.slab * P.k_tot << P.slab_shift);
             mbar_arrive_expect_tx(full, bytes);
             bulk_load_once(smem_u32(my_ring + st * kCommUnitBytes), src, bytes, full, y_policy);   // Y is read once
         }
@@ -1469,8 +1467,8 @@ __device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &p
                 }
                 orow_n = reinterpret_cast<__nv_bfloat16 *>(P.out[d]) + (size_t)(tok - d * P.tok_blk) * (size_t)P.H + s * P.split_w + c0;
                 if (lane == 0) {
-                    const uint32_t bytes = (uint32_t)(P.Q * row_bytes_n), bar = full + 8u * (uint32_t)(k & 1);
-                    const __nv_bfloat16 *src = Y + (((size_t)tok * P.L + s) * (size_t)P.split_w + c0) * (size_t)P.Q;
+                    const uint32_t bytes = (uint32_t)(P.k_tot * row_bytes_n), bar = full + 8u * (uint32_t)(k & 1);
+                    const __nv_bfloat16 *src = Y + (((size_t)tok * P.L + s) * (size_t)P.split_w + c0) * (size_t)P.k_tot;
                     mbar_arrive_expect_tx(bar, bytes);
                     bulk_load_once(smem_u32(stages + (k & 1) * kCommUnitBytes), src, bytes, bar, y_policy);   // Y is read once
                 }
@@ -1551,7 +1549,7 @@ __device__ __forceinline__ Part launch_part(const FusedParams &P)
     Part pt = {P.W_comp, P.C, P.P};
     if (P.S_dev) {
         const int S = ld_chained_uniform(P.S_dev);
-        pt.W_comp = min(S, P.S) * P.TP * P.NTs;
+        pt.W_comp = min(S, P.S) * P.NTs;
         if (P.c_table_n > 0) {
             pt.C = P.c_table[max(0, min(S - P.c_table_first, P.c_table_n - 1))];
             pt.P = (P.G - pt.C) / P.slot_sms;

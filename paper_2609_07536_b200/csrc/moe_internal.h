@@ -55,7 +55,7 @@ struct alignas(64) FusedParams {
     const int32_t *pad_row;
     const int32_t *perm;
     const float *topk_w;
-    void *Y;                       // bf16 [T][L][slabs][Q][slab cols], token-major
+    void *Y;                       // bf16 [T][L][slabs][k_tot][slab cols], token-major
     uint32_t *flags;               // [L * W_comp] readiness per global tile (== epoch when ready)
     uint32_t *split_done;          // [L] tiles finished per split (this launch)
     uint32_t *split_done_next;     // [L] counters of the next launch, zeroed by this one
@@ -67,7 +67,7 @@ struct alignas(64) FusedParams {
     void *out[MOE_MAX_EP];
     unsigned long long wait_ns;
     long long R_pad;
-    int32_t T, H, K, TP, EP, L, k_tot;
+    int32_t T, H, EP, L, k_tot;
     int32_t S, tile_m, NTs, split_w, W_comp;
     int32_t C, P, mode, withhold;
     unsigned long long *mail;           // != nullptr: the tile counts (S_dev - E_tot) are mailed to the host by this launch
@@ -91,7 +91,7 @@ struct alignas(64) FusedParams {
                                         // co-resident warp is asked for and the epilogue needs no staging buffer
     int32_t tile_order;                 // 0: split-major tile sequence (the paper's); 1: m-tile-major across splits
     int32_t flag_parts;                 // readiness flags per tile: 1, or 2 for a CTA-pair tile
-    int32_t Q, slab_cols, slab_shift;   // Q = k_tot * TP rows per unit; slab_cols = 1 << slab_shift
+    int32_t slab_cols, slab_shift;      // slab_cols = 1 << slab_shift; a unit is k_tot rows of a slab
     int32_t wide_store;                 // every 16-column group of a Y row is whole and 32-byte aligned: 256-bit epilogue stores
     uint32_t epoch;
 };

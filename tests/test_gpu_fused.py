@@ -271,6 +271,28 @@ def test_ep_concat_invariance_and_tp_within_tolerance():
         assert np.max(np.abs(got - expect)) <= G.tolerance(expect), TP
 
 
+@pytest.mark.parametrize("tile", [(64, 64), (128, 256), (256, 256)])
+@pytest.mark.parametrize("drain_help", [0, 1])
+def test_shards_are_summed_in_the_accumulator(tile, drain_help):
+    # one fp32 sum over all of I whatever TP is: the same bits, with shards that end inside a k-block (80 columns of 64-wide blocks)
+    w = replace(wl.TINY, name="shards", T=150, H=520, I=320, E=4, k=3, TP=1, EP=2, L=1, tile_m=tile[0], tile_n=tile[1])
+    idx, wt, _ = wl.make_routing(w)
+    x, W2 = wl.make_data(w)
+    base, *_ = G.run_layer(w, idx, wt, x, W2, force_C=3, drain_help=drain_help)
+    for TP in (2, 4):
+        outs, plan, *_ = G.run_layer(replace(w, TP=TP), idx, wt, x, W2, force_C=3, drain_help=drain_help)
+        assert all(np.array_equal(a, b, equal_nan=True) for a, b in zip(base, outs)), TP
+    # a withheld tile is named by its shard as well; its flag is that of the tile over all shards
+    h, wt_ = G.handle(), replace(w, TP=2)
+    S, NT = rr.build_routing(idx, w.E_tot, w.tile_m)["S"], -(-w.H // w.tile_n)
+    B.moe_set_wait_limit_ns(h, 20_000_000)
+    try:
+        *_, st = G.run_layer(wt_, idx, wt, x, W2, force_C=3, drain_help=drain_help, withhold=((S - 1) * 2 + 1) * NT, check_status=False)
+        assert st.code == B.MOE_DEV_TIMEOUT
+    finally:
+        B.moe_set_wait_limit_ns(h, 2_000_000_000)
+
+
 def test_identity_weights_make_the_combine_exact():
     # W2_e = identity (I = H), small integer activations, power-of-two weights: every partial
     # sum is exactly representable in bf16, so the GPU output must equal the gather exactly
