@@ -275,36 +275,53 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            G1Tile t_next = g1_decode<TN>(min(b + stride, total_tiles - 1), P);
-            int f[kSteps], f_next[kSteps];
-            g1_load_perm(P, g1_decode<TN>(b, P), rank, first, f);
-            for (int g = b; g < total_tiles && ok; g += stride) {
-                // fetched ahead: the table entries two tiles, the rows' assignments one tile
-                const G1Tile t_nn = g1_decode<TN>(min(g + 2 * stride, total_tiles - 1), P);
-                g1_load_perm(P, t_next, rank, first, f_next);
-                const __nv_bfloat16 *src[kSteps];
+            // where this thread's chunk of its rows begins (nullptr: the tile has no such row)
+            const auto rows_of = [&](const int (&f)[kSteps], const __nv_bfloat16 *(&src)[kSteps]) {
 #pragma unroll
                 for (int i = 0; i < kSteps; ++i)
                     src[i] = f[i] >= 0 ? P.hidden + (size_t)min(f[i] / P.k_tot, P.T - 1) * (size_t)P.H + chunk * 8 : nullptr;
+            };
+            G1Tile t_next = g1_decode<TN>(min(b + stride, total_tiles - 1), P);
+            int f_next[kSteps];
+            const __nv_bfloat16 *src[kSteps], *src_next[kSteps];
+            g1_load_perm(P, g1_decode<TN>(b, P), rank, first, f_next);
+            rows_of(f_next, src);
+            for (int g = b; g < total_tiles && ok; g += stride) {
+                // Fetched ahead: the table entries two tiles, the rows' assignments one tile; their addresses (a division each) are
+                // worked out between two k-blocks, so that nothing but copies stands between the last k-block of a tile and
+                // the first of the next.  The way from a freed stage to its next rows is the longest of the ring: with the
+                // divisions at the head of the tile and a test per row in every k-block the stage took 1270 us at the DeepSeek
+                // shape T = 16384, now 1177 (20 more instructions a k-block for something else: 1400).
+                const G1Tile t_nn = g1_decode<TN>(min(g + 2 * stride, total_tiles - 1), P);
+                g1_load_perm(P, t_next, rank, first, f_next);
+                bool whole = true;               // the tile has all rows of this warp
+#pragma unroll
+                for (int i = 0; i < kSteps; ++i) whole = whole && src[i] != nullptr;
+                whole = __all_sync(0xffffffffu, whole);
+                const int ahead_at = min(4, P.num_kb - 1);
                 int left = P.H - chunk * 8;      // columns from this chunk on
                 for (int kb = 0; kb < P.num_kb; ++kb, left -= kBlockK) {
-                    ok = g1_wait_warp(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 55u);
-                    if (!ok) break;
+                    if (!mbar_test_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u))
+                        ok = g1_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 55u);
+                    if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
                     const uint32_t dst = smem_u32(ring + stage * C::kStageBytes) + dst0;
                     if (left > 0) {              // (past the last column: no MMA reads it)
+                        if (whole) {
 #pragma unroll
-                        for (int i = 0; i < kSteps; ++i)
-                            if (src[i]) {
-                                cp_async_16(dst + (uint32_t)(i * kG1RowsPerStep * 128), src[i]);
-                                src[i] += kBlockK;
-                            }
+                            for (int i = 0; i < kSteps; ++i) cp_async_16(dst + (uint32_t)(i * kG1RowsPerStep * 128), src[i] + kb * kBlockK);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < kSteps; ++i)
+                                if (src[i]) cp_async_16(dst + (uint32_t)(i * kG1RowsPerStep * 128), src[i] + kb * kBlockK);
+                        }
                     }
                     cp_async_arrive(smem_u32(&ctl->rows[stage]));
                     if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+                    if (kb == ahead_at) rows_of(f_next, src_next);
                 }
                 t_next = t_nn;
 #pragma unroll
-                for (int i = 0; i < kSteps; ++i) f[i] = f_next[i];
+                for (int i = 0; i < kSteps; ++i) src[i] = src_next[i];
             }
             cp_async_wait_all();
         }
