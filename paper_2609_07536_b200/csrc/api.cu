@@ -35,7 +35,7 @@ int32_t require_handle_device(moe_handle *h, const char *who)
 const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name)
 {
     if (!h->maps && !(h->maps = new (std::nothrow) MapEntry[kMapEntries]())) return nullptr;
-    const uint64_t mixed = (reinterpret_cast<uintptr_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull;
+    const uint64_t mixed = ((reinterpret_cast<uintptr_t>(ptr) >> 8) + (uint64_t)box_rows) * 0x9E3779B97F4A7C15ull;
     MapEntry &m = h->maps[mixed >> 57];
     static_assert(kMapEntries == 1 << (64 - 57), "the hash's upper bits index the table");
     if (m.ptr == ptr && m.rows == rows && m.cols == cols && m.planes == planes && m.box_rows == box_rows) return &m.map;
@@ -96,11 +96,6 @@ int32_t n_routing_warps(const moe_shape *s)
 }  // namespace moe
 
 using namespace moe;
-
-#ifndef MOE_PAIR_SEVENTH_STAGE
-#define MOE_PAIR_SEVENTH_STAGE 1
-#endif
-static constexpr bool kPairSeventhStage = MOE_PAIR_SEVENTH_STAGE != 0;
 
 extern "C" {
 
@@ -660,6 +655,9 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     }
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
     p.tok_blk = (int32_t)ceil_div(s->T, s->EP);
+    p.token_shift = 30u;                                     // exact below 2^30: token_mul exceeds the quotient by less than k_tot / 2^shift
+    while ((1u << (p.token_shift - 30u)) < (uint32_t)s->k_tot) ++p.token_shift;
+    p.token_mul = (uint32_t)(((1ull << p.token_shift) + (uint32_t)s->k_tot - 1) / (uint32_t)s->k_tot);
     p.comm_cols = (int32_t)ceil_div(p.split_w, kCommTileN);
     p.num_kb = (int32_t)ceil_div(s->I, kBlockK);
     p.last_ksteps = (s->I - (p.num_kb - 1) * kBlockK) / kUmmaK;
@@ -674,24 +672,19 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.slab_cols = 1 << p.slab_shift;
     p.topk_w = topk_w;
     p.Y = y_ws;
-    p.wide_store = (p.slab_cols >= 32 && p.split_w % 16 == 0 && s->H % 16 == 0 &&
-                    (reinterpret_cast<uintptr_t>(y_ws) & 31u) == 0) ? 1 : 0;
     p.status = status_dev;
     for (int d = 0; d < s->EP; ++d) p.out[d] = out[d];
     if (feed) {
         p.x_ready = feed->ready;
         p.wait_ns += feed->extra_wait_ns;
     }
-    // Co-resident communication warps need the dynamic hand-out (they pull from the queues), the aux region
-    // of shared memory (free only when the epilogue stores straight from registers) and units of at most 16
+    // Co-resident communication warps need the dynamic hand-out (they pull from the queues) and units of at most 16
     // rows; where one of these does not hold the launch runs without them (same result, bit for bit).
     p.co_warps = plan->co_warps < fused_co_warps_max() ? plan->co_warps : fused_co_warps_max();
-    if (!p.drain_help || !p.wide_store || s->k_tot > 16) p.co_warps = 0;
+    if (!p.drain_help || s->k_tot > 16) p.co_warps = 0;
     // warps 16-19 of a compute CTA: co-resident communication warps, or -- when none is asked for -- a fourth
     // epilogue column group (a third less epilogue work per warp: what bounds tiles with a short K)
-    p.epi_warps = (p.co_warps == 0 && p.wide_store) ? 16 : 12;
-    // CTA-pair kernel: with the aux region free during the GEMM it becomes a seventh operand stage
-    p.pair_stages = (pair && p.co_warps == 0 && p.wide_store && kPairSeventhStage) ? 7 : 6;
+    p.epi_warps = p.co_warps == 0 ? 16 : 12;
     // Tile sequence: split-major (the paper's) whenever something consumes a split while the next one is
     // computed; m-tile-major across the splits (x is read from DRAM once) when nothing does
     p.tile_order = (plan->drain_help && p.co_warps == 0) ? 1 : 0;
@@ -747,12 +740,16 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.flags = flags_ws + kSplitCounterWords;
 
     // operands (Section II-A): x_routed [R, I] and W2 [E_tot, H, I], k contiguous; a pair CTA loads half the n-tile's rows
-    const CUtensorMap *mA = operand_map(h, x_routed, 0, R, s->I, pair ? kMmaM : kXBoxRows, "x_routed");
-    if (!mA) return MOE_ERR_CUDA;
-    p.tmA = *mA;
+    CUtensorMap *const mA[3] = {&p.tmA, &p.tmA64, &p.tmA32};
+    for (int i = 0; i < (pair ? 2 : 3); ++i) {
+        const CUtensorMap *m = operand_map(h, x_routed, 0, R, s->I, 128 >> i, "x_routed");
+        if (!m) return MOE_ERR_CUDA;
+        *mA[i] = *m;
+    }
     const CUtensorMap *mB = operand_map(h, W2, s->E_tot, s->H, s->I, pair ? TN / 2 : TN, "W2");
     if (!mB) return MOE_ERR_CUDA;
     p.tmB = *mB;
+    p.stages = fused_stages(pair, TN, p.co_warps == 0);
     const int grid = pair ? ((ctas_c + 1) & ~1) + 2 * ctas_p : ctas_c + ctas_p;
     p.timeline = nullptr;
     if (h->timeline && h->timeline_bytes >= ((size_t)grid * kTimelineSlots + MOE_MAX_L) * sizeof(unsigned long long))

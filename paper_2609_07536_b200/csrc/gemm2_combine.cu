@@ -14,16 +14,16 @@
 //   warps 0, 2  TMA producers (one thread each): warp 0 the x_routed tile (up to 128 rows x 64 k), warp 2 the
 //               W2 tile (tile_n rows x 64 k) of every k-block, into a ring of 128B-swizzled stages;
 //   warp 1      MMA issuer (the warp runs the loop converged, an elected lane issues; all operands warp-uniform):
-//               tcgen05.mma (M = 128, N = tile_n, K = 16, bf16 -> fp32) into one of two TMEM accumulator
-//               buffers; tcgen05.commit frees stages / publishes the tile;
-//   warps 4-15  epilogue: tcgen05.ld -> bf16 -> Y (three column groups x four TMEM lane quarters; warps 16-19
-//               are a fourth column group when the launch carries no co-resident communication warp);
+//               tcgen05.mma (M = 128 output columns, N = the tile's rows, K = 16, bf16 -> fp32; two of them for 256 columns) into one
+//               of two TMEM accumulator buffers; tcgen05.commit frees stages / publishes the tile;
+//   warps 4-15  epilogue: tcgen05.ld -> bf16, transposed -> Y (three groups of four warps, one per TMEM lane quarter; warps 16-19
+//               are a fourth group when the launch carries no co-resident communication warp);
 //   warp 3      publisher (one thread): once the epilogue warps have stored a tile, release fence, then the
 //               tile's readiness flag and the split counter (one fence for all tiles stored by then).
 // Compute CTA pair (256 x 256 tiles): the same roles in both CTAs of a cluster of two; one
-//   tcgen05.mma.cta_group::2 spans both SMs, each CTA loads only its own operand halves; six operand
+//   tcgen05.mma.cta_group::2 (M = 256) spans both SMs, each CTA loads only its own operand halves; six operand
 //   stages, seven when the aux region of shared memory is free while the GEMM runs.
-// Y is token-major: the epilogue scatters each accumulator row to its (token, slot) place, so
+// Y is token-major: the epilogue scatters each routed row to its (token, slot) place, so
 //   that the k_tot rows of one (token, split, column slab) form one contiguous block.  The sum over the tensor-parallel
 //   K-shards (Section II-A: each rank's partial product, here all on one GPU) is taken in the accumulator, in fp32: a tile runs over
 //   all of I.  With a tile and a bf16 row of Y per shard, each partial was rounded, stored, read back and added by the combine:
@@ -92,15 +92,19 @@ enum { kProbeSkipOddW2 = 1, kProbeSkipAllW2 = 2, kProbeSkipYStores = 4, kProbeSk
 
 // --------------------------------------------------------------------------- shared memory
 
+// Weights on the M side of the MMA, tokens on the N side: an accumulator lane is a column of the output, an accumulator column a
+// routed row, and N is the tile's row count rounded up to 16 (a pair: 32).  (With the rows on the M side every tile was computed for
+// 128 or 256 rows.  Whole calls, us, rows on M -> on N: DeepSeek shape T = 16 58.9 -> 53.5, T = 256 81 -> 72, Qwen shape T = 8192
+// 239 -> 229, its whole layer T = 48 187 -> 170, T = 3000 126 -> 116; where hardly a row is padding, Granite shape T = 13784, equal.)
 template <int TN>
 struct Cfg {
-    static constexpr int kABytes = kMmaM * kBlockK * 2;          // 16 KB
-    static constexpr int kBBytes = TN * kBlockK * 2;             // 8 / 16 / 32 KB
-    static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = kStageBytesTotal / kStageBytes;  // 8 / 6 / 4
-    static constexpr int kTmemCols = 2 * TN;                     // two accumulator buffers
-    // epilogue: warps 4..15 (three column groups x four TMEM lane quarters), plus warps 16..19 as a fourth
-    // column group when the launch carries no co-resident communication warps (FusedParams::epi_warps)
+    static constexpr int kWBytes = TN * kBlockK * 2;             // 8 / 16 / 32 KB: the tile's rows of W2
+    static constexpr int kXBytes = kMmaM * kBlockK * 2;          // 16 KB: up to 128 routed rows
+    static constexpr int kStageBytes = kWBytes + kXBytes;
+    static constexpr int kStages = kStageBytesTotal / kStageBytes;  // 8 / 6 / 4 
+    static constexpr int kBlocks = TN > kMmaM ? 2 : 1;           // blocks of 128 output columns, an MMA each (TN = 64: half of one is used)
+    static constexpr int kAccCols = kBlocks * kMmaM;             // TMEM columns of an accumulator buffer
+    static constexpr int kTmemCols = 2 * kAccCols;               // two of them
 };
 
 // Tiles a CTA may have stored but not yet published: the publisher's release fence takes thousands of cycles,
@@ -116,20 +120,14 @@ struct Control {
     unsigned long long pub_done[kPubSlots];   // the publisher warp has raised that tile's flag
     uint32_t tmem_base;
     volatile uint32_t abort;
+    volatile uint32_t tile_n[8];        // N of a tile's MMAs (tile number mod 8), from the x producer to the MMA issuer
     unsigned long long comm_full[24];   // communication CTA: one barrier per warp and stage
     unsigned long long co_full[8];      // co-resident communication warps: one barrier per warp and stage
 };
 
-// 32 KB after the control block, used by one role per CTA:
-//   communication CTA: per-row weights of the unit each warp reduces (12 warps x 256 floats)
-//   compute CTA      : per-epilogue-warp staging (12 warps x 2.5 KB + row pointers) for coalesced Y stores
-constexpr int kAuxBytes = 12 * 2560 + 12 * 256;
-constexpr int kEpiStagePitch = 80;    // 64 data bytes + 16 pad: conflict-free 16-byte stores
-struct EpiStage {
-    uint8_t data[32 * kEpiStagePitch];        // 32 rows x 32 bf16
-    unsigned long long rowptr[32];            // destination of each row for the group in hand (0 = skip)
-};
-static_assert(sizeof(EpiStage) * 12 <= kAuxBytes, "epilogue staging exceeds the aux region");
+// 33 KB after the control block: per-row weights of the unit each communication warp reduces (12 warps x 256 floats), or the stages
+// and weights of co-resident communication warps
+constexpr int kAuxBytes = 33 * 1024;
 static_assert(12 * 256 * 4 <= kAuxBytes, "communication weights exceed the aux region");
 
 // Bounded mbarrier wait, warp-collective: lane 0 polls (32 lanes polling the same barrier would
@@ -182,44 +180,73 @@ __device__ __forceinline__ void sync_compute_warps(const FusedParams &P)
 {
     asm volatile("bar.sync 1, %0;" ::"r"(kThreads + 32 * (P.epi_warps - 12)) : "memory");
 }
-// 32-column rounds of a TN-wide tile dealt to `groups` epilogue column groups (3 or 4)
-__device__ __forceinline__ int epi_cols_per_group(int tn, int groups)
-{
-    return ((tn / 32 + groups - 1) / groups) * 32;
-}
+// token of flat assignment f (< 2^30): the quotient by k_tot, exact (token_mul = ceil(2^token_shift / k_tot))
+__device__ __forceinline__ int token_of(const FusedParams &P, int f) { return (int)((unsigned long long)(uint32_t)f * P.token_mul >> P.token_shift); }
+// N of a tile's MMAs: its rows, rounded up to what the instruction takes (M = 128: 16, M = 256 over a pair: 32)
+template <bool kPair>
+__device__ __forceinline__ int mma_n_of(int valid) { return kPair ? (valid + 31) & ~31 : (valid + 15) & ~15; }
+
+// The MMA issuer's N of its tile `it`, behind the tile's first full barrier.  The producer knows the tile's rows; looked up by the issuer
+// itself, the table entry is a load in the issuer's way.  (A place is written again
+// eight tiles later, when the MMAs of the tile before the last seven stages are over.)
+template <typename Ctl>
+__device__ __forceinline__ int tile_n(const Ctl *ctl, int it) { return (int)__reduce_max_sync(0xffffffffu, ctl->tile_n[it & 7]); }   // (warp-uniform)
 
 // What a launch's roles are divided by: compute tiles per split (Eq. 5), communication CTAs, compute slots.
 struct Part {
-    int W_comp, C, P;
+    int W_comp, S, C, P;     // S: m-tiles
 };
 
 struct Tile {
     int s, mu, i_n;
     int id;   // canonical tile number s * W_comp + mu * NTs + i_n: indexes the readiness flags
 };
-// Tile g of the processing sequence.  Split-major (Section III-C: all tiles of split s precede those of
-// s + 1; inside a split the expert problems are contiguous), or, when the work is handed out dynamically
+// The tiles of the processing sequence that a compute slot takes: b, b + P, b + 2 P, ...  Split-major (Section III-C: all tiles of
+// split s precede those of s + 1; inside a split the expert problems are contiguous), or, when the work is handed out dynamically
 // and nothing waits for an early split (drain help), m-tile-major: the n-tiles of ALL splits of one
 // m-tile are adjacent, so that the x rows are read from DRAM once instead of once per split.
-__device__ __forceinline__ Tile decode_tile(int g, const FusedParams &P, int W_comp)
-{
-    Tile t;
-    if (P.tile_order == 0) {
-        t.s = g / W_comp;
-        const int idx = g - t.s * W_comp;
-        t.mu = idx / P.NTs;
-        t.i_n = idx - t.mu * P.NTs;
-        t.id = g;
-    } else {
-        const int per_m = P.L * P.NTs;
-        t.mu = g / per_m;
-        const int j = g - t.mu * per_m;
-        t.s = j / P.NTs;
-        t.i_n = j - t.s * P.NTs;
-        t.id = t.s * W_comp + t.mu * P.NTs + t.i_n;
+// A position is a number of three digits (split, m-tile, n-tile), the step another one: no division per tile (with two for every
+// look-up the epilogue warps spent 2500 cycles of a tile's 6200 between tiles at the Granite shape, and paced it).
+struct TileWalk {
+    int W_comp, NTs, n_mid, last_mu;     // n_mid: values of the middle digit
+    bool m_major;
+    int top, mid, low, d_top, d_mid, d_low;
+    __device__ __forceinline__ TileWalk(const FusedParams &P, const Part &pt, int b)
+    {
+        W_comp = pt.W_comp;
+        NTs = P.NTs;
+        m_major = P.tile_order != 0;
+        n_mid = m_major ? P.L : pt.S;
+        last_mu = pt.S - 1;
+        split(b, top, mid, low);
+        split(pt.P, d_top, d_mid, d_low);
     }
-    return t;
-}
+    __device__ __forceinline__ void split(int g, int &t, int &m, int &l) const
+    {
+        const int r = g / NTs;
+        l = g - r * NTs;
+        t = r / n_mid;
+        m = r - t * n_mid;
+    }
+    __device__ __forceinline__ void next()
+    {
+        low += d_low;
+        mid += d_mid;
+        top += d_top;
+        if (low >= NTs) { low -= NTs; ++mid; }
+        if (mid >= n_mid) { mid -= n_mid; ++top; }
+    }
+    // (past the end of the sequence: some tile of the table, for look-ups that nobody uses)
+    __device__ __forceinline__ Tile tile() const
+    {
+        Tile t;
+        t.s = m_major ? mid : top;
+        t.mu = m_major ? min(top, last_mu) : mid;
+        t.i_n = low;
+        t.id = t.s * W_comp + t.mu * NTs + low;
+        return t;
+    }
+};
 
 // x_routed that is still being copied in (FusedParams::x_ready): waits until the rows up to `last_row` have arrived.  One
 // thread; `seen`: rows known to have arrived.  The copies were issued before this launch, so the wait ends on its own.
@@ -245,181 +272,77 @@ __device__ __forceinline__ bool wait_rows(const FusedParams &P, int last_row, ui
 
 // --------------------------------------------------------------------------- epilogue helper
 
-// One thread = one accumulator row (TMEM lane).  Reads COLS fp32 columns starting at `col_first` of
-// the accumulator at `taddr`, rounds to bf16 and writes them to the row's place in the token-major Y:
-// slab = column slab inside the split, q = row of the unit (slot j).
-__device__ __forceinline__ void store_accumulator_rows(const FusedParams &P, uint32_t taddr, int col_first, int n_cols, bool row_ok,
-                                                       __nv_bfloat16 *ybase, int q, int n0, int col_end, int cis0)
+// 32 rows x 32 columns of the accumulator at `taddr` -> bf16 -> Y, one warp.  The accumulator has the columns in its lanes, Y has
+// them contiguous: 8 x 8 blocks are transposed in registers, then the four lanes that hold a row's 32 columns in pairs deal them
+// out in eights, so that one store instruction covers 64 contiguous bytes of eight rows.  (By way of shared memory, 256 contiguous
+// bytes a row: the staging buffers take an operand stage, and the GEMM phase grows by it, DeepSeek shape T = 16384 578 -> 696 us.)
+// `dst`: lane i, where the first of the 32 columns of row i goes (nullptr: nowhere); `cols`: columns that exist.
+__device__ __forceinline__ void store_rows(const FusedParams &P, const uint32_t (&lo)[16], const uint32_t (&hi)[16], __nv_bfloat16 *dst, int cols)
 {
-#pragma unroll 1
-    for (int cc = 0; cc < n_cols; cc += 32) {
-        const int col = col_first + cc;
-        uint32_t r[32];
-        tmem_ld_32x32(taddr + (uint32_t)col, r);
-        tmem_ld_wait(r);
-        if (row_ok) {
+    const int lane = threadIdx.x & 31, c = lane & 3;
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int c0 = n0 + col + v * 8;
-                if (c0 < col_end) {
-                    const int cis = cis0 + col + v * 8;
-                    const int slab = cis >> P.slab_shift;
-                    const int cin = cis & (P.slab_cols - 1);
-                    const int wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
-                    uint4 pk;
-                    __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 0]), __uint_as_float(r[v * 8 + 1]));
-                    __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 2]), __uint_as_float(r[v * 8 + 3]));
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 4]), __uint_as_float(r[v * 8 + 5]));
-                    __nv_bfloat162 h3 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 6]), __uint_as_float(r[v * 8 + 7]));
-                    pk.x = *reinterpret_cast<uint32_t *>(&h0);
-                    pk.y = *reinterpret_cast<uint32_t *>(&h1);
-                    pk.z = *reinterpret_cast<uint32_t *>(&h2);
-                    pk.w = *reinterpret_cast<uint32_t *>(&h3);
-                    *reinterpret_cast<uint4 *>(ybase + ((size_t)slab * P.k_tot << P.slab_shift) + (size_t)q * wslab + cin) = pk;
-                }
+    for (int j = 0; j < 4; ++j) {                // rows 8j..8j+7; this lane: row 8j + lane / 4
+        uint32_t v[4] = {transpose_8x8(pack_bf16(lo[4 * j], lo[4 * j + 1])), transpose_8x8(pack_bf16(lo[4 * j + 2], lo[4 * j + 3])),
+                         transpose_8x8(pack_bf16(hi[4 * j], hi[4 * j + 1])), transpose_8x8(pack_bf16(hi[4 * j + 2], hi[4 * j + 3]))};
+        // v[m]: columns 8m + 2c and the next one -> v[k]: columns 8c + 2k and the next one
+#pragma unroll
+        for (int d = 1; d < 4; d *= 2)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                if (m & d) continue;
+                const bool up = (c & d) != 0;
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? v[m] : v[m + d], d);
+                if (up) v[m] = got;
+                else v[m + d] = got;
             }
-        }
-    }
-}
-
-// Same job with 256-bit stores straight from registers (no shared memory).  Needs every 16-column group whole
-// and 32-byte aligned (FusedParams::wide_store).
-// One 32-column group of every lane's row, bf16.  The stores of two neighbouring lanes are joined: lanes 2k and
-// 2k+1 swap half of their rows' data, so that one store instruction covers 64 contiguous bytes of a row (one
-// request of two sectors instead of two requests of one sector).  Half as many write requests from the SM for
-// the same bytes: the GEMM phase gets 2 % shorter where K is long (the requests compete with the operand stream)
-// and 10 % where it is short (K = 256: the epilogue bounds the tile).  The whole warp runs this, also lanes
-// without a valid row.
-__device__ __forceinline__ void emit_wide_joined(const FusedParams &P, const uint32_t (&r)[32], int col, bool row_ok,
-                                                 __nv_bfloat16 *ybase, int q, int n0, int col_end, int cis0)
-{
-    const int lane = threadIdx.x & 31;
-    const bool odd = lane & 1;
-    const int cis = cis0 + col;
-    const int slab = cis >> P.slab_shift;
-    const int wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
-    __nv_bfloat16 *dst = ybase + ((size_t)slab * P.k_tot << P.slab_shift) + (size_t)q * wslab + (cis & (P.slab_cols - 1));
-    if (!row_ok || MOE_PROBE(kProbeSkipYStores)) dst = nullptr;
-    uint32_t w[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-        w[i] = *reinterpret_cast<uint32_t *>(&h);
-    }
-    // what the neighbour stores for this lane's row: the even lane hands over columns 16..31, the odd one 0..15
-    uint32_t other[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) other[i] = __shfl_xor_sync(0xffffffffu, odd ? w[i] : w[8 + i], 1);
-    const unsigned long long mine = reinterpret_cast<unsigned long long>(dst);
-    const unsigned long long theirs = __shfl_xor_sync(0xffffffffu, mine, 1);
-    // first instruction: the even lane's row (even lane: its columns 0..15; odd lane: the even lane's 16..31);
-    // second instruction: the odd lane's row (even lane: the odd lane's 0..15; odd lane: its own 16..31)
-    __nv_bfloat16 *p1 = reinterpret_cast<__nv_bfloat16 *>(odd ? theirs : mine);
-    __nv_bfloat16 *p2 = reinterpret_cast<__nv_bfloat16 *>(odd ? mine : theirs);
-    const int c1 = n0 + col + (odd ? 16 : 0);
-    uint32_t d1[8], d2[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        d1[i] = odd ? other[i] : w[i];
-        d2[i] = odd ? w[8 + i] : other[i];
-    }
-    if (p1 != nullptr && c1 < col_end) st_global_v8(p1 + (odd ? 16 : 0), d1);
-    if (p2 != nullptr && c1 < col_end) st_global_v8(p2 + (odd ? 16 : 0), d2);
-}
-__device__ __forceinline__ void store_accumulator_rows_wide(const FusedParams &P, uint32_t taddr, int col_first, int n_cols, bool row_ok,
-                                                            __nv_bfloat16 *ybase, int q, int n0, int col_end, int cis0)
-{
-    // (reading the next group from TMEM while this one is stored was measured: no gain, 13 more registers)
-#pragma unroll 1
-    for (int cc = 0; cc < n_cols; cc += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32(taddr + (uint32_t)(col_first + cc), r);
-        tmem_ld_wait(r);
-        emit_wide_joined(P, r, col_first + cc, row_ok, ybase, q, n0, col_end, cis0);
-    }
-}
-
-// Same job with the stores coalesced: the warp's 32 rows x 32 columns go through a padded staging
-// buffer, so that four lanes write one row's 64 contiguous bytes (two full sectors) instead of every
-// lane writing 16 bytes of a different row.  Needs the 32-column group inside one column slab.
-__device__ __forceinline__ void store_accumulator_rows_staged(const FusedParams &P, uint32_t taddr, int col_first, int n_cols, bool row_ok,
-                                                              __nv_bfloat16 *ybase, int q, int n0, int col_end, int cis0,
-                                                              EpiStage *stg)
-{
-    const int lane = threadIdx.x & 31;
-    const uint32_t stg_s = smem_u32(stg->data);
-    const uint32_t my_row_s = stg_s + (uint32_t)lane * kEpiStagePitch;
-    const int chunk = lane & 3;
-#pragma unroll 1
-    for (int cc = 0; cc < n_cols; cc += 32) {
-        const int col = col_first + cc;
-        uint32_t r[32];
-        tmem_ld_32x32(taddr + (uint32_t)col, r);
-        // where this thread's row goes for this 32-column group
-        const int cis = cis0 + col;
-        const int slab = cis >> P.slab_shift;
-        const int wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
-        stg->rowptr[lane] = row_ok ? (unsigned long long)(ybase + ((size_t)slab * P.k_tot << P.slab_shift) + (size_t)q * wslab +
-                                                          (cis & (P.slab_cols - 1)))
-                                   : 0ull;
-        tmem_ld_wait(r);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 0]), __uint_as_float(r[v * 8 + 1]));
-            __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 2]), __uint_as_float(r[v * 8 + 3]));
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 4]), __uint_as_float(r[v * 8 + 5]));
-            __nv_bfloat162 h3 = __floats2bfloat162_rn(__uint_as_float(r[v * 8 + 6]), __uint_as_float(r[v * 8 + 7]));
-            sts_v4(my_row_s + v * 16, *reinterpret_cast<uint32_t *>(&h0), *reinterpret_cast<uint32_t *>(&h1),
-                   *reinterpret_cast<uint32_t *>(&h2), *reinterpret_cast<uint32_t *>(&h3));
-        }
-        __syncwarp();
-        // four lanes per row, eight rows per store instruction
-        const bool col_ok = (n0 + col + chunk * 8) < col_end;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int row = i * 8 + (lane >> 2);
-            const unsigned long long dst = stg->rowptr[row];
-            const uint4 v = lds_v4(stg_s + (uint32_t)row * kEpiStagePitch + (uint32_t)chunk * 16u);
-            if (dst != 0ull && col_ok) *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(dst) + chunk * 8) = v;
-        }
-        __syncwarp();
+        __nv_bfloat16 *row = reinterpret_cast<__nv_bfloat16 *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), 8 * j + (lane >> 2)));
+        if (row != nullptr && c * 8 < cols && !MOE_PROBE(kProbeSkipYStores)) *reinterpret_cast<uint4 *>(row + c * 8) = make_uint4(v[0], v[1], v[2], v[3]);
     }
 }
 
 // --------------------------------------------------------------------------- epilogue and publisher roles
 //
-// Shared by the one-CTA and the CTA-pair compute roles (kPair: this CTA is rank `rank` of a pair and owns rows
-// rank * 128 ... of the 256-row tile; the accumulator buffer is handed back on the leader's barrier; the tile is
+// Shared by the one-CTA and the CTA-pair compute roles (kPair: this CTA is rank `rank` of a pair and owns columns
+// rank * 128 ... of the tile; the accumulator buffer is handed back on the leader's barrier; the tile is
 // published in two parts, one flag per CTA).
 
-// Epilogue, one warp: TMEM -> bf16 -> Y for the warp's TMEM lane quarter and column group of every tile of
-// this CTA, then the hand-over to the publisher warp.
+// Epilogue, one warp: TMEM -> bf16 -> Y of every tile of this CTA: its TMEM lane quarter (32 of 128 columns) of every third or fourth
+// piece of 32 rows x 128 columns, then the hand-over to the publisher warp.
 template <int TN, bool kPair>
-__device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &pt, Control *ctl, uint8_t *aux, int b,
+__device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &pt, Control *ctl, int b,
                                               uint32_t tmem_base, unsigned long long deadline, int rank)
 {
+    constexpr int kBlocks = kPair ? 1 : Cfg<TN>::kBlocks, kAccCols = kPair ? TN : Cfg<TN>::kAccCols;
+    constexpr int kPieces = 3;                 // pieces of a tile that a warp may have: 8, over at least three groups of warps
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int total_tiles = P.L * pt.W_comp;
     const int q4 = warp & 3;                   // TMEM lane quarter this warp may read
-    const int grp = (warp - 4) >> 2;           // column group of the tile
-    const int cols_per_group = epi_cols_per_group(TN, P.epi_warps >> 2);
-    const int col_first = grp * cols_per_group;
-    const int n_cols = max(0, min(cols_per_group, TN - col_first));
-    const int row_in_tile = (kPair ? rank * kMmaM : 0) + q4 * 32 + lane;
+    const int grp = (warp - 4) >> 2, groups = P.epi_warps >> 2;
     __nv_bfloat16 *Y = reinterpret_cast<__nv_bfloat16 *>(P.Y);
     // Row bookkeeping runs ahead of the accumulators: the m-tile table entries are fetched two tiles
-    // ahead and the row's flat assignment one tile ahead, so that these dependent global loads are
+    // ahead and the rows' flat assignments one tile ahead, so that these dependent global loads are
     // not in the way between an accumulator becoming ready and its first store.
-    int valid = 0, f_row = 0, valid_n = 0, first_n = 0;
+    int valid = 0, valid_n = 0, first_n = 0;
+    int f[kPieces];                            // piece i: assignment of row `lane` of it
+    const int max_pieces = groups == 3 ? 3 : 2;
+    const auto load_rows = [&](int first, int n, int (&fr)[kPieces]) {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            const int row = (grp + i * groups) / kBlocks * 32 + lane;
+            fr[i] = i < max_pieces && row < n ? ld_chained(&P.perm[first + row]) : -1;
+        }
+    };
     TL_DECL(long long tl_ew = 0, tl_ek = 0, tl_ep = 0, tl_q;)
+    TileWalk walk(P, pt, b);
+    Tile t = walk.tile(), t_n = t;
     if (b < total_tiles) {
-        const int mu0 = decode_tile(b, P, pt.W_comp).mu;
-        const int mu1 = decode_tile(min(b + pt.P, total_tiles - 1), P, pt.W_comp).mu;
-        valid = ld_chained(&P.mtile_valid[mu0]);
-        const int first0 = ld_chained(&P.mtile_first_row[mu0]);
-        valid_n = ld_chained(&P.mtile_valid[mu1]);
-        first_n = ld_chained(&P.mtile_first_row[mu1]);
-        if (row_in_tile < valid) f_row = ld_chained(&P.perm[first0 + row_in_tile]);
+        walk.next();
+        t_n = walk.tile();
+        valid = ld_chained(&P.mtile_valid[t.mu]);
+        const int first0 = ld_chained(&P.mtile_first_row[t.mu]);
+        valid_n = ld_chained(&P.mtile_valid[t_n.mu]);
+        first_n = ld_chained(&P.mtile_first_row[t_n.mu]);
+        load_rows(first0, valid, f);
     }
     // Round -1 (one-CTA tiles: small launches, whose tail counts) is dry: the store path runs once without a tile while the first operands are on their way, on whatever the
     // second accumulator buffer holds, so that its instructions are at hand when the first tile is done.
@@ -427,56 +350,73 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
 #pragma unroll 1
     for (int g = b; g < total_tiles;) {
         const bool dry = !kPair && it < 0;
-        const Tile t = decode_tile(g, P, pt.W_comp);
         const int a = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
-        int valid_nn = valid_n, first_nn = first_n, f_row_n = 0;
+        Tile t_nn = t_n;
+        int valid_nn = valid_n, first_nn = first_n, f_n[kPieces];
         bool ok = true;
         if (!dry) {
-            const int mu_nn = decode_tile(min(g + 2 * pt.P, total_tiles - 1), P, pt.W_comp).mu;
-            valid_nn = ld_chained(&P.mtile_valid[mu_nn]);
-            first_nn = ld_chained(&P.mtile_first_row[mu_nn]);
-            if (row_in_tile < valid_n) f_row_n = ld_chained(&P.perm[first_n + row_in_tile]);
+            walk.next();
+            t_nn = walk.tile();
+            valid_nn = ld_chained(&P.mtile_valid[t_nn.mu]);
+            first_nn = ld_chained(&P.mtile_first_row[t_nn.mu]);
+            load_rows(first_n, valid_n, f_n);
+        }
+        const int n_pieces = (dry ? 1 : (valid + 31) >> 5) * kBlocks;
+        const int mine = dry ? 1 : n_pieces > grp ? (n_pieces - grp + groups - 1) / groups : 0;
+        // destinations of this lane's rows: a routed row belongs to flat assignment f = (token, slot); Y is token-major so that the
+        // combine reads one contiguous block
+        __nv_bfloat16 *dst[kPieces];
+        int cols[kPieces];
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            const int block = (grp + i * groups) % kBlocks;
+            const int cis = t.i_n * TN + (kPair ? rank : block) * kMmaM + q4 * 32;       // first column, inside the split
+            cols[i] = min(min(P.H, (t.s + 1) * P.split_w) - t.s * P.split_w, t.i_n * TN + TN) - cis;
+            dst[i] = nullptr;
+            if (!dry && f[i] >= 0 && cols[i] > 0) {
+                const int tok = token_of(P, f[i]), q = f[i] - tok * P.k_tot;
+                const int slab = cis >> P.slab_shift, wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
+                dst[i] = Y + (size_t)(uint32_t)(tok * P.L + t.s) * ((size_t)P.k_tot * (size_t)P.split_w) + ((size_t)slab * P.k_tot << P.slab_shift) +
+                         (uint32_t)(q * wslab + (cis & (P.slab_cols - 1)));
+            }
         }
         TL(tl_q = clock64());
         if (!dry) ok = wait_barrier(smem_u32(&ctl->tmem_full[a]), acc_phase, ctl, deadline, P.status, (uint32_t)g, 30u);
         TL(tl_ew += clock64() - tl_q; tl_q = clock64());
         if (ok) {
             tc_fence_after();
-            const int n0 = t.s * P.split_w + t.i_n * TN;
-            const int col_end = min(P.H, (t.s + 1) * P.split_w);
-            const bool row_ok = !dry && row_in_tile < valid;
-            // destination of this thread's row: the routed row belongs to flat assignment
-            // f = (token, slot); Y is token-major so that the combine reads one contiguous block
-            __nv_bfloat16 *ybase = Y;
-            int q = 0;
-            if (row_ok) {
-                const int f = f_row;
-                const int tok = f / P.k_tot;
-                q = f - tok * P.k_tot;
-                ybase = Y + ((size_t)tok * P.L + t.s) * (size_t)P.k_tot * (size_t)P.split_w;
+            const auto release = [&]() {
+                // the accumulator buffer (this CTA's half of it) may be overwritten by the MMA of the tile after next
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (kPair) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->tmem_empty[a]), 0u));   // the leader's barrier
+                    else mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
+                }
+            };
+#pragma unroll
+            for (int i = 0; i < kPieces; ++i) {
+                if (i >= mine) break;
+                const int piece = grp + i * groups, chunk = piece / kBlocks, block = piece - chunk * kBlocks;
+                if (dry || cols[i] > 0) {
+                    const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * kAccCols + (dry ? 0 : block * kMmaM + chunk * 32));
+                    uint32_t lo[16], hi[16];
+                    tmem_ld_16x256_x4(taddr, lo);
+                    tmem_ld_16x256_x4(taddr + (16u << 16), hi);
+                    tmem_ld_wait(lo);
+                    tmem_ld_wait(hi);
+                    if (!dry && i == mine - 1) release();
+                    store_rows(P, lo, hi, dst[i], cols[i]);
+                } else if (i == mine - 1) {
+                    release();
+                }
             }
-            const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * TN);
-            if (!dry && row_in_tile - lane >= valid) {
-                // none of the warp's 32 rows holds a token (small batches: most warps)
-            } else if (P.wide_store)
-                store_accumulator_rows_wide(P, taddr, col_first, n_cols, row_ok, ybase, q, n0, col_end, n0 - t.s * P.split_w);
-            else if (P.slab_cols >= 32)
-                store_accumulator_rows_staged(P, taddr, col_first, n_cols, row_ok, ybase, q, n0, col_end,
-                                              n0 - t.s * P.split_w, reinterpret_cast<EpiStage *>(aux) + (warp - 4));
-            else
-                store_accumulator_rows(P, taddr, col_first, n_cols, row_ok, ybase, q, n0, col_end, n0 - t.s * P.split_w);
-            // the accumulator buffer (this CTA's half of it) may be overwritten by the MMA of the tile after next
             if (dry) {
                 ++it;
                 continue;
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                if (kPair) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->tmem_empty[a]), 0u));   // the leader's barrier
-                else mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
-            }
+            if (mine == 0) release();
             TL(tl_ek += clock64() - tl_q);
         }
         // hand the tile to the publisher warp.  Its barrier is reused every kPubSlots tiles, so the warp first
@@ -491,7 +431,10 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
         __syncwarp();   // the lanes' stores are ordered before lane 0's arrival
         if (lane == 0) mbar_arrive(smem_u32(&ctl->epi_done[slot]));
         valid = valid_n;
-        f_row = f_row_n;
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) f[i] = f_n[i];
+        t = t_n;
+        t_n = t_nn;
         valid_n = valid_nn;
         first_n = first_nn;
         g += pt.P;
@@ -513,6 +456,7 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, const Part 
     const int total_tiles = P.L * pt.W_comp;
     if ((threadIdx.x & 31) == 0) {
         int it = 0;
+        TileWalk walk(P, pt, b);
         TL_DECL(long long tl_pw = 0, tl_pf = 0, tl_q;)
         for (int g = b; g < total_tiles;) {
             TL(tl_q = clock64());
@@ -527,8 +471,8 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, const Part 
                    mbar_test_wait(smem_u32(&ctl->epi_done[(it + n) & (kPubSlots - 1)]), (uint32_t)((it + n) / kPubSlots) & 1u))
                 ++n;
             fence_acq_rel_gpu();   // release: the epilogue warps' stores (observed through epi_done) come first
-            for (int j = 0; j < n; ++j, ++it, g += pt.P) {
-                const Tile t = decode_tile(g, P, pt.W_comp);
+            for (int j = 0; j < n; ++j, ++it, g += pt.P, walk.next()) {
+                const Tile t = walk.tile();
                 if (t.id != P.withhold) {
                     if (!P.even) st_relaxed_u32(&P.flags[kPair ? 2 * t.id + rank : t.id], P.epoch);
 #if MOE_TIMELINE
@@ -547,6 +491,114 @@ __device__ __forceinline__ void publisher_role(const FusedParams &P, const Part 
     __syncwarp();
 }
 
+struct PairCfg {
+    static constexpr int kTileN = 256;
+    static constexpr int kWBytes = kMmaM * kBlockK * 2;                 // 16 KB: this CTA's 128 W2 rows
+    static constexpr int kXBytes = (kTileN / 2) * kBlockK * 2;          // 16 KB: this CTA's half of the tile's rows
+    static constexpr int kStageBytes = kWBytes + kXBytes;               // 32 KB
+    static constexpr int kTmemCols = 2 * kTileN;                        // two accumulator buffers
+};
+
+// --------------------------------------------------------------------------- TMA producers
+//
+// One thread: kX the x_routed rows, else the W2 rows of every k-block of this CTA's tiles; both complete on the same full barrier
+// (two issuing threads halve the serial issue latency per k-block).  The way from a freed stage to its next copies is the longest
+// of the ring, so the loop over the k-blocks holds nothing but the wait, the copy and constants to add: a k-block of the rows is ONE
+// copy, of 128 rows or, where they suffice, 64 or 32 (two copies of 64 rows lengthen the GEMM phase of the DeepSeek shape T = 16384 from
+// 609 to 690 us, a number of copies and bytes that it looks up by 30), and the next tile is looked up between two k-blocks.
+template <int TN, bool kPair, bool kX>
+__device__ __forceinline__ void producer_role(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b, unsigned long long deadline, uint32_t rank)
+{
+    using C = typename std::conditional<kPair, PairCfg, Cfg<TN>>::type;
+    const int total_tiles = P.L * pt.W_comp, n_stages = P.stages;
+    // pair: the leader's full barriers, which lie at the same offsets in CTA 0
+    const uint32_t dst0 = smem_u32(ring) + (kX ? (uint32_t)C::kWBytes : 0u), empty0 = smem_u32(&ctl->empty[0]);
+    const uint32_t full0 = kPair ? smem_u32(&ctl->full[0]) & 0xFEFFFFFFu : smem_u32(&ctl->full[0]);
+    uint32_t dst = dst0, full_bar = full0, empty_bar = empty0;
+    int stage = 0, it = 0;
+    uint32_t phase = 0, seen = 0;
+    uint32_t armed = 0;  // bit s: stage s was handed to the TMA unit at least once
+    bool ok = true;
+    const unsigned long long w_policy = P.w2_once ? l2_evict_first_policy() : l2_evict_normal_policy();
+    TL_DECL(long long tl_pw = 0, tl_q;)
+    TileWalk walk(P, pt, b);
+    Tile t = walk.tile(), t_next = t;
+    int e = kX ? 0 : ld_chained(&P.mtile_expert[t.mu]), e_next = 0;
+    int row0 = kX ? ld_chained(&P.mtile_first_row[t.mu]) : 0, valid = kX ? ld_chained(&P.mtile_valid[t.mu]) : 0, row0_next = 0, valid_next = 0;
+    const int ahead_at = min(2, P.num_kb - 1);
+    for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
+        const int n0 = t.s * P.split_w + t.i_n * TN + (kPair ? (int)rank * (TN / 2) : 0);
+        const int n = mma_n_of<kPair>(valid), my_rows = kPair ? n >> 1 : n, my_row0 = row0 + (kPair ? (int)rank * my_rows : 0);
+        if (kX && P.x_ready && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
+        const auto kloop = [&](auto box_rows) {
+            constexpr int kRows = decltype(box_rows)::value;
+            constexpr uint32_t kXCopy = (uint32_t)(kRows * kBlockK * 2);
+            const CUtensorMap *const map = !kX ? &P.tmB : kRows == 128 ? &P.tmA : kRows == 64 ? &P.tmA64 : &P.tmA32;
+            int kx = 0;
+            for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
+                TL(tl_q = clock64());
+                ok = wait_barrier_1t(empty_bar, phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 10u);
+                if (!ok) break;
+                TL(tl_pw += clock64() - tl_q);
+                // (a probe that leaves a copy out completes its bytes by hand: every producer stays in the
+                // barrier's dependency chain, or the one that arms it could lap the others)
+                if (kX) {
+                    if (kb == 0) ctl->tile_n[it & 7] = (uint32_t)n;
+                    if (!kPair) mbar_arrive_expect_tx(full_bar, (uint32_t)C::kWBytes + kXCopy);
+                    else if (rank == 0) mbar_arrive_expect_tx(full_bar, 2u * ((uint32_t)C::kWBytes + kXCopy));
+                    if (MOE_PROBE(kProbeSkipX)) mbar_complete_tx_cluster(mapa_u32(smem_u32(&ctl->full[stage]), kPair ? 0u : cluster_ctarank()), kXCopy);
+                    else if (kPair) tma_load_2d_pair(dst, map, full_bar, kx, my_row0);
+                    else tma_load_2d(dst, map, full_bar, kx, my_row0);
+                } else if (MOE_PROBE(kProbeSkipAllW2) || (MOE_PROBE(kProbeSkipOddW2) && (kb & 1))) {
+                    mbar_complete_tx_cluster(mapa_u32(smem_u32(&ctl->full[stage]), kPair ? 0u : cluster_ctarank()), (uint32_t)C::kWBytes);
+                } else {
+                    if (kPair) tma_load_3d_pair(dst, map, full_bar, kx, n0, e);
+                    else tma_load_3d_hint(dst, map, full_bar, kx, n0, e, w_policy);
+                }
+                armed |= 1u << stage;
+                dst += (uint32_t)C::kStageBytes;
+                full_bar += 8u;
+                empty_bar += 8u;
+                if (++stage == n_stages) {
+                    stage = 0;
+                    phase ^= 1u;
+                    dst = dst0;
+                    full_bar = full0;
+                    empty_bar = empty0;
+                }
+                if (kb == ahead_at) {
+                    walk.next();
+                    t_next = walk.tile();
+                    if (kX) {
+                        row0_next = ld_chained(&P.mtile_first_row[t_next.mu]);
+                        valid_next = ld_chained(&P.mtile_valid[t_next.mu]);
+                    } else {
+                        e_next = ld_chained(&P.mtile_expert[t_next.mu]);
+                    }
+                }
+            }
+        };
+        if (!kX || my_rows > 64) kloop(std::integral_constant<int, 128>{});
+        else if (kPair || my_rows > 32) kloop(std::integral_constant<int, 64>{});
+        else kloop(std::integral_constant<int, 32>{});
+        t = t_next;
+        e = e_next;
+        row0 = row0_next;
+        valid = valid_next;
+    }
+    TL(if (kX) tl_put(P, kTlProducerWait, (unsigned long long)tl_pw));
+    if (!ok && rank == 0) {
+        // wind-down: let the copies already issued land before shared memory is released
+        // (bounded; a stage consumed meanwhile has completed its phase and passes at once)
+        const unsigned long long drain = globaltimer_ns() + 2000000ull;
+        for (int sidx = 0; sidx < n_stages; ++sidx) {
+            if (!(armed & (1u << sidx))) continue;
+            const uint32_t par = (sidx < stage) ? phase : (phase ^ 1u);
+            while (!mbar_try_wait(smem_u32(&ctl->full[sidx]), par) && globaltimer_ns() < drain) {}
+        }
+    }
+}
+
 // --------------------------------------------------------------------------- compute CTA
 
 // Barriers (thread 0) and TMEM (warp 1) of a compute CTA, before it is known that this CTA computes; a CTA-wide barrier of the
@@ -557,7 +609,7 @@ __device__ __forceinline__ void compute_setup(const FusedParams &P, Control *ctl
     using C = Cfg<TN>;
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < C::kStages; ++i) {
+        for (int i = 0; i < P.stages; ++i) {
             mbar_init(smem_u32(&ctl->full[i]), 1);
             mbar_init(smem_u32(&ctl->empty[i]), 1);
         }
@@ -576,82 +628,20 @@ __device__ __forceinline__ void compute_setup(const FusedParams &P, Control *ctl
 }
 
 template <int TN>
-__device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
+__device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b)
 {
     using C = Cfg<TN>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int total_tiles = P.L * pt.W_comp;
+    const int n_stages = P.stages;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
     const uint32_t tmem_base = ctl->tmem_base;
 
     if (warp == 0 || warp == 2) {
-        // ---------------- TMA producers: warp 0 loads the x_routed tile, warp 2 the W2 tile of every
-        // k-block; both complete on the same full barrier.  One thread per warp runs the whole loop (no
-        // per-iteration warp broadcast); the others park below.
-        const bool load_a = (warp == 0);
+        // ---------------- TMA producers: warp 0 loads the x_routed tile, warp 2 the W2 tile of every k-block
         if (lane == 0 && b < total_tiles) {
-            int stage = 0;
-            uint32_t phase = 0;
-            uint32_t armed = 0;  // bit s: stage s was handed to the TMA unit at least once
-            bool ok = true;
-            uint32_t seen = 0;
-            const unsigned long long w_policy = P.w2_once ? l2_evict_first_policy() : l2_evict_normal_policy();
-            TL_DECL(long long tl_pw = 0, tl_q;)
-            // the m-tile table entries of the NEXT tile are fetched while this tile's k-blocks are issued, so
-            // that the two dependent global loads never stall the stream of copies at a tile boundary
-            Tile t = decode_tile(b, P, pt.W_comp);
-            int e = ld_chained(&P.mtile_expert[t.mu]);
-            int row0 = ld_chained(&P.mtile_first_row[t.mu]);
-            int valid = ld_chained(&P.mtile_valid[t.mu]);
-            for (int g = b; g < total_tiles && ok; g += pt.P) {
-                const Tile t_next = decode_tile(min(g + pt.P, total_tiles - 1), P, pt.W_comp);
-                const int e_next = ld_chained(&P.mtile_expert[t_next.mu]);
-                const int row0_next = ld_chained(&P.mtile_first_row[t_next.mu]);
-                const int valid_next = ld_chained(&P.mtile_valid[t_next.mu]);
-                const int n0 = t.s * P.split_w + t.i_n * TN;
-                // rows come in boxes of kXBoxRows: those past the end of the expert's last tile are not fetched, nothing stored
-                // depends on them
-                const int boxes = min((valid + kXBoxRows - 1) / kXBoxRows, kMmaM / kXBoxRows);
-                if (load_a && P.x_ready && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
-                int kx = 0;
-                for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
-                    TL(tl_q = clock64());
-                    ok = wait_barrier_1t(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 10u);
-                    if (!ok) break;
-                    TL(tl_pw += clock64() - tl_q);
-                    const uint32_t full = smem_u32(&ctl->full[stage]);
-                    const uint32_t a_dst = smem_u32(ring + stage * C::kStageBytes);
-                    const bool skip_b = MOE_PROBE(kProbeSkipAllW2) || (MOE_PROBE(kProbeSkipOddW2) && (kb & 1));
-                    if (load_a) {
-                        mbar_arrive_expect_tx(full, (uint32_t)(boxes * kXBoxRows * kBlockK * 2 + C::kBBytes));
-                        for (int i = 0; i < boxes; ++i)
-                            tma_load_2d(a_dst + (uint32_t)(i * kXBoxRows * kBlockK * 2), &P.tmA, full, kx, row0 + i * kXBoxRows);
-                    } else if (!skip_b) {
-                        tma_load_3d_hint(a_dst + C::kABytes, &P.tmB, full, kx, n0, e, w_policy);
-                    } else {
-                        // a probe that leaves the copy out completes its bytes by hand: this producer stays in
-                        // the barrier's dependency chain, or the other one could lap it
-                        mbar_complete_tx_cluster(mapa_u32(full, cluster_ctarank()), (uint32_t)(C::kStageBytes - C::kABytes));
-                    }
-                    armed |= 1u << stage;
-                    if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
-                }
-                t = t_next;
-                e = e_next;
-                row0 = row0_next;
-                valid = valid_next;
-            }
-            TL(if (load_a) tl_put(P, kTlProducerWait, (unsigned long long)tl_pw));
-            if (!ok) {
-                // wind-down: let the copies already issued land before shared memory is released
-                // (bounded; a stage consumed meanwhile has completed its phase and passes at once)
-                const unsigned long long drain = globaltimer_ns() + 2000000ull;
-                for (int sidx = 0; sidx < C::kStages; ++sidx) {
-                    if (!(armed & (1u << sidx))) continue;
-                    const uint32_t par = (sidx < stage) ? phase : (phase ^ 1u);
-                    while (!mbar_try_wait(smem_u32(&ctl->full[sidx]), par) && globaltimer_ns() < drain) {}
-                }
-            }
+            if (warp == 0) producer_role<TN, false, true>(P, pt, ring, ctl, b, deadline, 0u);
+            else producer_role<TN, false, false>(P, pt, ring, ctl, b, deadline, 0u);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -660,11 +650,11 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
         // compute_cta_pair): a whole k-block (four MMAs and the commit) is one statement with 32-bit descriptor
         // arithmetic, addresses advance by additions, the barrier's first look is the non-suspending test.
         {
-            constexpr uint32_t idesc = make_idesc(kMmaM, TN);
-            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoB = (uint32_t)(C::kABytes >> 4);
+            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoX = (uint32_t)(C::kWBytes >> 4);
+            constexpr uint32_t kLoBlock = (uint32_t)(kMmaM * kBlockK * 2 >> 4);      // the next 128 rows of W2
             const uint32_t lo0 = smem_desc_lo(smem_u32(ring));
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-            uint32_t a_lo = lo0, full_bar = full0, empty_bar = empty0;
+            uint32_t w_lo = lo0, full_bar = full0, empty_bar = empty0;
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
@@ -673,6 +663,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
             for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
                 const int a = it & 1;
                 const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
+                uint32_t idesc = 0;
                 TL(tl_q = clock64());
                 if (!__all_sync(0xffffffffu, mbar_test_wait(smem_u32(&ctl->tmem_empty[a]), acc_phase ^ 1u))) {
                     // (every lane polls; the vote keeps `ok`, and with it the loop, provably warp-uniform)
@@ -681,7 +672,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                 }
                 TL(tl_wt += clock64() - tl_q);
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(a * TN);
+                const uint32_t d_tmem = tmem_base + (uint32_t)(a * C::kAccCols);
                 for (int kb = 0; kb < P.num_kb; ++kb) {
                     TL(tl_q = clock64());
                     if (!__all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) {
@@ -689,27 +680,31 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                         if (!ok) break;
                     }
                     TL(tl_wf += clock64() - tl_q; tl_q = clock64());
+                    if (kb == 0) idesc = make_idesc(kMmaM, tile_n(ctl, it));
                     tc_fence_after();
                     // advancing K by 16 bf16 = 32 bytes inside the swizzle row: +2 in the address field
                     if (elect_one_sync()) {
                         if (kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) {
-                            tc_kblock_bf16(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
+                            if (C::kBlocks == 2)
+                                tc_ksteps_bf16(d_tmem + kMmaM, w_lo + kLoBlock, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u);
+                            tc_kblock_bf16(d_tmem, w_lo, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u, empty_bar);
                         } else {
-                            const uint64_t a_desc = ((uint64_t)kSmemDescHi << 32) | a_lo, b_desc = a_desc + kLoB;
+                            const uint64_t w_desc = ((uint64_t)kSmemDescHi << 32) | w_lo, x_desc = w_desc + kLoX;
                             for (int k = 0; k < P.last_ksteps; ++k)
-                                tc_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                            (k > 0 || kb > 0) ? 1u : 0u);
+                                for (int i = 0; i < C::kBlocks; ++i)
+                                    tc_mma_bf16(d_tmem + (uint32_t)(i * kMmaM), w_desc + (uint64_t)(2 * k + i * (int)kLoBlock), x_desc + (uint64_t)(2 * k),
+                                                idesc, (k > 0 || kb > 0) ? 1u : 0u);
                             tc_commit(empty_bar);   // stage reusable once these MMAs have read it
                         }
                     }
                     TL(tl_is += clock64() - tl_q);
-                    a_lo += kLoStage;
+                    w_lo += kLoStage;
                     full_bar += 8u;
                     empty_bar += 8u;
-                    if (++stage == C::kStages) {
+                    if (++stage == n_stages) {
                         stage = 0;
                         phase ^= 1u;
-                        a_lo = lo0;
+                        w_lo = lo0;
                         full_bar = full0;
                         empty_bar = empty0;
                     }
@@ -725,7 +720,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        epilogue_role<TN, false>(P, pt, ctl, aux, b, tmem_base, deadline, 0);
+        epilogue_role<TN, false>(P, pt, ctl, b, tmem_base, deadline, 0);
     } else if (warp == 3) {
         publisher_role<false>(P, pt, ctl, b, deadline, 0);
     }
@@ -741,24 +736,16 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
 
 // --------------------------------------------------------------------------- compute CTA pair
 //
-// 256 x 256 pair tile: two CTAs of a cluster (two SMs) compute one tile with tcgen05.mma.cta_group::2.
-// CTA `rank` loads its own 128 rows of x_routed and its own 128 of the 256 W2 rows of every k-block
-// (no multicast: each CTA issues its own loads), so a k-block costs 32 KB per SM instead of 48 KB.
+// 256 x 256 pair tile: two CTAs of a cluster (two SMs) compute one tile with tcgen05.mma.cta_group::2, M = 256 columns of the
+// output, N = the tile's rows, rounded up to 32.  CTA `rank` loads its own half of those rows of x_routed and its own 128 of the
+// 256 W2 rows of every k-block (no multicast: each CTA issues its own loads), so a k-block costs 32 KB per SM instead of 48 KB.
 // Rank 0 (the leader) issues the MMAs; tcgen05.commit arrives on the barriers of both CTAs.
 //   full[stage]       only the leader's is used: armed by the leader for the bytes of both CTAs
 //   empty[stage]      one per CTA (its producer waits on it), signalled by the leader's commit
 //   tmem_full[a]      one per CTA (its epilogue waits on it), signalled by the leader's commit
 //   tmem_empty[a]     only the leader's is used: 12 local + 12 remote epilogue warps arrive
-struct PairCfg {
-    static constexpr int kTileN = 256;
-    static constexpr int kABytes = kMmaM * kBlockK * 2;                 // 16 KB: this CTA's 128 rows
-    static constexpr int kBBytes = (kTileN / 2) * kBlockK * 2;          // 16 KB: this CTA's 128 W2 rows
-    static constexpr int kStageBytes = kABytes + kBBytes;               // 32 KB
-    // kStageBytesTotal / kStageBytes = 6 stages; a seventh lies in the aux region when that is free (FusedParams::pair_stages)
-    static constexpr int kTmemCols = 2 * kTileN;                        // two accumulator buffers
-};
 
-__device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, uint8_t *aux, int b)
+__device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b)
 {
     using C = PairCfg;
     constexpr int TN = C::kTileN;
@@ -766,7 +753,7 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
     const uint32_t rank = cluster_ctarank();
     const bool leader_cta = (rank == 0);
     const int total_tiles = P.L * pt.W_comp;
-    const int n_stages = P.pair_stages;   // 6, or 7 with the aux region as one more stage
+    const int n_stages = P.stages;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
 
     if (threadIdx.x == 0) {
@@ -795,67 +782,10 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
 
     if (warp == 0 || warp == 2) {
         // ---------------- TMA producers (both CTAs): warp 0 loads this CTA's x_routed rows, warp 2 its W2
-        // rows; both complete on the leader's full barrier.  Two issuing threads halve the serial issue
-        // latency per k-block.  One thread per warp runs the whole loop; the others park below.
-        const bool load_a = (warp == 0);
+        // rows; both complete on the leader's full barrier.
         if (lane == 0 && b < total_tiles && !MOE_PROBE(kProbeFreeRunMma)) {
-            int stage = 0;
-            uint32_t phase = 0;
-            uint32_t armed = 0;
-            bool ok = true;
-            TL_DECL(long long tl_pw = 0, tl_q;)
-            // next tile's table entries are fetched one tile ahead (see compute_cta)
-            Tile t = decode_tile(b, P, pt.W_comp);
-            int e = ld_chained(&P.mtile_expert[t.mu]);
-            int row0 = ld_chained(&P.mtile_first_row[t.mu]) + (int)rank * kMmaM;
-            uint32_t seen = 0;
-            for (int g = b; g < total_tiles && ok; g += pt.P) {
-                const Tile t_next = decode_tile(min(g + pt.P, total_tiles - 1), P, pt.W_comp);
-                const int e_next = ld_chained(&P.mtile_expert[t_next.mu]);
-                const int row0_next = ld_chained(&P.mtile_first_row[t_next.mu]) + (int)rank * kMmaM;
-                const int n0 = t.s * P.split_w + t.i_n * TN + (int)rank * (TN / 2);
-                if (load_a && P.x_ready) {
-                    const int last = ld_chained(&P.mtile_first_row[t.mu]) + ld_chained(&P.mtile_valid[t.mu]) - 1;
-                    if (!(ok = wait_rows(P, last, seen, ctl, deadline))) break;
-                }
-                int kx = 0;
-                for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
-                    const uint32_t own_full = smem_u32(&ctl->full[stage]);
-                    TL(tl_q = clock64());
-                    ok = wait_barrier_1t(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 10u);
-                    if (!ok) break;
-                    TL(tl_pw += clock64() - tl_q);
-                    const uint32_t leader_full = own_full & 0xFEFFFFFFu;   // same offset in the leader CTA (rank 0)
-                    const uint32_t a_dst = smem_u32(ring + stage * C::kStageBytes);
-                    const bool skip_b = MOE_PROBE(kProbeSkipAllW2) || (MOE_PROBE(kProbeSkipOddW2) && (kb & 1));
-                    // (a probe that leaves a copy out completes its bytes by hand: every producer stays in the
-                    // barrier's dependency chain, or the leader's could lap the others)
-                    if (load_a) {
-                        if (leader_cta) mbar_arrive_expect_tx(own_full, 2u * (uint32_t)C::kStageBytes);
-                        if (!MOE_PROBE(kProbeSkipX)) tma_load_2d_pair(a_dst, &P.tmA, leader_full, kx, row0);
-                        else mbar_complete_tx_cluster(mapa_u32(own_full, 0u), (uint32_t)C::kABytes);
-                    } else if (!skip_b) {
-                        tma_load_3d_pair(a_dst + C::kABytes, &P.tmB, leader_full, kx, n0, e);
-                    } else {
-                        mbar_complete_tx_cluster(mapa_u32(own_full, 0u), (uint32_t)(C::kStageBytes - C::kABytes));
-                    }
-                    armed |= 1u << stage;
-                    if (++stage == n_stages) { stage = 0; phase ^= 1u; }
-                }
-                t = t_next;
-                e = e_next;
-                row0 = row0_next;
-            }
-            TL(if (load_a) tl_put(P, kTlProducerWait, (unsigned long long)tl_pw));
-            if (!ok && leader_cta) {
-                // wind-down: let the copies already issued land before shared memory is released
-                const unsigned long long drain = globaltimer_ns() + 2000000ull;
-                for (int sidx = 0; sidx < n_stages; ++sidx) {
-                    if (!(armed & (1u << sidx))) continue;
-                    const uint32_t par = (sidx < stage) ? phase : (phase ^ 1u);
-                    while (!mbar_try_wait(smem_u32(&ctl->full[sidx]), par) && globaltimer_ns() < drain) {}
-                }
-            }
+            if (warp == 0) producer_role<TN, true, true>(P, pt, ring, ctl, b, deadline, rank);
+            else producer_role<TN, true, false>(P, pt, ring, ctl, b, deadline, rank);
         }
         __syncwarp();
     } else if (warp == 1 && leader_cta) {
@@ -869,11 +799,10 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
         // moved over from ordinary registers, MMA by MMA; with warp-uniform values in warp-uniform control flow
         // and elect.sync around the issue the GEMM phase is 6 % faster.
         {
-            constexpr uint32_t idesc = make_idesc(2 * kMmaM, TN);
-            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoB = (uint32_t)(C::kABytes >> 4);
+            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoX = (uint32_t)(C::kWBytes >> 4);
             const uint32_t lo0 = smem_desc_lo(smem_u32(ring));
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-            uint32_t a_lo = lo0, full_bar = full0, empty_bar = empty0;
+            uint32_t w_lo = lo0, full_bar = full0, empty_bar = empty0;
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
@@ -891,43 +820,54 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
                 TL(tl_wt += clock64() - tl_q);
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(a * TN);
-                for (int kb = 0; kb < P.num_kb; ++kb) {
-                    TL(tl_q = clock64());
-                    if (!MOE_PROBE(kProbeFreeRunMma) && !__all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) {
-                        TL(++tl_late);
-                        ok = __all_sync(0xffffffffu, wait_barrier_1t(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 21u));
+                const auto wait_stage = [&]() {
+                    if (MOE_PROBE(kProbeFreeRunMma) || __all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) return;
+                    TL(++tl_late);
+                    ok = __all_sync(0xffffffffu, wait_barrier_1t(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 21u));
+                };
+                const auto kloop = [&](auto full, uint32_t n) {
+                    const uint32_t idesc = make_idesc(2 * kMmaM, decltype(full)::value ? TN : (int)n);
+                    for (int kb = 0; kb < P.num_kb; ++kb) {
+                        TL(tl_q = clock64());
+                        wait_stage();
                         if (!ok) break;
-                    }
-                    TL(tl_wf += clock64() - tl_q; tl_q = clock64());
-                    tc_fence_after();
-                    if (MOE_PROBE(kProbeSlowIssuer)) {   // 200 cycles in which nothing is issued
-                        const long long until = clock64() + 200;
-                        while (clock64() < until) {}
-                    }
-                    if (elect_one_sync()) {
-                        if ((kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) && !MOE_PROBE(kProbeFreeRunMma)) {
-                            tc_kblock_bf16_pair(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
-                        } else {
-                            const uint64_t a_desc = ((uint64_t)kSmemDescHi << 32) | a_lo, b_desc = a_desc + kLoB;
-                            const int ksteps = (kb == P.num_kb - 1) ? P.last_ksteps : (kBlockK / kUmmaK);
-                            for (int k = 0; k < ksteps; ++k)
-                                tc_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                                 (k > 0 || kb > 0) ? 1u : 0u);
-                            if (!MOE_PROBE(kProbeFreeRunMma)) tc_commit_pair(empty_bar);      // both CTAs may refill the stage
+                        TL(tl_wf += clock64() - tl_q; tl_q = clock64());
+                        tc_fence_after();
+                        if (MOE_PROBE(kProbeSlowIssuer)) {   // 200 cycles in which nothing is issued
+                            const long long until = clock64() + 200;
+                            while (clock64() < until) {}
+                        }
+                        if (elect_one_sync()) {
+                            if ((kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) && !MOE_PROBE(kProbeFreeRunMma)) {
+                                tc_kblock_bf16_pair(d_tmem, w_lo, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u, empty_bar);
+                            } else {
+                                const uint64_t w_desc = ((uint64_t)kSmemDescHi << 32) | w_lo, x_desc = w_desc + kLoX;
+                                const int ksteps = (kb == P.num_kb - 1) ? P.last_ksteps : (kBlockK / kUmmaK);
+                                for (int k = 0; k < ksteps; ++k)
+                                    tc_mma_bf16_pair(d_tmem, w_desc + (uint64_t)(2 * k), x_desc + (uint64_t)(2 * k), idesc,
+                                                     (k > 0 || kb > 0) ? 1u : 0u);
+                                if (!MOE_PROBE(kProbeFreeRunMma)) tc_commit_pair(empty_bar);      // both CTAs may refill the stage
+                            }
+                        }
+                        TL(tl_is += clock64() - tl_q);
+                        w_lo += kLoStage;
+                        full_bar += 8u;
+                        empty_bar += 8u;
+                        if (++stage == n_stages) {
+                            stage = 0;
+                            phase ^= 1u;
+                            w_lo = lo0;
+                            full_bar = full0;
+                            empty_bar = empty0;
                         }
                     }
-                    TL(tl_is += clock64() - tl_q);
-                    a_lo += kLoStage;
-                    full_bar += 8u;
-                    empty_bar += 8u;
-                    if (++stage == n_stages) {
-                        stage = 0;
-                        phase ^= 1u;
-                        a_lo = lo0;
-                        full_bar = full0;
-                        empty_bar = empty0;
-                    }
-                }
+                };
+                // full tiles in a loop of their own: with a constant N the issuer needs 27 cycles a k-block less
+                wait_stage();
+                if (!ok) break;
+                const uint32_t n = MOE_PROBE(kProbeFreeRunMma) ? 256u : ctl->tile_n[it & 7];
+                if (__all_sync(0xffffffffu, n == (uint32_t)TN)) kloop(std::true_type{}, 0u);
+                else kloop(std::false_type{}, __reduce_max_sync(0xffffffffu, n));
                 __syncwarp();
                 if (ok && elect_one_sync()) tc_commit_pair(smem_u32(&ctl->tmem_full[a]));   // both epilogues may start
                 TL(if (it == 0 && lane == 0) tl_put(P, kTlFirstAcc, globaltimer_ns()));
@@ -940,7 +880,7 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        epilogue_role<TN, true>(P, pt, ctl, aux, b, tmem_base, deadline, (int)rank);
+        epilogue_role<TN, true>(P, pt, ctl, b, tmem_base, deadline, (int)rank);
     } else if (warp == 3) {
         publisher_role<true>(P, pt, ctl, b, deadline, (int)rank);
     }
@@ -1067,15 +1007,13 @@ constexpr int kCommWarps = 12;
 constexpr int kCommUnitBytes = 8192;
 constexpr int kCommWarpBytes = 2 * kCommUnitBytes;
 static_assert(kCommWarps * kCommWarpBytes <= kStageBytesTotal, "communication stages exceed the ring");
-// Co-resident communication warps live in the aux region, which the epilogue leaves alone when it
-// stores straight from registers: two warps' stages (32 KB), then the per-row weights in compact
+// Co-resident communication warps live in the aux region: two warps' stages (32 KB), then the per-row weights in compact
 // 16-float slots -- four for co-resident warps, twelve for the CTA's own warps once they turn to
 // communication (their usual 256-float slots would overlap the co-resident stages).  Needs k_tot <= 16.
 constexpr int kCoWarpsAux = 2;          // co-resident warps whose stages fit the aux region
 constexpr int kCoWeightFloats = 16;
 constexpr int kCoWeightsOffset = kCoWarpsAux * kCommWarpBytes;
-static_assert(PairCfg::kStageBytes + ((sizeof(Control) + 127) & ~(size_t)127) <= kAuxBytes + ((sizeof(Control) + 127) & ~(size_t)127) &&
-              12 * 256 * 4 <= PairCfg::kStageBytes, "a seventh pair stage plus the control block exceed the allocation");
+static_assert(PairCfg::kStageBytes <= kAuxBytes && 12 * 256 * 4 <= PairCfg::kStageBytes, "a seventh pair stage exceeds the allocation");
 static_assert(kCoWeightsOffset + (kCoWarpsMax + kCommWarps) * kCoWeightFloats * 4 <= kAuxBytes,
               "co-resident stages and weights exceed the aux region");
 
@@ -1143,10 +1081,11 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
             if (done >= (uint32_t)(pt.W_comp * P.flag_parts)) {
                 ready_mask |= 1u << u.s;
             } else {
-                // per tile: every (slot j, n-tile under this slab)
-                const int cs0 = u.slab << P.slab_shift;
-                const int in0 = cs0 / TN;
-                const int nt = (cs0 + u.ucols - 1) / TN - in0 + 1;
+                // per tile: every (slot j, n-tile under this slab); a pair tile is published in two parts, one per CTA: its
+                // column halves
+                const int cs0 = u.slab << P.slab_shift, flag_cols = P.flag_parts == 2 ? TN / 2 : TN;
+                const int in0 = cs0 / flag_cols;
+                const int nt = (cs0 + u.ucols - 1) / flag_cols - in0 + 1;
                 bool failed = false;
                 for (int chk = lane; chk < P.k_tot * nt && !failed; chk += 32) {
                     const int j = chk / nt;
@@ -1154,9 +1093,7 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
                     const int row = ld_chained(&P.pad_row[(size_t)u.t * P.k_tot + j]);
                     if (row < 0 || row >= P.R_pad) continue;
                     const int mu = row / P.tile_m;
-                    // a pair tile is published in two parts, one per CTA: the row's part is its 128-row half
-                    const int part = (P.flag_parts == 2) ? ((row - mu * P.tile_m) >> 7) : 0;
-                    const int g = (u.s * pt.W_comp + mu * P.NTs + in0 + tn) * P.flag_parts + part;
+                    const int g = (u.s * pt.W_comp + mu * P.NTs) * P.flag_parts + in0 + tn;
                     uint32_t spins = 0;
                     TL_DECL(const unsigned long long tl_f0 = globaltimer_ns();)
                     while (ld_acquire_u32(&P.flags[g]) != P.epoch) {
@@ -1505,8 +1442,7 @@ __device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &p
     }
 }
 
-// Co-resident communication warp `cw` of a compute CTA: stages and weights in the aux region (free when
-// the epilogue stores straight from registers, which the host checks before it asks for such warps).
+// Co-resident communication warp `cw` of a compute CTA: stages and weights in the aux region.
 template <int TN>
 __device__ __forceinline__ void co_resident_warp(const FusedParams &P, const Part &pt, Control *ctl, uint8_t *aux, int cw)
 {
@@ -1546,10 +1482,11 @@ __device__ __forceinline__ void init_comm_barriers(Control *ctl)
 // routing build and this launch.
 __device__ __forceinline__ Part launch_part(const FusedParams &P)
 {
-    Part pt = {P.W_comp, P.C, P.P};
+    Part pt = {P.W_comp, P.S, P.C, P.P};
     if (P.S_dev) {
         const int S = ld_chained_uniform(P.S_dev);
-        pt.W_comp = min(S, P.S) * P.NTs;
+        pt.S = min(S, P.S);
+        pt.W_comp = pt.S * P.NTs;
         if (P.c_table_n > 0) {
             pt.C = P.c_table[max(0, min(S - P.c_table_first, P.c_table_n - 1))];
             pt.P = (P.G - pt.C) / P.slot_sms;
@@ -1609,7 +1546,7 @@ moe_gemm2_combine_kernel(const __grid_constant__ FusedParams P)
         if (co_warp_number(warp) < P.co_warps) co_resident_warp<TN>(P, pt, ctl, aux, co_warp_number(warp));
         return;
     } else {
-        compute_cta<TN>(P, pt, ring, ctl, aux, (int)blockIdx.x - pt.C);
+        compute_cta<TN>(P, pt, ring, ctl, (int)blockIdx.x - pt.C);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         // out of GEMM tiles: help with the communication that is left (all TMA and TMEM traffic is over)
         if (queued && !ctl->abort) comm_cta<TN>(P, pt, ring, ctl, aux, kRoleBack);
@@ -1625,11 +1562,10 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    // Layout: six operand stages, the control block, the aux region -- or, when nothing needs the aux region
-    // while the GEMM runs (256-bit epilogue stores, no co-resident communication warp), seven stages and the
-    // control block; the seventh stage then serves as the aux region of the communication role, which only
-    // starts after the CTA's last MMA (drain help) or never computes (communication CTA).
-    const bool seven = (P.pair_stages == 7);
+    // Layout: six operand stages, the control block, the aux region -- or, when no co-resident communication warp needs the aux region
+    // while the GEMM runs, seven stages and the control block; the seventh stage then serves as the aux region of the
+    // communication role, which only starts after the CTA's last MMA (drain help) or never computes (communication CTA).
+    const bool seven = P.stages == 7;
     Control *ctl = reinterpret_cast<Control *>(ring + kStageBytesTotal + (seven ? PairCfg::kStageBytes : 0));
     uint8_t *aux = seven ? ring + kStageBytesTotal
                          : reinterpret_cast<uint8_t *>(ring + kStageBytesTotal + ((sizeof(Control) + 127) & ~(size_t)127));
@@ -1669,7 +1605,7 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
         cluster_wait();
         return;
     } else {
-        compute_cta_pair(P, pt, ring, ctl, aux, ((int)blockIdx.x - c_even) >> 1);
+        compute_cta_pair(P, pt, ring, ctl, ((int)blockIdx.x - c_even) >> 1);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         if (queued && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack);
     }
@@ -1683,6 +1619,10 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
 }  // namespace
 
 int fused_co_warps_max() { return kCoWarpsAux; }
+int fused_stages(bool pair, int tile_n, bool aux_free)
+{
+    return pair ? kStageBytesTotal / PairCfg::kStageBytes + (aux_free ? 1 : 0) : tile_n == 64 ? Cfg<64>::kStages : tile_n == 128 ? Cfg<128>::kStages : Cfg<256>::kStages;
+}
 bool fused_timeline_build() { return MOE_TIMELINE != 0; }
 
 size_t fused_smem_bytes(int) { return (size_t)kStageBytesTotal + 1024 + ((sizeof(Control) + 127) & ~(size_t)127) + kAuxBytes; }

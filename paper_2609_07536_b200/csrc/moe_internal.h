@@ -19,7 +19,6 @@ constexpr int kFusedThreads = kThreads + 32 * kCoWarpsMax;   // block size of th
 constexpr int kBlockK = 64;            // bf16 elements per k-block: one 128-byte swizzle row
 constexpr int kUmmaK = 16;             // K of one tcgen05.mma.kind::f16 instruction
 constexpr int kMmaM = 128;             // M of the MMA (tile_m = 64 stores the first 64 rows only)
-constexpr int kXBoxRows = 32;          // rows of one x_routed box of a one-CTA tile of the fused kernel
 constexpr int kStageBytesTotal = 192 * 1024;  // operand ring, all stages together
 constexpr int kCommTileM = 32;         // T_M^comm: the piece in which the selector counts communication work (a CTA's units are 8 KB)
 constexpr int kCommTileN = 1024;       // T_N^comm
@@ -45,7 +44,7 @@ constexpr int kInlineMaxR = 2048;      // assignments up to which a kernel build
 // Parameters of one fused launch.  Passed by value (__grid_constant__): the two tensor maps
 // must sit in kernel parameter space, 64-byte aligned.
 struct alignas(64) FusedParams {
-    CUtensorMap tmA;   // x_routed [R, I]      box 64 x 32 rows (one-CTA tiles) or 128 (pair), 128B swizzle
+    CUtensorMap tmA, tmA64, tmA32;   // x_routed [R, I]   boxes 64 x 128, 64 and (one-CTA tiles) 32 rows, 128B swizzle
     CUtensorMap tmB;   // W2 [E_tot, H, I]     box 64 x tile_n rows (a pair's CTA: half of them) x 1, 128B swizzle
     const int32_t *mtile_expert;
     const int32_t *mtile_first_row;
@@ -77,6 +76,7 @@ struct alignas(64) FusedParams {
     int32_t c_table_first, c_table_n;   // c_table[i]: communication CTAs when S = c_table_first + i (0 entries: C and P above hold)
     uint8_t c_table[kPlanTableMax];
     int32_t tok_blk, comm_cols;
+    uint32_t token_mul, token_shift;    // see token_of
     int32_t even;                       // the communication work is dealt evenly to all warps once all tiles are done (no per-tile
                                         // flags, no queue)
     int32_t balance;                    // (even) P counts all compute slots; the kernel divides them by whole waves of its tiles
@@ -85,14 +85,13 @@ struct alignas(64) FusedParams {
     int32_t num_kb, last_ksteps;
     int32_t drain_help;                 // compute CTAs serve communication tiles once their GEMM tiles are done
     int32_t co_warps;                   // co-resident communication warps per compute CTA (0..2)
-    int32_t pair_stages;                // operand stages of the CTA-pair kernel: 6, or 7 when the aux region of shared memory is
-                                        // free during the GEMM (256-bit epilogue stores, no co-resident warp)
+    int32_t stages;                     // operand stages of a compute CTA: as many as fit the ring; a pair's has one more where the aux
+                                        // region of shared memory is free during the GEMM (no co-resident warp)
     int32_t epi_warps;                  // epilogue warps of a compute CTA: 12 (warps 4-15), or 16 (warps 4-19) when no
-                                        // co-resident warp is asked for and the epilogue needs no staging buffer
+                                        // co-resident warp is asked for
     int32_t tile_order;                 // 0: split-major tile sequence (the paper's); 1: m-tile-major across splits
     int32_t flag_parts;                 // readiness flags per tile: 1, or 2 for a CTA-pair tile
     int32_t slab_cols, slab_shift;      // slab_cols = 1 << slab_shift; a unit is k_tot rows of a slab
-    int32_t wide_store;                 // every 16-column group of a Y row is whole and 32-byte aligned: 256-bit epilogue stores
     uint32_t epoch;
 };
 
@@ -233,6 +232,7 @@ size_t fused_smem_bytes(int tile_n);
 cudaError_t fused_occupancy(int tile_n, int *blocks_per_sm);
 cudaError_t fused_launch(int tile_n, const FusedParams &p, int grid, cudaStream_t stream);
 int fused_co_warps_max();
+int fused_stages(bool pair, int tile_n, bool aux_free);   // operand stages of a compute CTA; aux_free: no co-resident warps
 bool fused_timeline_build();   // the library was compiled with -DMOE_TIMELINE=1   // co-resident communication warps a compute CTA has shared memory for
 // CTA-pair kernel (256 x 256 tiles, clusters of two)
 cudaError_t pair_occupancy(int *blocks_per_sm, int *max_clusters);

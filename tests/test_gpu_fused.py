@@ -271,6 +271,24 @@ def test_ep_concat_invariance_and_tp_within_tolerance():
         assert np.max(np.abs(got - expect)) <= G.tolerance(expect), TP
 
 
+@pytest.mark.parametrize("tile", [(64, 64), (128, 128), (128, 256), (256, 256)])
+@pytest.mark.parametrize("H,L", [(328, 1), (272, 2)])
+def test_row_counts_at_the_edges_of_a_tile(tile, H, L):
+    # an expert per row count: N of the MMA is the tile's rows rounded up (16, a pair 32), its copies are boxes of 32, 64 or 128 rows, the
+    # epilogue takes 32 rows at a time; columns that end inside a 128-column block and inside its quarters
+    counts = [1, 15, 16, 17, 31, 32, 33, 47, 64, 65, 96, 97, 127, 128, 129, 159, 160, 161, 192, 193, 224, 255, 256, 257, 300]
+    w = replace(wl.TINY, name="rows", T=sum(counts), H=H, I=80, E=len(counts), k=1, TP=1, EP=3, L=L, tile_m=tile[0], tile_n=tile[1])
+    rng = np.random.default_rng(5)
+    idx = rng.permutation(np.repeat(np.arange(len(counts)), counts)).astype(np.int32)[:, None]
+    wt = rng.random((w.T, 1)).astype(np.float32)
+    x, W2 = wl.make_data(w)
+    expect, _ = _oracle_tokens(w, idx, wt, x, W2)
+    for kw in ({"drain_help": 1}, {"drain_help": 0, "force_C": 5}):
+        outs, plan, ws, S, st = G.run_layer(w, idx, wt, x, W2, **kw)
+        got = np.concatenate([o[:len(G.tokens_of_rank(w.T, w.EP, d))] for d, o in enumerate(outs)])
+        assert st.code == 0 and np.max(np.abs(got - expect)) <= G.tolerance(expect)
+
+
 @pytest.mark.parametrize("tile", [(64, 64), (128, 256), (256, 256)])
 @pytest.mark.parametrize("drain_help", [0, 1])
 def test_shards_are_summed_in_the_accumulator(tile, drain_help):
