@@ -32,7 +32,9 @@ int32_t require_handle_device(moe_handle *h, const char *who)
     return MOE_OK;
 }
 
-const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name)
+// The table's entry for these arguments, encoded if it is another one's.
+static const CUtensorMap *cached_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, int rank,
+                                     const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, const char *name)
 {
     if (!h->maps && !(h->maps = new (std::nothrow) MapEntry[kMapEntries]())) return nullptr;
     const uint64_t mixed = ((reinterpret_cast<uintptr_t>(ptr) >> 8) + (uint64_t)box_rows) * 0x9E3779B97F4A7C15ull;
@@ -42,12 +44,10 @@ const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, i
     typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                       const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                       CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
-    const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * (cuuint64_t)rows};
-    const cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)box_rows, 1}, es[3] = {1, 1, 1};
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     m.ptr = nullptr;
     const CUresult cr = reinterpret_cast<EncodeTiledFn>(h->encode_tiled)(
-        &m.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, planes ? 3 : 2, const_cast<void *>(ptr), dims, strides, box, es,
+        &m.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(ptr), dims, strides, box, es,
         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) {
         snprintf(h->err, sizeof h->err, "cuTensorMapEncodeTiled(%s) failed: %d", name, (int)cr);
@@ -59,6 +59,23 @@ const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, i
     m.box_rows = box_rows;
     m.ptr = ptr;
     return &m.map;
+}
+
+const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name)
+{
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+    const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * (cuuint64_t)rows};
+    const cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)box_rows, 1};
+    return cached_map(h, ptr, planes, rows, cols, box_rows, planes ? 3 : 2, dims, strides, box, name);
+}
+
+const CUtensorMap *gate_up_map(moe_handle *h, const void *ptr, int32_t experts, int32_t inter, int32_t cols, int32_t box_inter, const char *name)
+{
+    const cuuint64_t row = (cuuint64_t)cols * 2, plane = row * (cuuint64_t)inter;
+    const cuuint64_t dims[5] = {(cuuint64_t)cols, 16, 2, (cuuint64_t)inter / 16, (cuuint64_t)experts};
+    const cuuint64_t strides[4] = {row, plane, 16 * row, 2 * plane};
+    const cuuint32_t box[5] = {(cuuint32_t)kBlockK, 16, 2, (cuuint32_t)box_inter / 16, 1};
+    return cached_map(h, ptr, -experts, inter, cols, box_inter, 5, dims, strides, box, name);
 }
 
 namespace {

@@ -12,27 +12,31 @@
 // shape, T = 4096: 120 -> 98 us).  (One TMA tile::gather4 copy per four rows does not keep up: 80 cycles each on an SM, 3660 us
 // for the stage.)  Rows past the end
 // of an expert's last tile are not fetched at all: nothing stored depends on them.
-//   tile_m <= 128: tile = 128 routed rows x 128 intermediate columns per CTA, four 48 KB stages;
-//   tile_m = 256 : tile = 256 rows x 128 columns per pair of CTAs (tcgen05 cta_group::2), seven 32 KB stages: CTA 0
-//                  holds rows 0..127 and loads the gate rows of W1, CTA 1 rows 128..255 and the up rows, so that a
-//                  k-block costs an SM 32 KB instead of 48.
-//   warp 0      TMA producer (one thread): the expert's 128 gate rows and 128 up rows of W1 for the same columns (64 k),
-//               which form one 256-row B operand;
+// The weights are on the M side of the MMA, the rows on its N side, as in the fused kernel: N is the tile's row count rounded up to 16
+// (a pair: 32), so that a tile costs what its rows cost.  The rows of W1 come in groups of 32, 16 gate rows and the 16 up rows of the
+// same columns: then the gate and the up projection of an output lie in one TMEM lane quarter, 16 lanes apart, and the 16-lane loads of
+// the epilogue put them into the same register of the same thread.
+// (Rows on the M side, every tile computed for 128 or 256 of them -> now, whole layer, us: DeepSeek shape T = 1 40.4 -> 39.0,
+// Qwen shape T = 48 179 -> 165, Granite shape T = 1003 84.3 -> 82.1, DeepSeek shape T = 16384, 6 % padding, 2106 -> 2091; same bits.)
+//   tile_m <= 128: tile = up to 128 routed rows x 128 intermediate columns per CTA (two MMAs of 64), four 48 KB stages;
+//   tile_m = 256 : tile = up to 256 rows x 128 columns per pair of CTAs (tcgen05 cta_group::2), seven 32 KB stages: each CTA
+//                  holds half of the rows and loads the gate and up rows of 64 columns, so that a k-block costs an SM 32 KB
+//                  instead of 48.
+//   warp 0      TMA producer (one thread): the expert's rows of W1 for the tile's columns (64 k), one copy;
 //   warps 12-15 loaders of the gathered rows; their copies arrive by themselves on the stage's `rows` barrier;
 //   warp 2      relay (one thread): waits for that barrier, makes the rows visible to the tensor core's proxy and
 //               arrives on the stage's full barrier (a fence in the issuing warp would cost every k-block its cycles).  Pair: the
 //               other CTA's relay arrives on the leader's barrier;
-//   warp 1      issues tcgen05.mma (converged warp, elected lane; N = 256, K = 16, bf16 -> fp32): accumulator
-//               columns 0..127 are the gate projection, 128..255 the up projection of the same outputs;
-//               two accumulator buffers in TMEM;
-//   warps 4-11  epilogue: tcgen05.ld of 16 gate and the matching 16 up columns, silu(g) * u in fp32,
-//               bf16, one 32-byte store per row (x_routed rows are contiguous: no scatter here).
+//   warp 1      issues tcgen05.mma (converged warp, elected lane; K = 16, bf16 -> fp32) into one of two accumulator buffers in TMEM;
+//   warps 4-11  epilogue: tcgen05.ld of the gate and the up values of 16 columns x 32 rows, silu(g) * u in fp32,
+//               bf16, transposed, one 32-byte store per row (x_routed rows are contiguous: no scatter here).
 // The n-tile index runs fastest in the tile sequence, so the CTAs of a wave share the gathered rows.
 // Every wait is bounded like in the fused kernel (status word, no trap).
 
 #include <cuda_bf16.h>
 
 #include <cstring>
+#include <type_traits>
 
 #include "moe_internal.h"
 #include "routing_device.cuh"
@@ -50,17 +54,19 @@ constexpr int kG1MaxStages = 7;
 // TN: intermediate columns per tile (a pair: 128)
 template <bool kPair, int TN>
 struct G1Cfg {
-    static constexpr int kABytes = kMmaM * kBlockK * 2;                              // 16 KB: this CTA's 128 rows
-    static constexpr int kBBytes = (kPair ? 1 : 2) * TN * kBlockK * 2;         // gate and up rows, or one of them
-    static constexpr int kStageBytes = kABytes + kBBytes;
+    static constexpr int kCols = kPair ? TN / 2 : TN;                                // intermediate columns whose weights this CTA loads
+    static constexpr int kWBytes = 2 * kCols * kBlockK * 2;                          // their gate and up rows
+    static constexpr int kXBytes = kMmaM * kBlockK * 2;                              // 16 KB: up to 128 rows of the hidden states
+    static constexpr int kStageBytes = kWBytes + kXBytes;                            // (TN = 96: the second MMA reads 64 rows past the weights, for lanes nobody reads)
     static constexpr int kStages = kPair || TN == 64 ? kG1MaxStages : TN == 96 ? 5 : 4;
-    static constexpr int kAccCols = TN == 64 ? 128 : 256;                            // columns from one accumulator to the next (2 TN used)
+    static constexpr int kBlocks = kPair || TN == 64 ? 1 : 2;                        // MMAs per K = 16, of 64 intermediate columns (a pair: 128)
+    static constexpr int kAccCols = kPair ? 2 * kMmaM : kBlocks * kMmaM;             // TMEM columns of an accumulator buffer
     static constexpr int kTmemCols = 2 * kAccCols;
     static constexpr int kRingBytes = kStages * kStageBytes;
 };
 
 struct alignas(64) G1Params {
-    CUtensorMap tmB;   // W1 as [E_tot * 2, I, H]    box 64 x tile columns (128, 96 or 64) x 1 plane
+    CUtensorMap tmW;   // W1 [E_tot][2][I][H] as [E_tot][I / 16][2][16][H]    box: a CTA's columns / 16 groups of 32 rows x 64
     const int32_t *mtile_expert;
     const int32_t *mtile_first_row;
     const int32_t *mtile_valid;
@@ -90,7 +96,9 @@ struct G1Control {
     unsigned long long tmem_empty[2];
     uint32_t tmem_base;
     volatile uint32_t abort;
+    volatile uint32_t tile_n[8];              // N of a tile's MMAs (tile number mod 8), from the W1 producer to the MMA issuer
 };
+static_assert(kG1MaxStages < 8, "a place in tile_n may be written again while its tile is still to be issued");
 
 template <bool kCluster = false>   // kCluster: what the other CTA of the pair released
 __device__ __forceinline__ bool g1_wait(uint32_t bar, uint32_t parity, G1Control *ctl, unsigned long long deadline,
@@ -135,16 +143,18 @@ __device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
     t.n0 = (g - mu * P.NT) * TN;
     return t;
 }
-// rows of the m-tile that CTA `rank` of a pair holds
-__device__ __forceinline__ int g1_rows_of(int valid, uint32_t rank) { return max(0, min(kMmaM, valid - (int)rank * kMmaM)); }
-// flat assignments of the rows this loader thread copies (step i of the stage: row 16 i + `first`)
+// N of a tile's MMAs: its rows, rounded up to what the instruction takes (M = 128: 16, M = 256 over a pair: 32)
+template <bool kPair>
+__device__ __forceinline__ int g1_mma_n(int valid) { return kPair ? (valid + 31) & ~31 : (valid + 15) & ~15; }
+// flat assignments of the rows this loader thread copies (step i of the stage: row 16 i + `first` of this CTA's)
+template <bool kPair>
 __device__ __forceinline__ void g1_load_perm(const G1Params &P, const G1Tile &t, uint32_t rank, int first, int (&f)[kMmaM / kG1RowsPerStep])
 {
-    const int rows = g1_rows_of(t.valid, rank);
+    const int held = kPair ? g1_mma_n<kPair>(t.valid) >> 1 : kMmaM, row0 = (int)rank * held, rows = min(held, t.valid - row0);
 #pragma unroll
     for (int i = 0; i < kMmaM / kG1RowsPerStep; ++i) {
         const int r = kG1RowsPerStep * i + first;
-        f[i] = r < rows ? ld_chained(&P.perm[t.row0 + (int)rank * kMmaM + r]) : -1;
+        f[i] = r < rows ? ld_chained(&P.perm[t.row0 + row0 + r]) : -1;
     }
 }
 
@@ -177,7 +187,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         ctl->abort = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        prefetch_tensormap(&P.tmB);
+        prefetch_tensormap(&P.tmW);
     }
     if (warp == 1) {
         if (kPair) tmem_alloc_pair(smem_u32(&ctl->tmem_base), C::kTmemCols);
@@ -214,21 +224,21 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             bool ok = true;
             const unsigned long long w_policy = P.w1_once ? l2_evict_first_policy() : l2_evict_normal_policy();
             G1Tile t = g1_decode<TN>(b, P);
-            for (int g = b; g < total_tiles && ok; g += stride) {
+            int it = 0;
+            for (int g = b; g < total_tiles && ok; g += stride, ++it) {
                 const G1Tile t_next = g1_decode<TN>(min(g + stride, total_tiles - 1), P);   // fetched one tile ahead
+                const int group = t.n0 / 16 + (kPair ? (int)rank * (TN / 32) : 0);
                 int kx = 0;
                 for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
                     ok = g1_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 50u);
                     if (!ok) break;
                     const uint32_t own_full = smem_u32(&ctl->full[stage]);
-                    const uint32_t b_dst = smem_u32(ring + stage * C::kStageBytes) + C::kABytes;
-                    if (rank == 0) mbar_arrive_expect_tx(own_full, (kPair ? 2u : 1u) * (uint32_t)C::kBBytes);
-                    if (kPair) {   // gate rows, or up rows; the barrier lies at the same offset in the leader CTA (rank 0)
-                        tma_load_3d_pair(b_dst, &P.tmB, own_full & 0xFEFFFFFFu, kx, t.n0, 2 * t.e + (int)rank);
-                    } else {
-                        tma_load_3d_hint(b_dst, &P.tmB, own_full, kx, t.n0, 2 * t.e, w_policy);                       // gate rows
-                        tma_load_3d_hint(b_dst + C::kBBytes / 2, &P.tmB, own_full, kx, t.n0, 2 * t.e + 1, w_policy);  // up rows
-                    }
+                    const uint32_t w_dst = smem_u32(ring + stage * C::kStageBytes);
+                    if (kb == 0 && rank == 0) ctl->tile_n[it & 7] = (uint32_t)g1_mma_n<kPair>(t.valid);
+                    if (rank == 0) mbar_arrive_expect_tx(own_full, (kPair ? 2u : 1u) * (uint32_t)C::kWBytes);
+                    // (pair: the barrier lies at the same offset in the leader CTA, rank 0)
+                    if (kPair) tma_load_5d_pair(w_dst, &P.tmW, own_full & 0xFEFFFFFFu, kx, 0, 0, group, t.e);
+                    else tma_load_5d_hint(w_dst, &P.tmW, own_full, kx, 0, 0, group, t.e, w_policy);
                     armed |= 1u << stage;
                     if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
                 }
@@ -284,7 +294,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             G1Tile t_next = g1_decode<TN>(min(b + stride, total_tiles - 1), P);
             int f_next[kSteps];
             const __nv_bfloat16 *src[kSteps], *src_next[kSteps];
-            g1_load_perm(P, g1_decode<TN>(b, P), rank, first, f_next);
+            g1_load_perm<kPair>(P, g1_decode<TN>(b, P), rank, first, f_next);
             rows_of(f_next, src);
             for (int g = b; g < total_tiles && ok; g += stride) {
                 // Fetched ahead: the table entries two tiles, the rows' assignments one tile; their addresses (a division each) are
@@ -293,7 +303,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                 // divisions at the head of the tile and a test per row in every k-block the stage took 1270 us at the DeepSeek
                 // shape T = 16384, now 1177 (20 more instructions a k-block for something else: 1400).
                 const G1Tile t_nn = g1_decode<TN>(min(g + 2 * stride, total_tiles - 1), P);
-                g1_load_perm(P, t_next, rank, first, f_next);
+                g1_load_perm<kPair>(P, t_next, rank, first, f_next);
                 bool whole = true;               // the tile has all rows of this warp
 #pragma unroll
                 for (int i = 0; i < kSteps; ++i) whole = whole && src[i] != nullptr;
@@ -304,7 +314,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                     if (!mbar_test_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u))
                         ok = g1_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 55u);
                     if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                    const uint32_t dst = smem_u32(ring + stage * C::kStageBytes) + dst0;
+                    const uint32_t dst = smem_u32(ring + stage * C::kStageBytes) + (uint32_t)C::kWBytes + dst0;
                     if (left > 0) {              // (past the last column: no MMA reads it)
                         if (whole) {
 #pragma unroll
@@ -333,11 +343,12 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         // operand and MMA, a whole k-block (four MMAs and the commit) is one statement with 32-bit descriptor
         // arithmetic, addresses advance by additions, the barrier's first look is the non-suspending test.
         {
-            constexpr uint32_t idesc = make_idesc(kPair ? 2 * kMmaM : kMmaM, 2 * TN);
-            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoB = (uint32_t)(C::kABytes >> 4);
+            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoX = (uint32_t)(C::kWBytes >> 4);
+            constexpr uint32_t kLoBlock = (uint32_t)(kMmaM * kBlockK * 2 >> 4);      // the next 128 rows of W1: 64 columns
+            constexpr int kFullN = kPair ? 2 * kMmaM : kMmaM;
             const uint32_t lo0 = smem_desc_lo(smem_u32(ring));
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-            uint32_t a_lo = lo0, full_bar = full0, empty_bar = empty0;
+            uint32_t w_lo = lo0, full_bar = full0, empty_bar = empty0;
             int stage = 0, it = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -351,38 +362,54 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
                 }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(a * C::kAccCols);
-                for (int kb = 0; kb < P.num_kb; ++kb) {
-                    if (!__all_sync(0xffffffffu, kPair ? mbar_test_wait_cluster(full_bar, phase) : mbar_test_wait(full_bar, phase))) {
-                        ok = __all_sync(0xffffffffu, g1_wait<kPair>(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 52u));
+                const auto wait_stage = [&]() {
+                    if (__all_sync(0xffffffffu, kPair ? mbar_test_wait_cluster(full_bar, phase) : mbar_test_wait(full_bar, phase))) return;
+                    ok = __all_sync(0xffffffffu, g1_wait<kPair>(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 52u));
+                };
+                const auto kloop = [&](auto full, uint32_t n) {
+                    const uint32_t idesc = make_idesc(kPair ? 2 * kMmaM : kMmaM, decltype(full)::value ? kFullN : (int)n);
+                    for (int kb = 0; kb < P.num_kb; ++kb) {
+                        wait_stage();
                         if (!ok) break;
-                    }
-                    tc_fence_after();
-                    if (elect_one_sync()) {
-                        if (kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) {
-                            if (kPair) tc_kblock_bf16_pair(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
-                            else tc_kblock_bf16(d_tmem, a_lo, a_lo + kLoB, idesc, kb > 0 ? 1u : 0u, empty_bar);
-                        } else {
-                            const uint64_t a_desc = ((uint64_t)kSmemDescHi << 32) | a_lo, b_desc = a_desc + kLoB;
-                            for (int k = 0; k < P.last_ksteps; ++k) {
-                                const uint32_t acc = (k > 0 || kb > 0) ? 1u : 0u;
-                                if (kPair) tc_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
-                                else tc_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
+                        tc_fence_after();
+                        if (elect_one_sync()) {
+                            if (kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) {
+                                if (C::kBlocks == 2) tc_ksteps_bf16(d_tmem + kMmaM, w_lo + kLoBlock, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u);
+                                if (kPair) tc_kblock_bf16_pair(d_tmem, w_lo, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u, empty_bar);
+                                else tc_kblock_bf16(d_tmem, w_lo, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u, empty_bar);
+                            } else {
+                                const uint64_t w_desc = ((uint64_t)kSmemDescHi << 32) | w_lo, x_desc = w_desc + kLoX;
+                                for (int k = 0; k < P.last_ksteps; ++k) {
+                                    const uint32_t acc = (k > 0 || kb > 0) ? 1u : 0u;
+                                    for (int i = 0; i < C::kBlocks; ++i) {
+                                        const uint64_t wd = w_desc + (uint64_t)(2 * k + i * (int)kLoBlock), xd = x_desc + (uint64_t)(2 * k);
+                                        if (kPair) tc_mma_bf16_pair(d_tmem, wd, xd, idesc, acc);
+                                        else tc_mma_bf16(d_tmem + (uint32_t)(i * kMmaM), wd, xd, idesc, acc);
+                                    }
+                                }
+                                if (kPair) tc_commit_pair(empty_bar);
+                                else tc_commit(empty_bar);
                             }
-                            if (kPair) tc_commit_pair(empty_bar);
-                            else tc_commit(empty_bar);
+                        }
+                        w_lo += kLoStage;
+                        full_bar += 8u;
+                        empty_bar += 8u;
+                        if (++stage == C::kStages) {
+                            stage = 0;
+                            phase ^= 1u;
+                            w_lo = lo0;
+                            full_bar = full0;
+                            empty_bar = empty0;
                         }
                     }
-                    a_lo += kLoStage;
-                    full_bar += 8u;
-                    empty_bar += 8u;
-                    if (++stage == C::kStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                        a_lo = lo0;
-                        full_bar = full0;
-                        empty_bar = empty0;
-                    }
-                }
+                };
+                // the producer knows the tile's rows; looked up here, the table entry is a load in the issuer's way.  Full tiles of a
+                // pair in a loop of their own, with a constant N, as in the fused kernel.
+                wait_stage();
+                if (!ok) break;
+                const uint32_t n = ctl->tile_n[it & 7];
+                if (kPair && __all_sync(0xffffffffu, n == (uint32_t)kFullN)) kloop(std::true_type{}, 0u);
+                else kloop(std::false_type{}, __reduce_max_sync(0xffffffffu, n));
                 __syncwarp();
                 if (ok && elect_one_sync()) {
                     if (kPair) tc_commit_pair(smem_u32(&ctl->tmem_full[a]));
@@ -392,54 +419,72 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + kG1EpiWarps) {
-        // ---------------- epilogue: rounds of 16 columns (one 32-byte store per row), a contiguous half of the tile per column
-        // group.  Every division is a branch (its slow path), so a lane's divisions run one after the other: where a launch is
-        // one wave, that chain is its tail, and it is split evenly over the groups and holds nothing but the divisions (whole layer,
-        // DeepSeek shape, T = 1: 43.3 us in rounds of 32 columns with exponentials and divisions mixed, 41.3 so).
-        const int q4 = warp & 3;
-        const int grp = (warp - 4) >> 2;
-        const int row_in_tile = (int)rank * kMmaM + q4 * 32 + lane;
+        // ---------------- epilogue: pieces of 32 rows x 16 columns (this warp's lane quarter), dealt over the two groups of warps.
+        // Every division is a branch (its slow path), so a lane's divisions run one after the other: where a launch is
+        // one wave, that chain is its tail.  It holds nothing but the divisions, and those of eights of rows that the tile has.
+        const int q4 = warp & 3, grp = (warp - 4) >> 2, c = lane & 3;
         int it = 0;
         for (int g = b; g < total_tiles; g += stride, ++it) {
             const G1Tile t = g1_decode<TN>(g, P);
-            const int a = it & 1;
+            const int a = it & 1, pieces = ((t.valid + 31) >> 5) * C::kBlocks;
             const bool ok = g1_wait_warp(smem_u32(&ctl->tmem_full[a]), (uint32_t)(it >> 1) & 1u, ctl, deadline, P.status,
                                          (uint32_t)g, 53u);
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * C::kAccCols);
-            const bool row_ok = row_in_tile < t.valid;
-            __nv_bfloat16 *dst_row = P.x_routed + (size_t)(t.row0 + row_in_tile) * (size_t)P.I + t.n0;
+            const auto release = [&]() {
+                // everything this warp needs of the accumulator is in registers: hand the buffer back
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (kPair) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->tmem_empty[a]), 0u));   // the leader's barrier
+                    else mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
+                }
+            };
+            if (grp >= pieces) release();
 #pragma unroll 1
-            for (int col = grp * (TN / 2); col < (grp + 1) * (TN / 2); col += 16) {
+            for (int piece = grp; piece < pieces; piece += kG1EpiWarps / 4) {
+                const int chunk = piece / C::kBlocks, block = piece % C::kBlocks;
+                const int col = (kPair ? (int)rank : block) * (kMmaM / 2) + q4 * 16;      // first column, inside the tile
+                const bool live = col < TN && t.n0 + col < P.I;
                 uint32_t gt[16], up[16];
-                tmem_ld_32x16(taddr + (uint32_t)col, gt);
-                tmem_ld_32x16(taddr + (uint32_t)(TN + col), up);
-                tmem_ld_wait(gt);
-                tmem_ld_wait(up);
-                if (col + 16 == (grp + 1) * (TN / 2)) {
-                    // everything this warp needs of the accumulator is in registers: hand the buffer back
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if (kPair) mbar_arrive_cluster_relaxed(mapa_u32(smem_u32(&ctl->tmem_empty[a]), 0u));   // the leader's barrier
-                        else mbar_arrive(smem_u32(&ctl->tmem_empty[a]));
-                    }
+                if (live) {
+                    tmem_ld_16x256_x4(taddr + (uint32_t)(block * kMmaM + chunk * 32), gt);
+                    tmem_ld_16x256_x4(taddr + (16u << 16) + (uint32_t)(block * kMmaM + chunk * 32), up);
+                    tmem_ld_wait(gt);
+                    tmem_ld_wait(up);
                 }
-                if (row_ok && t.n0 + col < P.I) {
-                    float x[16], d[16];
+                if (piece + kG1EpiWarps / 4 >= pieces) release();
+                if (!live) continue;
+                const int rows = t.valid - chunk * 32;
+                // registers 4j..4j+3: rows 8j + 2c and the next one, of columns lane / 4 (4j, 4j + 1) and 8 + lane / 4
+                float d[16];
+                uint32_t w[8];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) d[i] = silu_divisor(__uint_as_float(gt[i]));
+                for (int i = 0; i < 16; ++i) d[i] = silu_divisor(__uint_as_float(gt[i]));
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(gt[i]) / d[i];
-                    uint32_t w[8];
+                for (int j = 0; j < 4; ++j) {
+                    w[j] = w[4 + j] = 0u;
+                    if (8 * j >= rows) continue;
+                    float y[4];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * i] * __uint_as_float(up[2 * i]), x[2 * i + 1] * __uint_as_float(up[2 * i + 1]));
-                        w[i] = *reinterpret_cast<uint32_t *>(&h);
-                    }
-                    st_global_v8(dst_row + col, w);
+                    for (int i = 0; i < 4; ++i) y[i] = __uint_as_float(gt[4 * j + i]) / d[4 * j + i] * __uint_as_float(up[4 * j + i]);
+                    w[j] = transpose_8x8(pack_bf16(__float_as_uint(y[0]), __float_as_uint(y[1])));
+                    w[4 + j] = transpose_8x8(pack_bf16(__float_as_uint(y[2]), __float_as_uint(y[3])));
                 }
+                // w[j], w[4 + j]: columns 2c and 8 + 2c and the next ones of row 8j + lane / 4 -> all 16 columns of row 8c + lane / 4
+#pragma unroll
+                for (int x = 1; x < 4; x *= 2)
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) {
+                        if (m & x) continue;
+                        const bool hi = (c & x) != 0;
+                        const uint32_t got = __shfl_xor_sync(0xffffffffu, hi ? w[m] : w[m + x], x);
+                        if (hi) w[m] = got;
+                        else w[m + x] = got;
+                    }
+                const int row = 8 * c + (lane >> 2);
+                if (row < rows) st_global_v8(P.x_routed + (size_t)(t.row0 + chunk * 32 + row) * (size_t)P.I + t.n0 + col, w);
             }
         }
     }
@@ -551,10 +596,10 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     p.last_ksteps = (s->H - (p.num_kb - 1) * kBlockK) / kUmmaK;
     if ((int64_t)n_mtiles * p.NT >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
 
-    // W1 [E_tot][2][I][H] seen as [E_tot * 2 planes][I rows][H]: rows past I of a plane read zeros
-    const CUtensorMap *mB = operand_map(h, W1, 2 * s->E_tot, s->I, s->H, TN, "W1");
-    if (!mB) return MOE_ERR_CUDA;
-    p.tmB = *mB;
+    // columns past I read zeros
+    const CUtensorMap *mW = gate_up_map(h, W1, s->E_tot, s->I, s->H, pair ? TN / 2 : TN, "W1");
+    if (!mW) return MOE_ERR_CUDA;
+    p.tmW = *mW;
 
     const int64_t tiles_bound = (int64_t)n_mtiles * p.NT;
     const int slots = pair ? h->max_pairs : h->G;

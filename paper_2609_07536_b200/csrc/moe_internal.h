@@ -99,7 +99,7 @@ struct alignas(64) FusedParams {
 
 namespace moe {
 // An operand tensor map (bf16, k contiguous, 64 x box_rows boxes, 128B swizzle) and what it was encoded for: [rows, cols], or
-// [planes, rows, cols].  Encoding one costs a microsecond of host time per launch: the handle keeps the maps of the operands that
+// [planes, rows, cols], or gate and up planes of `-planes` experts.  Encoding one costs a microsecond of host time per launch: the handle keeps the maps of the operands that
 // it has seen (a model's layers, the buffers of a loop of steps) in a small direct-mapped table.
 struct alignas(64) MapEntry {
     CUtensorMap map;
@@ -227,6 +227,9 @@ int32_t cuda_fail(moe_handle *h, cudaError_t e, const char *what);
 int32_t require_handle_device(moe_handle *h, const char *who);
 // the tensor map of an operand (planes = 0: two dimensions); nullptr, with a message in the handle, when it cannot be encoded
 const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name);
+// ... of the gate and up weights [experts][2][inter][cols]: boxes of box_inter intermediate columns (a multiple of 16), in groups of 16
+// gate rows followed by the 16 up rows of the same columns; inter % 16 == 0
+const CUtensorMap *gate_up_map(moe_handle *h, const void *ptr, int32_t experts, int32_t inter, int32_t cols, int32_t box_inter, const char *name);
 // fused kernel (gemm2_combine.cu)
 size_t fused_smem_bytes(int tile_n);
 cudaError_t fused_occupancy(int tile_n, int *blocks_per_sm);
