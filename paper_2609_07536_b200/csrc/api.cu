@@ -706,6 +706,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     // computed; m-tile-major across the splits (x is read from DRAM once) when nothing does
     p.tile_order = (plan->drain_help && p.co_warps == 0) ? 1 : 0;
     const int64_t R = (int64_t)s->T * s->k_tot;
+    p.dry_rows = (int32_t)(R / s->E_tot < occ->tile_m ? R / s->E_tot + 1 : occ->tile_m);
     p.w2_once = R <= (int64_t)s->E_tot * kMmaM;    // at most one 128-row tile per expert on average
     // Even shares or the queue (few_units).  Co-resident warps draw on the queue; a launch with a withheld tile is about that
     // tile's flag.

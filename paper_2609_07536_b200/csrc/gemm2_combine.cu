@@ -507,7 +507,8 @@ struct PairCfg {
 // copy, of 128 rows or, where they suffice, 64 or 32 (two copies of 64 rows lengthen the GEMM phase of the DeepSeek shape T = 16384 from
 // 609 to 690 us, a number of copies and bytes that it looks up by 30), and the next tile is looked up between two k-blocks.
 template <int TN, bool kPair, bool kX>
-__device__ __forceinline__ void producer_role(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b, unsigned long long deadline, uint32_t rank)
+__device__ __forceinline__ void producer_role(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b, unsigned long long deadline, uint32_t rank,
+                                              bool dry)
 {
     using C = typename std::conditional<kPair, PairCfg, Cfg<TN>>::type;
     const int total_tiles = P.L * pt.W_comp, n_stages = P.stages;
@@ -523,13 +524,20 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
     TL_DECL(long long tl_pw = 0, tl_q;)
     TileWalk walk(P, pt, b);
     Tile t = walk.tile(), t_next = t;
-    int e = kX ? 0 : ld_chained(&P.mtile_expert[t.mu]), e_next = 0;
-    int row0 = kX ? ld_chained(&P.mtile_first_row[t.mu]) : 0, valid = kX ? ld_chained(&P.mtile_valid[t.mu]) : 0, row0_next = 0, valid_next = 0;
+    int e = 0, e_next = 0, row0 = 0, valid = P.dry_rows, row0_next = 0, valid_next = 0;
+    if (!dry) {
+        if (kX) {
+            row0 = ld_chained(&P.mtile_first_row[t.mu]);
+            valid = ld_chained(&P.mtile_valid[t.mu]);
+        } else {
+            e = ld_chained(&P.mtile_expert[t.mu]);
+        }
+    }
     const int ahead_at = min(2, P.num_kb - 1);
     for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
         const int n0 = t.s * P.split_w + t.i_n * TN + (kPair ? (int)rank * (TN / 2) : 0);
         const int n = mma_n_of<kPair>(valid), my_rows = kPair ? n >> 1 : n, my_row0 = row0 + (kPair ? (int)rank * my_rows : 0);
-        if (kX && P.x_ready && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
+        if (kX && P.x_ready && !dry && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
         const auto kloop = [&](auto box_rows) {
             constexpr int kRows = decltype(box_rows)::value;
             constexpr uint32_t kXCopy = (uint32_t)(kRows * kBlockK * 2);
@@ -542,7 +550,8 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
                 TL(tl_pw += clock64() - tl_q);
                 // (a probe that leaves a copy out completes its bytes by hand: every producer stays in the
                 // barrier's dependency chain, or the one that arms it could lap the others)
-                if (kX) {
+                if (dry) {
+                } else if (kX) {
                     if (kb == 0) ctl->tile_n[it & 7] = (uint32_t)n;
                     if (!kPair) mbar_arrive_expect_tx(full_bar, (uint32_t)C::kWBytes + kXCopy);
                     else if (rank == 0) mbar_arrive_expect_tx(full_bar, 2u * ((uint32_t)C::kWBytes + kXCopy));
@@ -566,6 +575,7 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
                     full_bar = full0;
                     empty_bar = empty0;
                 }
+                if (dry) break;
                 if (kb == ahead_at) {
                     walk.next();
                     t_next = walk.tile();
@@ -581,6 +591,7 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
         if (!kX || my_rows > 64) kloop(std::integral_constant<int, 128>{});
         else if (kPair || my_rows > 32) kloop(std::integral_constant<int, 64>{});
         else kloop(std::integral_constant<int, 32>{});
+        if (dry) return;
         t = t_next;
         e = e_next;
         row0 = row0_next;
@@ -640,8 +651,8 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
     if (warp == 0 || warp == 2) {
         // ---------------- TMA producers: warp 0 loads the x_routed tile, warp 2 the W2 tile of every k-block
         if (lane == 0 && b < total_tiles) {
-            if (warp == 0) producer_role<TN, false, true>(P, pt, ring, ctl, b, deadline, 0u);
-            else producer_role<TN, false, false>(P, pt, ring, ctl, b, deadline, 0u);
+            if (warp == 0) producer_role<TN, false, true>(P, pt, ring, ctl, b, deadline, 0u, false);
+            else producer_role<TN, false, false>(P, pt, ring, ctl, b, deadline, 0u, false);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -745,19 +756,12 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
 //   tmem_full[a]      one per CTA (its epilogue waits on it), signalled by the leader's commit
 //   tmem_empty[a]     only the leader's is used: 12 local + 12 remote epilogue warps arrive
 
-__device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b)
+// Barriers (thread 0) and TMEM (warp 1) of a CTA of a pair, before it is known that the pair computes; the cluster barrier behind it
+// makes the peer's barriers exist before anything arrives on them.
+__device__ __forceinline__ void pair_setup(const FusedParams &P, Control *ctl)
 {
-    using C = PairCfg;
-    constexpr int TN = C::kTileN;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();
-    const bool leader_cta = (rank == 0);
-    const int total_tiles = P.L * pt.W_comp;
-    const int n_stages = P.stages;
-    const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
-
     if (threadIdx.x == 0) {
-        for (int i = 0; i < n_stages; ++i) {
+        for (int i = 0; i < P.stages; ++i) {
             mbar_init(smem_u32(&ctl->full[i]), 1);
             mbar_init(smem_u32(&ctl->empty[i]), 1);
         }
@@ -772,20 +776,27 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc_pair(smem_u32(&ctl->tmem_base), C::kTmemCols);
-    tc_fence_before();
-    sync_compute_warps(P);
-    cluster_sync_all();          // the peer's barriers exist before anything arrives on them (the co-resident
-                                 // communication warps of both CTAs arrive on this cluster barrier too)
-    tc_fence_after();
+    if ((threadIdx.x >> 5) == 1) tmem_alloc_pair(smem_u32(&ctl->tmem_base), PairCfg::kTmemCols);
+}
+
+__device__ __forceinline__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b, bool dry)
+{
+    using C = PairCfg;
+    constexpr int TN = C::kTileN;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    const bool leader_cta = (rank == 0);
+    const int total_tiles = P.L * pt.W_comp;
+    const int n_stages = P.stages;
+    const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
     const uint32_t tmem_base = ctl->tmem_base;
 
     if (warp == 0 || warp == 2) {
         // ---------------- TMA producers (both CTAs): warp 0 loads this CTA's x_routed rows, warp 2 its W2
         // rows; both complete on the leader's full barrier.
         if (lane == 0 && b < total_tiles && !MOE_PROBE(kProbeFreeRunMma)) {
-            if (warp == 0) producer_role<TN, true, true>(P, pt, ring, ctl, b, deadline, rank);
-            else producer_role<TN, true, false>(P, pt, ring, ctl, b, deadline, rank);
+            if (warp == 0) producer_role<TN, true, true>(P, pt, ring, ctl, b, deadline, rank, dry);
+            else producer_role<TN, true, false>(P, pt, ring, ctl, b, deadline, rank, dry);
         }
         __syncwarp();
     } else if (warp == 1 && leader_cta) {
@@ -821,7 +832,7 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(a * TN);
                 const auto wait_stage = [&]() {
-                    if (MOE_PROBE(kProbeFreeRunMma) || __all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) return;
+                    if (MOE_PROBE(kProbeFreeRunMma) || __all_sync(0xffffffffu, mbar_test_wait(full_bar, phase) || dry)) return;
                     TL(++tl_late);
                     ok = __all_sync(0xffffffffu, wait_barrier_1t(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 21u));
                 };
@@ -837,6 +848,7 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
                             const long long until = clock64() + 200;
                             while (clock64() < until) {}
                         }
+                        if (dry) break;
                         if (elect_one_sync()) {
                             if ((kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) && !MOE_PROBE(kProbeFreeRunMma)) {
                                 tc_kblock_bf16_pair(d_tmem, w_lo, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u, empty_bar);
@@ -865,9 +877,10 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
                 // full tiles in a loop of their own: with a constant N the issuer needs 27 cycles a k-block less
                 wait_stage();
                 if (!ok) break;
-                const uint32_t n = MOE_PROBE(kProbeFreeRunMma) ? 256u : ctl->tile_n[it & 7];
+                const uint32_t n = MOE_PROBE(kProbeFreeRunMma) || dry ? 256u : ctl->tile_n[it & 7];
                 if (__all_sync(0xffffffffu, n == (uint32_t)TN)) kloop(std::true_type{}, 0u);
                 else kloop(std::false_type{}, __reduce_max_sync(0xffffffffu, n));
+                if (dry) break;
                 __syncwarp();
                 if (ok && elect_one_sync()) tc_commit_pair(smem_u32(&ctl->tmem_full[a]));   // both epilogues may start
                 TL(if (it == 0 && lane == 0) tl_put(P, kTlFirstAcc, globaltimer_ns()));
@@ -880,12 +893,13 @@ __device__ void compute_cta_pair(const FusedParams &P, const Part &pt, uint8_t *
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        epilogue_role<TN, true>(P, pt, ctl, b, tmem_base, deadline, (int)rank);
+        if (!dry) epilogue_role<TN, true>(P, pt, ctl, b, tmem_base, deadline, (int)rank);
     } else if (warp == 3) {
-        publisher_role<true>(P, pt, ctl, b, deadline, (int)rank);
+        if (!dry) publisher_role<true>(P, pt, ctl, b, deadline, (int)rank);
     }
+    if (dry) return;
     // ---------------- teardown: nobody leaves while its peer may still touch its memory (the co-resident
-    // communication warps arrived on this cluster barrier right after the set-up one)
+    // communication warps arrived on this cluster barrier at once)
     tc_fence_before();
     sync_compute_warps(P);
     cluster_sync_all();
@@ -1571,41 +1585,60 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
                          : reinterpret_cast<uint8_t *>(ring + kStageBytesTotal + ((sizeof(Control) + 127) & ~(size_t)127));
     const int warp = threadIdx.x >> 5;
 
+    // what does not depend on the predecessor is done before the wait for it
     init_comm_barriers(ctl);
+    if (P.P > 0) pair_setup(P, ctl);
     if (threadIdx.x == 96) {
         prefetch_tensormap(&P.tmA);
         prefetch_tensormap(&P.tmB);
     }
-    grid_dependency_wait();
-    if (blockIdx.x == 0 && threadIdx.x < (unsigned)P.L) {
-        P.split_done_next[threadIdx.x] = 0u;
-        P.queue_next[threadIdx.x] = 0ull;
-    }
-    const Part pt = launch_part(P);
-    __syncthreads();          // the only CTA-wide barrier all 20 warps share
-    TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < ((pt.C + 1) & ~1) ? 0u : 1u); });
-
-    const int c_even = (pt.C + 1) & ~1;
+    tc_fence_before();
+    cluster_sync_all();       // the only barrier all 20 warps share
+    tc_fence_after();
+    // Twice through the code of the producers and the issuer: dry, before the predecessor is waited for, then in earnest.  A launch runs
+    // cold: from the end of the wait to the first copy a producer took 8000 cycles, almost all of them misses of its instruction and constant
+    // caches, one after the other.  Behind a routing build this CTA has 10000 cycles to itself before the wait ends; with the dry round
+    // (4800 cycles) in them it is 3700 from there to the first copy (whole calls, with the set-up moved in front of the wait, us:
+    // Granite shape T = 4096 91.6 -> 89.1, its whole layer T = 1003 81.9 -> 80.7, Qwen shape T = 8192 236 -> 232).  The dry round
+    // touches neither barriers' phases nor memory, and reads nothing that the predecessor writes.  (With the combine's code in
+    // it as well it takes 12000 cycles, which is longer than the wait: whole layer T = 1003 +2 %.  In GEMM1: 0 to +1 %.)
     const bool queued = P.drain_help && !P.even;           // (drain help is a matter of fused launches)
-    if (P.mail && blockIdx.x == 0 && warp == kCommWarps)
-        mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
-    if ((int)blockIdx.x < pt.C) {
-        if (queued) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront);
-    } else if ((int)blockIdx.x < c_even) {
+    const bool co_resident = warp >= kThreads / 32 && P.epi_warps == 12;
+    Part pt = {1, 1, 0, 1};
+    int c_even = 0;
+#pragma unroll 1
+    for (int round = P.P > 0 ? 0 : 1; round < 2; ++round) {
+        const bool dry = round == 0;
+        if (!dry) {
+            grid_dependency_wait();
+            if (blockIdx.x == 0 && threadIdx.x < (unsigned)P.L) {
+                P.split_done_next[threadIdx.x] = 0u;
+                P.queue_next[threadIdx.x] = 0ull;
+            }
+            pt = launch_part(P);
+            c_even = (pt.C + 1) & ~1;
+            TL(if (threadIdx.x == 0) { tl_put(P, kTlBegin, globaltimer_ns()); tl_put(P, kTlRole, (int)blockIdx.x < c_even ? 0u : 1u); });
+            if (P.mail && blockIdx.x == 0 && warp == kCommWarps)
+                mail_counts(P.mail, P.mail_seq, P.E_tot, threadIdx.x & 31, [&](int x) { return ld_chained(P.S_dev - P.E_tot + x); });
+            if ((int)blockIdx.x < c_even) {
+                if (warp == 1 && P.P > 0) tmem_dealloc_pair(ctl->tmem_base, PairCfg::kTmemCols);
+                break;
+            }
+        }
+        if (!co_resident) compute_cta_pair(P, pt, ring, ctl, dry ? 0 : ((int)blockIdx.x - c_even) >> 1, dry);
+    }
+    if ((int)blockIdx.x < c_even) {
         // odd C: the last communication CTA's cluster-mate cannot compute (no partner).  With dynamic work
         // distribution it serves communication work as well; under the static map it has no tile list.
         if (queued) comm_cta<256>(P, pt, ring, ctl, aux, kRoleFront);
-    } else if (warp >= kThreads / 32 && P.epi_warps == 12) {
-        // The compute warps of both CTAs meet at two cluster barriers (set-up and teardown), and a cluster
-        // barrier counts every thread: these warps join the first, arrive at once on the second (they hold
-        // nothing a peer could touch) and pick its completion up when their own work is done.
-        cluster_sync_all();
+    } else if (co_resident) {
+        // The compute warps of both CTAs meet at a cluster barrier at the end, and a cluster barrier counts every thread: these
+        // warps arrive at once (they hold nothing a peer could touch) and pick its completion up when their own work is done.
         cluster_arrive();
         if (co_warp_number(warp) < P.co_warps) co_resident_warp<256>(P, pt, ctl, aux, co_warp_number(warp));
         cluster_wait();
         return;
     } else {
-        compute_cta_pair(P, pt, ring, ctl, ((int)blockIdx.x - c_even) >> 1);
         TL(if (threadIdx.x == 0) tl_put(P, kTlComputeEnd, globaltimer_ns()));
         if (queued && !ctl->abort) comm_cta<256>(P, pt, ring, ctl, aux, kRoleBack);
     }

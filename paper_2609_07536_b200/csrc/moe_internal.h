@@ -83,6 +83,7 @@ struct alignas(64) FusedParams {
     const uint32_t *x_ready;            // != nullptr: x_routed is still being copied in; the rows that have arrived
     int32_t w2_once;                    // W2 is read (about) once: its lines go first when L2 needs room
     int32_t num_kb, last_ksteps;
+    int32_t dry_rows;                   // rows of a tile as they are to be expected, for the dry round (pair kernel)
     int32_t drain_help;                 // compute CTAs serve communication tiles once their GEMM tiles are done
     int32_t co_warps;                   // co-resident communication warps per compute CTA (0..2)
     int32_t stages;                     // operand stages of a compute CTA: as many as fit the ring; a pair's has one more where the aux
