@@ -32,6 +32,15 @@ int32_t require_handle_device(moe_handle *h, const char *who)
     return MOE_OK;
 }
 
+Divisor divisor_of(int32_t d)
+{
+    // exact below 2^31: mul exceeds 2^shift / d by less than one
+    Divisor r = {0u, 31u};
+    while ((1ll << (r.shift - 31u)) < (long long)d) ++r.shift;
+    r.mul = (uint32_t)(((1ull << r.shift) + (uint32_t)d - 1) / (uint32_t)d);
+    return r;
+}
+
 // The table's entry for these arguments, encoded if it is another one's.
 static const CUtensorMap *cached_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, int rank,
                                      const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, const char *name)

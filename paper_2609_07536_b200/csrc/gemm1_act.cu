@@ -80,6 +80,7 @@ struct alignas(64) G1Params {
     unsigned long long wait_ns;
     int32_t S;                     // m-tiles of the routing workspace (or their bound with S_dev)
     int32_t T, k_tot, H;
+    Divisor by_k, by_NT, by_slots;   // k_tot, NT, CTAs (pairs) of the launch
     int32_t I, NT;                 // intermediate size, n-tiles = ceil(I / tile columns)
     int32_t num_kb, last_ksteps;
     int32_t w1_once;               // W1 is read (about) once: its lines go first when L2 needs room
@@ -135,7 +136,7 @@ struct G1Tile {
 template <int TN>
 __device__ __forceinline__ G1Tile g1_decode(int g, const G1Params &P)
 {
-    const int mu = g / P.NT;
+    const int mu = quotient(P.by_NT, g);
     G1Tile t;
     t.e = ld_chained(&P.mtile_expert[mu]);
     t.row0 = ld_chained(&P.mtile_first_row[mu]);
@@ -207,8 +208,8 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
         // as many waves as all CTAs need, over as few CTAs as then suffice: with all of them the same waves take longer, each
         // tile's share of the memory bandwidth being smaller (stage alone: Granite shape T = 16 30.7 -> 28.0 us, T = 400 32.5 -> 30.6,
         // DeepSeek shape T = 300 145.9 -> 140.8, Qwen shape T = 512 122.3 -> 118.1; large batches equal)
-        const int waves = max(1, (total_tiles + stride - 1) / stride);
-        stride = max(1, (total_tiles + waves - 1) / waves);
+        const int waves = max(1, quotient(P.by_slots, total_tiles + stride - 1));
+        stride = max(1, small_quotient(total_tiles + waves - 1, waves));
         if (b >= stride) b = total_tiles;
     }
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
@@ -289,7 +290,7 @@ moe_gemm1_act_kernel(const __grid_constant__ G1Params P)
             const auto rows_of = [&](const int (&f)[kSteps], const __nv_bfloat16 *(&src)[kSteps]) {
 #pragma unroll
                 for (int i = 0; i < kSteps; ++i)
-                    src[i] = f[i] >= 0 ? P.hidden + (size_t)min(f[i] / P.k_tot, P.T - 1) * (size_t)P.H + chunk * 8 : nullptr;
+                    src[i] = f[i] >= 0 ? P.hidden + (size_t)min(quotient(P.by_k, f[i]), P.T - 1) * (size_t)P.H + chunk * 8 : nullptr;
             };
             G1Tile t_next = g1_decode<TN>(min(b + stride, total_tiles - 1), P);
             int f_next[kSteps];
@@ -604,6 +605,9 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     const int64_t tiles_bound = (int64_t)n_mtiles * p.NT;
     const int slots = pair ? h->max_pairs : h->G;
     const int used = (int)(tiles_bound < slots ? (tiles_bound > 0 ? tiles_bound : 1) : slots);
+    p.by_k = divisor_of(s->k_tot);
+    p.by_NT = divisor_of(p.NT);
+    p.by_slots = divisor_of(used);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2] = {chained_launch_attribute()};
     attr[1].id = cudaLaunchAttributeClusterDimension;

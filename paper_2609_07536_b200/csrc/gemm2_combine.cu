@@ -206,7 +206,8 @@ struct Tile {
 // and nothing waits for an early split (drain help), m-tile-major: the n-tiles of ALL splits of one
 // m-tile are adjacent, so that the x rows are read from DRAM once instead of once per split.
 // A position is a number of three digits (split, m-tile, n-tile), the step another one: no division per tile (with two for every
-// look-up the epilogue warps spent 2500 cycles of a tile's 6200 between tiles at the Granite shape, and paced it).
+// look-up the epilogue warps spent 2500 cycles of a tile's 6200 between tiles at the Granite shape, and paced it).  Made once, for all
+// roles: a copy in each of them is code that has to be fetched, on the way to the first tile.
 struct TileWalk {
     int W_comp, NTs, n_mid, last_mu;     // n_mid: values of the middle digit
     bool m_major;
@@ -223,9 +224,9 @@ struct TileWalk {
     }
     __device__ __forceinline__ void split(int g, int &t, int &m, int &l) const
     {
-        const int r = g / NTs;
+        const int r = small_quotient(g, NTs);      // (g: a compute slot, or how many there are)
         l = g - r * NTs;
-        t = r / n_mid;
+        t = small_quotient(r, n_mid);
         m = r - t * n_mid;
     }
     __device__ __forceinline__ void next()
@@ -310,7 +311,7 @@ __device__ __forceinline__ void store_rows(const FusedParams &P, const uint32_t 
 // piece of 32 rows x 128 columns, then the hand-over to the publisher warp.
 template <int TN, bool kPair>
 __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &pt, Control *ctl, int b,
-                                              uint32_t tmem_base, unsigned long long deadline, int rank)
+                                              uint32_t tmem_base, unsigned long long deadline, int rank, TileWalk walk)
 {
     constexpr int kBlocks = kPair ? 1 : Cfg<TN>::kBlocks, kAccCols = kPair ? TN : Cfg<TN>::kAccCols;
     constexpr int kPieces = 3;                 // pieces of a tile that a warp may have: 8, over at least three groups of warps
@@ -333,7 +334,6 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
         }
     };
     TL_DECL(long long tl_ew = 0, tl_ek = 0, tl_ep = 0, tl_q;)
-    TileWalk walk(P, pt, b);
     Tile t = walk.tile(), t_n = t;
     if (b < total_tiles) {
         walk.next();
@@ -451,12 +451,11 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
 // whose epilogue has finished by then (up to kPubSlots).
 template <bool kPair>
 __device__ __forceinline__ void publisher_role(const FusedParams &P, const Part &pt, Control *ctl, int b,
-                                               unsigned long long deadline, int rank)
+                                               unsigned long long deadline, int rank, TileWalk walk)
 {
     const int total_tiles = P.L * pt.W_comp;
     if ((threadIdx.x & 31) == 0) {
         int it = 0;
-        TileWalk walk(P, pt, b);
         TL_DECL(long long tl_pw = 0, tl_pf = 0, tl_q;)
         for (int g = b; g < total_tiles;) {
             TL(tl_q = clock64());
@@ -508,7 +507,7 @@ struct PairCfg {
 // 609 to 690 us, a number of copies and bytes that it looks up by 30), and the next tile is looked up between two k-blocks.
 template <int TN, bool kPair, bool kX>
 __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &pt, uint8_t *ring, Control *ctl, int b, unsigned long long deadline, uint32_t rank,
-                                              bool dry)
+                                              bool dry, TileWalk walk)
 {
     using C = typename std::conditional<kPair, PairCfg, Cfg<TN>>::type;
     const int total_tiles = P.L * pt.W_comp, n_stages = P.stages;
@@ -522,7 +521,6 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
     bool ok = true;
     const unsigned long long w_policy = P.w2_once ? l2_evict_first_policy() : l2_evict_normal_policy();
     TL_DECL(long long tl_pw = 0, tl_q;)
-    TileWalk walk(P, pt, b);
     Tile t = walk.tile(), t_next = t;
     int e = 0, e_next = 0, row0 = 0, valid = P.dry_rows, row0_next = 0, valid_next = 0;
     if (!dry) {
@@ -647,12 +645,13 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
     const int n_stages = P.stages;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
     const uint32_t tmem_base = ctl->tmem_base;
+    const TileWalk walk(P, pt, b);
 
     if (warp == 0 || warp == 2) {
         // ---------------- TMA producers: warp 0 loads the x_routed tile, warp 2 the W2 tile of every k-block
         if (lane == 0 && b < total_tiles) {
-            if (warp == 0) producer_role<TN, false, true>(P, pt, ring, ctl, b, deadline, 0u, false);
-            else producer_role<TN, false, false>(P, pt, ring, ctl, b, deadline, 0u, false);
+            if (warp == 0) producer_role<TN, false, true>(P, pt, ring, ctl, b, deadline, 0u, false, walk);
+            else producer_role<TN, false, false>(P, pt, ring, ctl, b, deadline, 0u, false, walk);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -731,9 +730,9 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        epilogue_role<TN, false>(P, pt, ctl, b, tmem_base, deadline, 0);
+        epilogue_role<TN, false>(P, pt, ctl, b, tmem_base, deadline, 0, walk);
     } else if (warp == 3) {
-        publisher_role<false>(P, pt, ctl, b, deadline, 0);
+        publisher_role<false>(P, pt, ctl, b, deadline, 0, walk);
     }
     // ---------------- teardown
     tc_fence_before();
@@ -790,13 +789,14 @@ __device__ __forceinline__ void compute_cta_pair(const FusedParams &P, const Par
     const int n_stages = P.stages;
     const unsigned long long deadline = globaltimer_ns() + P.wait_ns;
     const uint32_t tmem_base = ctl->tmem_base;
+    const TileWalk walk(P, pt, b);
 
     if (warp == 0 || warp == 2) {
         // ---------------- TMA producers (both CTAs): warp 0 loads this CTA's x_routed rows, warp 2 its W2
         // rows; both complete on the leader's full barrier.
         if (lane == 0 && b < total_tiles && !MOE_PROBE(kProbeFreeRunMma)) {
-            if (warp == 0) producer_role<TN, true, true>(P, pt, ring, ctl, b, deadline, rank, dry);
-            else producer_role<TN, true, false>(P, pt, ring, ctl, b, deadline, rank, dry);
+            if (warp == 0) producer_role<TN, true, true>(P, pt, ring, ctl, b, deadline, rank, dry, walk);
+            else producer_role<TN, true, false>(P, pt, ring, ctl, b, deadline, rank, dry, walk);
         }
         __syncwarp();
     } else if (warp == 1 && leader_cta) {
@@ -893,9 +893,9 @@ __device__ __forceinline__ void compute_cta_pair(const FusedParams &P, const Par
         }
         __syncwarp();
     } else if (warp >= 4 && warp < 4 + P.epi_warps) {
-        if (!dry) epilogue_role<TN, true>(P, pt, ctl, b, tmem_base, deadline, (int)rank);
+        if (!dry) epilogue_role<TN, true>(P, pt, ctl, b, tmem_base, deadline, (int)rank, walk);
     } else if (warp == 3) {
-        if (!dry) publisher_role<true>(P, pt, ctl, b, deadline, (int)rank);
+        if (!dry) publisher_role<true>(P, pt, ctl, b, deadline, (int)rank, walk);
     }
     if (dry) return;
     // ---------------- teardown: nobody leaves while its peer may still touch its memory (the co-resident
@@ -1349,16 +1349,17 @@ __device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &p
     const __nv_bfloat16 *Y = reinterpret_cast<const __nv_bfloat16 *>(P.Y);
     // unit n of a split: token n / n_slabs, column slab n % n_slabs; this warp's next one is `workers` on
     const int n_slabs = (P.split_w + P.slab_cols - 1) >> P.slab_shift, workers = kCommWarps * n_ctas;
-    const int step_tok = workers / n_slabs, step_slab = workers - step_tok * n_slabs;
+    const int step_tok = small_quotient(workers, n_slabs), step_slab = workers - step_tok * n_slabs;
     int k = 0;                // copies issued so far: stage k & 1, parity (k >> 1) & 1
+    int n = warp * n_ctas + c, past = 0;      // this warp's first unit of the split; even: units of a split, modulo `workers`
 #pragma unroll 1
     for (int s = 0; s < P.L; ++s) {
-        int n = warp * n_ctas + c;
         if (P.even && s > 0) {     // the deal goes on where the split before ended
-            n -= (int)((long long)s * P.T * n_slabs % workers);
+            if (s == 1) past = P.T * n_slabs - small_quotient(P.T * n_slabs, workers) * workers;
+            n -= past;
             if (n < 0) n += workers;
         }
-        int tok = n / n_slabs, slab = n - tok * n_slabs, d = 0;
+        int tok = small_quotient(n, n_slabs), slab = n - tok * n_slabs, d = 0;
         // routing of a unit's token, fetched one unit ahead: lane j, row and weight of slot j
         int row = -1;
         float w = 0.f;
@@ -1503,7 +1504,7 @@ __device__ __forceinline__ Part launch_part(const FusedParams &P)
         pt.W_comp = pt.S * P.NTs;
         if (P.c_table_n > 0) {
             pt.C = P.c_table[max(0, min(S - P.c_table_first, P.c_table_n - 1))];
-            pt.P = (P.G - pt.C) / P.slot_sms;
+            pt.P = (P.G - pt.C) >> (P.slot_sms - 1);
         }
     }
     if (P.balance) {
@@ -1512,8 +1513,8 @@ __device__ __forceinline__ Part launch_part(const FusedParams &P)
         // (DeepSeek shape T = 128: 78.5 -> 74.6 us whole step, Qwen shape T = 512 74.3 -> 70.7).  Against the plan's C, with counts
         // on the device: DeepSeek shape T = 16 63.1 -> 57.2, T = 300 85.2 -> 77.1, T = 1024 120.9 -> 116.3; with counts on the
         // host: Granite shape T = 4096 89.1 -> 85.4, Qwen shape T = 8192 235.4 -> 233.1, others equal.
-        const int tiles = pt.W_comp * P.L, waves = max(1, (tiles + P.P - 1) / P.P);
-        pt.P = max(1, (tiles + waves - 1) / waves);
+        const int tiles = pt.W_comp * P.L, waves = max(1, small_quotient(tiles + P.P - 1, P.P));     // (few_units bounds the tiles)
+        pt.P = max(1, small_quotient(tiles + waves - 1, waves));
         pt.C = (P.P - pt.P) * P.slot_sms;
     }
     return pt;

@@ -33,6 +33,10 @@ struct RoutingOut {
     int32_t *counts, *offsets, *tiles, *tile_offsets, *mtile_expert, *mtile_first_row, *mtile_valid, *perm, *inv_perm, *pad_row;
 };
 
+// division by a number that the host knows, as a multiplication (quotient())
+struct Divisor {
+    uint32_t mul, shift;
+};
 // routing build inside a kernel that uses it (topk_idx = nullptr: the arrays are there already)
 struct InlineRouting {
     const int32_t *topk_idx;
@@ -180,6 +184,21 @@ inline cudaLaunchAttribute chained_launch_attribute()
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (after the wait, so that everything before this kernel is complete when a successor starts)
 __device__ __forceinline__ void grid_dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// n / d for a quotient below 2^20, n >= 0, d > 0.  A launch runs cold: what its critical path costs is the bytes of the instructions on it,
+// fetched one line after the other, and a division of integers is 25 of them at every place.
+// (Divisions out of the kernels' preambles, and the tile sequence set up once instead of in every role, whole calls, us: DeepSeek shape
+// T = 1 39.2 -> 37.7, T = 16 53.7 -> 53.1, Granite shape T = 1003 81.3 -> 78.7, tiny shape 13.4 -> 13.0.  Warming more code ahead
+// of time instead, by warps that wait, delays the code that is needed: +1 to +3 us.)
+__device__ __forceinline__ int small_quotient(int n, int d)
+{
+    int q = (int)__fdividef((float)n, (float)d);        // off by one at most
+    const int r = n - q * d;
+    if (r < 0) --q;
+    if (r >= d) ++q;
+    return q;
+}
+// n / d for 0 <= n < 2^31
+__device__ __forceinline__ int quotient(const Divisor &d, int n) { return (int)((unsigned long long)(uint32_t)n * d.mul >> d.shift); }
 // Load of what a predecessor may have written: an ordinary load that stays behind the wait (a read-only __ldg may be moved)
 template <typename T>
 __device__ __forceinline__ T ld_chained(const T *p)
@@ -226,6 +245,7 @@ int32_t cuda_fail(moe_handle *h, cudaError_t e, const char *what);
 // message in the handle) otherwise.  Every launching entry point checks it: kernels run on the
 // current device, the buffers and the cached residency belong to the handle's.
 int32_t require_handle_device(moe_handle *h, const char *who);
+Divisor divisor_of(int32_t d);     // d > 0
 // the tensor map of an operand (planes = 0: two dimensions); nullptr, with a message in the handle, when it cannot be encoded
 const CUtensorMap *operand_map(moe_handle *h, const void *ptr, int32_t planes, int64_t rows, int32_t cols, int32_t box_rows, const char *name);
 // ... of the gate and up weights [experts][2][inter][cols]: boxes of box_inter intermediate columns (a multiple of 16), in groups of 16

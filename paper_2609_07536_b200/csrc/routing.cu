@@ -356,7 +356,7 @@ routing_onepass(const int32_t *__restrict__ topk_idx, int R, int k_tot, int E_to
         }
     }
     // ---- exclusive prefixes over the experts: rows, tiles (Eq. 5, Eq. 16) and rows of this CTA (every CTA, for its own scatter)
-    const int tl = (cnt + tile_m - 1) / tile_m, n_scan = (E_tot + 31) / 32;
+    const int tl = small_quotient(cnt + tile_m - 1, tile_m), n_scan = (E_tot + 31) / 32;
     int ic = cnt, it = tl, io = own;
     if (w < n_scan) {
 #pragma unroll

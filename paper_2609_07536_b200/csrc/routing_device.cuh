@@ -57,8 +57,9 @@ __device__ __forceinline__ void rank_chunk(const int32_t *__restrict__ topk_idx,
     __syncwarp();
 
     // ---- ranks inside the chunk; bad ids are reported and left out, repeated experts reported and kept
-    int j = (begin + lane) % k_tot, m0 = begin % k_tot;             // slot of this lane's assignment, of the row's first
-    const int step = 32 % k_tot, id_bits = E_tot > 1 ? 32 - __clz(E_tot - 1) : 0;
+    const auto modulo_k = [&](int n) { return n - small_quotient(n, k_tot) * k_tot; };     // (begin < 2^18)
+    int j = modulo_k(begin + lane), m0 = modulo_k(begin);           // slot of this lane's assignment, of the row's first
+    const int step = modulo_k(32), id_bits = E_tot > 1 ? 32 - __clz(E_tot - 1) : 0;
 #pragma unroll
     for (int i = 0; i < kRows; ++i) {
         rk[i] = 0;
@@ -138,7 +139,7 @@ __device__ __forceinline__ void routing_inline(const InlineRouting &p, int k_tot
             }
         }
     }
-    const int tl = (cnt + tile_m - 1) / tile_m;
+    const int tl = small_quotient(cnt + tile_m - 1, tile_m);
     int ic = cnt, it = tl;
     if (w < n_scan) {
 #pragma unroll
