@@ -244,3 +244,14 @@ def test_tiles_dealt_by_whole_waves(tile_m, E):
     idx, _, _ = wl.make_routing(w)
     assert rr.build_routing(idx, E, tile_m)["S"] == E
     _check(w, n_rows=200, counts_on_device=True)
+
+
+@pytest.mark.parametrize("tile_m,tile_n", [(64, 64), (128, 128), (256, 256)], ids=str)
+@pytest.mark.parametrize("I", [16, 80, 144], ids=str)     # one group of columns, a tile that ends in its first half, in its second tile
+def test_row_counts_around_the_steps_of_the_mma(tile_m, tile_n, I):
+    # an m-tile is computed for its rows, rounded up to 16 (a pair: 32, half of them in each CTA)
+    counts = [8, 9, 15, 16, 17, 31, 32, 33, 47, 63, 64, 65, 95, 97, 159, 161, 223, 225, 0, 2]
+    idx = np.repeat(np.arange(len(counts)), counts).astype(np.int32)
+    idx = np.random.default_rng(3).permutation(idx)[:, None].copy()
+    w = replace(wl.TINY, name="rowsteps", T=len(idx), E=len(counts), k=1, H=144, I=I, tile_m=tile_m, tile_n=tile_n, TP=1, EP=1, L=1, data_seed=6)
+    _check(w, counts_on_device=True)
