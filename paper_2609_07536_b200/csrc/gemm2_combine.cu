@@ -377,8 +377,7 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
             if (!dry && f[i] >= 0 && cols[i] > 0) {
                 const int tok = token_of(P, f[i]), q = f[i] - tok * P.k_tot;
                 const int slab = cis >> P.slab_shift, wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
-                dst[i] = Y + (size_t)(uint32_t)(tok * P.L + t.s) * ((size_t)P.k_tot * (size_t)P.split_w) + ((size_t)slab * P.k_tot << P.slab_shift) +
-                         (uint32_t)(q * wslab + (cis & (P.slab_cols - 1)));
+                dst[i] = Y + y_unit(tok, t.s, slab << P.slab_shift, P.L, P.split_w, P.k_tot) + (uint32_t)(q * wslab + (cis & (P.slab_cols - 1)));
             }
         }
         TL(tl_q = clock64());
@@ -1136,8 +1135,7 @@ __device__ void comm_warp(const FusedParams &P, const Part &pt, Control *ctl, co
         if (lane == 0) {
             const uint32_t full = full_s + 8u * (uint32_t)st;
             const uint32_t bytes = (uint32_t)(P.k_tot * u.wslab) * 2u;
-            const __nv_bfloat16 *src = Y + ((size_t)u.t * P.L + u.s) * (size_t)P.k_tot * (size_t)P.split_w +
-                                       ((size_t)u.slab * P.k_tot << P.slab_shift);
+            const __nv_bfloat16 *src = Y + y_unit(u.t, u.s, u.slab << P.slab_shift, P.L, P.split_w, P.k_tot);
             mbar_arrive_expect_tx(full, bytes);
             bulk_load_once(smem_u32(my_ring + st * kCommUnitBytes), src, bytes, full, y_policy);   // Y is read once
         }
@@ -1420,7 +1418,7 @@ __device__ __forceinline__ void serve_shares(const FusedParams &P, const Part &p
                 orow_n = reinterpret_cast<__nv_bfloat16 *>(P.out[d]) + (size_t)(tok - d * P.tok_blk) * (size_t)P.H + s * P.split_w + c0;
                 if (lane == 0) {
                     const uint32_t bytes = (uint32_t)(P.k_tot * row_bytes_n), bar = full + 8u * (uint32_t)(k & 1);
-                    const __nv_bfloat16 *src = Y + (((size_t)tok * P.L + s) * (size_t)P.split_w + c0) * (size_t)P.k_tot;
+                    const __nv_bfloat16 *src = Y + y_unit(tok, s, c0, P.L, P.split_w, P.k_tot);
                     mbar_arrive_expect_tx(bar, bytes);
                     bulk_load_once(smem_u32(stages + (k & 1) * kCommUnitBytes), src, bytes, bar, y_policy);   // Y is read once
                 }

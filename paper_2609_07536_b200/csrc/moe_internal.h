@@ -181,6 +181,12 @@ inline cudaLaunchAttribute chained_launch_attribute()
     return a;
 }
 #ifdef __CUDACC__
+// Y [T][L][split_w columns in slabs][k_tot][slab's columns]: where the rows of (token, split, slab from column c0 of the split on) begin.
+// 64 bits from the first product on: T * L alone passes 2^32 at sizes that fit the card (T = 2^29 tokens of one expert each, L = 8).
+__host__ __device__ __forceinline__ size_t y_unit(int tok, int s, int c0, int L, int split_w, int k_tot)
+{
+    return (((size_t)tok * (size_t)L + (size_t)s) * (size_t)split_w + (size_t)c0) * (size_t)k_tot;
+}
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (after the wait, so that everything before this kernel is complete when a successor starts)
 __device__ __forceinline__ void grid_dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
