@@ -776,7 +776,10 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     const CUtensorMap *mB = operand_map(h, W2, s->E_tot, s->H, s->I, pair ? TN / 2 : TN, "W2");
     if (!mB) return MOE_ERR_CUDA;
     p.tmB = *mB;
-    p.stages = fused_stages(pair, TN, p.co_warps == 0);
+    // (no m-tile has more rows than there are assignments, whatever the routing)
+    const int64_t most_rows = R < occ->tile_m ? R : occ->tile_m;
+    p.x_rows = most_rows <= 32 ? 32 : most_rows <= 64 ? 64 : kMmaM;
+    p.stages = fused_stages(pair, TN, p.x_rows, p.co_warps == 0, &p.stage_bytes);
     const int grid = pair ? ((ctas_c + 1) & ~1) + 2 * ctas_p : ctas_c + ctas_p;
     p.timeline = nullptr;
     if (h->timeline && h->timeline_bytes >= ((size_t)grid * kTimelineSlots + MOE_MAX_L) * sizeof(unsigned long long))

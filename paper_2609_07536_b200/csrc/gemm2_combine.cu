@@ -98,10 +98,9 @@ enum { kProbeSkipOddW2 = 1, kProbeSkipAllW2 = 2, kProbeSkipYStores = 4, kProbeSk
 // 239 -> 229, its whole layer T = 48 187 -> 170, T = 3000 126 -> 116; where hardly a row is padding, Granite shape T = 13784, equal.)
 template <int TN>
 struct Cfg {
-    static constexpr int kWBytes = TN * kBlockK * 2;             // 8 / 16 / 32 KB: the tile's rows of W2
-    static constexpr int kXBytes = kMmaM * kBlockK * 2;          // 16 KB: up to 128 routed rows
-    static constexpr int kStageBytes = kWBytes + kXBytes;
-    static constexpr int kStages = kStageBytesTotal / kStageBytes;  // 8 / 6 / 4 
+    static constexpr int kWBytes = TN * kBlockK * 2;             // 8 / 16 / 32 KB: the tile's rows of W2, one k-block
+    static constexpr int kStageKb = TN == 256 ? 1 : 2;           // k-blocks of a stage
+    static constexpr int kThinKb = TN == 64 ? 4 : kStageKb;      // ... where no m-tile has more than 32 rows
     static constexpr int kBlocks = TN > kMmaM ? 2 : 1;           // blocks of 128 output columns, an MMA each (TN = 64: half of one is used)
     static constexpr int kAccCols = kBlocks * kMmaM;             // TMEM columns of an accumulator buffer
     static constexpr int kTmemCols = 2 * kAccCols;               // two of them
@@ -111,16 +110,29 @@ struct Cfg {
 // and one fence covers every tile whose epilogue is over by then.
 constexpr int kPubSlots = 4;
 
+// A stage of a one-CTA tile: the W2 rows of its k-blocks one after the other, then their routed rows, with room for as many as an m-tile
+// of the launch can have (FusedParams::x_rows: 32, 64 or 128).  Narrow tiles are bound by the instructions of the issuer's loop: about
+// 290 cycles of waiting, branching and the commit for a stage and 45 to 53 for an MMA (fitted to 500, 355 and 250 cycles for every 64
+// columns of I with one, two and four k-blocks a stage).  So a stage holds as many k-blocks as leave a ring of three or four.  That
+// counts where tiles are few and their chain of k-blocks is long: a tile over all of I has TP times the chain of one per K-shard.
+// Whole step, us, a tile per K-shard (TP as given) / over all of I, stages of one k-block and 128 rows / now:
+//   one token        Qwen shape, TP = 2, 15.4 / 17.0 / 15.9; DeepSeek shape, TP = 2, 18.8 / 18.2 / 17.5; 8 experts, k = 2, I = 14336,
+//                    TP = 8: H = 4096 46.5 / 69.3 / 53.4, H = 512 18.9 / 68.3 / 39.1 (16 tiles; the other SMs have none)
+//   T = 4096         DeepSeek shape, TP = 2, tiles of 64 x 64 974 / 732 / 556, 64 x 128 529 / 390 / 320, 128 x 128 369 / 268 / 258
+// (256 columns take two MMAs for every K = 16; one k-block a stage there.  More stages of one k-block instead, 16 in place of 8: 0.  The
+// issuer looking at the next stage's barrier ahead of its MMAs: +10 % on the long chains.)
+constexpr int kMaxStages = 8;
+
 struct Control {
-    unsigned long long full[8];
-    unsigned long long empty[8];
+    unsigned long long full[kMaxStages];
+    unsigned long long empty[kMaxStages];
     unsigned long long tmem_full[2];
     unsigned long long tmem_empty[2];
     unsigned long long epi_done[kPubSlots];   // every epilogue warp has stored its rows of the tile (tile number mod kPubSlots)
     unsigned long long pub_done[kPubSlots];   // the publisher warp has raised that tile's flag
     uint32_t tmem_base;
     volatile uint32_t abort;
-    volatile uint32_t tile_n[8];        // N of a tile's MMAs (tile number mod 8), from the x producer to the MMA issuer
+    volatile uint32_t tile_n[kMaxStages];   // N of a tile's MMAs (tile number mod kMaxStages), from the x producer to the MMA issuer
     unsigned long long comm_full[24];   // communication CTA: one barrier per warp and stage
     unsigned long long co_full[8];      // co-resident communication warps: one barrier per warp and stage
 };
@@ -187,10 +199,11 @@ template <bool kPair>
 __device__ __forceinline__ int mma_n_of(int valid) { return kPair ? (valid + 31) & ~31 : (valid + 15) & ~15; }
 
 // The MMA issuer's N of its tile `it`, behind the tile's first full barrier.  The producer knows the tile's rows; looked up by the issuer
-// itself, the table entry is a load in the issuer's way.  (A place is written again
-// eight tiles later, when the MMAs of the tile before the last seven stages are over.)
+// itself, the table entry is a load in the issuer's way.  (A place is written again kMaxStages tiles later, each of
+// at least one stage, behind the wait for the later tile's first stage: in a ring of kMaxStages or fewer that stage, or one that came
+// after it, was freed by MMAs of the earlier tile, so that the issuer is past the look.)
 template <typename Ctl>
-__device__ __forceinline__ int tile_n(const Ctl *ctl, int it) { return (int)__reduce_max_sync(0xffffffffu, ctl->tile_n[it & 7]); }   // (warp-uniform)
+__device__ __forceinline__ int tile_n(const Ctl *ctl, int it) { return (int)__reduce_max_sync(0xffffffffu, ctl->tile_n[it & (kMaxStages - 1)]); }   // (warp-uniform)
 
 // What a launch's roles are divided by: compute tiles per split (Eq. 5), communication CTAs, compute slots.
 struct Part {
@@ -494,8 +507,11 @@ struct PairCfg {
     static constexpr int kWBytes = kMmaM * kBlockK * 2;                 // 16 KB: this CTA's 128 W2 rows
     static constexpr int kXBytes = (kTileN / 2) * kBlockK * 2;          // 16 KB: this CTA's half of the tile's rows
     static constexpr int kStageBytes = kWBytes + kXBytes;               // 32 KB
+    static constexpr int kStageKb = 1, kThinKb = 1;                     // k-blocks of a stage
     static constexpr int kTmemCols = 2 * kTileN;                        // two accumulator buffers
 };
+// (a one-CTA ring: fused_stages)
+static_assert(kStageBytesTotal / PairCfg::kStageBytes + 1 <= kMaxStages && (kMaxStages & (kMaxStages - 1)) == 0, "barriers and tile_n of a ring");
 
 // --------------------------------------------------------------------------- TMA producers
 //
@@ -510,8 +526,11 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
 {
     using C = typename std::conditional<kPair, PairCfg, Cfg<TN>>::type;
     const int total_tiles = P.L * pt.W_comp, n_stages = P.stages;
+    const uint32_t stage_bytes = kPair ? (uint32_t)PairCfg::kStageBytes : (uint32_t)P.stage_bytes;
+    const bool thin = !kPair && P.x_rows == 32;
+    const int stage_kb = thin ? C::kThinKb : C::kStageKb;
     // pair: the leader's full barriers, which lie at the same offsets in CTA 0
-    const uint32_t dst0 = smem_u32(ring) + (kX ? (uint32_t)C::kWBytes : 0u), empty0 = smem_u32(&ctl->empty[0]);
+    const uint32_t dst0 = smem_u32(ring) + (kX ? (uint32_t)(C::kWBytes * stage_kb) : 0u), empty0 = smem_u32(&ctl->empty[0]);
     const uint32_t full0 = kPair ? smem_u32(&ctl->full[0]) & 0xFEFFFFFFu : smem_u32(&ctl->full[0]);
     uint32_t dst = dst0, full_bar = full0, empty_bar = empty0;
     int stage = 0, it = 0;
@@ -530,17 +549,20 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
             e = ld_chained(&P.mtile_expert[t.mu]);
         }
     }
-    const int ahead_at = min(2, P.num_kb - 1);
+    const int ahead_at = min(2, P.num_kb - 1) / stage_kb * stage_kb;
     for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
         const int n0 = t.s * P.split_w + t.i_n * TN + (kPair ? (int)rank * (TN / 2) : 0);
-        const int n = mma_n_of<kPair>(valid), my_rows = kPair ? n >> 1 : n, my_row0 = row0 + (kPair ? (int)rank * my_rows : 0);
+        const int n = mma_n_of<kPair>(kPair ? valid : min(valid, P.x_rows)), my_rows = kPair ? n >> 1 : n, my_row0 = row0 + (kPair ? (int)rank * my_rows : 0);
         if (kX && P.x_ready && !dry && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
-        const auto kloop = [&](auto box_rows) {
+        const auto kloop = [&](auto box_rows, auto kbs) {
+            constexpr int kKb = decltype(kbs)::value;
             constexpr int kRows = decltype(box_rows)::value;
             constexpr uint32_t kXCopy = (uint32_t)(kRows * kBlockK * 2);
             const CUtensorMap *const map = !kX ? &P.tmB : kRows == 128 ? &P.tmA : kRows == 64 ? &P.tmA64 : &P.tmA32;
             int kx = 0;
-            for (int kb = 0; kb < P.num_kb; ++kb, kx += kBlockK) {
+            for (int kb = 0; kb < P.num_kb; kb += kKb, kx += kBlockK * kKb) {
+                const bool whole = kKb == 1 || kb + kKb <= P.num_kb;
+                const uint32_t n_kb = whole ? (uint32_t)kKb : (uint32_t)(P.num_kb - kb);
                 TL(tl_q = clock64());
                 ok = wait_barrier_1t(empty_bar, phase ^ 1u, ctl, deadline, P.status, (uint32_t)g, 10u);
                 if (!ok) break;
@@ -549,20 +571,26 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
                 // barrier's dependency chain, or the one that arms it could lap the others)
                 if (dry) {
                 } else if (kX) {
-                    if (kb == 0) ctl->tile_n[it & 7] = (uint32_t)n;
-                    if (!kPair) mbar_arrive_expect_tx(full_bar, (uint32_t)C::kWBytes + kXCopy);
+                    if (kb == 0) ctl->tile_n[it & (kMaxStages - 1)] = (uint32_t)n;
+                    if (!kPair) mbar_arrive_expect_tx(full_bar, ((uint32_t)C::kWBytes + kXCopy) * n_kb);
                     else if (rank == 0) mbar_arrive_expect_tx(full_bar, 2u * ((uint32_t)C::kWBytes + kXCopy));
-                    if (MOE_PROBE(kProbeSkipX)) mbar_complete_tx_cluster(mapa_u32(smem_u32(&ctl->full[stage]), kPair ? 0u : cluster_ctarank()), kXCopy);
+                    if (MOE_PROBE(kProbeSkipX)) mbar_complete_tx_cluster(mapa_u32(smem_u32(&ctl->full[stage]), kPair ? 0u : cluster_ctarank()), kXCopy * n_kb);
                     else if (kPair) tma_load_2d_pair(dst, map, full_bar, kx, my_row0);
                     else tma_load_2d(dst, map, full_bar, kx, my_row0);
-                } else if (MOE_PROBE(kProbeSkipAllW2) || (MOE_PROBE(kProbeSkipOddW2) && (kb & 1))) {
-                    mbar_complete_tx_cluster(mapa_u32(smem_u32(&ctl->full[stage]), kPair ? 0u : cluster_ctarank()), (uint32_t)C::kWBytes);
+#pragma unroll
+                    for (int j = 1; j < kKb; ++j)
+                        if ((whole || kb + j < P.num_kb) && !MOE_PROBE(kProbeSkipX)) tma_load_2d(dst + (uint32_t)(j * P.x_rows * kBlockK * 2), map, full_bar, kx + j * kBlockK, my_row0);
+                } else if (MOE_PROBE(kProbeSkipAllW2) || (MOE_PROBE(kProbeSkipOddW2) && (kb / kKb & 1))) {   // (whole stages)
+                    mbar_complete_tx_cluster(mapa_u32(smem_u32(&ctl->full[stage]), kPair ? 0u : cluster_ctarank()), (uint32_t)C::kWBytes * n_kb);
                 } else {
                     if (kPair) tma_load_3d_pair(dst, map, full_bar, kx, n0, e);
                     else tma_load_3d_hint(dst, map, full_bar, kx, n0, e, w_policy);
+#pragma unroll
+                    for (int j = 1; j < kKb; ++j)
+                        if (whole || kb + j < P.num_kb) tma_load_3d_hint(dst + (uint32_t)(j * C::kWBytes), map, full_bar, kx + j * kBlockK, n0, e, w_policy);
                 }
                 armed |= 1u << stage;
-                dst += (uint32_t)C::kStageBytes;
+                dst += stage_bytes;
                 full_bar += 8u;
                 empty_bar += 8u;
                 if (++stage == n_stages) {
@@ -585,9 +613,11 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
                 }
             }
         };
-        if (!kX || my_rows > 64) kloop(std::integral_constant<int, 128>{});
-        else if (kPair || my_rows > 32) kloop(std::integral_constant<int, 64>{});
-        else kloop(std::integral_constant<int, 32>{});
+        const std::integral_constant<int, C::kStageKb> kbs;
+        if (C::kThinKb != C::kStageKb && thin) kloop(std::integral_constant<int, 32>{}, std::integral_constant<int, C::kThinKb>{});
+        else if (!kX || my_rows > 64) kloop(std::integral_constant<int, 128>{}, kbs);
+        else if (kPair || my_rows > 32) kloop(std::integral_constant<int, 64>{}, kbs);
+        else kloop(std::integral_constant<int, 32>{}, kbs);
         if (dry) return;
         t = t_next;
         e = e_next;
@@ -656,10 +686,13 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
     } else if (warp == 1) {
         // ---------------- MMA issuer: the whole warp runs the loop, converged, one elected lane issues; the loop
         // is as short as it can be and its operands are warp-uniform (both for the reasons given in
-        // compute_cta_pair): a whole k-block (four MMAs and the commit) is one statement with 32-bit descriptor
+        // compute_cta_pair): the four MMAs of a k-block (and the commit) are one statement with 32-bit descriptor
         // arithmetic, addresses advance by additions, the barrier's first look is the non-suspending test.
         {
-            constexpr uint32_t kLoStage = (uint32_t)(C::kStageBytes >> 4), kLoX = (uint32_t)(C::kWBytes >> 4);
+            const uint32_t lo_stage = (uint32_t)P.stage_bytes >> 4;
+            constexpr uint32_t kLoW = (uint32_t)(C::kWBytes >> 4);                   // the stage's next k-block
+            const uint32_t lo_x = (uint32_t)(P.x_rows * kBlockK * 2 >> 4);
+            const int all_ksteps = (P.num_kb - 1) * (kBlockK / kUmmaK) + P.last_ksteps;
             constexpr uint32_t kLoBlock = (uint32_t)(kMmaM * kBlockK * 2 >> 4);      // the next 128 rows of W2
             const uint32_t lo0 = smem_desc_lo(smem_u32(ring));
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
@@ -682,42 +715,51 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
                 TL(tl_wt += clock64() - tl_q);
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(a * C::kAccCols);
-                for (int kb = 0; kb < P.num_kb; ++kb) {
-                    TL(tl_q = clock64());
-                    if (!__all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) {
-                        ok = __all_sync(0xffffffffu, wait_barrier_1t(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 21u));
-                        if (!ok) break;
-                    }
-                    TL(tl_wf += clock64() - tl_q; tl_q = clock64());
-                    if (kb == 0) idesc = make_idesc(kMmaM, tile_n(ctl, it));
-                    tc_fence_after();
-                    // advancing K by 16 bf16 = 32 bytes inside the swizzle row: +2 in the address field
-                    if (elect_one_sync()) {
-                        if (kb < P.num_kb - 1 || P.last_ksteps == kBlockK / kUmmaK) {
-                            if (C::kBlocks == 2)
-                                tc_ksteps_bf16(d_tmem + kMmaM, w_lo + kLoBlock, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u);
-                            tc_kblock_bf16(d_tmem, w_lo, w_lo + kLoX, idesc, kb > 0 ? 1u : 0u, empty_bar);
-                        } else {
-                            const uint64_t w_desc = ((uint64_t)kSmemDescHi << 32) | w_lo, x_desc = w_desc + kLoX;
-                            for (int k = 0; k < P.last_ksteps; ++k)
-                                for (int i = 0; i < C::kBlocks; ++i)
-                                    tc_mma_bf16(d_tmem + (uint32_t)(i * kMmaM), w_desc + (uint64_t)(2 * k + i * (int)kLoBlock), x_desc + (uint64_t)(2 * k),
-                                                idesc, (k > 0 || kb > 0) ? 1u : 0u);
-                            tc_commit(empty_bar);   // stage reusable once these MMAs have read it
+                const auto kloop = [&](auto kbs) {
+                    constexpr int kKb = decltype(kbs)::value, kKsteps = kKb * (kBlockK / kUmmaK);
+                    for (int ks = 0; ks < all_ksteps; ks += kKsteps) {
+                        TL(tl_q = clock64());
+                        if (!__all_sync(0xffffffffu, mbar_test_wait(full_bar, phase))) {
+                            ok = __all_sync(0xffffffffu, wait_barrier_1t(full_bar, phase, ctl, deadline, P.status, (uint32_t)g, 21u));
+                            if (!ok) break;
+                        }
+                        TL(tl_wf += clock64() - tl_q; tl_q = clock64());
+                        if (ks == 0) idesc = make_idesc(kMmaM, tile_n(ctl, it));
+                        tc_fence_after();
+                        // advancing K by 16 bf16 = 32 bytes inside the swizzle row: +2 in the address field
+                        if (elect_one_sync()) {
+                            if (ks + kKsteps <= all_ksteps) {
+                                uint32_t wl = w_lo, xl = w_lo + kKb * kLoW, acc = ks > 0 ? 1u : 0u;
+                                if (C::kBlocks == 2) tc_ksteps_bf16(d_tmem + kMmaM, wl + kLoBlock, xl, idesc, acc);
+#pragma unroll
+                                for (int j = 1; j < kKb; ++j, wl += kLoW, xl += lo_x, acc = 1u) tc_ksteps_bf16(d_tmem, wl, xl, idesc, acc);
+                                tc_kblock_bf16(d_tmem, wl, xl, idesc, acc, empty_bar);
+                            } else {
+                                for (int k = 0; k < all_ksteps - ks; ++k) {
+                                    const uint32_t j = (uint32_t)k / (kBlockK / kUmmaK), in_row = 2u * ((uint32_t)k % (kBlockK / kUmmaK));
+                                    const uint64_t w_desc = ((uint64_t)kSmemDescHi << 32) | (w_lo + j * kLoW + in_row),
+                                                   x_desc = ((uint64_t)kSmemDescHi << 32) | (w_lo + kKb * kLoW + j * lo_x + in_row);
+                                    for (int i = 0; i < C::kBlocks; ++i)
+                                        tc_mma_bf16(d_tmem + (uint32_t)(i * kMmaM), w_desc + (uint64_t)(i * (int)kLoBlock), x_desc, idesc, (k > 0 || ks > 0) ? 1u : 0u);
+                                }
+                                tc_commit(empty_bar);   // stage reusable once these MMAs have read it
+                            }
+                        }
+                        TL(tl_is += clock64() - tl_q);
+                        w_lo += lo_stage;
+                        full_bar += 8u;
+                        empty_bar += 8u;
+                        if (++stage == n_stages) {
+                            stage = 0;
+                            phase ^= 1u;
+                            w_lo = lo0;
+                            full_bar = full0;
+                            empty_bar = empty0;
                         }
                     }
-                    TL(tl_is += clock64() - tl_q);
-                    w_lo += kLoStage;
-                    full_bar += 8u;
-                    empty_bar += 8u;
-                    if (++stage == n_stages) {
-                        stage = 0;
-                        phase ^= 1u;
-                        w_lo = lo0;
-                        full_bar = full0;
-                        empty_bar = empty0;
-                    }
-                }
+                };
+                if (C::kThinKb != C::kStageKb && P.x_rows == 32) kloop(std::integral_constant<int, C::kThinKb>{});
+                else kloop(std::integral_constant<int, C::kStageKb>{});
                 __syncwarp();
                 if (ok && elect_one_sync()) tc_commit(smem_u32(&ctl->tmem_full[a]));  // accumulator complete
                 TL(if (it == 0 && lane == 0) tl_put(P, kTlFirstAcc, globaltimer_ns()));
@@ -876,7 +918,7 @@ __device__ __forceinline__ void compute_cta_pair(const FusedParams &P, const Par
                 // full tiles in a loop of their own: with a constant N the issuer needs 27 cycles a k-block less
                 wait_stage();
                 if (!ok) break;
-                const uint32_t n = MOE_PROBE(kProbeFreeRunMma) || dry ? 256u : ctl->tile_n[it & 7];
+                const uint32_t n = MOE_PROBE(kProbeFreeRunMma) || dry ? 256u : ctl->tile_n[it & (kMaxStages - 1)];
                 if (__all_sync(0xffffffffu, n == (uint32_t)TN)) kloop(std::true_type{}, 0u);
                 else kloop(std::false_type{}, __reduce_max_sync(0xffffffffu, n));
                 if (dry) break;
@@ -1651,9 +1693,12 @@ moe_gemm2_combine_pair_kernel(const __grid_constant__ FusedParams P)
 }  // namespace
 
 int fused_co_warps_max() { return kCoWarpsAux; }
-int fused_stages(bool pair, int tile_n, bool aux_free)
+int fused_stages(bool pair, int tile_n, int x_rows, bool aux_free, int *stage_bytes)
 {
-    return pair ? kStageBytesTotal / PairCfg::kStageBytes + (aux_free ? 1 : 0) : tile_n == 64 ? Cfg<64>::kStages : tile_n == 128 ? Cfg<128>::kStages : Cfg<256>::kStages;
+    const int kbs = tile_n == 64 ? (x_rows == 32 ? Cfg<64>::kThinKb : Cfg<64>::kStageKb) : tile_n == 128 ? Cfg<128>::kStageKb : 1;
+    *stage_bytes = pair ? PairCfg::kStageBytes : (tile_n + x_rows) * kBlockK * 2 * kbs;
+    const int n = kStageBytesTotal / *stage_bytes + (pair && aux_free ? 1 : 0);
+    return n < kMaxStages ? n : kMaxStages;
 }
 bool fused_timeline_build() { return MOE_TIMELINE != 0; }
 

@@ -90,7 +90,8 @@ struct alignas(64) FusedParams {
     int32_t dry_rows;                   // rows of a tile as they are to be expected, for the dry round (pair kernel)
     int32_t drain_help;                 // compute CTAs serve communication tiles once their GEMM tiles are done
     int32_t co_warps;                   // co-resident communication warps per compute CTA (0..2)
-    int32_t stages;                     // operand stages of a compute CTA: as many as fit the ring; a pair's has one more where the aux
+    int32_t x_rows;                     // one-CTA tiles: the most rows that an m-tile of the launch can have, rounded up to a copy's 32, 64 or 128
+    int32_t stages, stage_bytes;        // operand stages of a compute CTA: as many as fit the ring; a pair's has one more where the aux
                                         // region of shared memory is free during the GEMM (no co-resident warp)
     int32_t epi_warps;                  // epilogue warps of a compute CTA: 12 (warps 4-15), or 16 (warps 4-19) when no
                                         // co-resident warp is asked for
@@ -262,7 +263,8 @@ size_t fused_smem_bytes(int tile_n);
 cudaError_t fused_occupancy(int tile_n, int *blocks_per_sm);
 cudaError_t fused_launch(int tile_n, const FusedParams &p, int grid, cudaStream_t stream);
 int fused_co_warps_max();
-int fused_stages(bool pair, int tile_n, bool aux_free);   // operand stages of a compute CTA; aux_free: no co-resident warps
+// operand stages of a compute CTA, and their size; x_rows: see FusedParams; aux_free: no co-resident warps
+int fused_stages(bool pair, int tile_n, int x_rows, bool aux_free, int *stage_bytes);
 bool fused_timeline_build();   // the library was compiled with -DMOE_TIMELINE=1   // co-resident communication warps a compute CTA has shared memory for
 // CTA-pair kernel (256 x 256 tiles, clusters of two)
 cudaError_t pair_occupancy(int *blocks_per_sm, int *max_clusters);

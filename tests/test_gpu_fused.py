@@ -311,6 +311,26 @@ def test_shards_are_summed_in_the_accumulator(tile, drain_help):
         B.moe_set_wait_limit_ns(h, 2_000_000_000)
 
 
+@pytest.mark.parametrize("rows", [32, 33, 64, 65])
+@pytest.mark.parametrize("tile_m", [64, 128])
+def test_stages_of_several_k_blocks(rows, tile_m):
+    # a stage has room for 32, 64 or 128 rows and holds one, two or four k-blocks: chains that end in every place of a stage, and in a
+    # k-block; more tiles a CTA than the ring has stages; one expert with all rows.  The order of the sum is the same in all of them.
+    for I in (16, 64, 80, 128, 208, 256, 272, 320, 784, 1040):
+        w = replace(wl.TINY, name="stages", T=rows, H=1096, I=I, E=2, k=1, TP=1, EP=1, L=1, tile_m=tile_m)
+        idx = np.ones((rows, 1), np.int32)
+        wt = np.random.default_rng(3).random((rows, 1)).astype(np.float32) + 0.5
+        x, W2 = wl.make_data(w)
+        expect, _ = _oracle_tokens(w, idx, wt, x, W2)
+        base = None
+        for tile_n in (64, 128, 256):
+            for kw in (dict(), dict(force_C=2, P_override=1)):
+                outs, _, _, _, st = G.run_layer(replace(w, tile_n=tile_n), idx, wt, x, W2, **kw)
+                assert st.code == 0 and np.max(np.abs(outs[0] - expect)) <= G.tolerance(expect), (I, tile_n, kw)
+                base = outs[0] if base is None else base
+                assert np.array_equal(base, outs[0]), (I, tile_n, kw)
+
+
 def test_identity_weights_make_the_combine_exact():
     # W2_e = identity (I = H), small integer activations, power-of-two weights: every partial
     # sum is exactly representable in bf16, so the GPU output must equal the gather exactly
