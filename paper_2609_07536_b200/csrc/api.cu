@@ -46,9 +46,7 @@ static const CUtensorMap *cached_map(moe_handle *h, const void *ptr, int32_t pla
                                      const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, const char *name)
 {
     if (!h->maps && !(h->maps = new (std::nothrow) MapEntry[kMapEntries]())) return nullptr;
-    const uint64_t mixed = ((reinterpret_cast<uintptr_t>(ptr) >> 8) + (uint64_t)box_rows) * 0x9E3779B97F4A7C15ull;
-    MapEntry &m = h->maps[mixed >> 57];
-    static_assert(kMapEntries == 1 << (64 - 57), "the hash's upper bits index the table");
+    MapEntry &m = h->maps[map_place(ptr, box_rows)];
     if (m.ptr == ptr && m.rows == rows && m.cols == cols && m.planes == planes && m.box_rows == box_rows) return &m.map;
     typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                       const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -767,18 +765,19 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.flags = flags_ws + kSplitCounterWords;
 
     // operands (Section II-A): x_routed [R, I] and W2 [E_tot, H, I], k contiguous; a pair CTA loads half the n-tile's rows
+    // (no m-tile has more rows than there are assignments, whatever the routing; a CTA of a pair holds half of them)
+    const int64_t most_rows = R < occ->tile_m ? R : occ->tile_m, cta_rows = pair ? ((most_rows + 31) & ~31ll) / 2 : most_rows;
+    p.x_rows = cta_rows <= 32 && !pair ? 32 : cta_rows <= 64 ? 64 : kMmaM;
     CUtensorMap *const mA[3] = {&p.tmA, &p.tmA64, &p.tmA32};
-    for (int i = 0; i < (pair ? 2 : 3); ++i) {
-        const CUtensorMap *m = operand_map(h, x_routed, 0, R, s->I, 128 >> i, "x_routed");
+    for (int i = 0, first = p.x_rows == kMmaM ? 0 : p.x_rows == 64 ? 1 : 2; i < (pair ? 2 : 3); ++i) {
+        // the boxes that the launch can need; in the place of a wider one a map that it does not use stands for the prefetch of the first
+        const CUtensorMap *m = operand_map(h, x_routed, 0, R, s->I, 128 >> (i < first ? first : i), "x_routed");
         if (!m) return MOE_ERR_CUDA;
         *mA[i] = *m;
     }
     const CUtensorMap *mB = operand_map(h, W2, s->E_tot, s->H, s->I, pair ? TN / 2 : TN, "W2");
     if (!mB) return MOE_ERR_CUDA;
     p.tmB = *mB;
-    // (no m-tile has more rows than there are assignments, whatever the routing)
-    const int64_t most_rows = R < occ->tile_m ? R : occ->tile_m;
-    p.x_rows = most_rows <= 32 ? 32 : most_rows <= 64 ? 64 : kMmaM;
     p.stages = fused_stages(pair, TN, p.x_rows, p.co_warps == 0, &p.stage_bytes);
     const int grid = pair ? ((ctas_c + 1) & ~1) + 2 * ctas_p : ctas_c + ctas_p;
     p.timeline = nullptr;

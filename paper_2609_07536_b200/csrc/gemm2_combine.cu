@@ -552,7 +552,7 @@ __device__ __forceinline__ void producer_role(const FusedParams &P, const Part &
     const int ahead_at = min(2, P.num_kb - 1) / stage_kb * stage_kb;
     for (int g = b; g < total_tiles && ok; g += pt.P, ++it) {
         const int n0 = t.s * P.split_w + t.i_n * TN + (kPair ? (int)rank * (TN / 2) : 0);
-        const int n = mma_n_of<kPair>(kPair ? valid : min(valid, P.x_rows)), my_rows = kPair ? n >> 1 : n, my_row0 = row0 + (kPair ? (int)rank * my_rows : 0);
+        const int n = mma_n_of<kPair>(min(valid, kPair ? 2 * P.x_rows : P.x_rows)), my_rows = kPair ? n >> 1 : n, my_row0 = row0 + (kPair ? (int)rank * my_rows : 0);
         if (kX && P.x_ready && !dry && !(ok = wait_rows(P, row0 + valid - 1, seen, ctl, deadline))) break;
         const auto kloop = [&](auto box_rows, auto kbs) {
             constexpr int kKb = decltype(kbs)::value;

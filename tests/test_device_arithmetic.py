@@ -38,3 +38,16 @@ def test_rows_of_y_beyond_32_bits(tmp_path):
         k, L = rng.randint(1, 32), rng.randint(1, 8)
         rows.append((rng.randrange((1 << 30) // k), rng.randrange(L), 128 * rng.randint(0, 60), L, 8 * rng.randint(1, 4000), k))
     assert _run(exe, rows) == [((t * L + s) * w + c) * k for t, s, c, L, w, k in rows]
+
+
+def test_places_of_the_operand_maps(tmp_path):
+    # one launch's maps, and those of buffers a power of two of bytes apart, never share a place (they would be encoded on every call)
+    exe = _compiled(tmp_path, '    unsigned long long p; int b;\n    while (scanf("%llu %d", &p, &b) == 2)\n'
+                              '        printf("%u\\n", moe::map_place(reinterpret_cast<const void *>(p), b));\n    return 0;')
+    rng = random.Random(2)
+    boxes, pairs = (32, 64, 96, 128, 256), [(0x7f0000000000 + 256 * rng.randrange(1 << 28), 1 << j) for j in range(8, 35) for _ in range(4)]
+    got = _run(exe, [(q, b) for p, d in pairs for q in (p, p + d) for b in boxes])
+    assert all(0 <= v < 128 for v in got)
+    for i in range(len(pairs)):
+        one, other = got[10 * i:10 * i + 5], got[10 * i + 5:10 * i + 10]
+        assert len(set(one)) == 5 and not set(one[:4]) & set(other[:4]), (hex(pairs[i][0]), pairs[i][1])
