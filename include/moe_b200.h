@@ -242,7 +242,7 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n,
 int32_t moe_select_tile(moe_handle *h, const moe_shape *shape, int32_t *tile_m, int32_t *tile_n);
 
 /* Sizes of the caller-allocated workspaces [bytes]: routing arrays, the tile-padded GEMM2
- * output Y (bf16, token-major: [T][L][k_tot][ceil(H/L)], with room for TP times as much), readiness flags + split counters +
+ * output Y (bf16, token-major: [T][L][k_tot][ceil(H/L)]), readiness flags + split counters +
  * work queues (must be zero-filled once before first use and not shared between handles), status
  * (16 bytes). */
 int32_t moe_workspace_bytes(const moe_shape *shape, int32_t tile_m, int32_t tile_n,

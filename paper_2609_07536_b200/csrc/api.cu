@@ -350,12 +350,13 @@ int32_t moe_workspace_bytes(const moe_shape *s, int32_t tile_m, int32_t tile_n, 
         b += align16((size_t)n_routing_warps(s) * E * 4); // per-warp histograms
         *routing_bytes = b + 16;
     }
-    if (y_bytes)   // token-major: [T][L][k_tot * TP][ceil(H/L)]
-        *y_bytes = align16((size_t)s->T * s->L * s->k_tot * s->TP * (size_t)ceil_div(s->H, s->L) * 2) + 16;
+    // (the sum over the K-shards is taken in the accumulators: neither depends on TP)
+    if (y_bytes)   // token-major: [T][L][k_tot][ceil(H/L)]
+        *y_bytes = align16((size_t)s->T * s->L * s->k_tot * (size_t)ceil_div(s->H, s->L) * 2) + 16;
     if (flags_bytes) {
         const size_t nts = (size_t)ceil_div(ceil_div(s->H, s->L), tile_n);
         const size_t parts = (tile_m == 256) ? 2 : 1;   // a pair tile is published in two parts
-        *flags_bytes = ((size_t)kSplitCounterWords + (size_t)s->L * s->TP * mt * nts * parts) * 4 + 16;
+        *flags_bytes = ((size_t)kSplitCounterWords + (size_t)s->L * mt * nts * parts) * 4 + 16;
     }
     if (status_bytes) *status_bytes = 16;
     return MOE_OK;

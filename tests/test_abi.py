@@ -89,6 +89,15 @@ def test_workspace_sizes_and_argument_errors():
     assert B.moe_host_arena_bytes(s, 64, 64) > rb + yb + fb
 
 
+def test_workspace_holds_one_row_per_assignment_whatever_tp_is():
+    # the sum over the K-shards is taken in the accumulator: no kernel writes a row of Y or a flag per shard
+    for tile_m, tile_n in ((64, 64), (128, 256), (256, 256)):
+        one = B.moe_workspace_bytes(B.make_shape(777, 2048, 1408, 66, 8, 1, 2, 2), tile_m, tile_n)
+        assert one[1] == 777 * 8 * 2048 * 2 + 16                # every column of every assignment, and the alignment's slack
+        for TP in (2, 4, 8):
+            assert B.moe_workspace_bytes(B.make_shape(777, 2048, 1408, 66, 8, TP, 2, 2), tile_m, tile_n) == one
+
+
 def test_header_is_plain_c():
     # the boundary is a C ABI: the header has to compile as C99 on its own (no C++-isms, no torch types)
     import shutil
