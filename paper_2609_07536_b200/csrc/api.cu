@@ -287,8 +287,6 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n, moe_o
         else if (tile_n == 256) rho->rho_ref = 3.04;
         else if (tile_n == 128) rho->rho_ref = 3.46;
         else rho->rho_ref = 3.46 * 2.0;          // 64-wide tiles: Eq. 14 tile-area scaling from 128x128
-        if (tile_m == 64) rho->rho_ref *= 1.0;     // a 64-row tile still occupies a 128-row MMA: same wave time
-        if (tile_n == 64) { rho->tile_n_ref = 64; }
         rho->D_ref = 2;
         rho->rows_ref = 8 * 2 + 1;
         rho->comm_cols_ref = 1024;
@@ -680,9 +678,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     }
     p.drain_help = (mode == MOE_MODE_FUSED && plan->drain_help) ? 1 : 0;
     p.tok_blk = (int32_t)ceil_div(s->T, s->EP);
-    p.token_shift = 30u;                                     // exact below 2^30: token_mul exceeds the quotient by less than k_tot / 2^shift
-    while ((1u << (p.token_shift - 30u)) < (uint32_t)s->k_tot) ++p.token_shift;
-    p.token_mul = (uint32_t)(((1ull << p.token_shift) + (uint32_t)s->k_tot - 1) / (uint32_t)s->k_tot);
+    p.by_k = divisor_of(s->k_tot);
     p.comm_cols = (int32_t)ceil_div(p.split_w, kCommTileN);
     p.num_kb = (int32_t)ceil_div(s->I, kBlockK);
     p.last_ksteps = (s->I - (p.num_kb - 1) * kBlockK) / kUmmaK;

@@ -192,8 +192,6 @@ __device__ __forceinline__ void sync_compute_warps(const FusedParams &P)
 {
     asm volatile("bar.sync 1, %0;" ::"r"(kThreads + 32 * (P.epi_warps - 12)) : "memory");
 }
-// token of flat assignment f (< 2^30): the quotient by k_tot, exact (token_mul = ceil(2^token_shift / k_tot))
-__device__ __forceinline__ int token_of(const FusedParams &P, int f) { return (int)((unsigned long long)(uint32_t)f * P.token_mul >> P.token_shift); }
 // N of a tile's MMAs: its rows, rounded up to what the instruction takes (M = 128: 16, M = 256 over a pair: 32)
 template <bool kPair>
 __device__ __forceinline__ int mma_n_of(int valid) { return kPair ? (valid + 31) & ~31 : (valid + 15) & ~15; }
@@ -388,7 +386,7 @@ __device__ __forceinline__ void epilogue_role(const FusedParams &P, const Part &
             cols[i] = min(min(P.H, (t.s + 1) * P.split_w) - t.s * P.split_w, t.i_n * TN + TN) - cis;
             dst[i] = nullptr;
             if (!dry && f[i] >= 0 && cols[i] > 0) {
-                const int tok = token_of(P, f[i]), q = f[i] - tok * P.k_tot;
+                const int tok = quotient(P.by_k, f[i]), q = f[i] - tok * P.k_tot;
                 const int slab = cis >> P.slab_shift, wslab = min(P.slab_cols, P.split_w - (slab << P.slab_shift));
                 dst[i] = Y + y_unit(tok, t.s, slab << P.slab_shift, P.L, P.split_w, P.k_tot) + (uint32_t)(q * wslab + (cis & (P.slab_cols - 1)));
             }
@@ -794,7 +792,7 @@ __device__ void compute_cta(const FusedParams &P, const Part &pt, uint8_t *ring,
 //   full[stage]       only the leader's is used: armed by the leader for the bytes of both CTAs
 //   empty[stage]      one per CTA (its producer waits on it), signalled by the leader's commit
 //   tmem_full[a]      one per CTA (its epilogue waits on it), signalled by the leader's commit
-//   tmem_empty[a]     only the leader's is used: 12 local + 12 remote epilogue warps arrive
+//   tmem_empty[a]     only the leader's is used: the epilogue warps of both CTAs arrive, 16 each (12 beside co-resident warps)
 
 // Barriers (thread 0) and TMEM (warp 1) of a CTA of a pair, before it is known that the pair computes; the cluster barrier behind it
 // makes the peer's barriers exist before anything arrives on them.

@@ -18,7 +18,7 @@ constexpr int kCoWarpsMax = 4;         // co-resident communication warps a comp
 constexpr int kFusedThreads = kThreads + 32 * kCoWarpsMax;   // block size of the fused kernel
 constexpr int kBlockK = 64;            // bf16 elements per k-block: one 128-byte swizzle row
 constexpr int kUmmaK = 16;             // K of one tcgen05.mma.kind::f16 instruction
-constexpr int kMmaM = 128;             // M of the MMA (tile_m = 64 stores the first 64 rows only)
+constexpr int kMmaM = 128;             // M of a one-CTA MMA: output columns (a pair's: twice that); also the rows of a one-CTA tile
 constexpr int kStageBytesTotal = 192 * 1024;  // operand ring, all stages together
 constexpr int kCommTileM = 32;         // T_M^comm: the piece in which the selector counts communication work (a CTA's units are 8 KB)
 constexpr int kCommTileN = 1024;       // T_N^comm
@@ -45,7 +45,7 @@ struct InlineRouting {
 };
 constexpr int kInlineMaxR = 2048;      // assignments up to which a kernel builds the routing itself: four rows of 32 per warp of 16 warps
 
-// Parameters of one fused launch.  Passed by value (__grid_constant__): the two tensor maps
+// Parameters of one fused launch.  Passed by value (__grid_constant__): the tensor maps
 // must sit in kernel parameter space, 64-byte aligned.
 struct alignas(64) FusedParams {
     CUtensorMap tmA, tmA64, tmA32;   // x_routed [R, I]   boxes 64 x 128, 64 and (one-CTA tiles) 32 rows, 128B swizzle
@@ -80,7 +80,7 @@ struct alignas(64) FusedParams {
     int32_t c_table_first, c_table_n;   // c_table[i]: communication CTAs when S = c_table_first + i (0 entries: C and P above hold)
     uint8_t c_table[kPlanTableMax];
     int32_t tok_blk, comm_cols;
-    uint32_t token_mul, token_shift;    // see token_of
+    Divisor by_k;                       // k_tot: flat assignment -> token
     int32_t even;                       // the communication work is dealt evenly to all warps once all tiles are done (no per-tile
                                         // flags, no queue)
     int32_t balance;                    // (even) P counts all compute slots; the kernel divides them by whole waves of its tiles
@@ -271,10 +271,10 @@ const CUtensorMap *gate_up_map(moe_handle *h, const void *ptr, int32_t experts, 
 size_t fused_smem_bytes(int tile_n);
 cudaError_t fused_occupancy(int tile_n, int *blocks_per_sm);
 cudaError_t fused_launch(int tile_n, const FusedParams &p, int grid, cudaStream_t stream);
-int fused_co_warps_max();
+int fused_co_warps_max();      // co-resident communication warps a compute CTA has shared memory for
 // operand stages of a compute CTA, and their size; x_rows: see FusedParams; aux_free: no co-resident warps
 int fused_stages(bool pair, int tile_n, int x_rows, bool aux_free, int *stage_bytes);
-bool fused_timeline_build();   // the library was compiled with -DMOE_TIMELINE=1   // co-resident communication warps a compute CTA has shared memory for
+bool fused_timeline_build();   // the library was compiled with -DMOE_TIMELINE=1
 // CTA-pair kernel (256 x 256 tiles, clusters of two)
 cudaError_t pair_occupancy(int *blocks_per_sm, int *max_clusters);
 cudaError_t pair_launch(const FusedParams &p, int grid, cudaStream_t stream);

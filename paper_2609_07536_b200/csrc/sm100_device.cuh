@@ -71,13 +71,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         ::"r"(dst), "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y, int z)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z)
-        : "memory");
-}
 // L2 priorities of the copies below: lines that are read once are marked evict-first, so that a stream of such reads does not
 // push out what is used again
 __device__ __forceinline__ unsigned long long l2_evict_first_policy()
@@ -106,15 +99,7 @@ __device__ __forceinline__ void tma_load_5d_hint(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(u), "r"(v), "l"(pol)
         : "memory");
 }
-// untiled bulk copy global -> shared; both addresses 16-byte aligned, size a multiple of 16
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-        ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-        : "memory");
-}
-// the same copy with an L2 priority
+// untiled bulk copy global -> shared, with an L2 priority; both addresses 16-byte aligned, size a multiple of 16
 __device__ __forceinline__ void bulk_load_once(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar, unsigned long long pol)
 {
     asm volatile(
@@ -297,6 +282,9 @@ __device__ __forceinline__ bool elect_one_sync()
 // the MMAs is on the critical path of the tensor pipe (the pipe buffers hardly any MMA ahead), so the
 // descriptors are kept as their low words (start address field and the constant leading offset) and
 // glued to the constant high word here instead of being rebuilt with 64-bit arithmetic per MMA.
+// The descriptor: a K-major, 128B-swizzled operand tile whose rows are 128 bytes (64 bf16); 8-row groups are 1024 bytes apart (stride
+// byte offset, bits [32,46)), the leading byte offset (bits [16,30)) is unused for swizzled K-major layouts, the start address (in units
+// of 16 bytes) has bits [0,14), the descriptor version (1) bits [46,48), the layout type (2) bits [61,64).
 constexpr uint32_t kSmemDescHi = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);   // stride offset, version, SWIZZLE_128B
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t smem_addr) { return ((smem_addr & 0x3FFFFu) >> 4) | (1u << 16); }
 __device__ __forceinline__ void tc_kblock_bf16_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate,
@@ -411,17 +399,6 @@ __device__ __forceinline__ uint32_t transpose_8x8(uint32_t x)
     asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
     return y;
 }
-// 32 lanes x 16 columns: thread i reads TMEM lane (base lane + i)
-__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
 // The wait for a tcgen05.ld, naming the registers it fills: the compiler then cannot move a use
 // of them above the wait (it sees only opaque asm statements, not the asynchronous write).
 __device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16])
@@ -443,16 +420,6 @@ __device__ __forceinline__ uint4 lds_v4(uint32_t addr)
 {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ void sts_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ float lds_f32(uint32_t addr)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
     return v;
 }
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p)
@@ -483,19 +450,6 @@ __device__ __forceinline__ void red_relaxed_add_u32(uint32_t *p, uint32_t v)
     asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Shared-memory matrix descriptor of a K-major, 128B-swizzled operand tile whose rows are
-// 128 bytes (64 bf16): 8-row groups are 1024 bytes apart (stride byte offset), the leading
-// byte offset is unused for swizzled K-major layouts, descriptor version 1, layout type 2.
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);        // start address, bits [0,14)
-    d |= (uint64_t)1 << 16;                               // leading byte offset (ignored), bits [16,30)
-    d |= (uint64_t)(1024 >> 4) << 32;                     // stride byte offset, bits [32,46)
-    d |= (uint64_t)1 << 46;                               // descriptor version, bits [46,48)
-    d |= (uint64_t)2 << 61;                               // SWIZZLE_128B, bits [61,64)
-    return d;
-}
 // Instruction descriptor, kind::f16: D fp32, A and B bf16, both K-major, M x N.
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N)
 {
