@@ -37,7 +37,7 @@ class Workload:
     E: int                 # routed experts
     k: int                 # routed experts per token
     n_shared: int = 0      # always-active shared experts
-    TP: int = 1            # emulated tensor-parallel shards (split-K partials)
+    TP: int = 1            # emulated tensor-parallel shards (K-shards of I / TP columns, summed in the accumulator)
     EP: int = 1            # emulated destination ranks (output buffers)
     tile_m: int = 128
     tile_n: int = 128

@@ -197,8 +197,8 @@ def test_co_resident_communication_warps_change_nothing_but_time():
     dict(T=777, E=5, k=2, H=1536, I=512, TP=2, EP=3, tile_m=128, tile_n=256, L=4),   # partial n-tile at the split end
     dict(T=1030, E=70, k=2, H=512, I=256, TP=2, EP=8, tile_m=128, tile_n=128, L=8),  # empty experts, L = 8
     dict(T=200, E=6, k=2, n_shared=2, H=256, I=128, TP=1, EP=1, tile_m=128, tile_n=64, L=2),  # shared experts
-    dict(T=900, E=9, k=4, H=1024, I=256, TP=4, EP=2, tile_m=256, tile_n=256, L=2),    # pair tiles, 16-row units
-    dict(T=333, E=12, k=3, H=264, I=80, tile_m=64, tile_n=64, EP=4, L=1),             # no room for them: dropped
+    dict(T=900, E=9, k=4, H=1024, I=256, TP=4, EP=2, tile_m=256, tile_n=256, L=2),    # pair tiles, four K-shards
+    dict(T=333, E=12, k=3, H=264, I=80, tile_m=64, tile_n=64, EP=4, L=1),             # a split width that is no multiple of 16
 ], ids=lambda kw: "-".join(f"{k}{v}" for k, v in kw.items()))
 def test_co_resident_warps_edge_shapes(kw):
     base = dict(name="co_edge", routing_seed=5, data_seed=6, TP=1, EP=1, L=1)
@@ -206,6 +206,36 @@ def test_co_resident_warps_edge_shapes(kw):
     w = replace(wl.TINY, **base)
     _check_against_oracle(w, drain_help=1, co_warps=2)
     _check_against_oracle(w, drain_help=1, co_warps=1, force_C=3)
+
+
+@pytest.mark.parametrize("k", [15, 16, 17, 32])
+@pytest.mark.parametrize("tile", [(64, 64), (128, 256), (256, 256)], ids=str)
+def test_units_of_many_rows(k, tile):
+    # a unit has k_tot rows: up to 16 for a co-resident warp (its slots for weights; above, the launch runs without them), slabs of 512
+    # columns at 8 rows, 256 at 15 and 16, 128 at 17 and more; a split width that is a multiple of 8 and of nothing larger.
+    # Even shares, the static map, the queue beside co-resident warps and without dedicated communication CTAs: the same bits.
+    w = replace(wl.TINY, name="rows", T=150, H=528, I=80, E=40, k=k, TP=1, EP=3, L=2, tile_m=tile[0], tile_n=tile[1], routing="zipf",
+                zipf_s=1.0, routing_seed=40 + k, data_seed=7)
+    idx, wt, _ = wl.make_routing(w)
+    x, W2 = wl.make_data(w)
+    base, _ = _check_against_oracle(w, drain_help=1)
+    own = [len(G.tokens_of_rank(w.T, w.EP, d)) for d in range(w.EP)]
+    all_slots = 148 // (2 if tile[0] == 256 else 1)
+    for kw in (dict(drain_help=0, force_C=5), dict(drain_help=1, co_warps=1), dict(drain_help=1, co_warps=2, force_C=3),
+               dict(drain_help=1, co_warps=2, force_C=1, C_override=0, P_override=all_slots)):
+        outs, _, _, _, st = G.run_layer(w, idx, wt, x, W2, **kw)
+        assert st.code == 0
+        for d, n in enumerate(own):
+            assert np.array_equal(base[d][:n], outs[d][:n]), (kw, d)
+
+
+def test_units_of_32_rows_from_the_queue():
+    # more units than are dealt evenly (32 a warp of 148 CTAs), 32 rows each, in slabs of 128 columns with a remainder of 8
+    w = replace(wl.TINY, name="rowsq", T=5800, H=1040, I=16, E=40, k=32, TP=1, EP=2, L=2, tile_m=256, tile_n=256, routing_seed=41,
+                data_seed=8)
+    assert w.T * w.L * 5 > 32 * 12 * 148
+    _check_against_oracle(w, n_random=48, drain_help=1)
+    _check_against_oracle(replace(w, tile_m=128), n_random=48, drain_help=1)
 
 
 def test_dsv2lite_with_co_resident_warps_sampled():
@@ -710,7 +740,7 @@ def test_the_selection_of_the_whole_step_call_is_the_selector_s(kw, limits):
     dict(T=1, E=9, k=3, H=208, I=80),                        # one wave of 64-column tiles, the last one partial
     dict(T=1, E=40, k=8, H=1536, I=512, TP=2),               # one wave, tiles of the plan's CTAs filled by bound
     dict(T=33, E=2, k=2, H=256, I=64, L=8, EP=8),            # 32-column splits, ranks without a token
-    dict(T=70, E=12, k=9, H=264, I=64, TP=2),                # 18 rows per unit, 16-byte stores, ragged width
+    dict(T=70, E=12, k=9, H=264, I=64, TP=2),                # 9 rows per unit, 16-byte stores, ragged width
     dict(T=300, E=5, k=2, H=512, I=128, tile_m=64),          # 33, 64 and more rows in a 64-row tile: boxes of 32 rows
     dict(T=600, E=3, k=2, H=1024, I=192, tile_m=256, L=2),   # CTA pairs
 ], ids=str)
