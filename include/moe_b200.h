@@ -60,8 +60,8 @@ enum { MOE_MODE_FUSED = 0, MOE_MODE_GEMM_ONLY = 1, MOE_MODE_COMBINE_ONLY = 2 };
 /* MOE_RHO_PAPER: Eq. 14 as printed (K, tile area and D/D_ref terms).
  * MOE_RHO_LOCAL: the re-derivation Section III-E asks of a new kernel family, for ranks
  * emulated inside one GPU: no ring term D/D_ref; a communication tile costs in proportion
- * to the rows it moves per token (k_tot * TP read + 1 written) and to its real width
- * min(T_N^comm, ceil(H/L)). */
+ * to the rows per token (k_tot * TP read + 1 written, a row per K-shard as the count of compute
+ * tiles has them; the launch reads k_tot) and to its real width min(T_N^comm, ceil(H/L)). */
 enum { MOE_RHO_PAPER = 0, MOE_RHO_LOCAL = 1 };
 enum { MOE_DEP_SPLIT = 0, MOE_DEP_TILE = 1 };
 #define MOE_MAX_EP 8
@@ -237,7 +237,7 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n,
  * kernel; the resource manager then reads that kernel's tile shape and residency).  Chooses the GEMM tile
  * family for `shape`: the widest n-tile the split width ceil(H/L) holds (256, 128 or 64), and 256-row
  * CTA-pair tiles when the experts hold at least 192 routed rows on average (T * k_tot / E_tot), 128-row
- * single-CTA tiles below (small and decode-sized token counts: less row padding, every SM its own tile).
+ * single-CTA tiles below (small and decode-sized token counts: every SM its own tile).
  * The result is a valid (tile_m, tile_n) for every other call.  [host] */
 int32_t moe_select_tile(moe_handle *h, const moe_shape *shape, int32_t *tile_m, int32_t *tile_n);
 

@@ -280,6 +280,11 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n, moe_o
         // share of the SMs at C = 32: time per communication wave (of 32-row tiles: the work is dealt out in units, so
         // that whole 128-row tiles per CTA would make the selector see waves that are not there) / time per compute wave.
         //   128x256: 19.7 us / 6.47 us ; 256x256 (CTA pair): 19.5 / 4.68 ; 128x128: 18.8 / 5.43
+        // That was with a tile and a row of Y per K-shard, which the selector still counts (g = TP; k_tot * TP + 1 rows).  The launch has
+        // tiles over all of I and k_tot + 1 rows whatever TP is; the same run on it: 10.0 / 5.56 ; 10.4 / 4.18 ; 10.4 / 3.12 for half
+        // of a tile, that is 1.80, 2.50 and 3.35.  No constant is right for every TP, as the rows of the count grow with it.  Static
+        // partition, 162 workloads of the DeepSeek shape, mean distance from the best C at TP = 1 / 2: these constants 2.9 / 1.8 %,
+        // the ones measured now 4.8 / 1.9 %, the same restated for TP = 1 (9 rows, K = 1408) 1.7 / 2.4 %; with drain help 1.9 to 2.4 % for all.
         rho->K_ref = 704;
         rho->tile_m_ref = tile_m;
         rho->tile_n_ref = tile_n;
@@ -314,15 +319,17 @@ int32_t moe_select_tile(moe_handle *h, const moe_shape *s, int32_t *tile_m, int3
     if (!h || !s || !tile_m || !tile_n) return MOE_ERR_NULL;
     if (!shape_ok(s)) return MOE_ERR_SHAPE;
     // Conventional kernel dispatch (Section III-E: it runs before the resource manager and hands it the tile
-    // shape and residency of the kernel it chose).  Widest n-tile the split holds; rows: the 256-row CTA-pair
-    // tile moves a third less operand traffic per FLOP but pads every expert's last tile to 256 rows and needs
-    // two co-scheduled SMs, so it pays once an expert fills most of one such tile on average.  Measured, whole fused step and
-    // whole layer, 128 x 256 against 256 x 256, us, at 128 / 192 / 256 / 512 rows per expert:
-    //   Granite shape  step 53/54  59/59  67/65  93/89    layer  80/87   99/90  105/103  143/142
-    //   Qwen shape     step 117/115  143/129  170/146  273/237    layer  232/251  309/282  368/337  587/565
-    //   DeepSeek shape step 136/135  149/145  195/177  357/319    layer  267/312  322/330  418/400  789/779
-    // From 192 on the pair is at most 3 % behind for a layer (DeepSeek shape, 192 and 224), up to 10 % ahead; at 160 and below
-    // 128-row tiles are at most 4 % behind for a step, up to a quarter ahead for a layer.
+    // shape and residency of the kernel it chose).  Widest n-tile the split holds; rows: a tile costs the rows that it has, rounded
+    // up to 16 (a pair's: 32), in both families.  The 256-row CTA-pair tile moves a third less operand traffic per FLOP, and an
+    // expert of 129 to 256 rows is one tile that reads its weights once, not two; it needs two co-scheduled SMs, so that there are half as
+    // many places for tiles.  Measured, whole fused step and whole layer, 128 x 256 against 256 x 256, us, skewed routing, at
+    // 64 / 128 / 160 / 192 / 256 / 400 rows per expert:
+    //   Granite shape  step 40/39  44/42  45/44  49/44  52/48  64/56   layer  77/78  82/82  87/85  100/85  102/88  122/114
+    //   Qwen shape     step 88/95  98/99  111/104  120/108  139/118  178/157   layer  208/215  234/234  258/241  286/255  336/299  453/420
+    //   DeepSeek shape step 95/103  110/112  122/117  126/120  152/132  190/157   layer  234/244  258/269  287/277  308/293  371/325  490/428
+    // From 192 on the pair is ahead by 5 to 17 % in all of them, up to 128 rows 128-row tiles are, by up to 8 % (Granite shape: equal).
+    // Between 129 and 191 the pair is ahead at these shapes too, by 2 to 16 %, once most experts have more than 128 rows; not where
+    // experts are so few that their 128-row tiles fit one wave on narrow columns, and the line has not been drawn between the two.
     const int64_t split_w = ceil_div(s->H, s->L);
     const int32_t tn = split_w >= 256 ? 256 : split_w >= 128 ? 128 : 64;
     const int64_t rows_per_expert = (int64_t)s->T * s->k_tot / s->E_tot;
@@ -494,9 +501,14 @@ int slab_shift_of(const moe_shape *s)
 }
 // Who serves what when the compute CTAs help: a queue per split, or, up to 32 units (of 8 KB) a warp, an even share for every
 // warp once the tiles are done.  Hardly any token is complete before the last tiles are, so the queue's early start is
-// worth little, while its atomics and its polling cost microseconds at the end (whole launch, queue -> even: DeepSeek shape
-// T = 16 67 -> 58 us, 256 92 -> 76, 2048 149 -> 142; Granite shape T = 1003 40 -> 30, 4096 120 -> 107; Qwen shape T = 8192 240 ->
-// 233); with more units the queue's balance wins (DeepSeek shape T = 16384, 74 units: 804 -> 815, 37 units: 719 -> 745).
+// worth little, while its atomics and its polling cost microseconds at the end; with many units the queue's balance wins.  Whole
+// step, queue / even, us, timed in turns, at 8 / 16 / 24 / 32 / 40 / 48 / 64 units a warp:
+//   Granite shape, L = 1   102/91  165/152  228/217  294/286  357/353  425/421  564/567 (T = 4736 to 37888)
+//   Qwen shape, L = 1      187/170  321/288  467/429  612/574  760/716  905/866  1194/1167 (T = 7104 to 56832)
+//   DeepSeek shape, L = 1  178/172  297/292  427/421  560/564  699/716  838/860  1137/1175 (T = 3552 to 28416)
+//   DeepSeek shape, L = 2  183/175  307/294  435/424  569/565  717/724  848/861  1139/1157
+// The lines lie between 26 and 56 units; up to 32 the even shares are at most 1 % behind, above it up to 6 % ahead (Qwen shape) or 3 %
+// behind (DeepSeek shape).
 bool few_units(const moe_handle *h, const moe_shape *s)
 {
     const int64_t split_w = ceil_div(s->H, s->L);

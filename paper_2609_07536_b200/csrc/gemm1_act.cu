@@ -583,7 +583,7 @@ int32_t moe::launch_gemm1_act(moe_handle *h, const void *hidden, const void *W1,
     const bool pair = tile_m == 256;
     // Narrow tiles where every one that this routing can have then still finds an SM of its own: the time of the only wave is the
     // time to stream one tile's weights (Granite shape, T = 2, 64 columns: 14.6 -> 12.7 us; DeepSeek shape, T = 1, 96 columns: 20.4
-    // -> 18.8).  With more tiles than SMs the wide ones are faster at every size: a k-block costs ~300 cycles whatever its width.
+    // -> 18.8).  With more tiles than SMs the wide ones are faster at every size (64 columns: +1 to +8 % over a layer).
     int TN = kG1TileN;
     if (!pair) {
         const int64_t R = (int64_t)s->T * s->k_tot, used = R < s->E_tot ? R : s->E_tot, bound = (R - used) / tile_m + used;
