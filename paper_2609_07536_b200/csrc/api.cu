@@ -267,9 +267,9 @@ int32_t moe_query_occupancy(moe_handle *h, int32_t tile_m, int32_t tile_n, moe_o
         // Lower end of the co-resident family's legal set (one-time sweep).  One-CTA tiles: below 24 compute waves
         // co-resident warps lost 2-5 % (T = 1024: 19 waves; T = 2048: 37).  CTA-pair tiles: a co-resident warp takes
         // the shared memory of the seventh operand stage.  In a loop of equal steps w = 0 is the fastest at every size
-        // (w = 0 / 1 / 2, 20 steps: T = 8192 425 / 433 / 429 us, 16384 783 / 802 / 793, 32768 1516 / 1541 / 1521; 400 steps, where
-        // the power cap sets the clock: 496 / 503 / 502, 902 / 914 / 911, 1718 / 1743 / 1743); only between launches of other
-        // candidates (the sweep) was w = 2 ahead, by up to 3 % from T = 16384 on.  The family is not offered (a forced w is
+        // (w = 0 / 1 / 2, 20 steps: T = 8192 346 / 362 / 357 us, 16384 663 / 681 / 672, 32768 1296 / 1326 / 1310; 400 steps, where
+        // the power cap sets the clock: 386 / 412 / 405, 733 / 769 / 744, 1477 / 1536 / 1519); only between launches of other
+        // candidates (the sweep) was w = 2 ahead, by 7 to 9 % from T = 16384 on.  The family is not offered (a forced w is
         // still honoured).
         limits->co_min_waves = (tile_m == 256) ? INT32_MAX : 24;
     }
