@@ -368,12 +368,14 @@ def launched_division(w, lim, plan, S):
     while slab > 8 and w.k_tot * slab * 2 > 8192:
         slab //= 2
     units = w.T * w.L * -(-split_w // slab)
-    if not lim.drain_help or lim.force_comm_ctas > 0 or lim.selector_off or plan.co_warps or units > 32 * 12 * lim.G:
+    used = min(w.R, w.E_tot)
+    S_max = (w.R - used) // w.tile_m + used
+    waves_most = -(-S_max * w.L * -(-split_w // w.tile_n) // ((lim.G - min(lim.C_co_max, lim.C_max)) // slot))
+    by_plan = plan.co_warps and (lim.force_co_warps >= 0 or waves_most >= lim.co_min_waves)
+    if not lim.drain_help or lim.force_comm_ctas > 0 or lim.selector_off or by_plan or units > 32 * 12 * lim.G:
         return {"comm_ctas": plan.comm_ctas, "P": plan.P, "by": "plan"}
     slots, tn = lim.G // slot, w.tile_n
     if slot == 1:
-        used = min(w.R, w.E_tot)
-        S_max = (w.R - used) // w.tile_m + used
         tn = next((n for n in (64, 128, 256) if n <= w.tile_n and S_max * w.L * -(-split_w // n) <= slots), w.tile_n)
     tiles = S * w.L * -(-split_w // tn)
     waves = max(1, -(-tiles // slots))

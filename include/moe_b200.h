@@ -363,8 +363,9 @@ int32_t moe_clear_status(moe_handle *h, uint32_t *status_dev, void *stream);
  * the words (bounded: it gives up with MOE_ERR_CUDA when the stream finishes or fails without them, or
  * after the handle's wait limit plus two seconds), copies the counts to tile_counts_pinned and plans.
  * Where the combine is dealt out evenly after the GEMM (drain help, up to 32 units of 8 KB per warp), limits ask for no
- * particular C and no co-resident warp can be picked, the kernel divides its CTAs by whole waves of the tiles it counts on the
- * device, whatever the selection: it is launched at once, at every batch size from the first call on, and the host waits and
+ * particular C and the tiles that the launch can have are too few waves for co-resident warps (co_min_waves; at TP > 1 the selector
+ * counts TP times as many, and plan_out may name co-resident warps that the launch does without), the kernel divides its CTAs by
+ * whole waves of the tiles it counts on the device, whatever the selection: it is launched at once, at every batch size from the first call on, and the host waits and
  * plans beside it; plan_out holds the selector's pick (the division launched: waves = ceil(tiles / slots), with
  * ceil(tiles / waves) of the slots computing).  Other launches need the pick.  The selector sees the counts through their sum S
  * alone: the first two calls with a shape and limits wait for the counts, the second tabulates the picks for every S that a

@@ -518,21 +518,23 @@ bool few_units(const moe_handle *h, const moe_shape *s)
 // Whether a whole-step launch with these limits divides its CTAs by itself whatever the counts turn out to be (even shares, no C
 // asked for, no co-resident warps): such a launch needs no selection, and goes out before the counts are on the host, at a
 // batch size that was never seen before as well (32 sizes in turn, 15 us a step as with repeated ones; 52 when the picks for all
-// counts had to be tabulated first).
+// counts had to be tabulated first).  The tiles are those of the launch, over all of I: counted per K-shard, as the selector does, the same
+// launch at TP = 2 took co-resident warps, the queue, or the wait for the counts that it does without at TP = 1 (whole step, TP = 1 / 2, us: H = 4096,
+// otherwise the DeepSeek shape, L = 2, T = 1200 196 / 203, T = 1500 215 / 226; the DeepSeek shape on 128 x 128 tiles, T = 1024 110 / 117, T = 2048 158 / 169).
 bool divides_itself(const moe_handle *h, const moe_shape *s, const moe_occupancy *occ, const moe_sm_limits *lim)
 {
     if (!lim->drain_help || lim->force_comm_ctas > 0 || lim->selector_off || lim->C_max < 1 || s->T < 1 || !few_units(h, s)) return false;
     const int slot = occ->comp_slot_sms;
     if (occ->o_comp != 1 || occ->o_comm != 1 || lim->G <= slot || lim->G > (slot == 2 ? 2 * h->max_pairs : h->G)) return false;   // (else: what the launch says to the plan)
     const int64_t NTs = ceil_div(ceil_div(s->H, s->L), occ->tile_n);
-    if ((int64_t)s->TP * max_mtiles_of(s, occ->tile_m) * NTs * s->L >= (int64_t)1 << 30) return false;     // (too many tiles: the wait knows better)
+    if ((int64_t)max_mtiles_of(s, occ->tile_m) * NTs * s->L >= (int64_t)1 << 30) return false;     // (too many tiles: the wait knows better)
     const int32_t w_top = lim->force_co_warps >= 0 && lim->force_co_warps < lim->co_warps_max ? lim->force_co_warps : lim->co_warps_max;
     if (w_top < 1) return true;
     if (lim->force_co_warps >= 0) return false;
     // the selector tries co-resident warps from co_min_waves waves on, with C up to C_co_max
     const int32_t C_most = lim->C_co_max < lim->C_max ? lim->C_co_max : lim->C_max;
     if (C_most < 1) return true;
-    const int64_t P_least = (lim->G - C_most) / slot, tiles = (int64_t)s->L * s->TP * most_mtiles(s, occ->tile_m) * NTs;
+    const int64_t P_least = (lim->G - C_most) / slot, tiles = (int64_t)s->L * most_mtiles(s, occ->tile_m) * NTs;
     return P_least >= 1 && ceil_div(tiles, P_least) < lim->co_min_waves;
 }
 
@@ -668,7 +670,7 @@ int32_t launch_gemm2_combine(moe_handle *h, const void *x_routed, const void *W2
     p.split_w = (int32_t)ceil_div(s->H, s->L);
     p.NTs = (int32_t)ceil_div(p.split_w, occ->tile_n);
     const int64_t Wc = (int64_t)n_mtiles * p.NTs;
-    if (Wc * s->TP * s->L * 2 >= (int64_t)1 << 31) return MOE_ERR_SHAPE;
+    if (Wc * s->TP * s->L * 2 >= (int64_t)1 << 31) return MOE_ERR_SHAPE;   // (the plan's count, a tile per K-shard)
     p.W_comp = (int32_t)Wc;
     p.S_dev = counts_on_device ? r->tiles + s->E_tot : nullptr;
     p.C = C; p.P = Pc; p.mode = mode;
@@ -803,7 +805,8 @@ struct Selection {
     moe_occupancy occ;
     moe_sm_limits lim;
     moe_rho rho;
-    bool divides;          // divides_itself, with the counts on the host wanted
+    bool alone;            // divides_itself
+    bool divides;          // ... with the counts on the host wanted
     PlanTable *table;      // else, with the counts on the host wanted: plan_table
     // whether the fused launch goes out before the counts are on the host
     bool launch_first() const { return divides || (table && table->n > 0); }
@@ -816,7 +819,8 @@ int32_t selection_of(moe_handle *h, const moe_shape *s, int32_t tile_m, int32_t 
     if (rc != MOE_OK) return rc;
     if (limits_or_null) sel->lim = *limits_or_null;
     const bool mailed = host_counts && h->mail_dev;
-    sel->divides = mailed && divides_itself(h, s, &sel->occ, &sel->lim);
+    sel->alone = divides_itself(h, s, &sel->occ, &sel->lim);
+    sel->divides = mailed && sel->alone;
     sel->table = mailed && !sel->divides ? plan_table(h, s, &sel->occ, &sel->lim) : nullptr;
     return MOE_OK;
 }
@@ -858,7 +862,9 @@ int32_t select_and_launch(moe_handle *h, const void *x_routed, const void *W2, c
     }
     if (ev_before) cudaEventRecord(static_cast<cudaEvent_t>(ev_before), st);
     const bool own_division = sel.lim.force_comm_ctas <= 0 && !sel.lim.selector_off;
-    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &plan, own_division, table, first ? mail_seq : 0u, topk_idx, feed, out, y_ws,
+    moe_plan launched = plan;
+    if (sel.alone) launched.co_warps = 0;               // (the selector counts a tile per K-shard, and may have found waves enough for them)
+    rc = launch_gemm2_combine(h, x_routed, W2, topk_w, s, &sel.occ, routing, n_mtiles, &launched, own_division, table, first ? mail_seq : 0u, topk_idx, feed, out, y_ws,
                               flags_ws, status_dev, st);
     if (ev_after) cudaEventRecord(static_cast<cudaEvent_t>(ev_after), st);
     if (rc == MOE_OK && first) rc = counts_and_plan();

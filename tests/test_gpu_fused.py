@@ -899,6 +899,31 @@ def test_tabulated_selection_from_the_first_call_to_the_third(kw, limits):
     B.moe_destroy(h)
 
 
+@pytest.mark.parametrize("on_device", [False, True], ids=["counts_on_host", "counts_on_device"])
+def test_a_whole_step_divides_its_ctas_by_the_tiles_it_launches(on_device):
+    # a tile runs over all of I whatever TP is: at TP = 2 the selector counts twice the tiles (and finds waves enough for co-resident warps), the
+    # launch is that of TP = 1, dealt evenly.  Even shares raise no tile flags, every other launch of the dynamic mode does.
+    h = G.handle()
+    w = replace(wl.TINY, name="alone", T=900, E=24, k=4, H=2048, I=256, EP=2, L=2, tile_m=64, tile_n=64)
+    idx, wt, _ = wl.make_routing(w)
+    x, W2 = wl.make_data(w)
+    xd, Wd, idx_d, wt_d = x.cuda(), W2.cuda(), torch.from_numpy(idx).cuda(), torch.from_numpy(wt).cuda()
+    outs = []
+    for TP in (1, 2):
+        ws = B.alloc_workspace(G.shape_of(replace(w, TP=TP)), w.tile_m, w.tile_n)
+        for _ in range(3):      # the first call, the second (tabulates where the launch waits for the counts) and one after it
+            plan = B.moe_layer(h, xd, Wd, idx_d, wt_d, ws, counts_on_device=on_device)
+        torch.cuda.synchronize()
+        assert B.moe_get_status(h, ws.status).code == 0
+        assert plan.co_warps == 0 if TP == 1 else plan.co_warps > 0      # the plan that comes back is the selector's
+        words = ws.flags_ws[:ws.flags_ws.numel() // 4 * 4].view(torch.int32)
+        assert int(words[64:].abs().max()) == 0, TP                     # behind the split counters and the queues: the tiles' flags
+        outs.append([o.float().cpu().numpy() for o in ws.out])
+        B.moe_release_workspace(h, ws.flags_ws)
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("k,n_shared", [(3, 0), (2, 2), (9, 0)])       # Q = 3, 4, 9 rows a unit: short of a multiple of four or eight, and not
 def test_an_infinity_stays_one_on_every_route(k, n_shared):
     # a partial result over the bf16 range: its token's column is infinite (not NaN) whether the units are dealt evenly, drawn from
